@@ -300,6 +300,33 @@ int reflex_partitioned_attention(reflex_cache_t *cache, int layer, const void *q
 int reflex_flow_step(void *x, const void *v, void *x_lowp, int B, int T, int A, int k, int K,
                      int dtype, void *stream);
 
+/* A whole denoising step of the action expert (Sec. 2.1, Sec. 3.1-3.3), one host call: the gates of all 2L + 1 norms, the input
+ * projection of the action chunk, L layers of (norm + Q/K/V, partitioned attention, output projection + residual, norm +
+ * SwiGLU, down projection + residual), the velocity head behind the last norm and the Euler update of the chunk:
+ *   h = W_in a;   per layer  h += W_O Attention(W_QKV AdaRMSNorm(h; gamma_2l));  h += W_D SwiGLU(W_GU AdaRMSNorm(h; gamma_2l+1))
+ *   vel = W_out AdaRMSNorm(h; gamma_2L);   a <- a - vel / K
+ * The same results as the single calls in that order (reflex_adarmsnorm_gate, reflex_linear_residual, ...), to rounding.
+ * Nothing inside the step writes weights or cache regions, so its kernels may ask for them ahead of their turn; the first kernel
+ * waits for everything ahead of it on the stream. No other work on the device may write the weights or the cache regions that
+ * are being read while a step runs (reflex_cache_stage_static, which writes the idle bank, may).
+ * All tensors device, dense, 16-byte aligned, in the cache's dtype unless said otherwise; L, B, Hq, Hkv, d are the cache's. */
+typedef struct {
+    int32_t T, D, F, A, Cd, Hd;           /* tokens per stream, model / SwiGLU / action / conditioning / gate-MLP widths */
+    float eps;
+    int32_t reserved;
+    const void *W_in, *W_out;             /* [D][A], [A][D]                                                     */
+    const void *Wqkv, *Wo, *Wgu, *Wd;     /* stacked over layers: [L][(Hq+2Hkv)d][D], [L][D][Hq d], [L][2F][D], [L][D][F] */
+    const void *W1, *b1, *W2, *b2;        /* gate MLPs of the 2L + 1 norms, as reflex_adarmsnorm_gate takes them  */
+    float *gates;                         /* fp32 [(2L+1) B (D + Hd)]                                             */
+    void *h, *y;                          /* [B][T][D]: residual stream (out: its last state); scratch for normalised rows  */
+    void *q, *k, *v, *o;                  /* scratch [B][T][Hq][d], [B][T][Hkv][d] x 2, [B][T][Hq][d]             */
+    void *m;                              /* scratch [B][T][F]                                                    */
+    void *vel, *a_lowp;                   /* [B][T][A]: velocity (out); scratch                                   */
+    float *row_sums;                      /* fp32 scratch, 2 * B * T * ceil(D / 32) floats                        */
+} reflex_expert;
+/* a  fp32 [B][T][A], updated in place;  cond [B][Cd];  k, K as in reflex_flow_step. Errors as the single calls. */
+int reflex_expert_step(reflex_cache_t *cache, const reflex_expert *expert, float *a, const void *cond, int k, int K, void *stream);
+
 /* ---- Sec. 3.4 "Stream Throughput: Asynchronous Pipeline", Algorithm 1 (future-conditional overlap scheduling), Eq. 3 ----
  * Host logic only; no device work. A control loop calls reflex_overlap_tick once per control period:
  *   - the event names the action to execute (chunk index, position in the chunk; Algorithm 1 line 5);

@@ -28,9 +28,16 @@ EXPORTS = [
     "reflex_cache_set_attention_impl", "reflex_cache_check_status", "reflex_cache_selftest_wait_limit", "reflex_cache_init_static", "reflex_cache_stage_static",
     "reflex_cache_commit_static", "reflex_cache_append_sliding",
     "reflex_adarmsnorm", "reflex_adarmsnorm_gate", "reflex_adarmsnorm_noalloc", "reflex_adarmsnorm_qkv", "reflex_adarmsnorm_swiglu", "reflex_linear_residual", "reflex_partitioned_attention",
-    "reflex_flow_step", "reflex_overlap_create", "reflex_overlap_destroy", "reflex_overlap_tick", "reflex_overlap_inference_done",
+    "reflex_flow_step", "reflex_expert_step", "reflex_overlap_create", "reflex_overlap_destroy", "reflex_overlap_tick", "reflex_overlap_inference_done",
     "reflex_overlap_simulate",
 ]
+
+
+class ExpertDesc(ctypes.Structure):
+    """struct reflex_expert: the tensors of a whole expert step."""
+    _fields_ = ([(n, ctypes.c_int32) for n in ("T", "D", "F", "A", "Cd", "Hd")] + [("eps", ctypes.c_float), ("reserved", ctypes.c_int32)] +
+                [(n, ctypes.c_void_p) for n in ("W_in", "W_out", "Wqkv", "Wo", "Wgu", "Wd", "W1", "b1", "W2", "b2", "gates", "h", "y", "q", "k", "v", "o", "m",
+                                                "vel", "a_lowp", "row_sums")])
 
 
 class OverlapEvent(ctypes.Structure):
@@ -91,6 +98,7 @@ def load():
     lib.reflex_linear_residual.argtypes = [vp, vp, vp, vp, vp, i, i, i, i, i, vp]
     lib.reflex_partitioned_attention.argtypes = [vp, i, vp, vp, vp, vp, i, f, i, vp]
     lib.reflex_flow_step.argtypes = [vp, vp, vp, i, i, i, i, i, i, vp]
+    lib.reflex_expert_step.argtypes = [vp, ctypes.POINTER(ExpertDesc), vp, vp, i, i, vp]
     dbl = ctypes.c_double
     lib.reflex_overlap_create.argtypes = [i, dbl, dbl, ctypes.POINTER(vp)]
     lib.reflex_overlap_destroy.argtypes = [vp]
@@ -307,6 +315,12 @@ def reflex_flow_step(x, v, x_lowp, k, K, stream=None):
     B, T, A = x.shape
     _check(load().reflex_flow_step(_ptr(x), _ptr(v), _ptr(x_lowp), B, T, A, int(k), int(K), dtype_code(v), _stream(stream)))
     return x
+
+
+def reflex_expert_step(cache: Cache, desc: ExpertDesc, a, cond, k, K, stream=None):
+    """One whole expert step on the fp32 chunk a [B][T][A] (in place); desc holds the pointers of weights and buffers."""
+    _check(load().reflex_expert_step(cache.handle, ctypes.byref(desc), _ptr(a), _ptr(cond), int(k), int(K), _stream(stream)))
+    return a
 
 
 # ---- prepared calls: arguments marshalled once, then replayed with ~1 us of host overhead per call ----

@@ -2,7 +2,7 @@
 
     python -m paper_2607_14695_b200.build [--force] [--verbose]
 
-Extra compiler flags (debug builds with in-kernel timelines: -DREFLEX_TRACE, -DREFLEX_QK_TRACE, -DREFLEX_LIN_TRACE) can be
+Extra compiler flags (debug builds with in-kernel timelines: -DREFLEX_TRACE, -DREFLEX_QK_TRACE, -DREFLEX_LIN_TRACE, -DREFLEX_CG_TRACE) can be
 given in the environment variable REFLEX_NVCC_FLAGS.
 """
 from __future__ import annotations

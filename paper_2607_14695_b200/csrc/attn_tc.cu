@@ -562,27 +562,27 @@ EncodeTiledFn encode_fn()
     return fn;
 }
 
-// rank-3 map over rows of [rows][Hkv][d] bf16, box = 64 rows x 1 head x 64 elements, 128-byte swizzle
-bool make_kv_map(CUtensorMap *m, const void *ptr, uint64_t rows, int Hkv, int d)
+// rank-3 map over rows of [rows][Hkv][d] bf16, box = box_rows rows x 1 head x 64 elements, 128-byte swizzle
+bool make_kv_map(CUtensorMap *m, const void *ptr, uint64_t rows, int Hkv, int d, int box_rows = kBN)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)Hkv, rows};
     cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)Hkv * d * 2};
-    cuuint32_t box[3] = {64, 1, (cuuint32_t)kBN};
+    cuuint32_t box[3] = {64, 1, (cuuint32_t)box_rows};
     cuuint32_t es[3] = {1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(ptr), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// rank-4 map over q [B][T][Hq][d], box = (64 elements, G heads, 128/G tokens, 1 stream): rows land as (token, head)
-bool make_q_map(CUtensorMap *m, const void *ptr, int B, int T, int Hq, int d, int G)
+// rank-4 map over q [B][T][Hq][d], box = (64 elements, heads, tokens, 1 stream): rows land as (token, head)
+bool make_q_map(CUtensorMap *m, const void *ptr, int B, int T, int Hq, int d, int heads, int tokens)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)Hq, (cuuint64_t)T, (cuuint64_t)B};
     cuuint64_t strides[3] = {(cuuint64_t)d * 2, (cuuint64_t)Hq * d * 2, (cuuint64_t)T * Hq * d * 2};
-    cuuint32_t box[4] = {64, (cuuint32_t)G, (cuuint32_t)(kBM / G), 1};
+    cuuint32_t box[4] = {64, (cuuint32_t)heads, (cuuint32_t)tokens, 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(ptr), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -605,6 +605,12 @@ struct MapCache {
         *out = m;
         return true;
     }
+    bool put(const CUtensorMap *m, const void *ptr, int kind, int a, int b, int c, int d)
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        maps[std::make_tuple(ptr, kind, a, b, c, d)] = *m;
+        return true;
+    }
 };
 
 MapCache &cache() { static MapCache c; return c; }
@@ -612,7 +618,7 @@ MapCache &cache() { static MapCache c; return c; }
 bool mk_slab(CUtensorMap *m, const void *ptr, int rows, int Hkv, int d, int) { return make_kv_map(m, ptr, (uint64_t)rows, Hkv, d); }
 bool mk_q(CUtensorMap *m, const void *ptr, int BT /*B<<16|T not used*/, int Hq, int d, int G)
 {
-    return make_q_map(m, ptr, BT >> 16, BT & 0xFFFF, Hq, d, G);
+    return make_q_map(m, ptr, BT >> 16, BT & 0xFFFF, Hq, d, G, kBM / G);
 }
 
 template <int HD>
@@ -717,6 +723,19 @@ bool tensor_map_2d_bf16(CUtensorMap *out, const void *ptr, int inner, int rows, 
         return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(p_), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     });
+}
+
+bool tensor_map_kv_bf16(CUtensorMap *out, const void *ptr, int rows, int Hkv, int d, int box_rows)
+{
+    return cache().get(out, ptr, 4, rows, Hkv, d, box_rows, [](CUtensorMap *m, const void *p_, int rows_, int Hkv_, int d_, int box_) -> bool {
+        return make_kv_map(m, p_, (uint64_t)rows_, Hkv_, d_, box_);
+    });
+}
+
+bool tensor_map_q_bf16(CUtensorMap *out, const void *ptr, int B, int T, int Hq, int d, int heads, int tokens)
+{
+    return cache().get(out, ptr, 5 | heads << 8, B << 16 | T, Hq, d, tokens, [](CUtensorMap *, const void *, int, int, int, int) -> bool { return false; }) ||
+           (make_q_map(out, ptr, B, T, Hq, d, heads, tokens) && cache().put(out, ptr, 5 | heads << 8, B << 16 | T, Hq, d, tokens));
 }
 
 bool tc_supported(const AttnParams &p)

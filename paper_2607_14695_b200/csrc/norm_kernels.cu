@@ -522,6 +522,15 @@ __global__ void flow_step_kernel(float *__restrict__ x, const T *__restrict__ v,
 }
 
 template <typename T>
+__global__ void cast_kernel(const float *__restrict__ x, T *__restrict__ y, size_t n)
+{
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        if constexpr (sizeof(T) == 2) y[i] = __float2bfloat16_rn(x[i]);
+        else y[i] = x[i];
+    }
+}
+
+template <typename T>
 static cudaError_t launch_gate_wide_t(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, float *gate_buf, int L, int B,
                                       int D, int Cd, int Hd, cudaStream_t st)
 {
@@ -563,6 +572,15 @@ cudaError_t launch_flow_step(float *x, const void *v, void *x_lowp, size_t n, fl
         flow_step_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(x, (const __nv_bfloat16 *)v, (__nv_bfloat16 *)x_lowp, n, dt);
     else
         flow_step_kernel<float><<<blocks, 256, 0, st>>>(x, (const float *)v, (float *)x_lowp, n, dt);
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cast(const float *x, void *y, size_t n, int dtype, cudaStream_t st)
+{
+    const unsigned blocks = (unsigned)((n + 255) / 256 < 592 ? (n + 255) / 256 : 592);
+    if (dtype == REFLEX_DTYPE_BF16) cast_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(x, (__nv_bfloat16 *)y, n);
+    else cast_kernel<float><<<blocks, 256, 0, st>>>(x, (float *)y, n);
     count_launch();
     return cudaGetLastError();
 }

@@ -7,6 +7,7 @@
 #include <new>
 #include <vector>
 
+#include "chain.cuh"
 #include "reflex_internal.cuh"
 
 using namespace reflex;
@@ -451,8 +452,8 @@ int reflex_linear_residual(reflex_cache_t *c, const void *a, const void *W, cons
     return REFLEX_OK;
 }
 
-int reflex_partitioned_attention(reflex_cache_t *c, int layer, const void *q, const void *k_dyn, const void *v_dyn,
-                                 void *out, int T, float scale, int dyn_mask, void *stream)
+static int attention(reflex_cache_t *c, int layer, const void *q, const void *k_dyn, const void *v_dyn, void *out, int T, float scale, int dyn_mask,
+                     bool early, const ChainPrefetch *pf, void *stream)
 {
     if (!c) return fail(REFLEX_ERR_INVALID_ARG, "cache is NULL");
     const reflex_cache_desc &d = c->desc;
@@ -485,6 +486,8 @@ int reflex_partitioned_attention(reflex_cache_t *c, int layer, const void *q, co
     if (c->attn_impl == REFLEX_ATTN_SIMT || !tc_ok) {
         p.nsplit = simt_choose_splits(p, c->lay.partial_bytes, c->sm_count);
         e = launch_attention_simt(p, (cudaStream_t)stream);
+    } else if (c->attn_impl == REFLEX_ATTN_AUTO && chain_attn_supported(p, c->sm_count)) {
+        e = launch_chain_attn(p, status, early, pf, (cudaStream_t)stream);
     } else {
         // Batched shapes take the two-CTA kernel (with a key split when the streams alone do not fill the SM pairs);
         // a single stream or a few take one CTA per query tile with a finer key split.
@@ -495,6 +498,12 @@ int reflex_partitioned_attention(reflex_cache_t *c, int layer, const void *q, co
     }
     if (e != cudaSuccess) return cuda_fail(e, "attention launch");
     return REFLEX_OK;
+}
+
+int reflex_partitioned_attention(reflex_cache_t *c, int layer, const void *q, const void *k_dyn, const void *v_dyn,
+                                 void *out, int T, float scale, int dyn_mask, void *stream)
+{
+    return attention(c, layer, q, k_dyn, v_dyn, out, T, scale, dyn_mask, false, nullptr, stream);
 }
 
 int reflex_flow_step(void *x, const void *v, void *x_lowp, int B, int T, int A, int k, int K, int dtype, void *stream)
@@ -508,6 +517,118 @@ int reflex_flow_step(void *x, const void *v, void *x_lowp, int B, int T, int A, 
     cudaError_t e = launch_flow_step((float *)x, v, x_lowp, (size_t)B * T * A, dt, dtype, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "flow_step launch");
     return REFLEX_OK;
+}
+
+// The step's projections through the chained kernels (chain_gemm.cu): every projection's shape has a tile choice that fits the SMs at once.
+static bool expert_chained(const reflex_cache_desc &d, const reflex_expert &e)
+{
+    const int M = d.B * e.T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
+    if (d.dtype != REFLEX_DTYPE_BF16 || e.D % 64 != 0 || !(e.A == 8 || e.A == 16 || e.A == 32)) return false;
+    return chain_proj_supported(CG_QKV, M, e.D, nq + 2 * nk) && chain_proj_supported(CG_RES, M, nq, e.D) && chain_proj_supported(CG_SWIGLU, M, e.D, e.F) &&
+           chain_proj_supported(CG_RES, M, e.F, e.D) && chain_proj_supported(CG_OUT, M, e.D, e.A);
+}
+
+static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float *a, float dt, void *stream)
+{
+    const reflex_cache_desc &d = c->desc;
+    typedef __nv_bfloat16 bf;
+    const int L = d.L, B = d.B, T = e.T, D = e.D, M = B * T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
+    cudaStream_t st = (cudaStream_t)stream;
+    // partial sums of squares of the residual rows: two areas, so that a projection never writes the one its predecessor reads
+    float *ss[2] = {e.row_sums, e.row_sums + (size_t)M * ((D + 31) / 32)};
+    auto gate = [&](int i) { return (const float *)e.gates + (size_t)i * B * D; };
+    // what a later kernel of the step reads is asked into the L2 one or two kernels ahead, so that the 34 MB of a layer come from
+    // memory while the chain is busy with latencies
+    auto range = [](ChainPrefetch &pf, int i, const void *base, size_t first, size_t n) {
+        pf.ptr[i] = (const char *)base + first * 2; pf.bytes[i] = n * 2 & ~(size_t)15;
+    };
+    const size_t kv_layer = (size_t)B * (ring_off(d) + d.N) * d.Hkv * d.d;
+    cudaError_t err = launch_chain_in(a, (const bf *)e.W_in, gate(0), (bf *)e.h, (bf *)e.y, ss[0], B, T, D, e.A, st);
+    if (err != cudaSuccess) return cuda_fail(err, "expert input projection launch");
+    int slots = 1;
+    for (int l = 0; l < L; ++l) {
+        ChainProj p = {};
+        p.B = B; p.R = T; p.D = D; p.eps = e.eps; p.status = (uint32_t *)(c->ws + c->lay.status_off);
+        ChainProj qkv = p;
+        qkv.mode = CG_QKV; qkv.x = (const bf *)e.y; qkv.W = (const bf *)e.Wqkv; qkv.w_rows = L * (nq + 2 * nk); qkv.w_row0 = l * (nq + 2 * nk);
+        qkv.K = D; qkv.N = nq + 2 * nk; qkv.ss_in = ss[0]; qkv.slots_in = slots; qkv.q = (bf *)e.q; qkv.k = (bf *)e.k; qkv.v = (bf *)e.v; qkv.nq = nq; qkv.nk = nk;
+        range(qkv.pf, 0, e.Wo, (size_t)l * D * nq, (size_t)D * nq);
+        err = launch_chain_proj(qkv, st);
+        if (err != cudaSuccess) return cuda_fail(err, "expert q/k/v projection launch");
+        ChainPrefetch apf = {};
+        range(apf, 0, e.Wgu, (size_t)l * 2 * e.F * D, (size_t)2 * e.F * D);
+        const int rc = attention(c, l, e.q, e.k, e.v, e.o, T, 0.f, 0, true, &apf, stream);
+        if (rc != REFLEX_OK) return rc;
+        ChainProj o = p;
+        o.mode = CG_RES; o.x = (const bf *)e.o; o.W = (const bf *)e.Wo; o.w_rows = L * D; o.w_row0 = l * D; o.K = nq; o.N = D; o.res = (const bf *)e.h;
+        o.h = (bf *)e.h; o.xg = (bf *)e.y; o.gate = gate(2 * l + 1); o.ss_out = ss[1];
+        range(o.pf, 0, e.Wd, (size_t)l * D * e.F, (size_t)D * e.F);
+        err = launch_chain_proj(o, st);
+        if (err != cudaSuccess) return cuda_fail(err, "expert output projection launch");
+        ChainProj gu = p;
+        gu.mode = CG_SWIGLU; gu.x = (const bf *)e.y; gu.W = (const bf *)e.Wgu; gu.w_rows = L * 2 * e.F; gu.w_row0 = l * 2 * e.F; gu.K = D; gu.N = e.F;
+        gu.h = (bf *)e.m; gu.ss_in = ss[1]; gu.slots_in = (D + 31) / 32;
+        if (l + 1 < L) {
+            range(gu.pf, 0, c->k_slab, (size_t)(l + 1) * kv_layer, kv_layer);
+            range(gu.pf, 1, c->v_slab, (size_t)(l + 1) * kv_layer, kv_layer);
+            range(gu.pf, 2, e.Wqkv, (size_t)(l + 1) * (nq + 2 * nk) * D, (size_t)(nq + 2 * nk) * D);
+        }
+        err = launch_chain_proj(gu, st);
+        if (err != cudaSuccess) return cuda_fail(err, "expert gate/up projection launch");
+        ChainProj dn = p;
+        dn.mode = CG_RES; dn.x = (const bf *)e.m; dn.W = (const bf *)e.Wd; dn.w_rows = L * D; dn.w_row0 = l * D; dn.K = e.F; dn.N = D; dn.res = (const bf *)e.h;
+        dn.h = (bf *)e.h; dn.xg = (bf *)e.y; dn.gate = gate(2 * l + 2); dn.ss_out = ss[0];
+        err = launch_chain_proj(dn, st);
+        if (err != cudaSuccess) return cuda_fail(err, "expert down projection launch");
+        slots = (D + 31) / 32;
+    }
+    ChainProj out = {};
+    out.mode = CG_OUT; out.B = B; out.R = T; out.D = D; out.eps = e.eps; out.status = (uint32_t *)(c->ws + c->lay.status_off);
+    out.x = (const bf *)e.y; out.W = (const bf *)e.W_out; out.w_rows = e.A; out.w_row0 = 0; out.K = D; out.N = e.A; out.h = (bf *)e.vel; out.ss_in = ss[0];
+    out.slots_in = slots; out.a = a; out.dt = dt;
+    err = launch_chain_proj(out, st);
+    if (err != cudaSuccess) return cuda_fail(err, "expert velocity head launch");
+    return REFLEX_OK;
+}
+
+int reflex_expert_step(reflex_cache_t *c, const reflex_expert *ep, float *a, const void *cond, int k, int K, void *stream)
+{
+    if (!c || !ep || !a || !cond) return fail(REFLEX_ERR_INVALID_ARG, "NULL argument");
+    const reflex_cache_desc &d = c->desc;
+    const reflex_expert &e = *ep;
+    const void *ptrs[] = {a, cond, e.W_in, e.W_out, e.Wqkv, e.Wo, e.Wgu, e.Wd, e.W1, e.b1, e.W2, e.b2, e.gates, e.h, e.y, e.q, e.k, e.v, e.o, e.m, e.vel, e.a_lowp, e.row_sums};
+    for (const void *p : ptrs) {
+        if (!p) return fail(REFLEX_ERR_INVALID_ARG, "NULL tensor of the expert");
+        if (!aligned16(p)) return fail(REFLEX_ERR_ALIGN, "a tensor of the expert is not 16-byte aligned");
+    }
+    if (K < 1 || k < 0 || k >= K) return fail(REFLEX_ERR_INVALID_ARG, "step k=%d outside [0, K=%d)", k, K);
+    if (e.T < 1 || e.T > d.T_max) return fail(REFLEX_ERR_SHAPE, "T=%d outside [1, T_max=%d]", e.T, d.T_max);
+    if (e.A < 1) return fail(REFLEX_ERR_SHAPE, "A=%d must be >= 1", e.A);
+    if (!(e.eps >= 0.f)) return fail(REFLEX_ERR_INVALID_ARG, "eps must be >= 0");
+    for (int b = 0; b < d.B; ++b)
+        if (c->static_len[b] < 0) return fail(REFLEX_ERR_STATE, "stream %d: static prefix never initialised (reflex_cache_init_static, S = 0 allowed)", b);
+    const int L = d.L, B = d.B, T = e.T, D = e.D, M = B * T, nq = d.Hq * d.d, nk = d.Hkv * d.d, dt_ = d.dtype;
+    int rc = reflex_adarmsnorm_gate(cond, e.W1, e.b1, e.W2, e.b2, e.gates, 2 * L + 1, B, D, e.Cd, e.Hd, dt_, stream);
+    if (rc != REFLEX_OK) return rc;
+    if (expert_chained(d, e)) return expert_step_chained(c, e, a, -1.0f / (float)K, stream);
+    // any other dtype or shape: the single calls in order
+    const size_t es = elem_size(dt_);
+    auto off = [&](const void *p, size_t elems) -> const void * { return (const char *)p + elems * es; };
+    auto gate = [&](int i) { return (const float *)e.gates + (size_t)i * B * D; };
+    cudaError_t err = launch_cast(a, e.a_lowp, (size_t)M * e.A, dt_, (cudaStream_t)stream);
+    if (err != cudaSuccess) return cuda_fail(err, "action chunk cast launch");
+    rc = reflex_linear_residual(c, e.a_lowp, e.W_in, nullptr, e.h, M, e.A, D, dt_, 0, stream);
+    for (int l = 0; l < L && rc == REFLEX_OK; ++l) {
+        rc = reflex_adarmsnorm_qkv(c, e.h, gate(2 * l), off(e.Wqkv, (size_t)l * (nq + 2 * nk) * D), e.q, e.k, e.v, B, T, D, d.Hq, d.Hkv, d.d, e.eps, dt_, 0, stream);
+        if (rc == REFLEX_OK) rc = reflex_partitioned_attention(c, l, e.q, e.k, e.v, e.o, T, 0.f, 0, stream);
+        if (rc == REFLEX_OK) rc = reflex_linear_residual(c, e.o, off(e.Wo, (size_t)l * D * nq), e.h, e.h, M, nq, D, dt_, 0, stream);
+        if (rc == REFLEX_OK) rc = reflex_adarmsnorm_swiglu(c, e.h, gate(2 * l + 1), off(e.Wgu, (size_t)l * 2 * e.F * D), e.m, B, T, D, e.F, e.eps, dt_, 0, stream);
+        if (rc == REFLEX_OK) rc = reflex_linear_residual(c, e.m, off(e.Wd, (size_t)l * D * e.F), e.h, e.h, M, e.F, D, dt_, 0, stream);
+    }
+    if (rc == REFLEX_OK) rc = reflex_adarmsnorm(e.h, e.y, nullptr, nullptr, nullptr, nullptr, nullptr, (float *)gate(2 * L), B, T, D, 0, 0, e.eps, dt_, stream);
+    if (rc == REFLEX_OK) rc = reflex_linear_residual(c, e.y, e.W_out, nullptr, e.vel, M, D, e.A, dt_, 0, stream);
+    if (rc == REFLEX_OK) rc = reflex_flow_step(a, e.vel, nullptr, B, T, e.A, k, K, dt_, stream);
+    return rc;
 }
 
 }  // extern "C"

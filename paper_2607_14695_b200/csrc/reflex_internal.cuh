@@ -105,16 +105,24 @@ cudaError_t launch_adarmsnorm(const void *x, void *y, const void *cond, const vo
                               cudaStream_t st);
 cudaError_t launch_adarmsnorm_gate(const void *cond, const void *W1, const void *b1, const void *W2, const void *b2, float *gate_buf,
                                    int L, int B, int D, int Cd, int Hd, int dtype, cudaStream_t st);
+cudaError_t launch_cast(const float *x, void *y, size_t n, int dtype, cudaStream_t st);   // y = x rounded to dtype
 cudaError_t launch_flow_step(float *x, const void *v, void *x_lowp, size_t n, float dt, int dtype, cudaStream_t st);
 cudaError_t launch_attention_simt(const AttnParams &p, cudaStream_t st);
 int simt_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count);
 cudaError_t launch_attention_merge(const AttnParams &p, cudaStream_t st);  // combines nsplit (m, l, acc) partials
 bool tc_supported(const AttnParams &p);
 bool tensor_map_2d_bf16(CUtensorMap *out, const void *ptr, int inner, int rows, int box_rows);
+bool tensor_map_kv_bf16(CUtensorMap *out, const void *ptr, int rows, int Hkv, int d, int box_rows);   // [rows][Hkv][d], box = box_rows x 1 head x 64
+bool tensor_map_q_bf16(CUtensorMap *out, const void *ptr, int B, int T, int Hq, int d, int heads, int tokens);   // [B][T][Hq][d], box = tokens x heads x 64
 int tc_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count);
 bool tc2_supported(const AttnParams &p);
 int tc2_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count);
 cudaError_t launch_attention_tc(const AttnParams &p, uint32_t *status, bool two_cta, int sm_count, cudaStream_t st);
+// one or two streams (chain_attn.cu): one head and an eighth of the keys per CTA, merged inside clusters of eight. early: the caller
+// vouches that the cached regions are not written by work that may still be running
+bool chain_attn_supported(const AttnParams &p, int sm_count);
+struct ChainPrefetch;
+cudaError_t launch_chain_attn(const AttnParams &p, uint32_t *status, bool early, const ChainPrefetch *pf, cudaStream_t st);
 // gate MLP of AdaRMSNorm on tcgen05 (bf16): false when the shapes or the driver do not allow it (the caller falls back)
 // adaptive norm + packed Q/K/V projection (qkv_tc.cu). impl: 0 = tensor cores where supported, 1 = plain kernel,
 // 2 = tensor cores with 256-column tiles only

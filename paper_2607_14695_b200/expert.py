@@ -40,6 +40,7 @@ class ActionExpert:
         self.m = e(B, T, F)
         self.vel = e(B, T, w.A)
         self.a_lowp = e(B, T, w.A)
+        self.row_sums = torch.empty((2 * B * T * ((D + 31) // 32),), dtype=torch.float32, device=self.dev)
 
     def gate(self, i: int):
         w = self.w
@@ -48,21 +49,18 @@ class ActionExpert:
 
     def step(self, a: torch.Tensor, cond: torch.Tensor, k: int, stream=None):
         """One Euler step on the fp32 action chunk a [B][T][A] (updated in place); cond [B][Cd] in the storage dtype."""
-        w, W = self.w, self.W
-        B, T, D = w.B, w.T, w.D
-        rb.reflex_adarmsnorm_gate(cond, W["W1"], W["b1"], W["W2"], W["b2"], self.gates, stream=stream)   # all 2L + 1 gates
-        self.a_lowp.copy_(a)
-        rb.reflex_linear_residual(self.a_lowp.view(B * T, w.A), W["W_in"], None, self.h.view(B * T, D), cache=self.cache, stream=stream)
-        for l in range(w.L):
-            rb.reflex_adarmsnorm_qkv(self.h, self.gate(2 * l), W["Wqkv"][l], self.q, self.k, self.v, cache=self.cache, stream=stream)
-            rb.reflex_partitioned_attention(self.cache, l, self.q, self.k, self.v, self.o, stream=stream)
-            rb.reflex_linear_residual(self.o.view(B * T, w.Hq * w.d), W["Wo"][l], self.h, self.h, cache=self.cache, stream=stream)
-            rb.reflex_adarmsnorm_swiglu(self.h, self.gate(2 * l + 1), W["Wgu"][l], self.m, cache=self.cache, stream=stream)
-            rb.reflex_linear_residual(self.m.view(B * T, self.F), W["Wd"][l], self.h, self.h, cache=self.cache, stream=stream)
-        rb.reflex_adarmsnorm(self.h, self.y, None, None, None, None, None, gate_buf=self.gate(2 * w.L), stream=stream)
-        rb.reflex_linear_residual(self.y.view(B * T, D), W["W_out"], None, self.vel.view(B * T, w.A), cache=self.cache, stream=stream)
-        rb.reflex_flow_step(a, self.vel, None, k, w.K, stream=stream)
-        return a
+        d, w, W = rb.ExpertDesc(self.w.T, self.w.D, self.F, self.w.A, self.w.Cd, self.w.Hd, 1e-6, 0), self.w, self.W
+        for n in _WEIGHTS:
+            if not W[n].is_contiguous():
+                raise ValueError(f"weight {n} must be contiguous")
+            setattr(d, n, W[n].data_ptr())
+        for n in _BUFFERS:
+            setattr(d, n, getattr(self, n).data_ptr())
+        return rb.reflex_expert_step(self.cache, d, a, cond, k, w.K, stream=stream)
+
+
+_BUFFERS = ("gates", "h", "y", "q", "k", "v", "o", "m", "vel", "a_lowp", "row_sums")
+_WEIGHTS = ("W_in", "W_out", "Wqkv", "Wo", "Wgu", "Wd", "W1", "b1", "W2", "b2")
 
 
 def expert_weights(w: synth.Workload, F: int, std_scale: float = 1.0) -> dict:

@@ -336,6 +336,32 @@ def test_edge_shapes(U, case, impl):
     tw.attention(0, 6, scale=0.05, what=name + " scale override")
 
 
+FEW_STREAMS = [
+    # B, Hq, Hkv, S_max, prefix lengths, N, T, appends: the edges of the kernel that splits keys over clusters of eight CTAs
+    (1, 8, 1, 816, [816], 32, 50, [32, 7]),          # 32-row tiles, ring wrapped
+    (1, 8, 1, 896, [890], 64, 64, [64, 64, 1]),      # largest slices, ring and dynamic tile; 64-row tiles
+    (2, 8, 1, 300, [300, 0], 5, 50, [3]),            # one stream without a prefix, ring partly filled
+    (1, 4, 2, 7, [3], 1, 1, []),                     # slices without keys, one row per head, no ring tokens
+    (3, 2, 1, 130, [130, 129, 1], 9, 33, [9, 2]),    # tiles of 16 tokens, last one ragged
+    (1, 32, 1, 100, [64], 33, 13, [20]),             # every token fills a tile
+]
+
+
+@pytest.mark.parametrize("case", FEW_STREAMS, ids=[f"B{c[0]}_h{c[1]}kv{c[2]}_S{c[3]}_N{c[5]}_T{c[6]}" for c in FEW_STREAMS])
+def test_attention_of_few_streams(U, case):
+    B, Hq, Hkv, S_max, S_list, N, T, appends = case
+    w = synth.Workload("few", 78, synth.DTYPE_BF16, B=B, L=2, Hq=Hq, Hkv=Hkv, d=256, S=S_max, S_max=S_max, N=N, T=T, D=64, Cd=8, Hd=8, A=4, K=2)
+    tw = U.Twin(w, head0=[(3 * b + 2) % N for b in range(B)], poison=True)
+    tw.init_static(list(range(B)), S_list)
+    for i, m in enumerate(appends):
+        tw.append(list(range(B)), m, i)
+    for layer in range(w.L):
+        tw.attention(layer, 0, what="few streams")
+    tw.attention(0, 1, q_scale=8.0, what="few streams, wide logits")
+    if T > 1:
+        tw.attention(1, 2, T=T - 1, what="few streams, T < T_max")
+
+
 def _random_attention_cases(n, seed):
     """Seeded shapes across what the kernels branch on: head_dim, queries per KV head, KV heads, prefix lengths that differ per
     stream (0 included), ring capacity and fill (empty, partly filled, wrapped), dynamic tokens from 1 to beyond one tile."""
@@ -1045,6 +1071,20 @@ def test_expert_step_bf16(U):
     accumulate; the velocity stays within 2 % of the double-precision chain."""
     w = synth.CONFIGS["cfg2"].with_(B=2, L=2, S=200, S_max=208)
     _expert_case(U, w, 1024, 2e-2, "expert bf16")
+
+
+CHAINS = [
+    # B, T, F, A, Hq, Hkv, D
+    (1, 50, 4096, 32, 8, 1, 1024), (2, 64, 1024, 8, 8, 1, 1024), (1, 1, 512, 16, 4, 1, 512), (3, 33, 1536, 32, 4, 2, 768), (1, 32, 328, 32, 8, 1, 1024),
+]
+
+
+@pytest.mark.parametrize("case", CHAINS, ids=["B%d_T%d_F%d_A%d_h%dkv%d_D%d" % c for c in CHAINS])
+def test_expert_step_bf16_few_rows(U, case):
+    """Row counts, widths and tile edges of the chained projections (up to 128 rows; the last shape's F takes the single calls)."""
+    B, T, F, A, Hq, Hkv, D = case
+    w = synth.CONFIGS["cfg2"].with_(B=B, L=2, T=T, A=A, Hq=Hq, Hkv=Hkv, D=D, S=200, S_max=208)
+    _expert_case(U, w, F, 2e-2, "expert bf16, few rows")
 
 
 def test_expert_step_bf16_batched(U):
