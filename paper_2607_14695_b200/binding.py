@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+from array import array
 from typing import Optional, Sequence
 
 import torch
@@ -79,17 +80,17 @@ def load():
     lib.reflex_kernel_launch_count.restype = ctypes.c_ulonglong
     lib.reflex_cache_slab_bytes.argtypes = [dp]; lib.reflex_cache_slab_bytes.restype = ctypes.c_size_t
     lib.reflex_workspace_bytes.argtypes = [dp]; lib.reflex_workspace_bytes.restype = ctypes.c_size_t
-    lib.reflex_cache_create.argtypes = [dp, vp, vp, vp, i32p, vp, ctypes.POINTER(vp)]
+    lib.reflex_cache_create.argtypes = [dp, vp, vp, vp, vp, vp, ctypes.POINTER(vp)]
     lib.reflex_cache_destroy.argtypes = [vp]
     lib.reflex_cache_get_state.argtypes = [vp, i32p, i32p, i32p, i64p, vp]
     lib.reflex_cache_slot_map.argtypes = [vp, i, i32p]
     lib.reflex_cache_set_attention_impl.argtypes = [vp, i]
     lib.reflex_cache_check_status.argtypes = [vp, vp]
     lib.reflex_cache_selftest_wait_limit.argtypes = [vp, i, vp]
-    lib.reflex_cache_init_static.argtypes = [vp, i32p, i, vp, vp, i, i32p, vp]
-    lib.reflex_cache_stage_static.argtypes = [vp, i32p, i, vp, vp, i, i32p, vp]
-    lib.reflex_cache_commit_static.argtypes = [vp, i32p, i, vp]
-    lib.reflex_cache_append_sliding.argtypes = [vp, i32p, i, vp, vp, i, i32p, vp]
+    lib.reflex_cache_init_static.argtypes = [vp, vp, i, vp, vp, i, vp, vp]
+    lib.reflex_cache_stage_static.argtypes = [vp, vp, i, vp, vp, i, vp, vp]
+    lib.reflex_cache_commit_static.argtypes = [vp, vp, i, vp]
+    lib.reflex_cache_append_sliding.argtypes = [vp, vp, i, vp, vp, i, vp, vp]
     lib.reflex_adarmsnorm.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, i, i, i, i, i, f, i, vp]
     lib.reflex_adarmsnorm_gate.argtypes = [vp, vp, vp, vp, vp, vp, i, i, i, i, i, i, vp]
     lib.reflex_adarmsnorm_noalloc.argtypes = [vp, vp, vp, vp, vp, vp, vp, i, i, i, i, i, f, i, vp]
@@ -116,24 +117,41 @@ def _check(rc: int):
         raise ReflexError(rc, load().reflex_last_error_string().decode())
 
 
+# A direct call costs the host its marshalling: pointers, streams and id lists therefore go through as plain integers (the argument
+# types convert them in C), and nothing is built per call that is not needed (tick of the tiny configuration, 18 calls: 190 us of
+# host time with a ctypes object per argument and a torch Stream per call).
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
         return None
     if not t.is_contiguous():
         raise ValueError("tensor must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+
+
+class _I32(array):
+    """Host int32 array that a c_void_p parameter takes (ctypes keeps the argument alive for the call)."""
+
+    def __new__(cls, seq):
+        return array.__new__(cls, "i", seq)
+
+    @property
+    def _as_parameter_(self):
+        return self.buffer_info()[0]
 
 
 def _i32(seq: Optional[Sequence[int]]):
     if seq is None:
         return None
-    return (ctypes.c_int32 * len(seq))(*[int(v) for v in seq])
+    try:
+        return _I32(seq)
+    except TypeError:
+        return _I32([int(v) for v in seq])
 
 
 def torch_dtype(dtype: int) -> torch.dtype:
@@ -251,7 +269,7 @@ def reflex_cache_append_sliding(cache: Cache, stream_ids, k_new, v_new, stream=N
     """k_new, v_new: device [n][L][m][Hkv][d]. Returns the per-stream eviction counts."""
     n = len(stream_ids)
     m = int(k_new.shape[2])
-    ev = (ctypes.c_int32 * n)()
+    ev = _I32(bytes(4 * n))
     _check(load().reflex_cache_append_sliding(cache.handle, _i32(stream_ids), n, _ptr(k_new), _ptr(v_new), m, ev, _stream(stream)))
     return list(ev)
 
@@ -327,7 +345,7 @@ def reflex_expert_step(cache: Cache, desc: ExpertDesc, a, cond, k, K, stream=Non
 
 def stream_handle(stream=None) -> ctypes.c_void_p:
     """ctypes handle of a torch stream (default: the current one), for the prepared calls below."""
-    return _stream(stream)
+    return ctypes.c_void_p(_stream(stream))
 
 
 def _prepared(fn, args):
