@@ -34,8 +34,13 @@ template <int DPL> struct RowIO<__nv_bfloat16, DPL> {
 };
 template <int DPL> struct RowIO<float, DPL> {
     static __device__ __forceinline__ void load(const float *p, float (&f)[DPL]) {
+        if constexpr (DPL % 4 == 0) {
 #pragma unroll
-        for (int i = 0; i < DPL; ++i) f[i] = p[i];
+            for (int i = 0; i < DPL; i += 4) { const float4 v = *reinterpret_cast<const float4 *>(p + i); f[i] = v.x; f[i + 1] = v.y; f[i + 2] = v.z; f[i + 3] = v.w; }
+        } else {
+#pragma unroll
+            for (int i = 0; i < DPL; ++i) f[i] = p[i];
+        }
     }
     static __device__ __forceinline__ void store(float *p, const float (&f)[DPL]) {
 #pragma unroll
@@ -43,45 +48,63 @@ template <int DPL> struct RowIO<float, DPL> {
     }
 };
 
-template <typename T> __device__ __forceinline__ float ld_f(const T *p);
-template <> __device__ __forceinline__ float ld_f<float>(const float *p) { return *p; }
-template <> __device__ __forceinline__ float ld_f<__nv_bfloat16>(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
-
-// dot of a K row (global, storage type) with a query row (shared, fp32), 8 elements per step
-template <typename T>
-__device__ __forceinline__ float dot_row(const T *__restrict__ k, const float *__restrict__ q_s, int d)
+// dot of a K row (global, storage type) with a query row (shared, fp32), 8 elements per step; the loads of 64 elements in flight together
+template <typename T, int D>
+__device__ __forceinline__ float dot_row(const T *__restrict__ k, const float *__restrict__ q_s)
 {
+    constexpr int CH = D < 64 ? D : 64;
     float acc0 = 0.f, acc1 = 0.f;
-    for (int e = 0; e < d; e += 8) {
-        float f[8];
-        RowIO<T, 8>::load(k + e, f);
-        const float4 qa = *reinterpret_cast<const float4 *>(q_s + e);
-        const float4 qb = *reinterpret_cast<const float4 *>(q_s + e + 4);
-        acc0 = fmaf(f[0], qa.x, acc0); acc1 = fmaf(f[1], qa.y, acc1);
-        acc0 = fmaf(f[2], qa.z, acc0); acc1 = fmaf(f[3], qa.w, acc1);
-        acc0 = fmaf(f[4], qb.x, acc0); acc1 = fmaf(f[5], qb.y, acc1);
-        acc0 = fmaf(f[6], qb.z, acc0); acc1 = fmaf(f[7], qb.w, acc1);
+#pragma unroll 1
+    for (int e0 = 0; e0 < D; e0 += CH) {
+        float f[CH / 8][8];
+#pragma unroll
+        for (int c = 0; c < CH / 8; ++c) RowIO<T, 8>::load(k + e0 + 8 * c, f[c]);
+#pragma unroll
+        for (int c = 0; c < CH / 8; ++c) {
+            const float4 qa = *reinterpret_cast<const float4 *>(q_s + e0 + 8 * c);
+            const float4 qb = *reinterpret_cast<const float4 *>(q_s + e0 + 8 * c + 4);
+            acc0 = fmaf(f[c][0], qa.x, acc0); acc1 = fmaf(f[c][1], qa.y, acc1);
+            acc0 = fmaf(f[c][2], qa.z, acc0); acc1 = fmaf(f[c][3], qa.w, acc1);
+            acc0 = fmaf(f[c][4], qb.x, acc0); acc1 = fmaf(f[c][5], qb.y, acc1);
+            acc0 = fmaf(f[c][6], qb.z, acc0); acc1 = fmaf(f[c][7], qb.w, acc1);
+        }
     }
     return acc0 + acc1;
 }
 
-constexpr int kSimtWarps = 4;
+constexpr int kSimtWarps = 4;      // rows of a block, a warp each (WPR = 1)
+constexpr int kSimtRowWarps = 8;   // warps that share a row (WPR = kSimtRowWarps)
 
-// grid = (ceil(T*Hq / kSimtWarps), B, nsplit)
-template <typename T, int DPL>
-__global__ void __launch_bounds__(kSimtWarps * 32)
+// WPR: warps per query row. 1: a block takes kSimtWarps rows, grid = (ceil(T Hq / kSimtWarps), B, nsplit). kSimtRowWarps: a block
+// takes one row, its warps every eighth tile of the slice, and merges their (m, l, acc) through shared memory, grid = (T Hq, B, nsplit).
+// What bounds small problems is the latency of a tile, not the arithmetic: the rows of K and then batches of V rows are
+// loaded with all loads in flight, and with few rows the tiles go to different warps (16 rows, 88 keys, fp32: 22.1 us with a warp
+// per row, one load at a time and 3 tiles in a row).
+template <typename T, int DPL, int WPR>
+__global__ void __launch_bounds__(WPR == 1 ? kSimtWarps * 32 : WPR * 32)
 attn_simt_kernel(AttnParams p)
 {
     constexpr int d = DPL * 32;
-    __shared__ __align__(16) float q_s[kSimtWarps][d];
+    constexpr int NB = DPL >= 8 ? 8 : DPL == 4 ? 16 : 32;      // V rows in flight
+    __shared__ __align__(16) float q_s[WPR == 1 ? kSimtWarps : 1][d];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b = blockIdx.y, split = blockIdx.z;
     const int rows = p.T * p.Hq;
-    const int r = blockIdx.x * kSimtWarps + warp;
-    if (r >= rows) return;  // no block-wide barrier below
+    const int r = WPR == 1 ? blockIdx.x * kSimtWarps + warp : blockIdx.x;
+    if (WPR == 1 && r >= rows) return;  // no block-wide barrier below
     const int t = r / p.Hq, h = r % p.Hq;
     const int kv = h / (p.Hq / p.Hkv);
+    float *qs = q_s[WPR == 1 ? warp : 0];
 
+    const T *q_row = (const T *)p.q + (((size_t)b * p.T + t) * p.Hq + h) * d;
+    if (WPR == 1 || warp == 0) {
+        float f[DPL];
+        RowIO<T, DPL>::load(q_row + lane * DPL, f);
+#pragma unroll
+        for (int i = 0; i < DPL; ++i) qs[lane * DPL + i] = f[i];
+    }
     const StreamState st = p.state[b];
     const int S = st.static_len > 0 ? st.static_len : 0;
     const int N = p.N;
@@ -100,22 +123,14 @@ attn_simt_kernel(AttnParams p)
     const T *v_blk = (const T *)p.v_slab + blk * row_elems + (size_t)kv * d;
     const T *k_dyn = (const T *)p.k_dyn + (size_t)b * p.T * row_elems + (size_t)kv * d;
     const T *v_dyn = (const T *)p.v_dyn + (size_t)b * p.T * row_elems + (size_t)kv * d;
-
-    const T *q_row = (const T *)p.q + (((size_t)b * p.T + t) * p.Hq + h) * d;
-    {
-        float f[DPL];
-        RowIO<T, DPL>::load(q_row + lane * DPL, f);
-#pragma unroll
-        for (int i = 0; i < DPL; ++i) q_s[warp][lane * DPL + i] = f[i];
-    }
-    __syncwarp();
+    if (WPR == 1) __syncwarp(); else __syncthreads();
 
     float m = -INFINITY, l = 0.f;
     float acc[DPL];
 #pragma unroll
     for (int i = 0; i < DPL; ++i) acc[i] = 0.f;
 
-    for (int tile = tile0; tile < tile1; ++tile) {
+    for (int tile = tile0 + (WPR == 1 ? 0 : warp); tile < tile1; tile += WPR) {
         const int idx = tile * 32 + lane;
         const T *kp = nullptr, *vp = nullptr;
         if (idx < S) {
@@ -131,8 +146,23 @@ attn_simt_kernel(AttnParams p)
             const int j = idx - S - N;
             if (!(p.dyn_mask && j > t)) { kp = k_dyn + (size_t)j * row_elems; vp = v_dyn + (size_t)j * row_elems; }
         }
+        const unsigned long long vaddr = (unsigned long long)vp;
+        // a dead key's V row is never read (it may hold stale or poisoned bytes)
+        float f[NB][DPL];
+        auto load_v = [&](int j0) {
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                const unsigned long long va = __shfl_sync(0xffffffffu, vaddr, j0 + j);
+                if (va != 0ull) RowIO<T, DPL>::load((const T *)va + lane * DPL, f[j]);
+                else {
+#pragma unroll
+                    for (int i = 0; i < DPL; ++i) f[j][i] = 0.f;
+                }
+            }
+        };
+        load_v(0);
         float s = -INFINITY;
-        if (kp) s = dot_row<T>(kp, q_s[warp], d) * p.scale;
+        if (kp) s = dot_row<T, d>(kp, qs) * p.scale;
         float tmax = s;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
@@ -147,18 +177,40 @@ attn_simt_kernel(AttnParams p)
         m = m_new;
 #pragma unroll
         for (int i = 0; i < DPL; ++i) acc[i] *= alpha;
-        const unsigned long long vaddr = (unsigned long long)vp;
-        for (int j = 0; j < 32; ++j) {
-            const float w = __shfl_sync(0xffffffffu, pj, j);
-            const unsigned long long va = __shfl_sync(0xffffffffu, vaddr, j);
-            if (va == 0ull) continue;  // dead key: its V row is never read (may hold stale or poisoned bytes)
-            float f[DPL];
-            RowIO<T, DPL>::load((const T *)va + lane * DPL, f);
+#pragma unroll 1
+        for (int j0 = 0; j0 < 32; j0 += NB) {
+            if (j0 > 0) load_v(j0);
 #pragma unroll
-            for (int i = 0; i < DPL; ++i) acc[i] = fmaf(w, f[i], acc[i]);
+            for (int j = 0; j < NB; ++j) {
+                const float w = __shfl_sync(0xffffffffu, pj, j0 + j);
+#pragma unroll
+                for (int i = 0; i < DPL; ++i) acc[i] = fmaf(w, f[j][i], acc[i]);
+            }
         }
     }
 
+    if constexpr (WPR > 1) {
+        // the warps' partial results: warp 0 adds them up
+        __shared__ float part[WPR][d + 2];
+        part[warp][d] = m; part[warp][d + 1] = l;
+#pragma unroll
+        for (int i = 0; i < DPL; ++i) part[warp][lane * DPL + i] = acc[i];
+        __syncthreads();
+        if (warp > 0) return;
+        const int live = min(WPR, tile1 - tile0);       // warps that had a tile
+        for (int w = 1; w < live; ++w) m = fmaxf(m, part[w][d]);
+        l = 0.f;
+#pragma unroll
+        for (int i = 0; i < DPL; ++i) acc[i] = 0.f;
+        for (int w = 0; w < live; ++w) {
+            const float mw = part[w][d];
+            if (mw == -INFINITY) continue;
+            const float a = expf(mw - m);
+            l = fmaf(part[w][d + 1], a, l);
+#pragma unroll
+            for (int i = 0; i < DPL; ++i) acc[i] = fmaf(part[w][lane * DPL + i], a, acc[i]);
+        }
+    }
     if (p.nsplit == 1) {
         const float inv = 1.f / l;  // l > 0: a dynamic query always sees itself
 #pragma unroll
@@ -243,13 +295,18 @@ attn_merge_kernel(AttnParams p)
     RowIO<T, DPL>::store(out + lane * DPL, acc);
 }
 
+// Few rows: a block per row, its eight warps share the keys. The line lies where warps with a row each would no longer leave SMs idle.
+static bool simt_row_blocks(const AttnParams &p) { return (long long)p.T * p.Hq * p.B <= 2048; }
+
 int simt_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count)
 {
     const int rows = p.T * p.Hq;
-    const int blocks = ((rows + kSimtWarps - 1) / kSimtWarps) * p.B;
+    const bool rb = simt_row_blocks(p);
+    const int blocks = rb ? rows * p.B : ((rows + kSimtWarps - 1) / kSimtWarps) * p.B;
     const int n_tiles = (p.S_max + p.N + p.T + 31) / 32;
     int want = (4 * sm_count + blocks - 1) / blocks;  // aim at ~4 blocks per SM
-    if (want > n_tiles / 2) want = n_tiles / 2;       // at least two key tiles per split
+    const int per = rb ? 2 * kSimtRowWarps : 2;       // at least two key tiles per split and warp
+    if (want > n_tiles / per) want = n_tiles / per;
     if (want > kMaxSplits) want = kMaxSplits;
     const size_t per_split = (size_t)p.B * rows * (p.d + 2) * sizeof(float);
     if (per_split > 0 && (size_t)want * per_split > partial_bytes) want = (int)(partial_bytes / per_split);
@@ -257,20 +314,35 @@ int simt_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count)
     return want;
 }
 
+template <typename T, int DPL>
+static cudaError_t launch_simt_d(const AttnParams &p, cudaStream_t st)
+{
+    const int rows = p.T * p.Hq;
+    const bool rb = simt_row_blocks(p);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = rb ? dim3(rows, p.B, p.nsplit) : dim3((rows + kSimtWarps - 1) / kSimtWarps, p.B, p.nsplit);
+    cfg.blockDim = dim3(32 * (rb ? kSimtRowWarps : kSimtWarps));
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return rb ? cudaLaunchKernelEx(&cfg, attn_simt_kernel<T, DPL, kSimtRowWarps>, p) : cudaLaunchKernelEx(&cfg, attn_simt_kernel<T, DPL, 1>, p);
+}
+
 template <typename T>
 static cudaError_t launch_simt_t(const AttnParams &p, cudaStream_t st)
 {
-    const int rows = p.T * p.Hq;
-    dim3 grid((rows + kSimtWarps - 1) / kSimtWarps, p.B, p.nsplit);
+    cudaError_t e;
     switch (p.d / 32) {
-        case 1: attn_simt_kernel<T, 1><<<grid, kSimtWarps * 32, 0, st>>>(p); break;
-        case 2: attn_simt_kernel<T, 2><<<grid, kSimtWarps * 32, 0, st>>>(p); break;
-        case 4: attn_simt_kernel<T, 4><<<grid, kSimtWarps * 32, 0, st>>>(p); break;
-        case 8: attn_simt_kernel<T, 8><<<grid, kSimtWarps * 32, 0, st>>>(p); break;
+        case 1: e = launch_simt_d<T, 1>(p, st); break;
+        case 2: e = launch_simt_d<T, 2>(p, st); break;
+        case 4: e = launch_simt_d<T, 4>(p, st); break;
+        case 8: e = launch_simt_d<T, 8>(p, st); break;
         default: return cudaErrorInvalidValue;
     }
     count_launch();
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || p.nsplit == 1) return e;
     return launch_attention_merge(p, st);
 }

@@ -42,53 +42,55 @@ template <typename T> __device__ __forceinline__ float to_f(T v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
 
+// emit(j, w_j . v) for j in [j0, j1): rows w_j of length len (a multiple of 8) in global memory, v in shared memory. 1 to 32 lanes per
+// row, eight elements a lane, so that a short row leaves no lane idle and a warp has several rows' loads in flight at once.
+template <typename T, typename F>
+__device__ __forceinline__ void dot_rows(const T *__restrict__ W, int len, int j0, int j1, const float *v, F &&emit)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    int group = 32;
+    while (group > 1 && group * 4 >= len) group >>= 1;
+    const int per_warp = 32 / group, sub = lane / group, l = lane % group;
+    for (int jj = j0 + warp * per_warp; jj < j1; jj += nwarp * per_warp) {
+        const int j = jj + sub;
+        float acc = 0.f;
+        if (j < j1) {
+            const T *w = W + (size_t)j * len;
+            for (int e = l * 8; e < len; e += group * 8) {
+                float f[8];
+                Vec8<T>::load(w + e, f);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc = fmaf(f[i], v[e + i], acc);
+            }
+        }
+        for (int o = group / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (l == 0 && j < j1) emit(j, acc);
+    }
+}
+
 // hidden = SiLU(W1 c + b1) for one stream into shared memory; c_s is scratch of Cd floats.
 template <typename T>
 __device__ void gate_hidden(const T *__restrict__ cond_b, const T *__restrict__ W1, const T *__restrict__ b1, int Cd, int Hd,
                             float *c_s, float *hid_s)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     for (int e = threadIdx.x; e < Cd; e += blockDim.x) c_s[e] = to_f<T>(cond_b[e]);
     __syncthreads();
-    for (int j = warp; j < Hd; j += nwarp) {
-        const T *w = W1 + (size_t)j * Cd;
-        float acc = 0.f;
-        for (int e = lane * 8; e < Cd; e += 256) {
-            float f[8];
-            Vec8<T>::load(w + e, f);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) acc = fmaf(f[i], c_s[e + i], acc);
-        }
-        acc = warp_sum(acc);
-        if (lane == 0) {
-            const float z = acc + to_f<T>(b1[j]);
-            hid_s[j] = z / (1.f + expf(-z));
-        }
-    }
+    dot_rows<T>(W1, Cd, 0, Hd, c_s, [&](int j, float acc) {
+        const float z = acc + to_f<T>(b1[j]);
+        hid_s[j] = z / (1.f + expf(-z));
+    });
     __syncthreads();
 }
 
-// gate[i] = 1 + b2[i] + W2[i] . hidden for columns [i0, i1): one warp per column.
+// gate[i] = 1 + b2[i] + W2[i] . hidden for columns [i0, i1).
 template <typename T>
 __device__ void gate_columns(const T *__restrict__ W2, const T *__restrict__ b2, int Hd, int i0, int i1, const float *hid_s,
                              float *gate_out /* indexed by i - i0 */)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    for (int i = i0 + warp; i < i1; i += nwarp) {
-        const T *w = W2 + (size_t)i * Hd;
-        float acc = 0.f;
-        for (int e = lane * 8; e < Hd; e += 256) {
-            float f[8];
-            Vec8<T>::load(w + e, f);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) acc = fmaf(f[k], hid_s[e + k], acc);
-        }
-        acc = warp_sum(acc);
-        if (lane == 0) gate_out[i - i0] = 1.f + (acc + to_f<T>(b2[i]));
-    }
+    dot_rows<T>(W2, Hd, i0, i1, hid_s, [&](int i, float acc) { gate_out[i - i0] = 1.f + (acc + to_f<T>(b2[i])); });
 }
 
-// grid = (column chunks, B): writes gate_buf[b][i].
+// grid = (column chunks, B, layers): writes gate_buf[layer][b][i]; every block computes the hidden layer for itself.
 template <typename T>
 __global__ void __launch_bounds__(256)
 gate_kernel(const T *__restrict__ cond, const T *__restrict__ W1, const T *__restrict__ b1, const T *__restrict__ W2,
@@ -97,10 +99,13 @@ gate_kernel(const T *__restrict__ cond, const T *__restrict__ W1, const T *__res
     extern __shared__ float smem[];
     float *c_s = smem, *hid_s = smem + Cd;
     const int b = blockIdx.y;
-    gate_hidden<T>(cond + (size_t)b * Cd, W1, b1, Cd, Hd, c_s, hid_s);
+    const size_t l = blockIdx.z;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    gate_hidden<T>(cond + (size_t)b * Cd, W1 + l * Hd * Cd, b1 + l * Hd, Cd, Hd, c_s, hid_s);
     const int i0 = blockIdx.x * cols_per_block;
     const int i1 = min(D, i0 + cols_per_block);
-    gate_columns<T>(W2, b2, Hd, i0, i1, hid_s, gate_buf + (size_t)b * D + i0);
+    gate_columns<T>(W2 + l * D * Hd, b2 + l * D, Hd, i0, i1, hid_s, gate_buf + (l * gridDim.y + b) * D + i0);
 }
 
 // grid = (row chunks, B); one warp per row. FUSED: the block computes its stream's gate itself.
@@ -374,6 +379,26 @@ static bool gate_scratch_fits(int Cd, int Hd)
 // gamma_l(c) = 1 + W2_l SiLU(W1_l c + b1_l) + b2_l for L layers (stacked weights) and B streams: gates into
 // gate_buf[L][B][D], hidden activations into gate_buf + L*B*D ([L][B][Hd]). Two launches whatever L is.
 template <typename T>
+static cudaError_t launch_gate_blocks(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, float *gate_buf, int L, int B,
+                                      int D, int Cd, int Hd, cudaStream_t st)
+{
+    const int cols = 64;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((D + cols - 1) / cols, B, L);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = (size_t)(Cd + Hd) * 4;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gate_kernel<T>, cond, W1, b1, W2, b2, gate_buf, D, Cd, Hd, cols);
+    count_launch();
+    return e;
+}
+
+template <typename T>
 static cudaError_t launch_gate_t(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, float *gate_buf, int L, int B,
                                  int D, int Cd, int Hd, cudaStream_t st)
 {
@@ -398,6 +423,10 @@ static cudaError_t launch_gate_t(const T *cond, const T *W1, const T *b1, const 
             if (e != cudaErrorInvalidValue) return e;   // invalid value: no tensor maps from this driver, fall through
         }
     }
+    // A small MLP for a few streams: one launch whose blocks compute the hidden layer each for themselves. Up to 8 K hidden products
+    // that costs a block less than the second launch (3.4 us for the two, tiny configuration). The rule does not depend on L: one call
+    // for L layers and L calls give the same bits.
+    if (Hd * Cd <= 8192 && B <= 8) return launch_gate_blocks<T>(cond, W1, b1, W2, b2, gate_buf, L, B, D, Cd, Hd, st);
     const int groups = (B + kGateStreams - 1) / kGateStreams;
     const size_t tiled_h = (size_t)(kTileUnits + kGateStreams) * (Cd + 4) * 4, tiled_g = (size_t)(kTileUnits + kGateStreams) * (Hd + 4) * 4;
     if (L > 1 && tiled_h <= 200 * 1024 && tiled_g <= 200 * 1024) {
@@ -461,10 +490,7 @@ static cudaError_t launch_norm_t(const T *x, T *y, const T *cond, const T *W1, c
         after_gate = true;
     } else if (cond && gate_buf) {
         // very wide conditioning / hidden layers: per-block gate (shared-memory staging of 16 streams would not fit)
-        const int cols = 64;
-        gate_kernel<T><<<dim3((D + cols - 1) / cols, B), 256, (size_t)(Cd + Hd) * 4, st>>>(cond, W1, b1, W2, b2, gate_buf, D, Cd, Hd, cols);
-        count_launch();
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = launch_gate_blocks<T>(cond, W1, b1, W2, b2, gate_buf, 1, B, D, Cd, Hd, st);
         if (e != cudaSuccess) return e;
     }
     if (gate_buf && D <= 2048) return launch_rows_t<T>(x, y, gate_buf, B, R, D, eps, after_gate, st);
@@ -511,6 +537,8 @@ cudaError_t launch_adarmsnorm(const void *x, void *y, const void *cond, const vo
 template <typename T>
 __global__ void flow_step_kernel(float *__restrict__ x, const T *__restrict__ v, T *__restrict__ x_lowp, size_t n, float dt)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float nx = fmaf(dt, to_f<T>(v[i]), x[i]);
         x[i] = nx;
@@ -530,30 +558,15 @@ __global__ void cast_kernel(const float *__restrict__ x, T *__restrict__ y, size
     }
 }
 
-template <typename T>
-static cudaError_t launch_gate_wide_t(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, float *gate_buf, int L, int B,
-                                      int D, int Cd, int Hd, cudaStream_t st)
-{
-    const int cols = 64;
-    for (int l = 0; l < L; ++l) {
-        gate_kernel<T><<<dim3((D + cols - 1) / cols, B), 256, (size_t)(Cd + Hd) * 4, st>>>(
-            cond, W1 + (size_t)l * Hd * Cd, b1 + (size_t)l * Hd, W2 + (size_t)l * D * Hd, b2 + (size_t)l * D, gate_buf + (size_t)l * B * D, D, Cd, Hd, cols);
-        count_launch();
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
 cudaError_t launch_adarmsnorm_gate(const void *cond, const void *W1, const void *b1, const void *W2, const void *b2, float *gate_buf,
                                    int L, int B, int D, int Cd, int Hd, int dtype, cudaStream_t st)
 {
     if (!gate_scratch_fits(Cd, Hd)) {
-        // conditioning or hidden layers too wide to stage 32 streams' vectors in shared memory: the per-stream kernel, layer by layer
+        // conditioning or hidden layers too wide to stage 32 streams' vectors in shared memory: the per-stream kernel
         if (dtype == REFLEX_DTYPE_BF16)
-            return launch_gate_wide_t<__nv_bfloat16>((const __nv_bfloat16 *)cond, (const __nv_bfloat16 *)W1, (const __nv_bfloat16 *)b1,
+            return launch_gate_blocks<__nv_bfloat16>((const __nv_bfloat16 *)cond, (const __nv_bfloat16 *)W1, (const __nv_bfloat16 *)b1,
                                                      (const __nv_bfloat16 *)W2, (const __nv_bfloat16 *)b2, gate_buf, L, B, D, Cd, Hd, st);
-        return launch_gate_wide_t<float>((const float *)cond, (const float *)W1, (const float *)b1, (const float *)W2, (const float *)b2,
+        return launch_gate_blocks<float>((const float *)cond, (const float *)W1, (const float *)b1, (const float *)W2, (const float *)b2,
                                          gate_buf, L, B, D, Cd, Hd, st);
     }
     if (dtype == REFLEX_DTYPE_BF16)
@@ -568,12 +581,20 @@ cudaError_t launch_flow_step(float *x, const void *v, void *x_lowp, size_t n, fl
     int blocks = (int)((n + 255) / 256);
     if (blocks > 1184) blocks = 1184;
     if (blocks < 1) blocks = 1;
-    if (dtype == REFLEX_DTYPE_BF16)
-        flow_step_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(x, (const __nv_bfloat16 *)v, (__nv_bfloat16 *)x_lowp, n, dt);
-    else
-        flow_step_kernel<float><<<blocks, 256, 0, st>>>(x, (const float *)v, (float *)x_lowp, n, dt);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = dtype == REFLEX_DTYPE_BF16
+                        ? cudaLaunchKernelEx(&cfg, flow_step_kernel<__nv_bfloat16>, x, (const __nv_bfloat16 *)v, (__nv_bfloat16 *)x_lowp, n, dt)
+                        : cudaLaunchKernelEx(&cfg, flow_step_kernel<float>, x, (const float *)v, (float *)x_lowp, n, dt);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_cast(const float *x, void *y, size_t n, int dtype, cudaStream_t st)
