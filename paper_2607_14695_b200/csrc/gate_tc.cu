@@ -42,7 +42,7 @@ struct GateTcSmem {
 // SILU: first layer (writes hi/lo bf16 hidden activations); else second layer (writes fp32 gates 1 + z). PASSES: 1 = one
 // bf16 vector per stream (tm_v0), 2 = hi and lo halves (tm_v0, tm_v1).
 template <bool SILU, int PASSES>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(256, 1)
 gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_v0, const __grid_constant__ CUtensorMap tm_v1,
                const __nv_bfloat16 *__restrict__ bias, float *out_f32, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, int B, int len, int units,
                int vec_rows_per_layer, uint32_t *status)
@@ -56,7 +56,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + S::OFF_BAR + 16);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int layer = blockIdx.z, u0 = blockIdx.x * kGtUnits;
-    const int chunks = (len + 63) / 64, ksteps = len / 16;
+    const int chunks = (len + 63) / 64;
     // A CTA keeps its 128 weight rows in shared memory and walks the groups of 64 streams that fall to it (blockIdx.y takes
     // a contiguous share of the groups): with many streams -- the conditioning vectors of all steps of a control tick
     // stacked -- the weights are fetched once per CTA instead of once per group, and the next group's vectors come in
@@ -73,7 +73,17 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
         prefetch_tmap(&tm_w); prefetch_tmap(&tm_v0);
         if (PASSES == 2) prefetch_tmap(&tm_v1);
     }
-    if (warp == 0) tmem_alloc(smem_u32((const void *)tmem_slot), 64);
+    // weights and (first group of) vectors on one barrier. The second layer asks for its weights before the wait for the first layer's
+    // kernel: that kernel writes none, and whatever precedes the call was complete before this one could start.
+    auto load_weights = [&]() {
+        mbar_expect_tx_elect(bar_load, (uint32_t)chunks * (S::A_CHUNK + PASSES * S::B_CHUNK));
+        for (int c = 0; c < chunks; ++c) tma_load_2d_elect(base + S::OFF_A + c * S::A_CHUNK, &tm_w, bar_load, c * 64, layer * units + u0);
+    };
+    if (warp == 0) {
+        __syncwarp();
+        if (!SILU && ng > 0) load_weights();
+    }
+    if (warp == 1) tmem_alloc(smem_u32((const void *)tmem_slot), 64);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -92,22 +102,22 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
         if (status) atomicCAS(status, 0u, 0x80000000u | ((code + 64u) << 16) | (blockIdx.x & 0xFFFFu));
         return false;
     };
-    auto load_vectors = [&](int g) {   // the (up to) 64 vectors of group g, one or two bf16 arrays
+    auto load_vectors = [&](int g) {   // the (up to) 64 vectors of group g, one or two bf16 arrays (the warp is converged)
         for (int c = 0; c < chunks; ++c) {
-            tma_load_2d(base + S::OFF_B + c * S::B_CHUNK, &tm_v0, bar_load, c * 64, layer * vec_rows_per_layer + g * kGtStreams);
+            tma_load_2d_elect(base + S::OFF_B + c * S::B_CHUNK, &tm_v0, bar_load, c * 64, layer * vec_rows_per_layer + g * kGtStreams);
             if (PASSES == 2)
-                tma_load_2d(base + S::OFF_B + (kGtMaxChunks + c) * S::B_CHUNK, &tm_v1, bar_load, c * 64, layer * vec_rows_per_layer + g * kGtStreams);
+                tma_load_2d_elect(base + S::OFF_B + (kGtMaxChunks + c) * S::B_CHUNK, &tm_v1, bar_load, c * 64, layer * vec_rows_per_layer + g * kGtStreams);
         }
     };
 
     bool ok = true;
-    if (warp == 0 && lane == 0 && ng > 0) {
-        mbar_expect_tx(bar_load, (uint32_t)chunks * (S::A_CHUNK + PASSES * S::B_CHUNK));
-        for (int c = 0; c < chunks; ++c) tma_load_2d(base + S::OFF_A + c * S::A_CHUNK, &tm_w, bar_load, c * 64, layer * units + u0);
+    if (warp == 0 && ng > 0) {
+        if (SILU) load_weights();
         load_vectors(g_first);
     }
-    const int u = u0 + warp * 32 + lane;
-    const uint32_t lane_addr = (uint32_t)(warp * 32) << 16;
+    const int quarter = warp & 3, half = warp >> 2;
+    const int u = u0 + quarter * 32 + lane;
+    const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const float bi = u < units ? __bfloat162float(bias[(size_t)layer * units + u]) : 0.f;
 #pragma unroll 1
     for (int i = 0; i < ng; ++i) {
@@ -122,10 +132,15 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
 #pragma unroll 1
                 for (int pass = 0; pass < PASSES; ++pass) {
 #pragma unroll 1
-                    for (int kk = 0; kk < ksteps; ++kk) {
-                        const uint32_t a = base + S::OFF_A + (kk >> 2) * S::A_CHUNK + (kk & 3) * 32;
-                        const uint32_t b = base + S::OFF_B + (pass * kGtMaxChunks + (kk >> 2)) * S::B_CHUNK + (kk & 3) * 32;
-                        umma_ss_elect(tmem, umma_desc_sw128(a, 16, 1024), umma_desc_sw128(b, 16, 1024), idesc, (pass > 0 || kk > 0) ? 1u : 0u);
+                    for (int c = 0; c < chunks; ++c) {      // (columns past the contraction's end are zeros on both sides)
+                        uint64_t ad = umma_desc_sw128(base + S::OFF_A + c * S::A_CHUNK, 16, 1024);
+                        uint64_t bd = umma_desc_sw128(base + S::OFF_B + (pass * kGtMaxChunks + c) * S::B_CHUNK, 16, 1024);
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            umma_ss_elect(tmem, ad, bd, idesc, (pass > 0 || c > 0 || kk > 0) ? 1u : 0u);
+                            umma_desc_advance(ad, 32);
+                            umma_desc_advance(bd, 32);
+                        }
                     }
                 }
             }
@@ -134,47 +149,46 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
         ok = wait(bar_mma, ph, 2) && ok;
         tc_fence_after();
         // the MMAs that read this group's vectors are complete: the next group's may land on them
-        if (warp == 0 && lane == 0 && i + 1 < ng) {
-            mbar_expect_tx(bar_load, (uint32_t)chunks * (PASSES * S::B_CHUNK));
+        if (warp == 0 && i + 1 < ng) {
+            mbar_expect_tx_elect(bar_load, (uint32_t)chunks * (PASSES * S::B_CHUNK));
             load_vectors(g_first + i + 1);
         }
-        // epilogue: thread = weight row (TMEM lane), 64 columns = streams
-        uint32_t acc[64];
-        tmem_ld32(tmem + lane_addr, *reinterpret_cast<uint32_t(*)[32]>(acc));
-        tmem_ld32(tmem + lane_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(acc + 32));
-        tmem_wait_ld();
-        tc_fence_before();
-        __syncthreads();      // every warp holds its accumulators in registers: the next group's MMAs may overwrite them
+        // epilogue: thread = weight row (TMEM lane), columns = streams, the two warps of a lane quarter take 32 each in groups of eight.
+        // Groups without a stream are skipped by a branch: as predicated code over all 64 columns the SiLU layer's epilogue took 4.7 us
+        // for a single stream.
         const int nb = min(kGtStreams, B - b0);
-        if (!ok && u < units) {
-            // a bounded wait ran out: this CTA's slice of the output is marked invalid (quiet NaN) instead of keeping the
-            // previous call's values, so whatever consumes the gates shows it
-            for (int n = 0; n < nb; ++n) {
-                const size_t o = ((size_t)layer * B + b0 + n) * units + u;
-                if (SILU) { out_hi[o] = __float2bfloat16_rn(__int_as_float(0x7fc00000)); out_lo[o] = __float2bfloat16_rn(0.f); }
-                else out_f32[o] = __int_as_float(0x7fc00000);
-            }
-        }
-        if (ok && u < units) {
+#pragma unroll 1
+        for (int g = 0; g < 4; ++g) {
+            const int n0 = half * 32 + g * 8;
+            if (n0 >= nb) break;
+            uint32_t acc[8];
+            tmem_ld8(tmem + lane_addr + n0, acc);
+            tmem_wait_ld();
+            if (u < units) {
+                const size_t o0 = ((size_t)layer * B + b0 + n0) * units + u;
 #pragma unroll
-            for (int n = 0; n < kGtStreams; ++n) {
-                if (n >= nb) continue;   // (fully unrolled: the accumulator stays in registers)
-                const float z = __uint_as_float(acc[n]) + bi;
-                const size_t o = ((size_t)layer * B + b0 + n) * units + u;
-                if (SILU) {
-                    const float h = z / (1.f + expf(-z));
-                    const __nv_bfloat16 hi = __float2bfloat16_rn(h);
-                    out_hi[o] = hi;
-                    out_lo[o] = __float2bfloat16_rn(h - __bfloat162float(hi));
-                } else {
-                    out_f32[o] = 1.f + z;
+                for (int n = 0; n < 8; ++n) {
+                    // (after a bounded wait that ran out this CTA's slice of the output is marked invalid, a quiet NaN, instead of keeping
+                    // the previous call's values: whatever consumes the gates shows it)
+                    const float z = ok ? __uint_as_float(acc[n]) + bi : __int_as_float(0x7fc00000);
+                    if (n0 + n >= nb) continue;
+                    if (SILU) {
+                        const float h = z / (1.f + expf(-z));
+                        const __nv_bfloat16 hi = __float2bfloat16_rn(h);
+                        out_hi[o0 + (size_t)n * units] = hi;
+                        out_lo[o0 + (size_t)n * units] = __float2bfloat16_rn(h - __bfloat162float(hi));
+                    } else {
+                        out_f32[o0 + (size_t)n * units] = 1.f + z;
+                    }
                 }
             }
         }
+        tc_fence_before();
+        __syncthreads();      // every warp has read its accumulators: the next group's MMAs may overwrite them
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, 64);
+    if (warp == 1) tmem_dealloc(tmem, 64);
 }
 
 template <bool SILU, int PASSES>
@@ -193,7 +207,7 @@ cudaError_t launch_one(const CUtensorMap &mw, const CUtensorMap &mv0, const CUte
     int gy = 148 / (ux * L);
     gy = gy < 1 ? 1 : (gy > n_groups ? n_groups : gy);
     cfg.gridDim = dim3(ux, gy, L);
-    cfg.blockDim = dim3(128);
+    cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = GateTcSmem::TOTAL;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
