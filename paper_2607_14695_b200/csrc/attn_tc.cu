@@ -783,9 +783,9 @@ bool tc2_supported(const AttnParams &p) { return tc_supported(p) && (p.d == 128 
 // the columns is whole 16-byte stores. Measured against the split with partials: 4466 keys, 16 streams 41.2 -> 35.6 us
 // (two slices); 898 keys, 4 streams 18.5 -> 16.5 (four slices); one stream 15.5 merged in four against 14.4 with eight
 // slices and the merge kernel, and 2 streams 16.5 merged in four against 15.9 with partials. The model therefore charges
-// the in-cluster merge 5.5 us (three cluster barriers and the staged reduction keep every CTA of the cluster that long)
-// and uses it only where the partials' round trip would cost more.
-static constexpr double kTc2MergedUs = 5.5;
+// the in-cluster merge 6.6 us (three cluster barriers and the staged reduction keep every CTA of the cluster that long; 4 streams
+// x 4466 keys: 23.0 merged in four, 19.0 with eight slices and partials) and uses it only where the partials' round trip would cost more.
+static constexpr double kTc2MergedUs = 6.6;
 static double tc2_partials_us(const AttnParams &p, int nsplit)   // merge launch + fp32 partials written and read back
 {
     const double per_split_bytes = (double)p.B * p.T * p.Hq * (p.d + 2) * sizeof(float);
@@ -820,10 +820,13 @@ int tc2_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count)
     const double per_split_bytes = (double)p.B * p.T * p.Hq * (p.d + 2) * sizeof(float);
     int best = 1;
     double best_us = 1e30;
-    for (int ns = 1; ns <= 8; ns *= 2) {
+    // Long keys want many slices: one stream x 13666 keys takes 29.2 us in 8, 23.3 in 12, 19.5 in 24, 20.9 in 32; 12 streams x 4466
+    // keys 33.6 merged in two, 31.2 in three.
+    static const int kSlices[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24};
+    for (const int ns : kSlices) {
         if (ns > tiles) break;
         const bool merged = ns > 1 && tc2_cluster_merge_ok(p, ns, sm_count);
-        if (ns > 1 && !merged && per_split_bytes * ns > (double)partial_bytes) break;
+        if (ns > 1 && !merged && per_split_bytes * ns > (double)partial_bytes) continue;
         const int waves = merged ? 1 : (units * ns + clusters - 1) / clusters;
         const double loop_us = 1.3 * waves * ((tiles + ns - 1) / ns);
         const double split_us = ns == 1 ? 0.0 : (merged ? kTc2MergedUs : tc2_partials_us(p, ns));
@@ -899,3 +902,4 @@ extern "C" int reflex_debug_tc2_trace(long long *out)
     return (int)cudaMemcpyFromSymbol(out, reflex::g_tc2_trace, sizeof(long long) * 2 * 4 * 16 * 16);
 }
 #endif
+
