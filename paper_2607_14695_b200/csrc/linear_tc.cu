@@ -53,6 +53,7 @@ struct LinSmem {
 };
 
 struct LinParams {
+    int early_w;        // weights may be asked for before the preceding kernel is complete
     int M, K, N;
     int m_tiles;          // 256-row tiles
     int has_res;
@@ -124,6 +125,15 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     if (threadIdx.x == 64) LIN_TRACE(1);
+    auto load_w = [&](int s, int ks) {
+        // both CTAs' loads complete on the leader's barrier: the issuing thread there waits for all four at once
+        if (rank == 0) mbar_expect_tx(bar(S::C_FULL + s), 2 * (S::A_STAGE + S::B_STAGE));
+        lin_tma2_load_2d(base + S::OFF_B + s * S::B_STAGE, &tm_w, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * kLinBK, n0 + (int)rank * (BN / 2));
+    };
+    // inside an expert step (early_w) the weights of the first steps are asked for before the wait for the preceding kernel
+    const int head = p.early_w ? (nk_steps < NST ? nk_steps : NST) : 0;
+    if (threadIdx.x == 0)
+        for (int ks = 0; ks < head; ++ks) load_w(ks, ks);
     // programmatic dependent launch: whatever produced a and res is complete from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -154,10 +164,8 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
                 const int s = ks % NST;
                 if (ks >= NST) ok = wait(S::C_EMPTY + s, (uint32_t)(ks / NST - 1) & 1u, 1);
                 if (!ok) break;
-                // both CTAs' loads complete on the leader's barrier: the issuing thread there waits for all four at once
-                if (rank == 0) mbar_expect_tx(bar(S::C_FULL + s), 2 * (S::A_STAGE + S::B_STAGE));
+                if (ks >= head) load_w(s, ks);
                 lin_tma2_load_2d(base + S::OFF_A + s * S::A_STAGE, &tm_a, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * kLinBK, m0);
-                lin_tma2_load_2d(base + S::OFF_B + s * S::B_STAGE, &tm_w, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * kLinBK, n0 + (int)rank * (BN / 2));
             }
             if (ok) {
                 // the residual tile goes last: it is not needed before the epilogue, and ahead of the main loop's operands it
@@ -433,16 +441,16 @@ bool linear_tc_supported(int dtype, int M, int K, int N)
 
 // impl: 0 = tensor cores where supported, 1 = plain kernel, 2 = tensor cores, the 256-row tiles whatever M is
 cudaError_t launch_linear_residual(const void *a, const void *W, const void *res, void *out, int M, int K, int N, int dtype, int impl,
-                                   uint32_t *status, cudaStream_t st)
+                                   uint32_t *status, bool early_w, cudaStream_t st)
 {
     const bool tc = impl != 1 && linear_tc_supported(dtype, M, K, N);
     if (!tc) {
         if ((size_t)K * sizeof(float) > 48 * 1024) return cudaErrorInvalidValue;
         return dtype == REFLEX_DTYPE_BF16 ? launch_lin_simt<__nv_bfloat16>(a, W, res, out, M, K, N, st) : launch_lin_simt<float>(a, W, res, out, M, K, N, st);
     }
-    if (impl == 0 && linear_small_takes(M, K, N)) return launch_linear_small(a, W, res, out, M, K, N, status, st);
+    if (impl == 0 && linear_small_takes(M, K, N)) return launch_linear_small(a, W, res, out, M, K, N, status, early_w, st);
     LinParams p;
-    p.M = M; p.K = K; p.N = N; p.m_tiles = (M + 2 * kLinBM - 1) / (2 * kLinBM); p.has_res = res ? 1 : 0; p.status = status;
+    p.M = M; p.K = K; p.N = N; p.m_tiles = (M + 2 * kLinBM - 1) / (2 * kLinBM); p.has_res = res ? 1 : 0; p.status = status; p.early_w = early_w ? 1 : 0;
     // 256-column tiles unless they would leave more than half of the SM pairs without one: then 128-column tiles, twice as
     // many pairs at work on a contraction that is as long (every CTA then fetches 24 KB per step for half the MMA work)
     const bool narrow = p.m_tiles * ((N + 255) / 256) * 2 <= 74;

@@ -75,6 +75,7 @@ struct QkParams {
     uint32_t *status;
     const __nv_bfloat16 *res;   // plain projection only (few-rows kernel with PLAIN): residual [M][nq] added to the output, or NULL
     int ksplit;                 // few-rows kernel: CTAs of a cluster that share one feature tile, each taking a slice of the contraction
+    int early;                  // weights and gates may be read before the preceding kernel is complete (inside an expert step)
     int tma_out;                // 256-row kernel: the output tile leaves through TMA stores (tensor maps over q / k / v given)
 };
 
@@ -159,6 +160,31 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     if (threadIdx.x == 64) QK_TRACE(2, 30, 0);
+    auto load_w = [&](int s, int ks, int n0) {
+        if (rank == 0) mbar_expect_tx(bar(Q_BFULL + s), 2 * S::B_STAGE);
+#pragma unroll
+        for (int j = 0; j < NACC; ++j)
+            tma2_load_2d(base + S::OFF_B + s * S::B_STAGE + j * S::B_HALF, &tm_w, bar(Q_BFULL + s) & kPeerBitMask, ks * kQkBK,
+                         (swiglu ? j * p.swiglu_F + n0 : n0 + j * kQkBN) + (int)rank * (kQkBN / 2));
+    };
+    // the gates of the streams under this CTA's 128 rows, [stream][D]
+    auto stage_gates = [&](int m0) {
+        const int b_first = min(m0 / p.R, p.B - 1), b_last = min((m0 + kQkBM - 1) / p.R, p.B - 1);
+        const int n4 = (b_last - b_first + 1) * p.D / 4;
+        const float4 *src = reinterpret_cast<const float4 *>(p.gate + (size_t)b_first * p.D);
+        float4 *gsm = reinterpret_cast<float4 *>(smem + S::OFF_GATE);
+        for (int i = threadIdx.x - 64; i < n4; i += 256) gsm[i] = src[i];
+    };
+    // Inside an expert step the weights and gates of the first tile are read before the wait for the preceding kernel: nothing in the step
+    // writes weights, and the gates come from kernels that were complete before the preceding one passed its own wait.
+    const int head = p.early && my_tiles > 0 ? (nk_steps < kQkStages ? nk_steps : kQkStages) : 0;
+    if (head > 0) {
+        if (threadIdx.x == 0) {
+            for (int ks = 0; ks < head; ++ks) load_w(ks, ks, tile_n0(0));
+        } else if (warp >= 2) {
+            stage_gates(tile_m0(0));
+        }
+    }
     // programmatic dependent launch: whatever produced x and the gate is complete from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -197,14 +223,6 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                     mbar_expect_tx(bar(Q_XFULL + s), S::X_STAGE);
                     tma_load_2d(base + S::OFF_X + s * S::X_STAGE, &tm_x, bar(Q_XFULL + s), ks * kQkBK, m0);
                 };
-                auto load_w = [&](int ks) {
-                    const int s = (g0 + ks) % kQkStages;
-                    if (rank == 0) mbar_expect_tx(bar(Q_BFULL + s), 2 * S::B_STAGE);
-#pragma unroll
-                    for (int j = 0; j < NACC; ++j)
-                        tma2_load_2d(base + S::OFF_B + s * S::B_STAGE + j * S::B_HALF, &tm_w, bar(Q_BFULL + s) & kPeerBitMask, ks * kQkBK,
-                                     (swiglu ? j * p.swiglu_F + n0 : n0 + j * kQkBN) + (int)rank * (kQkBN / 2));
-                };
                 int ks = 0;
                 if (it > 0) {
                     // head of a later tile: the weights of its first steps go out while the last tile's epilogue still owns the
@@ -214,7 +232,7 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                     if (w_staged) ok = wait(Q_STAGEFREE, ph, 7);
                     for (int h = 0; h < nh && ok; ++h) {
                         ok = stage_free(h);
-                        if (ok) load_w(h);
+                        if (ok) load_w((g0 + h) % kQkStages, h, n0);
                     }
                     if (ok && !w_staged) ok = wait(Q_STAGEFREE, ph, 7);
                     for (int h = 0; h < nh && ok; ++h) load_x(h);
@@ -225,7 +243,7 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                     if (!ok) break;
                     QK_TRACE(0, ks, 0);
                     load_x(ks);
-                    load_w(ks);
+                    if (it > 0 || ks >= head) load_w((g0 + ks) % kQkStages, ks, n0);
                 }
             }
         }
@@ -289,13 +307,9 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         // the gates of the streams under this CTA's 128 rows go to shared memory once per tile: every step needs 128 fresh bytes
         // of them per thread, and as global loads those were an L2 round trip per step on the critical path. (Every warp is
         // through with the last tile's gates: they are read in the step loop only, and all eight warps have met since.)
-        const int b_first = min(m0 / p.R, p.B - 1), b_last = min((m0 + kQkBM - 1) / p.R, p.B - 1);
-        {
-            const int n4 = (b_last - b_first + 1) * p.D / 4;
-            const float4 *src = reinterpret_cast<const float4 *>(p.gate + (size_t)b_first * p.D);
-            for (int i = threadIdx.x - 64; i < n4; i += 256) reinterpret_cast<float4 *>(gsm)[i] = __ldg(src + i);
-            asm volatile("bar.sync 1, 256;" ::: "memory");
-        }
+        const int b_first = min(m0 / p.R, p.B - 1);
+        if (it > 0 || head == 0) stage_gates(m0);
+        asm volatile("bar.sync 1, 256;" ::: "memory");
         const float *grow = gsm + (size_t)(b - b_first) * p.D + half * 32;
         uint64_t ss2 = 0ull;
         for (int ks = 0; ks < nk_steps; ++ks) {
@@ -567,6 +581,32 @@ norm_linear_small_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     if (threadIdx.x == 64) QK_TRACE(2, 30, 0);
+    // one barrier for both operands of a step: the threads that rewrite x wait for it, so their hand-over to the MMA warp also says
+    // that the weights are in place (one wait less per step in the issuing loop)
+    auto load_w = [&](int s, int ks) {
+        mbar_expect_tx(bar(S_XFULL + s), S::X_STAGE + S::W_STAGE);
+#pragma unroll
+        for (int cc = 0; cc < CPS; ++cc)
+#pragma unroll
+            for (int j = 0; j < NACC; ++j)
+                tma_load_2d(base + S::OFF_W + s * S::W_STAGE + (j * CPS + cc) * S::W_TILE, &tm_w, bar(S_XFULL + s), (chunk0 + ks * CPS + cc) * kQkBK, j * p.swiglu_F + f0);
+    };
+    auto stage_gates = [&]() {        // the gates of the streams under this group's rows (they fit: checked by the launcher)
+        const int b_first = min(row0 / p.R, p.B - 1), b_last = min((row0 + NT - 1) / p.R, p.B - 1);
+        const int n4 = (b_last - b_first + 1) * p.D / 4;
+        const float4 *src = reinterpret_cast<const float4 *>(p.gate + (size_t)b_first * p.D);
+        float4 *gsm = reinterpret_cast<float4 *>(smem + S::OFF_GATE);
+        for (int i = threadIdx.x - 64; i < n4; i += 256) gsm[i] = src[i];
+    };
+    // inside an expert step weights and gates are read ahead of the wait for the preceding kernel, as in the kernel above
+    const int head = p.early ? (nk_steps < kSmStages ? nk_steps : kSmStages) : 0;
+    if (head > 0) {
+        if (threadIdx.x == 0) {
+            for (int ks = 0; ks < head; ++ks) load_w(ks, ks);
+        } else if (!PLAIN && warp >= 2) {
+            stage_gates();
+        }
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (threadIdx.x == 64) QK_TRACE(2, 30, 1);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -594,17 +634,10 @@ norm_linear_small_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
                 const int s = ks % kSmStages;
                 if (ks >= kSmStages) ok = wait(S_EMPTY + s, (uint32_t)(ks / kSmStages - 1) & 1u, 1);
                 if (!ok) break;
-                // one barrier for both operands of the step: the threads that rewrite x wait for it, so their hand-over to the
-                // MMA warp also says that the weights are in place (one wait less per step in the issuing loop)
-                mbar_expect_tx(bar(S_XFULL + s), S::X_STAGE + S::W_STAGE);
+                if (ks >= head) load_w(s, ks);
 #pragma unroll
-                for (int cc = 0; cc < CPS; ++cc) {
-                    const int col = (chunk0 + ks * CPS + cc) * kQkBK;
-                    tma_load_2d(base + S::OFF_X + s * S::X_STAGE + cc * S::X_TILE, &tm_x, bar(S_XFULL + s), col, row0);
-#pragma unroll
-                    for (int j = 0; j < NACC; ++j)
-                        tma_load_2d(base + S::OFF_W + s * S::W_STAGE + (j * CPS + cc) * S::W_TILE, &tm_w, bar(S_XFULL + s), col, j * p.swiglu_F + f0);
-                }
+                for (int cc = 0; cc < CPS; ++cc)
+                    tma_load_2d(base + S::OFF_X + s * S::X_STAGE + cc * S::X_TILE, &tm_x, bar(S_XFULL + s), (chunk0 + ks * CPS + cc) * kQkBK, row0);
             }
         }
     } else if (warp == 1) {
@@ -643,12 +676,10 @@ norm_linear_small_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
         const int kpart = tid / NT;                    // which 64 / TP columns of every step
         constexpr int KW = kQkBK / TP;                 // columns per thread and step: 16 or 32
         const int b = min((row0 + row) / p.R, p.B - 1);
-        const int b_first = min(row0 / p.R, p.B - 1), b_last = min((row0 + NT - 1) / p.R, p.B - 1);   // streams under this group's rows
+        const int b_first = min(row0 / p.R, p.B - 1);
         float *gsm = reinterpret_cast<float *>(smem + S::OFF_GATE);
         if constexpr (!PLAIN) {
-            const int n4 = (b_last - b_first + 1) * p.D / 4;     // (they fit: checked by the launcher)
-            const float4 *src = reinterpret_cast<const float4 *>(p.gate + (size_t)b_first * p.D);
-            for (int i = tid; i < n4; i += 256) reinterpret_cast<float4 *>(gsm)[i] = __ldg(src + i);
+            if (head == 0) stage_gates();
             asm volatile("bar.sync 1, 256;" ::: "memory");
         }
         if (threadIdx.x == 64) QK_TRACE(2, 30, 2);
@@ -1033,7 +1064,7 @@ static cudaError_t launch_small(const CUtensorMap &mx, const CUtensorMap &mw, Qk
 // swiglu_F = 0: W = W_QKV, outputs q / k / v with nq and nk columns. swiglu_F = F > 0: W = [W_gate; W_up] ([2F][D]),
 // q = the [M][F] output SiLU(gate) * up; nq, nk, k, v unused.
 cudaError_t launch_adarmsnorm_qkv(const void *x, const float *gate, const void *W, void *q, void *k, void *v, int B, int R, int D, int nq, int nk,
-                                  int swiglu_F, float eps, int dtype, int impl, int sm_count, uint32_t *status, cudaStream_t st)
+                                  int swiglu_F, float eps, int dtype, int impl, int sm_count, uint32_t *status, bool early, cudaStream_t st)
 {
     const int M = B * R;
     if (swiglu_F > 0) { nq = swiglu_F; nk = 0; }
@@ -1065,7 +1096,7 @@ cudaError_t launch_adarmsnorm_qkv(const void *x, const float *gate, const void *
         QkParams sp;
         sp.gate = gate; sp.q = (__nv_bfloat16 *)q; sp.k = (__nv_bfloat16 *)k; sp.v = (__nv_bfloat16 *)v;
         sp.M = M; sp.R = R; sp.B = B; sp.D = D; sp.nq = nq; sp.nk = nk; sp.m_tiles = 1; sp.n_tiles = 1; sp.swiglu_F = swiglu_F;
-        sp.eps = eps; sp.status = status; sp.res = nullptr; sp.tma_out = 0;
+        sp.eps = eps; sp.status = status; sp.res = nullptr; sp.tma_out = 0; sp.early = early ? 1 : 0;
         // The contraction split over 4 CTAs per (feature tile, row group) where the chain has 8 steps or more and the grid stays
         // within the SMs, every slice keeping whole steps: the slices' sums meet through distributed shared memory, four
         // features per thread and all slices' loads in flight together (one stream: Q/K/V 6.4 -> 5.9 us, gate/up 11.1 -> 8.6;
@@ -1088,7 +1119,7 @@ cudaError_t launch_adarmsnorm_qkv(const void *x, const float *gate, const void *
     p.M = M; p.R = R; p.B = B; p.D = D; p.nq = nq; p.nk = nk;
     p.m_tiles = (M + 2 * kQkBM - 1) / (2 * kQkBM);
     p.swiglu_F = swiglu_F;
-    p.eps = eps; p.status = status; p.res = nullptr; p.ksplit = 1; p.tma_out = 0;
+    p.eps = eps; p.status = status; p.res = nullptr; p.ksplit = 1; p.tma_out = 0; p.early = early ? 1 : 0;
     if (swiglu_F > 0) return launch_tc<2>(mx, mw, p, (swiglu_F + kQkBN - 1) / kQkBN, sm_count, st);
     int nacc = qk_choose_nacc(M, R, D, nq + 2 * nk, sm_count > 0 ? sm_count : 148);
     if (impl == 2 && nacc == 2) nacc = 1;     // (forced 256-column tiles, for tests and timing)
@@ -1115,7 +1146,7 @@ bool linear_small_takes(int M, int K, int N)
     return K % kQkBK == 0 && linear_small_groups(M, K, N) > 0;
 }
 
-cudaError_t launch_linear_small(const void *a, const void *W, const void *res, void *out, int M, int K, int N, uint32_t *status, cudaStream_t st)
+cudaError_t launch_linear_small(const void *a, const void *W, const void *res, void *out, int M, int K, int N, uint32_t *status, bool early_w, cudaStream_t st)
 {
     const int ftiles = (N + 127) / 128;
     const int groups = linear_small_groups(M, K, N);
@@ -1125,7 +1156,7 @@ cudaError_t launch_linear_small(const void *a, const void *W, const void *res, v
     QkParams sp;
     sp.gate = nullptr; sp.q = (__nv_bfloat16 *)out; sp.k = nullptr; sp.v = nullptr;
     sp.M = M; sp.R = M; sp.B = 1; sp.D = K; sp.nq = N; sp.nk = 0; sp.m_tiles = 1; sp.n_tiles = 1; sp.swiglu_F = 0;
-    sp.eps = 0.f; sp.status = status; sp.res = (const __nv_bfloat16 *)res; sp.tma_out = 0;
+    sp.eps = 0.f; sp.status = status; sp.res = (const __nv_bfloat16 *)res; sp.tma_out = 0; sp.early = early_w ? 1 : 0;
     // split the contraction over up to 8 CTAs per (feature tile, row group) while every slice keeps whole steps of two 64-column
     // chunks and the grid stays within the SMs
     const int chunks = K / kQkBK;

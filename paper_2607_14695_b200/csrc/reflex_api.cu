@@ -397,8 +397,8 @@ int reflex_adarmsnorm_gate(const void *cond, const void *W1, const void *b1, con
     return REFLEX_OK;
 }
 
-int reflex_adarmsnorm_qkv(reflex_cache_t *c, const void *x, const float *gate, const void *Wqkv, void *q, void *k_dyn, void *v_dyn,
-                          int B, int R, int D, int Hq, int Hkv, int d, float eps, int dtype, int impl, void *stream)
+static int norm_qkv(reflex_cache_t *c, const void *x, const float *gate, const void *Wqkv, void *q, void *k_dyn, void *v_dyn,
+                          int B, int R, int D, int Hq, int Hkv, int d, float eps, int dtype, int impl, bool early, void *stream)
 {
     if (dtype != REFLEX_DTYPE_BF16 && dtype != REFLEX_DTYPE_F32) return fail(REFLEX_ERR_INVALID_ARG, "unknown dtype %d", dtype);
     if (impl < 0 || impl > 2) return fail(REFLEX_ERR_INVALID_ARG, "impl must be 0 (auto), 1 (plain kernel) or 2 (tensor cores, 256-column tiles)");
@@ -411,14 +411,20 @@ int reflex_adarmsnorm_qkv(reflex_cache_t *c, const void *x, const float *gate, c
     if (!aligned16(x) || !aligned16(gate) || !aligned16(Wqkv) || !aligned16(q) || !aligned16(k_dyn) || !aligned16(v_dyn))
         return fail(REFLEX_ERR_ALIGN, "x / gate / Wqkv / q / k_dyn / v_dyn not 16-byte aligned");
     uint32_t *status = c ? (uint32_t *)(c->ws + c->lay.status_off) : nullptr;
-    cudaError_t e = launch_adarmsnorm_qkv(x, gate, Wqkv, q, k_dyn, v_dyn, B, R, D, Hq * d, Hkv * d, 0, eps, dtype, impl, c ? c->sm_count : 0, status,
+    cudaError_t e = launch_adarmsnorm_qkv(x, gate, Wqkv, q, k_dyn, v_dyn, B, R, D, Hq * d, Hkv * d, 0, eps, dtype, impl, c ? c->sm_count : 0, status, early,
                                           (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "adarmsnorm qkv launch");
     return REFLEX_OK;
 }
 
-int reflex_adarmsnorm_swiglu(reflex_cache_t *c, const void *x, const float *gate, const void *Wgu, void *h, int B, int R, int D, int F,
-                             float eps, int dtype, int impl, void *stream)
+int reflex_adarmsnorm_qkv(reflex_cache_t *c, const void *x, const float *gate, const void *Wqkv, void *q, void *k_dyn, void *v_dyn,
+                          int B, int R, int D, int Hq, int Hkv, int d, float eps, int dtype, int impl, void *stream)
+{
+    return norm_qkv(c, x, gate, Wqkv, q, k_dyn, v_dyn, B, R, D, Hq, Hkv, d, eps, dtype, impl, false, stream);
+}
+
+static int norm_swiglu(reflex_cache_t *c, const void *x, const float *gate, const void *Wgu, void *h, int B, int R, int D, int F,
+                             float eps, int dtype, int impl, bool early, void *stream)
 {
     if (dtype != REFLEX_DTYPE_BF16 && dtype != REFLEX_DTYPE_F32) return fail(REFLEX_ERR_INVALID_ARG, "unknown dtype %d", dtype);
     if (impl != 0 && impl != 1) return fail(REFLEX_ERR_INVALID_ARG, "impl must be 0 (auto) or 1 (plain kernel)");
@@ -429,14 +435,20 @@ int reflex_adarmsnorm_swiglu(reflex_cache_t *c, const void *x, const float *gate
     if (!(eps >= 0.f)) return fail(REFLEX_ERR_INVALID_ARG, "eps must be >= 0");
     if (!aligned16(x) || !aligned16(gate) || !aligned16(Wgu) || !aligned16(h)) return fail(REFLEX_ERR_ALIGN, "x / gate / Wgu / h not 16-byte aligned");
     uint32_t *status = c ? (uint32_t *)(c->ws + c->lay.status_off) : nullptr;
-    cudaError_t e = launch_adarmsnorm_qkv(x, gate, Wgu, h, nullptr, nullptr, B, R, D, 0, 0, F, eps, dtype, impl, c ? c->sm_count : 0, status,
+    cudaError_t e = launch_adarmsnorm_qkv(x, gate, Wgu, h, nullptr, nullptr, B, R, D, 0, 0, F, eps, dtype, impl, c ? c->sm_count : 0, status, early,
                                           (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "adarmsnorm swiglu launch");
     return REFLEX_OK;
 }
 
-int reflex_linear_residual(reflex_cache_t *c, const void *a, const void *W, const void *res, void *out, int M, int K, int N, int dtype,
-                           int impl, void *stream)
+int reflex_adarmsnorm_swiglu(reflex_cache_t *c, const void *x, const float *gate, const void *Wgu, void *h, int B, int R, int D, int F,
+                             float eps, int dtype, int impl, void *stream)
+{
+    return norm_swiglu(c, x, gate, Wgu, h, B, R, D, F, eps, dtype, impl, false, stream);
+}
+
+static int linear_residual(reflex_cache_t *c, const void *a, const void *W, const void *res, void *out, int M, int K, int N, int dtype,
+                           int impl, bool early, void *stream)
 {
     if (dtype != REFLEX_DTYPE_BF16 && dtype != REFLEX_DTYPE_F32) return fail(REFLEX_ERR_INVALID_ARG, "unknown dtype %d", dtype);
     if (impl < 0 || impl > 2) return fail(REFLEX_ERR_INVALID_ARG, "impl must be 0 (auto), 1 (plain kernel) or 2 (tensor cores, 256-row tiles)");
@@ -447,9 +459,15 @@ int reflex_linear_residual(reflex_cache_t *c, const void *a, const void *W, cons
     if (!aligned16(a) || !aligned16(W) || !aligned16(out) || (res && !aligned16(res))) return fail(REFLEX_ERR_ALIGN, "a / W / res / out not 16-byte aligned");
     if (a == out) return fail(REFLEX_ERR_INVALID_ARG, "out may alias res, not a");
     uint32_t *status = c ? (uint32_t *)(c->ws + c->lay.status_off) : nullptr;
-    cudaError_t e = launch_linear_residual(a, W, res, out, M, K, N, dtype, impl, status, (cudaStream_t)stream);
+    cudaError_t e = launch_linear_residual(a, W, res, out, M, K, N, dtype, impl, status, early, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "linear residual launch");
     return REFLEX_OK;
+}
+
+int reflex_linear_residual(reflex_cache_t *c, const void *a, const void *W, const void *res, void *out, int M, int K, int N, int dtype,
+                           int impl, void *stream)
+{
+    return linear_residual(c, a, W, res, out, M, K, N, dtype, impl, false, stream);
 }
 
 static int attention(reflex_cache_t *c, int layer, const void *q, const void *k_dyn, const void *v_dyn, void *out, int T, float scale, int dyn_mask,
@@ -611,22 +629,23 @@ int reflex_expert_step(reflex_cache_t *c, const reflex_expert *ep, float *a, con
     int rc = reflex_adarmsnorm_gate(cond, e.W1, e.b1, e.W2, e.b2, e.gates, 2 * L + 1, B, D, e.Cd, e.Hd, dt_, stream);
     if (rc != REFLEX_OK) return rc;
     if (expert_chained(d, e)) return expert_step_chained(c, e, a, -1.0f / (float)K, stream);
-    // any other dtype or shape: the single calls in order
+    // any other dtype or shape: the single calls in order, allowed to read weights and gates ahead of the preceding kernel (nothing in
+    // the step writes weights; the gates are complete before the input projection starts)
     const size_t es = elem_size(dt_);
     auto off = [&](const void *p, size_t elems) -> const void * { return (const char *)p + elems * es; };
     auto gate = [&](int i) { return (const float *)e.gates + (size_t)i * B * D; };
     cudaError_t err = launch_cast(a, e.a_lowp, (size_t)M * e.A, dt_, (cudaStream_t)stream);
     if (err != cudaSuccess) return cuda_fail(err, "action chunk cast launch");
-    rc = reflex_linear_residual(c, e.a_lowp, e.W_in, nullptr, e.h, M, e.A, D, dt_, 0, stream);
+    rc = linear_residual(c, e.a_lowp, e.W_in, nullptr, e.h, M, e.A, D, dt_, 0, true, stream);
     for (int l = 0; l < L && rc == REFLEX_OK; ++l) {
-        rc = reflex_adarmsnorm_qkv(c, e.h, gate(2 * l), off(e.Wqkv, (size_t)l * (nq + 2 * nk) * D), e.q, e.k, e.v, B, T, D, d.Hq, d.Hkv, d.d, e.eps, dt_, 0, stream);
-        if (rc == REFLEX_OK) rc = reflex_partitioned_attention(c, l, e.q, e.k, e.v, e.o, T, 0.f, 0, stream);
-        if (rc == REFLEX_OK) rc = reflex_linear_residual(c, e.o, off(e.Wo, (size_t)l * D * nq), e.h, e.h, M, nq, D, dt_, 0, stream);
-        if (rc == REFLEX_OK) rc = reflex_adarmsnorm_swiglu(c, e.h, gate(2 * l + 1), off(e.Wgu, (size_t)l * 2 * e.F * D), e.m, B, T, D, e.F, e.eps, dt_, 0, stream);
-        if (rc == REFLEX_OK) rc = reflex_linear_residual(c, e.m, off(e.Wd, (size_t)l * D * e.F), e.h, e.h, M, e.F, D, dt_, 0, stream);
+        rc = norm_qkv(c, e.h, gate(2 * l), off(e.Wqkv, (size_t)l * (nq + 2 * nk) * D), e.q, e.k, e.v, B, T, D, d.Hq, d.Hkv, d.d, e.eps, dt_, 0, true, stream);
+        if (rc == REFLEX_OK) rc = attention(c, l, e.q, e.k, e.v, e.o, T, 0.f, 0, true, nullptr, stream);
+        if (rc == REFLEX_OK) rc = linear_residual(c, e.o, off(e.Wo, (size_t)l * D * nq), e.h, e.h, M, nq, D, dt_, 0, true, stream);
+        if (rc == REFLEX_OK) rc = norm_swiglu(c, e.h, gate(2 * l + 1), off(e.Wgu, (size_t)l * 2 * e.F * D), e.m, B, T, D, e.F, e.eps, dt_, 0, true, stream);
+        if (rc == REFLEX_OK) rc = linear_residual(c, e.m, off(e.Wd, (size_t)l * D * e.F), e.h, e.h, M, e.F, D, dt_, 0, true, stream);
     }
     if (rc == REFLEX_OK) rc = reflex_adarmsnorm(e.h, e.y, nullptr, nullptr, nullptr, nullptr, nullptr, (float *)gate(2 * L), B, T, D, 0, 0, e.eps, dt_, stream);
-    if (rc == REFLEX_OK) rc = reflex_linear_residual(c, e.y, e.W_out, nullptr, e.vel, M, D, e.A, dt_, 0, stream);
+    if (rc == REFLEX_OK) rc = linear_residual(c, e.y, e.W_out, nullptr, e.vel, M, D, e.A, dt_, 0, true, stream);
     if (rc == REFLEX_OK) rc = reflex_flow_step(a, e.vel, nullptr, B, T, e.A, k, K, dt_, stream);
     return rc;
 }

@@ -124,18 +124,19 @@ bool chain_attn_supported(const AttnParams &p, int sm_count);
 struct ChainPrefetch;
 cudaError_t launch_chain_attn(const AttnParams &p, uint32_t *status, bool early, const ChainPrefetch *pf, cudaStream_t st);
 // gate MLP of AdaRMSNorm on tcgen05 (bf16): false when the shapes or the driver do not allow it (the caller falls back)
+// early: inside an expert step weights and gates may be read before the preceding kernel on the stream is complete.
 // adaptive norm + packed Q/K/V projection (qkv_tc.cu). impl: 0 = tensor cores where supported, 1 = plain kernel,
 // 2 = tensor cores with 256-column tiles only
 bool norm_qkv_tc_supported(int dtype, int B, int R, int D, int nq, int nk);
 // swiglu_F > 0: W = [W_gate; W_up] and q receives SiLU(gate) * up, [B*R][F]
 cudaError_t launch_adarmsnorm_qkv(const void *x, const float *gate, const void *W, void *q, void *k, void *v, int B, int R, int D, int nq, int nk,
-                                  int swiglu_F, float eps, int dtype, int impl, int sm_count, uint32_t *status, cudaStream_t st);
+                                  int swiglu_F, float eps, int dtype, int impl, int sm_count, uint32_t *status, bool early, cudaStream_t st);
 // plain projection with residual (linear_tc.cu): out [M][N] = res + a [M][K] W [N][K]^T. impl: 0 = tensor cores where supported,
 // 1 = plain kernel, 2 = tensor cores with 256-row tiles whatever M is
 cudaError_t launch_linear_residual(const void *a, const void *W, const void *res, void *out, int M, int K, int N, int dtype, int impl,
-                                   uint32_t *status, cudaStream_t st);
+                                   uint32_t *status, bool early_w, cudaStream_t st);
 bool linear_small_takes(int M, int K, int N);
-cudaError_t launch_linear_small(const void *a, const void *W, const void *res, void *out, int M, int K, int N, uint32_t *status, cudaStream_t st);
+cudaError_t launch_linear_small(const void *a, const void *W, const void *res, void *out, int M, int K, int N, uint32_t *status, bool early_w, cudaStream_t st);
 bool gate_tc_supported(int B, int D, int Cd, int Hd);
 cudaError_t launch_gate_tc(const void *cond, const void *W1, const void *b1, const void *W2, const void *b2, float *gate_buf, int L, int B,
                            int D, int Cd, int Hd, cudaStream_t st);
