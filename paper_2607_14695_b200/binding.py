@@ -8,7 +8,6 @@ from __future__ import annotations
 
 import ctypes
 import os
-from array import array
 from typing import Optional, Sequence
 
 import torch
@@ -62,6 +61,7 @@ class ReflexError(RuntimeError):
 
 
 _lib = None
+_marshal = None
 
 
 def load():
@@ -71,7 +71,7 @@ def load():
         return _lib
     if not os.path.exists(LIB_PATH):
         raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2607_14695_b200.build`")
-    lib = ctypes.CDLL(LIB_PATH)
+    lib = ctypes.CDLL(LIB_PATH, mode=ctypes.RTLD_GLOBAL)      # (the marshalling module takes its symbols from here)
     vp, i, f = ctypes.c_void_p, ctypes.c_int, ctypes.c_float
     i32p, i64p = ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int64)
     dp = ctypes.POINTER(CacheDesc)
@@ -112,14 +112,25 @@ def load():
     return lib
 
 
+def _native():
+    """The native marshalling of the calls that a control loop makes many times per tick."""
+    global _marshal
+    if _marshal is None:
+        load()
+        from . import _marshal as m      # built beside the library; there is no fallback
+        _marshal = m
+    return _marshal
+
+
+def _handle(cache) -> Optional[int]:
+    return None if cache is None or cache.handle is None else cache.handle.value
+
+
 def _check(rc: int):
     if rc != OK:
         raise ReflexError(rc, load().reflex_last_error_string().decode())
 
 
-# A direct call costs the host its marshalling: pointers, streams and id lists therefore go through as plain integers (the argument
-# types convert them in C), and nothing is built per call that is not needed (tick of the tiny configuration, 18 calls: 190 us of
-# host time with a ctypes object per argument and a torch Stream per call).
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
         return None
@@ -134,24 +145,10 @@ def _stream(stream) -> int:
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
-class _I32(array):
-    """Host int32 array that a c_void_p parameter takes (ctypes keeps the argument alive for the call)."""
-
-    def __new__(cls, seq):
-        return array.__new__(cls, "i", seq)
-
-    @property
-    def _as_parameter_(self):
-        return self.buffer_info()[0]
-
-
 def _i32(seq: Optional[Sequence[int]]):
     if seq is None:
         return None
-    try:
-        return _I32(seq)
-    except TypeError:
-        return _I32([int(v) for v in seq])
+    return (ctypes.c_int32 * len(seq))(*[int(v) for v in seq])
 
 
 def torch_dtype(dtype: int) -> torch.dtype:
@@ -246,41 +243,39 @@ def reflex_cache_selftest_wait_limit(cache: Cache, limit_us: int = 2000, stream=
 
 def reflex_cache_init_static(cache: Cache, stream_ids, k_static, v_static, S=None, stream=None):
     """k_static, v_static: device [n][L][S_src][Hkv][d]."""
-    n = len(stream_ids)
-    S_src = int(k_static.shape[2]) if k_static is not None else 0
-    _check(load().reflex_cache_init_static(cache.handle, _i32(stream_ids), n, _ptr(k_static), _ptr(v_static), S_src,
-                                           _i32(S), _stream(stream)))
+    rc = _native().write_static(0, _handle(cache), stream_ids, k_static, v_static, S, stream)
+    if rc:
+        _check(rc)
 
 
 def reflex_cache_stage_static(cache: Cache, stream_ids, k_static, v_static, S=None, stream=None):
     """Write a new prefix into the static bank that attention is not reading (cache created with static_banks=2)."""
-    n = len(stream_ids)
-    S_src = int(k_static.shape[2]) if k_static is not None else 0
-    _check(load().reflex_cache_stage_static(cache.handle, _i32(stream_ids), n, _ptr(k_static), _ptr(v_static), S_src,
-                                            _i32(S), _stream(stream)))
+    rc = _native().write_static(1, _handle(cache), stream_ids, k_static, v_static, S, stream)
+    if rc:
+        _check(rc)
 
 
 def reflex_cache_commit_static(cache: Cache, stream_ids, stream=None):
     """Make the staged prefix of these streams the one attention reads (index flip on `stream`)."""
-    _check(load().reflex_cache_commit_static(cache.handle, _i32(stream_ids), len(stream_ids), _stream(stream)))
+    rc = _native().commit_static(_handle(cache), stream_ids, stream)
+    if rc:
+        _check(rc)
 
 
 def reflex_cache_append_sliding(cache: Cache, stream_ids, k_new, v_new, stream=None):
     """k_new, v_new: device [n][L][m][Hkv][d]. Returns the per-stream eviction counts."""
-    n = len(stream_ids)
-    m = int(k_new.shape[2])
-    ev = _I32(bytes(4 * n))
-    _check(load().reflex_cache_append_sliding(cache.handle, _i32(stream_ids), n, _ptr(k_new), _ptr(v_new), m, ev, _stream(stream)))
-    return list(ev)
+    out = _native().append_sliding(_handle(cache), stream_ids, k_new, v_new, stream)
+    if type(out) is int:
+        _check(out)
+    return out
 
 
 def reflex_adarmsnorm(x, y, cond, W1, b1, W2, b2, gate_buf=None, eps=1e-6, stream=None):
     """x, y [B][R][D]; cond [B][Cd] or None (then gate_buf [B][D] fp32 is the precomputed gate).
     With cond given, gate_buf (optional) must hold B*(D+Hd) floats: gate, then hidden-layer scratch."""
-    B, R, D = x.shape
-    Hd, Cd = (W1.shape if W1 is not None else (0, 0))
-    _check(load().reflex_adarmsnorm(_ptr(x), _ptr(y), _ptr(cond), _ptr(W1), _ptr(b1), _ptr(W2), _ptr(b2), _ptr(gate_buf),
-                                    B, R, D, int(Cd), int(Hd), float(eps), dtype_code(x), _stream(stream)))
+    rc = _native().adarmsnorm(x, y, cond, W1, b1, W2, b2, gate_buf, eps, stream)
+    if rc:
+        _check(rc)
     return y
 
 
@@ -294,9 +289,9 @@ def _gate_dims(cond, W1, W2):
 def reflex_adarmsnorm_gate(cond, W1, b1, W2, b2, gate_buf, stream=None):
     """gate_buf[:L*B*D] <- 1 + W2_l SiLU(W1_l c + b1_l) + b2_l (fp32) for the L stacked layers; gate_buf holds
     L*B*(D+Hd) floats."""
-    L, B, D, Cd, Hd = _gate_dims(cond, W1, W2)
-    _check(load().reflex_adarmsnorm_gate(_ptr(cond), _ptr(W1), _ptr(b1), _ptr(W2), _ptr(b2), _ptr(gate_buf), L, B, D, Cd, Hd,
-                                         dtype_code(cond), _stream(stream)))
+    rc = _native().adarmsnorm_gate(cond, W1, b1, W2, b2, gate_buf, stream)
+    if rc:
+        _check(rc)
     return gate_buf
 
 
@@ -312,26 +307,25 @@ def reflex_adarmsnorm_noalloc(x, y, cond, W1, b1, W2, b2, eps=1e-6, stream=None)
 
 def reflex_adarmsnorm_qkv(x, gate, Wqkv, q, k_dyn, v_dyn, eps=1e-6, impl=0, cache=None, stream=None):
     """x [B][R][D], gate fp32 [B][D], Wqkv [(Hq + 2 Hkv) d][D] -> q [B][R][Hq][d], k_dyn / v_dyn [B][R][Hkv][d]."""
-    B, R, D = x.shape
-    Hq, d = int(q.shape[2]), int(q.shape[3])
-    Hkv = int(k_dyn.shape[2])
-    _check(load().reflex_adarmsnorm_qkv(cache.handle if cache is not None else None, _ptr(x), _ptr(gate), _ptr(Wqkv), _ptr(q), _ptr(k_dyn),
-                                        _ptr(v_dyn), B, R, D, Hq, Hkv, d, float(eps), dtype_code(x), int(impl), _stream(stream)))
+    rc = _native().adarmsnorm_qkv(_handle(cache), x, gate, Wqkv, q, k_dyn, v_dyn, eps, impl, stream)
+    if rc:
+        _check(rc)
     return q, k_dyn, v_dyn
 
 
 def reflex_partitioned_attention(cache: Cache, layer, q, k_dyn, v_dyn, out, scale=0.0, dyn_mask=0, stream=None):
     """q, out [B][T][Hq][d]; k_dyn, v_dyn [B][T][Hkv][d]."""
-    T = int(q.shape[1])
-    _check(load().reflex_partitioned_attention(cache.handle, int(layer), _ptr(q), _ptr(k_dyn), _ptr(v_dyn), _ptr(out), T,
-                                               float(scale), int(dyn_mask), _stream(stream)))
+    rc = _native().partitioned_attention(_handle(cache), layer, q, k_dyn, v_dyn, out, scale, dyn_mask, stream)
+    if rc:
+        _check(rc)
     return out
 
 
 def reflex_flow_step(x, v, x_lowp, k, K, stream=None):
     """x [B][T][A] fp32 in place; v [B][T][A] storage dtype; x_lowp optional mirror."""
-    B, T, A = x.shape
-    _check(load().reflex_flow_step(_ptr(x), _ptr(v), _ptr(x_lowp), B, T, A, int(k), int(K), dtype_code(v), _stream(stream)))
+    rc = _native().flow_step(x, v, x_lowp, k, K, stream)
+    if rc:
+        _check(rc)
     return x
 
 
@@ -375,19 +369,17 @@ def prepare_adarmsnorm_gate(cond, W1, b1, W2, b2, gate_buf):
 
 def reflex_adarmsnorm_swiglu(x, gate, Wgu, h, eps=1e-6, impl=0, cache=None, stream=None):
     """x [B][R][D], gate fp32 [B][D], Wgu [2F][D] = [W_gate; W_up] -> h [B][R][F] = SiLU(y W_gate^T) * (y W_up^T)."""
-    B, R, D = x.shape
-    F = int(h.shape[2])
-    _check(load().reflex_adarmsnorm_swiglu(cache.handle if cache is not None else None, _ptr(x), _ptr(gate), _ptr(Wgu), _ptr(h), B, R, D, F,
-                                           float(eps), dtype_code(x), int(impl), _stream(stream)))
+    rc = _native().adarmsnorm_swiglu(_handle(cache), x, gate, Wgu, h, eps, impl, stream)
+    if rc:
+        _check(rc)
     return h
 
 
 def reflex_linear_residual(a, W, res, out, impl=0, cache=None, stream=None):
     """a [..., K] (all leading axes are rows), W [N][K], res [..., N] or None -> out [..., N] = res + a W^T; out may be res."""
-    K, N = int(a.shape[-1]), int(W.shape[0])
-    M = a.numel() // K
-    _check(load().reflex_linear_residual(cache.handle if cache is not None else None, _ptr(a), _ptr(W), _ptr(res), _ptr(out), M, K, N,
-                                         dtype_code(a), int(impl), _stream(stream)))
+    rc = _native().linear_residual(_handle(cache), a, W, res, out, impl, stream)
+    if rc:
+        _check(rc)
     return out
 
 

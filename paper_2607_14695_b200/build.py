@@ -1,4 +1,4 @@
-"""Builds libreflex_b200.so (the C-ABI library, sm_100a only) in-tree with nvcc.
+"""Builds libreflex_b200.so (the C-ABI library, sm_100a only) and the binding's argument marshalling (_marshal, plain C++) in-tree.
 
     python -m paper_2607_14695_b200.build [--force] [--verbose]
 
@@ -11,11 +11,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libreflex_b200.so")
+MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
+MARSHAL = os.path.join(HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 
 def sources():
@@ -37,7 +40,25 @@ def nvcc_path() -> str:
     return "nvcc"
 
 
+def build_marshal(force: bool = False) -> str:
+    """The marshalling module takes the library's symbols from the process (binding.load() opens the library first)."""
+    deps = (MARSHAL_SRC, os.path.join(ROOT, "include", "reflex.h"))
+    if not force and os.path.exists(MARSHAL) and all(os.path.getmtime(p) <= os.path.getmtime(MARSHAL) for p in deps):
+        return MARSHAL
+    import torch
+    torch_dir = os.path.dirname(torch.__file__)
+    tmp = MARSHAL + f".tmp{os.getpid()}"
+    cuda = os.path.dirname(os.path.dirname(nvcc_path())) or "/usr/local/cuda"
+    inc = [sysconfig.get_paths()["include"], os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include"), os.path.join(ROOT, "include")]
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] +
+                          [f"-I{p}" for p in inc] + ["-o", tmp, MARSHAL_SRC, "-L" + os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
+    os.replace(tmp, MARSHAL)
+    return MARSHAL
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_marshal(force)
     if not force and not _stale():
         return LIB
     tmp = LIB + f".tmp{os.getpid()}"
