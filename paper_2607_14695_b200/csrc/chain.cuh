@@ -56,6 +56,12 @@ struct ChainProj {
 // Do the chain's projections take this shape (all CTAs of the launch on the SMs at once)?
 bool chain_proj_supported(int mode, int M, int K, int N);
 cudaError_t launch_chain_proj(const ChainProj &p, cudaStream_t st);
+// The same projections for many rows: CG_QKV and CG_SWIGLU (tile_gemm.cu), CG_RES (linear_tc.cu; N a multiple of 256, tile_res_slots
+// partial sums of squares per row)
+bool tile_proj_supported(int mode, int M, int K, int nq, int nk, int F);
+cudaError_t launch_tile_proj(const ChainProj &p, cudaStream_t st);
+cudaError_t launch_tile_res(const ChainProj &p, cudaStream_t st);
+int tile_res_slots(int M, int K, int N);
 // h = bf16(a) W_in^T, xg = h * gate, ss_out [M] (one partial sum per row)
 cudaError_t launch_chain_in(const float *a, const __nv_bfloat16 *W_in, const float *gate, __nv_bfloat16 *h, __nv_bfloat16 *xg, float *ss_out, int B,
                             int R, int D, int A, cudaStream_t st);

@@ -475,7 +475,7 @@ cudaError_t cg_launch_mode(int mode, const CgConfig &c, const CUtensorMap &mx, c
 bool chain_proj_supported(int mode, int M, int K, int N)
 {
     CgConfig c;
-    return M >= 1 && M <= kCgMaxRows && K % 8 == 0 && N % 8 == 0 && cg_choose(mode, M, K, N, c);
+    return M >= 1 && (M <= kCgMaxRows || mode == CG_OUT) && K % 8 == 0 && N % 8 == 0 && cg_choose(mode, M, K, N, c);
 }
 
 cudaError_t launch_chain_proj(const ChainProj &a, cudaStream_t st)
@@ -507,67 +507,76 @@ cudaError_t launch_chain_proj(const ChainProj &a, cudaStream_t st)
 // ---- head of the step: the action chunk to tokens --------------------------------------------------------------------------
 namespace {
 
-constexpr int kCiRows = 4;       // rows per block
+constexpr int kCiRows = 4;       // rows at a time
 
-// h = bf16(a) W_in^T with a contraction of A <= 32: fp32 FMAs, four features per thread (their weights in registers before the
-// wait), kCiRows rows per block; the block holds whole rows, so it finishes their sums of squares.
+// h = bf16(a) W_in^T with a contraction of A <= 32: fp32 FMAs, four features per thread, their weights in registers for all the row groups
+// of the block; the block holds whole rows, so it finishes their sums of squares. (One group per block read the 64 KB of weights once
+// for every four rows: 27 us for 3200 rows.)
 template <int A>
 __global__ void __launch_bounds__(256)
 chain_in_kernel(const float *__restrict__ a, const __nv_bfloat16 *__restrict__ W, const float *__restrict__ gate, __nv_bfloat16 *__restrict__ h,
-                __nv_bfloat16 *__restrict__ xg, float *__restrict__ ss_out, int M, int R, int D)
+                __nv_bfloat16 *__restrict__ xg, float *__restrict__ ss_out, int M, int R, int D, int groups)
 {
-    __shared__ float as[kCiRows][A];
+    __shared__ __align__(16) float as[kCiRows][A];
     __shared__ float part[kCiRows][8];
+    uint4 w[4][A / 8];                                 // features f .. f + 3 of the first 1024
+    const int f0 = threadIdx.x * 4;
+    auto load_w = [&](int f) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int k8 = 0; k8 < A / 8; ++k8) w[j][k8] = f < D ? *reinterpret_cast<const uint4 *>(W + (size_t)(f + j) * A + k8 * 8) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    load_w(f0);                                        // (weights: nothing in a step writes them)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int row0 = blockIdx.x * kCiRows;
-    for (int i = threadIdx.x; i < kCiRows * A; i += 256) {
-        const int r = row0 + i / A;
-        as[i / A][i % A] = r < M ? __bfloat162float(__float2bfloat16_rn(a[(size_t)r * A + i % A])) : 0.f;
-    }
-    __syncthreads();
-    float ss[kCiRows];
+#pragma unroll 1
+    for (int g = 0; g < groups; ++g) {
+        const int row0 = (blockIdx.x * groups + g) * kCiRows;
+        if (row0 >= M) break;
+        for (int i = threadIdx.x; i < kCiRows * A; i += 256) {
+            const int r = row0 + i / A;
+            as[i / A][i % A] = r < M ? __bfloat162float(__float2bfloat16_rn(a[(size_t)r * A + i % A])) : 0.f;
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int fb = 0; fb < D; fb += 1024) {
+            const int f = fb + f0;
+            if (D > 1024) load_w(f);
+#pragma unroll 1
+            for (int r = 0; r < kCiRows; ++r) {
+                float ss = 0.f;
+                if (f < D && row0 + r < M) {
+                    float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int r = 0; r < kCiRows; ++r) ss[r] = 0.f;
-    for (int f = threadIdx.x * 4; f < D; f += 1024) {
-        float acc[kCiRows][4];
+                    for (int k8 = 0; k8 < A / 8; ++k8) {
+                        const float4 a0 = *reinterpret_cast<const float4 *>(&as[r][k8 * 8]), a1 = *reinterpret_cast<const float4 *>(&as[r][k8 * 8 + 4]);
+                        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
 #pragma unroll
-        for (int r = 0; r < kCiRows; ++r) { acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f; }
+                        for (int j = 0; j < 4; ++j) {
+                            const uint32_t ww[4] = {w[j][k8].x, w[j][k8].y, w[j][k8].z, w[j][k8].w};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-#pragma unroll
-            for (int k8 = 0; k8 < A / 8; ++k8) {
-                const uint4 w = *reinterpret_cast<const uint4 *>(W + (size_t)(f + j) * A + k8 * 8);
-                const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float w0 = __uint_as_float(ww[i] << 16), w1 = __uint_as_float(ww[i] & 0xFFFF0000u);
-#pragma unroll
-                    for (int r = 0; r < kCiRows; ++r) acc[r][j] = fmaf(as[r][k8 * 8 + 2 * i + 1], w1, fmaf(as[r][k8 * 8 + 2 * i], w0, acc[r][j]));
+                            for (int i = 0; i < 4; ++i)
+                                acc[j] = fmaf(av[2 * i + 1], __uint_as_float(ww[i] & 0xFFFF0000u), fmaf(av[2 * i], __uint_as_float(ww[i] << 16), acc[j]));
+                        }
+                    }
+                    const uint2 hv = pack4_bf16(acc[0], acc[1], acc[2], acc[3]);
+                    const float4 h4 = unpack4_bf16(hv), g4 = *reinterpret_cast<const float4 *>(gate + (size_t)((row0 + r) / R) * D + f);
+                    const size_t o = (size_t)(row0 + r) * D + f;
+                    *reinterpret_cast<uint2 *>(h + o) = hv;
+                    *reinterpret_cast<uint2 *>(xg + o) = pack4_bf16(h4.x * g4.x, h4.y * g4.y, h4.z * g4.z, h4.w * g4.w);
+                    ss = fmaf(h4.x, h4.x, fmaf(h4.y, h4.y, fmaf(h4.z, h4.z, h4.w * h4.w)));
                 }
+                for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                if ((threadIdx.x & 31) == 0) part[r][threadIdx.x >> 5] = fb == 0 ? ss : part[r][threadIdx.x >> 5] + ss;
             }
         }
-#pragma unroll
-        for (int r = 0; r < kCiRows; ++r) {
-            if (row0 + r >= M) continue;
-            const uint2 hv = pack4_bf16(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-            const float4 h4 = unpack4_bf16(hv), g4 = *reinterpret_cast<const float4 *>(gate + (size_t)((row0 + r) / R) * D + f);
-            const size_t o = (size_t)(row0 + r) * D + f;
-            *reinterpret_cast<uint2 *>(h + o) = hv;
-            *reinterpret_cast<uint2 *>(xg + o) = pack4_bf16(h4.x * g4.x, h4.y * g4.y, h4.z * g4.z, h4.w * g4.w);
-            ss[r] = fmaf(h4.x, h4.x, fmaf(h4.y, h4.y, fmaf(h4.z, h4.z, fmaf(h4.w, h4.w, ss[r]))));
+        __syncthreads();
+        if (threadIdx.x < kCiRows && row0 + (int)threadIdx.x < M) {
+            float s = 0.f;
+            for (int x = 0; x < 8; ++x) s += part[threadIdx.x][x];
+            ss_out[row0 + threadIdx.x] = s;
         }
-    }
-#pragma unroll
-    for (int r = 0; r < kCiRows; ++r) {
-        for (int o = 16; o > 0; o >>= 1) ss[r] += __shfl_xor_sync(0xffffffffu, ss[r], o);
-        if ((threadIdx.x & 31) == 0) part[r][threadIdx.x >> 5] = ss[r];
-    }
-    __syncthreads();
-    if (threadIdx.x < kCiRows && row0 + (int)threadIdx.x < M) {
-        float s = 0.f;
-        for (int w = 0; w < 8; ++w) s += part[threadIdx.x][w];
-        ss_out[row0 + threadIdx.x] = s;
     }
 }
 
@@ -578,7 +587,8 @@ cudaError_t launch_chain_in(const float *a, const __nv_bfloat16 *W_in, const flo
 {
     const int M = B * R;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((M + kCiRows - 1) / kCiRows));
+    const int all = (M + kCiRows - 1) / kCiRows, groups = (all + 295) / 296;       // about two blocks per SM
+    cfg.gridDim = dim3((unsigned)((all + groups - 1) / groups));
     cfg.blockDim = dim3(256);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -588,9 +598,9 @@ cudaError_t launch_chain_in(const float *a, const __nv_bfloat16 *W_in, const flo
     cfg.numAttrs = 1;
     cudaError_t e;
     switch (A) {
-        case 8: e = cudaLaunchKernelEx(&cfg, chain_in_kernel<8>, a, W_in, gate, h, xg, ss_out, M, R, D); break;
-        case 16: e = cudaLaunchKernelEx(&cfg, chain_in_kernel<16>, a, W_in, gate, h, xg, ss_out, M, R, D); break;
-        case 32: e = cudaLaunchKernelEx(&cfg, chain_in_kernel<32>, a, W_in, gate, h, xg, ss_out, M, R, D); break;
+        case 8: e = cudaLaunchKernelEx(&cfg, chain_in_kernel<8>, a, W_in, gate, h, xg, ss_out, M, R, D, groups); break;
+        case 16: e = cudaLaunchKernelEx(&cfg, chain_in_kernel<16>, a, W_in, gate, h, xg, ss_out, M, R, D, groups); break;
+        case 32: e = cudaLaunchKernelEx(&cfg, chain_in_kernel<32>, a, W_in, gate, h, xg, ss_out, M, R, D, groups); break;
         default: return cudaErrorInvalidValue;
     }
     count_launch();

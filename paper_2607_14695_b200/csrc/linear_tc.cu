@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "chain.cuh"
 #include "reflex_internal.cuh"
 #include "sm100_ptx.cuh"
 
@@ -54,6 +55,11 @@ struct LinSmem {
 
 struct LinParams {
     int early_w;        // weights may be asked for before the preceding kernel is complete
+    // Inside an expert step of many rows the epilogue also writes what the norm that follows needs of this residual stream: out * gate
+    // (through tm_xg) and every row's sums of squares over the columns of one thread, [M][slots].
+    const float *gate;  // [B][N], or NULL: none of that
+    float *ss_out;
+    int R, B, slots;
     int M, K, N;
     int m_tiles;          // 256-row tiles
     int has_res;
@@ -74,6 +80,52 @@ __device__ __forceinline__ void lin_tma2_load_2d(uint32_t dst, const CUtensorMap
                  ::"r"(dst), "l"(map), "r"(leader_bar), "r"(c0), "r"(c1)
                  : "memory");
 }
+__device__ __forceinline__ float lin_sum2(uint64_t v) { float a, b; unpack_f32x2(v, a, b); return a + b; }
+
+// The gates of the streams under a CTA's 128 rows, columns [n0, n0 + W), on their way to shared memory: the first ones in registers before
+// the accumulator is final, stored once the operand stages are idle. (Read from global memory by the threads as they need them, each
+// piece of eight columns was a round trip to the L2: +3.5 to 5.4 us per launch.)
+template <int W>
+struct LinGates {
+    float4 v[2];
+    __device__ __forceinline__ int count(const LinParams &p, int b_first, int m0) const { return (min((m0 + kLinBM - 1) / p.R, p.B - 1) - b_first + 1) * (W / 4); }
+    __device__ __forceinline__ float4 fetch(const LinParams &p, int b_first, int n0, int i) const
+    {
+        return *reinterpret_cast<const float4 *>(p.gate + (size_t)(b_first + i / (W / 4)) * p.N + n0 + (i % (W / 4)) * 4);
+    }
+    __device__ __forceinline__ void load(const LinParams &p, int b_first, int m0, int n0, int t)
+    {
+        const int n = count(p, b_first, m0);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (t + j * 256 < n) v[j] = fetch(p, b_first, n0, t + j * 256);
+    }
+    __device__ __forceinline__ void store(const LinParams &p, int b_first, int m0, int n0, int t, float *dst) const
+    {
+        const int n = count(p, b_first, m0);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (t + j * 256 < n) reinterpret_cast<float4 *>(dst)[t + j * 256] = v[j];
+        for (int i = t + 512; i < n; i += 256) reinterpret_cast<float4 *>(dst)[i] = fetch(p, b_first, n0, i);
+    }
+};
+// Eight columns of the new residual stream, as packed fp32 pairs before their rounding: times the gate into the swizzled staging chunk,
+// squares into ss.
+__device__ __forceinline__ void lin_gated_piece(const uint64_t (&v)[4], const float *gate, uint8_t *dst, uint64_t &ss)
+{
+    const ulonglong2 ga = *reinterpret_cast<const ulonglong2 *>(gate), gb = *reinterpret_cast<const ulonglong2 *>(gate + 4);
+    const uint64_t g[4] = {ga.x, ga.y, gb.x, gb.y};
+    uint32_t o[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        ss = fma_f32x2(v[k], v[k], ss);
+        float x0, x1;
+        unpack_f32x2(mul_f32x2(v[k], g[k]), x0, x1);
+        __nv_bfloat162 x = __floats2bfloat162_rn(x0, x1);
+        o[k] = *reinterpret_cast<uint32_t *>(&x);
+    }
+    *reinterpret_cast<uint4 *>(dst) = make_uint4(o[0], o[1], o[2], o[3]);
+}
 __device__ __forceinline__ void lin_tma_store_2d(const CUtensorMap *map, uint32_t src, int c0, int c1)
 {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");
@@ -86,7 +138,8 @@ __device__ __forceinline__ void lin_tma_store_2d(const CUtensorMap *map, uint32_
 template <int BN, int KS>
 __global__ void __launch_bounds__(kLinThreads, 1)
 linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
-                     const __grid_constant__ CUtensorMap tm_res, const __grid_constant__ CUtensorMap tm_out, LinParams p)
+                     const __grid_constant__ CUtensorMap tm_res, const __grid_constant__ CUtensorMap tm_out, const __grid_constant__ CUtensorMap tm_xg,
+                     LinParams p)
 {
     static_assert(KS == 1 || (KS == 2 && BN == 128), "contraction split");
     using S = LinSmem<BN>;
@@ -248,13 +301,26 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             rr[j] = make_uint4(0u, 0u, 0u, 0u);
             if (p.has_res) rr[j] = *reinterpret_cast<const uint4 *>(smem + S::OFF_RES + (half * CPT + j / 8) * S::CHUNK + row * 128 + (((j & 7) ^ (row & 7)) << 4));
         }
+        LinGates<BN> gates;
+        const int b_first = p.gate ? min(m0 / p.R, p.B - 1) : 0;
+        if (p.gate) gates.load(p, b_first, m0, n0, threadIdx.x - 64);
         ok = wait(S::C_ACC, 0u, 4) && ok;
         if (threadIdx.x == 64) LIN_TRACE(4);
         tc_fence_after();
+        uint64_t ss2 = 0ull;
+        const float *grow = nullptr;                  // this row's gates, in the idle stages of W
+        if (p.gate) {
+            float *gsm = reinterpret_cast<float *>(smem + S::OFF_B);
+            gates.store(p, b_first, m0, n0, threadIdx.x - 64, gsm);
+            grow = gsm + (size_t)(min((m0 + row) / p.R, p.B - 1) - b_first) * BN;
+            asm volatile("bar.sync 3, 256;" ::: "memory");
+        }
+        static_assert(S::NST * S::A_STAGE >= S::RES_BYTES, "the idle operand stages hold the gated tile");
 #pragma unroll
         for (int cc = 0; cc < CPT; ++cc) {
             const int ch = half * CPT + cc;
             uint8_t *rowp = smem + S::OFF_RES + ch * S::CHUNK + row * 128;
+            uint8_t *xrowp = smem + S::OFF_A + ch * S::CHUNK + row * 128;
 #pragma unroll
             for (int g = 0; g < 2; ++g) {             // 32 columns at a time
                 uint32_t acc[32];
@@ -265,14 +331,17 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
                     const uint4 t = rr[cc * 8 + g * 4 + i];
                     const uint32_t rv[4] = {t.x, t.y, t.z, t.w};
                     uint32_t ov[4];
+                    uint64_t vv[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         float v0 = __uint_as_float(acc[8 * i + 2 * k]) + __uint_as_float(rv[k] << 16);
                         float v1 = __uint_as_float(acc[8 * i + 2 * k + 1]) + __uint_as_float(rv[k] & 0xFFFF0000u);
                         if (!ok) v0 = v1 = __int_as_float(0x7fc00000);   // a wait ran out: the tile is marked invalid, not left stale
+                        vv[k] = pack_f32x2(v0, v1);
                         __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
                         ov[k] = *reinterpret_cast<uint32_t *>(&h);
                     }
+                    if (grow) lin_gated_piece(vv, grow + ch * 64 + g * 32 + i * 8, xrowp + (((g * 4 + i) ^ (row & 7)) << 4), ss2);
                     // 128-byte swizzle of the TMA box: 16-byte piece j of row r sits at j ^ (r % 8)
                     *reinterpret_cast<uint4 *>(rowp + (((g * 4 + i) ^ (row & 7)) << 4)) = make_uint4(ov[0], ov[1], ov[2], ov[3]);
                 }
@@ -282,9 +351,11 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
             if (quarter == 0 && lane == 0 && m0 < p.M && n0 + ch * 64 < p.N) {
                 lin_tma_store_2d(&tm_out, base + S::OFF_RES + ch * S::CHUNK, n0 + ch * 64, m0);
+                if (p.gate) lin_tma_store_2d(&tm_xg, base + S::OFF_A + ch * S::CHUNK, n0 + ch * 64, m0);
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
         }
+        if (grow && m0 + row < p.M) p.ss_out[(size_t)(m0 + row) * p.slots + (n0 / BN) * 2 + half] = lin_sum2(ss2);
         if (threadIdx.x == 64) LIN_TRACE(5);
         // (the staging buffer has been read; the writes themselves are complete when the grid is)
         if (quarter == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -295,6 +366,9 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     if constexpr (KS > 1) {
         // (cluster barriers are warp-aligned: the lanes of the producer warp that idled while lane 0 ran the loads must not
         // reach them before lane 0 does, so the CTA meets first)
+        LinGates<64> gates;
+        const int b_first = p.gate ? min(m0 / p.R, p.B - 1) : 0;
+        if (p.gate && warp >= 2) gates.load(p, b_first, m0, n0 + kq * 64, threadIdx.x - 64);
         __syncthreads();
         cluster_arrive();
         cluster_wait();       // every CTA's staged half is in place
@@ -323,6 +397,16 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             uint32_t acc[32];
             tmem_ld32(tmem + lane_addr + kq * 64 + half * 32, acc);
             tmem_wait_ld();
+            uint64_t ss2 = 0ull;
+            uint8_t *xrowp = smem + S::OFF_B + row * 128;         // (the stages of W are idle; those of a may still be read by the counterpart)
+            static_assert(S::NST * S::B_STAGE >= 2 * S::CHUNK, "the idle weight stages hold the gated chunk and the gates");
+            const float *grow = nullptr;
+            if (p.gate) {
+                float *gsm = reinterpret_cast<float *>(smem + S::OFF_B + S::CHUNK);
+                gates.store(p, b_first, m0, n0 + kq * 64, threadIdx.x - 64, gsm);
+                grow = gsm + (size_t)(min((m0 + row) / p.R, p.B - 1) - b_first) * 64 + half * 32;
+                asm volatile("bar.sync 1, 256;" ::: "memory");
+            }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const uint4 t = rr[i];
@@ -330,14 +414,17 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
                 const float4 q0 = pv[2 * i], q1 = pv[2 * i + 1];
                 const float pp[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
                 uint32_t ov[4];
+                uint64_t vv[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     float v0 = __uint_as_float(acc[8 * i + 2 * k]) + pp[2 * k] + __uint_as_float(rv[k] << 16);
                     float v1 = __uint_as_float(acc[8 * i + 2 * k + 1]) + pp[2 * k + 1] + __uint_as_float(rv[k] & 0xFFFF0000u);
                     if (!split_ok) v0 = v1 = __int_as_float(0x7fc00000);
+                    vv[k] = pack_f32x2(v0, v1);
                     __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
                     ov[k] = *reinterpret_cast<uint32_t *>(&h);
                 }
+                if (grow) lin_gated_piece(vv, grow + i * 8, xrowp + (((half * 4 + i) ^ (row & 7)) << 4), ss2);
                 *reinterpret_cast<uint4 *>(rowp + (((half * 4 + i) ^ (row & 7)) << 4)) = make_uint4(ov[0], ov[1], ov[2], ov[3]);
             }
             fence_proxy_async_smem();
@@ -345,10 +432,12 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             if (warp == 2 && lane == 0) {
                 if (m0 < p.M && n0 + kq * 64 < p.N) {
                     lin_tma_store_2d(&tm_out, base + S::OFF_RES + kq * S::CHUNK, n0 + kq * 64, m0);
+                    if (p.gate) lin_tma_store_2d(&tm_xg, base + S::OFF_B, n0 + kq * 64, m0);
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
                 asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             }
+            if (grow && m0 + row < p.M) p.ss_out[(size_t)(m0 + row) * p.slots + (n0 / 64 + kq) * 2 + half] = lin_sum2(ss2);
         }
     }
 
@@ -407,7 +496,7 @@ cudaError_t launch_lin_simt(const void *a, const void *W, const void *res, void 
 }
 
 template <int BN, int KS>
-cudaError_t launch_lin_tc(const CUtensorMap &ma, const CUtensorMap &mw, const CUtensorMap &mr, const CUtensorMap &mo, const LinParams &p, int n_tiles,
+cudaError_t launch_lin_tc(const CUtensorMap &ma, const CUtensorMap &mw, const CUtensorMap &mr, const CUtensorMap &mo, const CUtensorMap &mx, const LinParams &p, int n_tiles,
                           cudaStream_t st)
 {
     static std::atomic<unsigned long long> attr_set{0};
@@ -427,7 +516,7 @@ cudaError_t launch_lin_tc(const CUtensorMap &ma, const CUtensorMap &mw, const CU
     attr[1].val.clusterDim.x = 2u * KS; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, linear_res_tc_kernel<BN, KS>, ma, mw, mr, mo, p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, linear_res_tc_kernel<BN, KS>, ma, mw, mr, mo, mx, p);
     count_launch();
     return e;
 }
@@ -437,6 +526,51 @@ cudaError_t launch_lin_tc(const CUtensorMap &ma, const CUtensorMap &mw, const CU
 bool linear_tc_supported(int dtype, int M, int K, int N)
 {
     return dtype == REFLEX_DTYPE_BF16 && M >= 1 && K >= 8 && K % 8 == 0 && N >= 8 && N % 8 == 0 && (long long)M * N <= 0x3FFFFFFF;
+}
+
+// Tile shape of a problem: columns of a tile and the CTA pairs that share its contraction. 256-column tiles unless they would leave more
+// than half of the SM pairs without one: then 128-column tiles, twice as many pairs at work on a contraction that is as long (every CTA
+// then fetches 24 KB per step for half the MMA work) ...
+static void lin_tiles(int M, int K, int N, int &bn, int &ks)
+{
+    const int m_tiles = (M + 2 * kLinBM - 1) / (2 * kLinBM);
+    bn = m_tiles * ((N + 255) / 256) * 2 <= 74 ? 128 : 256;
+    // ... and the contraction in two halves on two pairs of a 4-CTA cluster while that still leaves every pair an SM pair of
+    // its own and the halves are long enough to pay for the exchange, which costs about 4 us (two cluster barriers, 32 KB
+    // per CTA through distributed shared memory, the slower pair's lag): 300-1000 rows x 4096 -> 1024 15.5-17.0 -> 12.9-15.0 us;
+    // x 2048 9.3-9.4 -> 9.8-11.0, so only contractions of 4096 and more are split
+    const int nk_all = (K + kLinBK - 1) / kLinBK;
+    ks = bn == 128 && m_tiles * ((N + 127) / 128) * 2 <= 74 && nk_all % 2 == 0 && nk_all >= 64 ? 2 : 1;
+}
+
+static cudaError_t launch_tiles(LinParams p, const void *a, const void *W, const void *res, void *out, void *xg, cudaStream_t st)
+{
+    p.m_tiles = (p.M + 2 * kLinBM - 1) / (2 * kLinBM);
+    p.has_res = res ? 1 : 0;
+    int bn, ks;
+    lin_tiles(p.M, p.K, p.N, bn, ks);
+    CUtensorMap ma, mw, mr, mo, mx;
+    if (!tensor_map_2d_bf16(&ma, a, p.K, p.M, kLinBM) || !tensor_map_2d_bf16(&mw, W, p.K, p.N, bn / 2) || !tensor_map_2d_bf16(&mo, out, p.N, p.M, kLinBM) ||
+        !tensor_map_2d_bf16(&mr, res ? res : out, p.N, p.M, kLinBM) || !tensor_map_2d_bf16(&mx, xg ? xg : out, p.N, p.M, kLinBM))
+        return cudaErrorInvalidValue;
+    p.slots = p.N / bn * 2 * (ks == 2 ? 2 : 1);
+    if (bn == 256) return launch_lin_tc<256, 1>(ma, mw, mr, mo, mx, p, (p.N + 255) / 256, st);
+    return ks == 2 ? launch_lin_tc<128, 2>(ma, mw, mr, mo, mx, p, (p.N + 127) / 128, st) : launch_lin_tc<128, 1>(ma, mw, mr, mo, mx, p, (p.N + 127) / 128, st);
+}
+
+// CG_RES of ChainProj for many rows: the residual projection together with what the norm behind it needs
+cudaError_t launch_tile_res(const ChainProj &a, cudaStream_t st)
+{
+    LinParams p = {};
+    p.M = a.B * a.R; p.K = a.K; p.N = a.N; p.status = a.status; p.early_w = 1; p.gate = a.gate; p.ss_out = a.ss_out; p.R = a.R; p.B = a.B;
+    return launch_tiles(p, a.x, a.W + (size_t)a.w_row0 * a.K, a.res, a.h, a.xg, st);
+}
+
+int tile_res_slots(int M, int K, int N)
+{
+    int bn, ks;
+    lin_tiles(M, K, N, bn, ks);
+    return N / bn * 2 * (ks == 2 ? 2 : 1);
 }
 
 // impl: 0 = tensor cores where supported, 1 = plain kernel, 2 = tensor cores, the 256-row tiles whatever M is
@@ -449,26 +583,9 @@ cudaError_t launch_linear_residual(const void *a, const void *W, const void *res
         return dtype == REFLEX_DTYPE_BF16 ? launch_lin_simt<__nv_bfloat16>(a, W, res, out, M, K, N, st) : launch_lin_simt<float>(a, W, res, out, M, K, N, st);
     }
     if (impl == 0 && linear_small_takes(M, K, N)) return launch_linear_small(a, W, res, out, M, K, N, status, early_w, st);
-    LinParams p;
-    p.M = M; p.K = K; p.N = N; p.m_tiles = (M + 2 * kLinBM - 1) / (2 * kLinBM); p.has_res = res ? 1 : 0; p.status = status; p.early_w = early_w ? 1 : 0;
-    // 256-column tiles unless they would leave more than half of the SM pairs without one: then 128-column tiles, twice as
-    // many pairs at work on a contraction that is as long (every CTA then fetches 24 KB per step for half the MMA work)
-    const bool narrow = p.m_tiles * ((N + 255) / 256) * 2 <= 74;
-    CUtensorMap ma, mw, mr, mo;
-    if (!tensor_map_2d_bf16(&ma, a, K, M, kLinBM) || !tensor_map_2d_bf16(&mw, W, K, N, narrow ? 64 : 128) || !tensor_map_2d_bf16(&mo, out, N, M, kLinBM))
-        return cudaErrorInvalidValue;
-    if (res) { if (!tensor_map_2d_bf16(&mr, res, N, M, kLinBM)) return cudaErrorInvalidValue; }
-    else mr = mo;
-    if (narrow) {
-        // ... and the contraction in two halves on two pairs of a 4-CTA cluster while that still leaves every pair an SM pair of
-        // its own and the halves are long enough to pay for the exchange, which costs about 4 us (two cluster barriers, 32 KB
-        // per CTA through distributed shared memory, the slower pair's lag): 300-1000 rows x 4096 -> 1024 15.5-17.0 -> 12.9-15.0 us;
-        // x 2048 9.3-9.4 -> 9.8-11.0, so only contractions of 4096 and more are split
-        const int n_tiles = (N + 127) / 128, nk_all = (K + kLinBK - 1) / kLinBK;
-        if (p.m_tiles * n_tiles * 2 <= 74 && nk_all % 2 == 0 && nk_all >= 64) return launch_lin_tc<128, 2>(ma, mw, mr, mo, p, n_tiles, st);
-        return launch_lin_tc<128, 1>(ma, mw, mr, mo, p, n_tiles, st);
-    }
-    return launch_lin_tc<256, 1>(ma, mw, mr, mo, p, (N + 255) / 256, st);
+    LinParams p = {};
+    p.M = M; p.K = K; p.N = N; p.status = status; p.early_w = early_w ? 1 : 0;
+    return launch_tiles(p, a, W, res, out, nullptr, st);
 }
 
 }  // namespace reflex

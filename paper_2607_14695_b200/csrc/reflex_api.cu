@@ -546,12 +546,24 @@ static bool expert_chained(const reflex_cache_desc &d, const reflex_expert &e)
            chain_proj_supported(CG_RES, M, e.F, e.D) && chain_proj_supported(CG_OUT, M, e.D, e.A);
 }
 
-static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float *a, float dt, void *stream)
+// ... or, for many rows, through the tile kernels on the same operands (tile_gemm.cu, linear_tc.cu). Up to 256 rows the single calls' few-rows
+// kernels split the two residual projections into more CTAs than tiles of 256 rows are (200 rows: 7.1 us each against 12 and 16).
+static bool expert_tiled(const reflex_cache_desc &d, const reflex_expert &e)
+{
+    const int M = d.B * e.T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
+    if (d.dtype != REFLEX_DTYPE_BF16 || e.D % 256 != 0 || !(e.A == 8 || e.A == 16 || e.A == 32) || M <= 256 || e.T < 4) return false;      // (T: the gates of the streams under 128 rows fit the idle stages)
+    return tile_proj_supported(CG_QKV, M, e.D, nq, nk, 0) && tile_proj_supported(CG_SWIGLU, M, e.D, 0, 0, e.F) && chain_proj_supported(CG_OUT, M, e.D, e.A) &&
+           nq % 8 == 0 && e.F % 8 == 0;
+}
+
+static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float *a, float dt, bool tiled, void *stream)
 {
     const reflex_cache_desc &d = c->desc;
     typedef __nv_bfloat16 bf;
     const int L = d.L, B = d.B, T = e.T, D = e.D, M = B * T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
     cudaStream_t st = (cudaStream_t)stream;
+    auto proj = [&](const ChainProj &p) { return !tiled ? launch_chain_proj(p, st) : p.mode == CG_RES ? launch_tile_res(p, st) : launch_tile_proj(p, st); };
+    auto slots_of = [&](int K) { return tiled ? tile_res_slots(M, K, D) : (D + 31) / 32; };
     // partial sums of squares of the residual rows: two areas, so that a projection never writes the one its predecessor reads
     float *ss[2] = {e.row_sums, e.row_sums + (size_t)M * ((D + 31) / 32)};
     auto gate = [&](int i) { return (const float *)e.gates + (size_t)i * B * D; };
@@ -561,9 +573,19 @@ static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float 
         pf.ptr[i] = (const char *)base + first * 2; pf.bytes[i] = n * 2 & ~(size_t)15;
     };
     const size_t kv_layer = (size_t)B * (ring_off(d) + d.N) * d.Hkv * d.d;
-    cudaError_t err = launch_chain_in(a, (const bf *)e.W_in, gate(0), (bf *)e.h, (bf *)e.y, ss[0], B, T, D, e.A, st);
-    if (err != cudaSuccess) return cuda_fail(err, "expert input projection launch");
+    cudaError_t err;
     int slots = 1;
+    if (tiled && M > 1024) {       // (64 streams: 18.9 us as fp32 FMAs, 8 with the cast in front of the tensor cores; 429 rows: 6.2 against 7.7)
+        err = launch_cast(a, e.a_lowp, (size_t)M * e.A, d.dtype, st);
+        ChainProj in = {};
+        in.mode = CG_RES; in.B = B; in.R = T; in.D = D; in.status = (uint32_t *)(c->ws + c->lay.status_off);
+        in.x = (const bf *)e.a_lowp; in.W = (const bf *)e.W_in; in.w_rows = D; in.K = e.A; in.N = D; in.h = (bf *)e.h; in.xg = (bf *)e.y; in.gate = gate(0); in.ss_out = ss[0];
+        if (err == cudaSuccess) err = launch_tile_res(in, st);
+        slots = slots_of(e.A);
+    } else {
+        err = launch_chain_in(a, (const bf *)e.W_in, gate(0), (bf *)e.h, (bf *)e.y, ss[0], B, T, D, e.A, st);
+    }
+    if (err != cudaSuccess) return cuda_fail(err, "expert input projection launch");
     for (int l = 0; l < L; ++l) {
         ChainProj p = {};
         p.B = B; p.R = T; p.D = D; p.eps = e.eps; p.status = (uint32_t *)(c->ws + c->lay.status_off);
@@ -571,7 +593,7 @@ static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float 
         qkv.mode = CG_QKV; qkv.x = (const bf *)e.y; qkv.W = (const bf *)e.Wqkv; qkv.w_rows = L * (nq + 2 * nk); qkv.w_row0 = l * (nq + 2 * nk);
         qkv.K = D; qkv.N = nq + 2 * nk; qkv.ss_in = ss[0]; qkv.slots_in = slots; qkv.q = (bf *)e.q; qkv.k = (bf *)e.k; qkv.v = (bf *)e.v; qkv.nq = nq; qkv.nk = nk;
         range(qkv.pf, 0, e.Wo, (size_t)l * D * nq, (size_t)D * nq);
-        err = launch_chain_proj(qkv, st);
+        err = proj(qkv);
         if (err != cudaSuccess) return cuda_fail(err, "expert q/k/v projection launch");
         ChainPrefetch apf = {};
         range(apf, 0, e.Wgu, (size_t)l * 2 * e.F * D, (size_t)2 * e.F * D);
@@ -581,24 +603,24 @@ static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float 
         o.mode = CG_RES; o.x = (const bf *)e.o; o.W = (const bf *)e.Wo; o.w_rows = L * D; o.w_row0 = l * D; o.K = nq; o.N = D; o.res = (const bf *)e.h;
         o.h = (bf *)e.h; o.xg = (bf *)e.y; o.gate = gate(2 * l + 1); o.ss_out = ss[1];
         range(o.pf, 0, e.Wd, (size_t)l * D * e.F, (size_t)D * e.F);
-        err = launch_chain_proj(o, st);
+        err = proj(o);
         if (err != cudaSuccess) return cuda_fail(err, "expert output projection launch");
         ChainProj gu = p;
         gu.mode = CG_SWIGLU; gu.x = (const bf *)e.y; gu.W = (const bf *)e.Wgu; gu.w_rows = L * 2 * e.F; gu.w_row0 = l * 2 * e.F; gu.K = D; gu.N = e.F;
-        gu.h = (bf *)e.m; gu.ss_in = ss[1]; gu.slots_in = (D + 31) / 32;
+        gu.h = (bf *)e.m; gu.ss_in = ss[1]; gu.slots_in = slots_of(nq);
         if (l + 1 < L) {
             range(gu.pf, 0, c->k_slab, (size_t)(l + 1) * kv_layer, kv_layer);
             range(gu.pf, 1, c->v_slab, (size_t)(l + 1) * kv_layer, kv_layer);
             range(gu.pf, 2, e.Wqkv, (size_t)(l + 1) * (nq + 2 * nk) * D, (size_t)(nq + 2 * nk) * D);
         }
-        err = launch_chain_proj(gu, st);
+        err = proj(gu);
         if (err != cudaSuccess) return cuda_fail(err, "expert gate/up projection launch");
         ChainProj dn = p;
         dn.mode = CG_RES; dn.x = (const bf *)e.m; dn.W = (const bf *)e.Wd; dn.w_rows = L * D; dn.w_row0 = l * D; dn.K = e.F; dn.N = D; dn.res = (const bf *)e.h;
         dn.h = (bf *)e.h; dn.xg = (bf *)e.y; dn.gate = gate(2 * l + 2); dn.ss_out = ss[0];
-        err = launch_chain_proj(dn, st);
+        err = proj(dn);
         if (err != cudaSuccess) return cuda_fail(err, "expert down projection launch");
-        slots = (D + 31) / 32;
+        slots = slots_of(e.F);
     }
     ChainProj out = {};
     out.mode = CG_OUT; out.B = B; out.R = T; out.D = D; out.eps = e.eps; out.status = (uint32_t *)(c->ws + c->lay.status_off);
@@ -628,8 +650,9 @@ int reflex_expert_step(reflex_cache_t *c, const reflex_expert *ep, float *a, con
     const int L = d.L, B = d.B, T = e.T, D = e.D, M = B * T, nq = d.Hq * d.d, nk = d.Hkv * d.d, dt_ = d.dtype;
     int rc = reflex_adarmsnorm_gate(cond, e.W1, e.b1, e.W2, e.b2, e.gates, 2 * L + 1, B, D, e.Cd, e.Hd, dt_, stream);
     if (rc != REFLEX_OK) return rc;
-    if (expert_chained(d, e)) return expert_step_chained(c, e, a, -1.0f / (float)K, stream);
-    // any other dtype or shape: the single calls in order, allowed to read weights and gates ahead of the preceding kernel (nothing in
+    const bool chained = expert_chained(d, e);
+    if (chained || expert_tiled(d, e)) return expert_step_chained(c, e, a, -1.0f / (float)K, !chained, stream);
+    // any other dtype, shape or row count: the single calls in order, allowed to read weights and gates ahead of the preceding kernel (nothing in
     // the step writes weights; the gates are complete before the input projection starts)
     const size_t es = elem_size(dt_);
     auto off = [&](const void *p, size_t elems) -> const void * { return (const char *)p + elems * es; };

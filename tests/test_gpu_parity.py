@@ -1074,17 +1074,19 @@ def test_expert_step_bf16(U):
 
 
 CHAINS = [
-    # B, T, F, A, Hq, Hkv, D
+    # B, T, F, A, Hq, Hkv, D: up to 128 rows ...
     (1, 50, 4096, 32, 8, 1, 1024), (2, 64, 1024, 8, 8, 1, 1024), (1, 1, 512, 16, 4, 1, 512), (3, 33, 1536, 32, 4, 2, 768), (1, 32, 328, 32, 8, 1, 1024),
+    # ... and more than 256: 128- and 256-column tiles, split contraction, ragged rows and widths, many streams under one tile
+    (6, 50, 4096, 32, 8, 1, 1024), (13, 33, 1000, 16, 8, 1, 512), (67, 4, 328, 8, 4, 2, 256), (24, 50, 4104, 32, 8, 1, 1024), (5, 64, 1024, 32, 16, 1, 768),
 ]
 
 
 @pytest.mark.parametrize("case", CHAINS, ids=["B%d_T%d_F%d_A%d_h%dkv%d_D%d" % c for c in CHAINS])
-def test_expert_step_bf16_few_rows(U, case):
-    """Row counts, widths and tile edges of the chained projections (up to 128 rows; the last shape's F takes the single calls)."""
+def test_expert_step_bf16_chained(U, case):
+    """Row counts, widths and tile edges of the chained projections (F = 328 at 32 rows takes the single calls)."""
     B, T, F, A, Hq, Hkv, D = case
     w = synth.CONFIGS["cfg2"].with_(B=B, L=2, T=T, A=A, Hq=Hq, Hkv=Hkv, D=D, S=200, S_max=208)
-    _expert_case(U, w, F, 2e-2, "expert bf16, few rows")
+    _expert_case(U, w, F, 2e-2, "expert bf16, chained", streams=None if B <= 6 else [0, B // 2, B - 1])
 
 
 def test_expert_step_bf16_batched(U):
