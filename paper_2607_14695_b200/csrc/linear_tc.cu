@@ -273,13 +273,14 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
         if constexpr (KS > 1) {
             // Contraction split: thread (row, half) holds this pair's share of columns [64 half, 64 half + 64) of its row. The
             // half that the counterpart CTA (same rank, other pair) finishes goes to shared memory as fp32, 16-byte pieces at
-            // [row][piece ^ (row % 16)]; the other half stays in tensor memory until the cluster has met.
+            // [piece][row], so that the counterpart's warps read 512 contiguous bytes through distributed shared memory (scattered 16-byte
+            // pieces, [row][piece ^ (row % 16)], took 3.3 us for the 32 KB); the other half stays in tensor memory until the cluster has met.
             ok = wait(S::C_ACC, 0u, 4) && ok;
             if (threadIdx.x == 64) LIN_TRACE(4);
             tc_fence_after();
             split_ok = ok;
             if (half != kq) {
-                uint4 *stage = reinterpret_cast<uint4 *>(smem + S::OFF_A);     // [128 rows][16 pieces]; the stage ring is idle
+                uint4 *stage = reinterpret_cast<uint4 *>(smem + S::OFF_A);     // [16 pieces][128 rows]; the stage ring is idle
                 static_assert(S::NST * S::A_STAGE >= 128u * 64u * 4u, "staging area of the split");
 #pragma unroll
                 for (int g = 0; g < 2; ++g) {
@@ -288,7 +289,7 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
                     tmem_wait_ld();
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
-                        stage[row * 16 + ((g * 8 + i) ^ (row & 15))] = ok ? make_uint4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3])
+                        stage[(g * 8 + i) * 128 + row] = ok ? make_uint4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3])
                                                                            : make_uint4(0x7fc00000u, 0x7fc00000u, 0x7fc00000u, 0x7fc00000u);
                 }
             }
@@ -379,11 +380,11 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
             // the counterpart's share of this thread's 32 columns: 8 loads through distributed shared memory, all in flight
             const uint32_t peer = crank ^ 2u;
-            const uint32_t st0 = base + S::OFF_A + (uint32_t)row * 256u;
+            const uint32_t st0 = base + S::OFF_A + (uint32_t)row * 16u;
             float4 pv[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const uint32_t a = mapa(st0 + (uint32_t)(((half * 8 + j) ^ (row & 15)) << 4), peer);
+                const uint32_t a = mapa(st0 + (uint32_t)(half * 8 + j) * (128u * 16u), peer);
                 asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(pv[j].x), "=f"(pv[j].y), "=f"(pv[j].z), "=f"(pv[j].w) : "r"(a) : "memory");
             }
             uint8_t *rowp = smem + S::OFF_RES + kq * S::CHUNK + row * 128;     // residual in, output out: one chunk of 64 columns
@@ -536,11 +537,11 @@ static void lin_tiles(int M, int K, int N, int &bn, int &ks)
     const int m_tiles = (M + 2 * kLinBM - 1) / (2 * kLinBM);
     bn = m_tiles * ((N + 255) / 256) * 2 <= 74 ? 128 : 256;
     // ... and the contraction in two halves on two pairs of a 4-CTA cluster while that still leaves every pair an SM pair of
-    // its own and the halves are long enough to pay for the exchange, which costs about 4 us (two cluster barriers, 32 KB
-    // per CTA through distributed shared memory, the slower pair's lag): 300-1000 rows x 4096 -> 1024 15.5-17.0 -> 12.9-15.0 us;
-    // x 2048 9.3-9.4 -> 9.8-11.0, so only contractions of 4096 and more are split
+    // its own and the halves are long enough to pay for the exchange, which costs about 2 us (two cluster barriers, 32 KB
+    // per CTA through distributed shared memory, the slower pair's lag): 300-1000 rows x 4096 -> 1024 14.3-15.2 -> 12.2-12.9 us,
+    // x 2048 10.2-10.4 -> 8.4-9.4
     const int nk_all = (K + kLinBK - 1) / kLinBK;
-    ks = bn == 128 && m_tiles * ((N + 127) / 128) * 2 <= 74 && nk_all % 2 == 0 && nk_all >= 64 ? 2 : 1;
+    ks = bn == 128 && m_tiles * ((N + 127) / 128) * 2 <= 74 && nk_all % 2 == 0 && nk_all >= 32 ? 2 : 1;
 }
 
 static cudaError_t launch_tiles(LinParams p, const void *a, const void *W, const void *res, void *out, void *xg, cudaStream_t st)
