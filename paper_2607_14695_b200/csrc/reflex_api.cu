@@ -504,7 +504,7 @@ static int attention(reflex_cache_t *c, int layer, const void *q, const void *k_
     if (c->attn_impl == REFLEX_ATTN_SIMT || !tc_ok) {
         p.nsplit = simt_choose_splits(p, c->lay.partial_bytes, c->sm_count);
         e = launch_attention_simt(p, (cudaStream_t)stream);
-    } else if (c->attn_impl == REFLEX_ATTN_AUTO && chain_attn_supported(p, c->sm_count)) {
+    } else if (c->attn_impl == REFLEX_ATTN_AUTO && chain_attn_supported(p, early, c->sm_count)) {
         e = launch_chain_attn(p, status, early, pf, (cudaStream_t)stream);
     } else {
         // Batched shapes take the two-CTA kernel (with a key split when the streams alone do not fill the SM pairs);

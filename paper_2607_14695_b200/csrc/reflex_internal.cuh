@@ -118,9 +118,9 @@ int tc_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count);
 bool tc2_supported(const AttnParams &p);
 int tc2_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count);
 cudaError_t launch_attention_tc(const AttnParams &p, uint32_t *status, bool two_cta, int sm_count, cudaStream_t st);
-// one or two streams (chain_attn.cu): one head and an eighth of the keys per CTA, merged inside clusters of eight. early: the caller
+// a few streams (chain_attn.cu): key slices merged inside clusters of eight or four. early: the caller
 // vouches that the cached regions are not written by work that may still be running
-bool chain_attn_supported(const AttnParams &p, int sm_count);
+bool chain_attn_supported(const AttnParams &p, bool early, int sm_count);
 struct ChainPrefetch;
 cudaError_t launch_chain_attn(const AttnParams &p, uint32_t *status, bool early, const ChainPrefetch *pf, cudaStream_t st);
 // gate MLP of AdaRMSNorm on tcgen05 (bf16): false when the shapes or the driver do not allow it (the caller falls back)

@@ -1025,12 +1025,12 @@ def test_context_window_and_chunk_sweep(U, frames, T):
 # ------------------------------------------------------------------------------------------------
 # a whole action-expert denoising step chained from the library's calls
 # ------------------------------------------------------------------------------------------------
-def _expert_case(U, w, F, tol_v, what, streams=None):
+def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None):
     from oracle import expert_oracle as eo
     from paper_2607_14695_b200 import expert as ex
     rb = U.rb
     tw = U.Twin(w, head0=[3] * w.B, poison=True)
-    tw.init_static(list(range(w.B)), [w.S] * w.B)
+    tw.init_static(list(range(w.B)), S_list or [w.S] * w.B)
     for i in range(3):
         tw.append(list(range(w.B)), 2, i)
     W = ex.expert_weights(w, F, std_scale=0.5)
@@ -1087,6 +1087,20 @@ def test_expert_step_bf16_chained(U, case):
     B, T, F, A, Hq, Hkv, D = case
     w = synth.CONFIGS["cfg2"].with_(B=B, L=2, T=T, A=A, Hq=Hq, Hkv=Hkv, D=D, S=200, S_max=208)
     _expert_case(U, w, F, 2e-2, "expert bf16, chained", streams=None if B <= 6 else [0, B // 2, B - 1])
+
+
+CLUSTERS_OF_FOUR = [
+    # B, T, Hq, Hkv, S_max, prefix lengths, N: edges of the attention that merges four key slices per 128 rows (three to eight streams)
+    (4, 50, 8, 1, 816, [816, 700, 0, 113], 32), (8, 64, 8, 1, 896, [896] * 8, 64), (6, 60, 4, 2, 300, [300, 1, 2, 7, 8, 299], 5),
+    (5, 33, 16, 1, 64, [64] * 5, 4),
+]
+
+
+@pytest.mark.parametrize("case", CLUSTERS_OF_FOUR, ids=["B%d_T%d_h%dkv%d_S%d" % c[:5] for c in CLUSTERS_OF_FOUR])
+def test_expert_step_bf16_attention_of_a_few_streams(U, case):
+    B, T, Hq, Hkv, S_max, S_list, N = case
+    w = synth.CONFIGS["cfg2"].with_(B=B, L=1, T=T, Hq=Hq, Hkv=Hkv, D=512, S=S_max, S_max=S_max, N=N)
+    _expert_case(U, w, 512, 2e-2, "expert bf16, a few streams", streams=[0, 1, B // 2, B - 1], S_list=S_list)
 
 
 def test_expert_step_bf16_batched(U):
