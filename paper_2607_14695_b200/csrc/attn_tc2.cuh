@@ -101,7 +101,7 @@ template <int HD> struct Tc2Smem {
     // mbarrier indices
     static constexpr int C_QFULL = 0, C_QEMPTY = 1, C_KFULL = 2, C_KEMPTY = C_KFULL + NKS, C_VLAND = C_KEMPTY + NKS,
                          C_VEMPTY = C_VLAND + NVS, C_SFULL = C_VEMPTY + NVS, C_PFULL = C_SFULL + 2, C_PVDONE = C_PFULL + 2,
-                         C_OFREE = C_PVDONE + 2, C_COUNT = C_OFREE + 1;   // P V completion: one barrier per S/P buffer
+                         C_OFREE = C_PVDONE + 2, C_MFREE = C_OFREE + 1, C_INBOX = C_MFREE + 1, C_COUNT = C_INBOX + 1;   // P V completion: one barrier per S/P buffer
     static_assert(8 * C_COUNT + 8 <= BAR_BYTES, "barrier area");
 };
 
@@ -115,7 +115,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     using L = Tc2Smem<HD>;
     constexpr int CH = L::CH, VCH = L::VCH, NKS = L::NKS, NVS = L::NVS;
     constexpr int C_QFULL = L::C_QFULL, C_QEMPTY = L::C_QEMPTY, C_KFULL = L::C_KFULL, C_KEMPTY = L::C_KEMPTY, C_VLAND = L::C_VLAND,
-                  C_VEMPTY = L::C_VEMPTY, C_SFULL = L::C_SFULL, C_PFULL = L::C_PFULL, C_PVDONE = L::C_PVDONE, C_OFREE = L::C_OFREE,
+                  C_VEMPTY = L::C_VEMPTY, C_SFULL = L::C_SFULL, C_PFULL = L::C_PFULL, C_PVDONE = L::C_PVDONE, C_OFREE = L::C_OFREE, C_MFREE = L::C_MFREE, C_INBOX = L::C_INBOX,
                   C_COUNT = L::C_COUNT;
     constexpr uint32_t kTmemCols = 512;
     // O: HD fp32 columns. S: 2 x 128 fp32 columns; P(j) (bf16, two keys per column) overwrites the first 64 columns of
@@ -187,10 +187,15 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (threadIdx.x == 0) {
         for (int i = 0; i < C_COUNT; ++i) {
             const bool both = (i == C_PFULL || i == C_PFULL + 1 || i == C_OFREE);
-            mbar_init(bar(i), both ? (uint32_t)(8 * kTc2Parts) : 1u);   // "both": one arrival per softmax warp of either CTA
+            mbar_init(bar(i), both ? (uint32_t)(8 * kTc2Parts) : i == C_MFREE ? (uint32_t)p.nsplit : 1u);   // "both": one arrival per softmax warp of either CTA
         }
         *abort_flag = 0u;
         fence_mbar_init();
+        if (p.cluster_merge) {     // what the other slices' CTAs will send: (m, l) of every row that exists and this CTA's columns of their O
+            const int t0 = (2 * ((u_start / p.nsplit) % n_pairs) + (int)rank) * p.tile_tokens;
+            const int rows = max(0, min(128, (p.T - t0) * p.G));
+            mbar_expect_tx(bar(C_INBOX), (uint32_t)((p.nsplit - 1) * rows) * (uint32_t)(HD / p.nsplit * 4 + 8));
+        }
         prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); prefetch_tmap(&tm_v); prefetch_tmap(&tm_kd); prefetch_tmap(&tm_vd); prefetch_tmap(&tm_o);
     }
     if (warp == 1) tmem_alloc2(smem_u32((const void *)tmem_slot), kTmemCols);
@@ -755,138 +760,133 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (threadIdx.x == 64) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // all stores of this CTA are complete
     }
 
-    if (p.cluster_merge) {
+    if (p.cluster_merge && warp >= 2) {
         // ---- merge of the key slices inside the cluster ----
-        // Pair q of the cluster holds slice q of the keys for the same 256 query rows; CTAs of equal rank inside their pairs
-        // hold the same 128 rows. 1. every row's (m, l) is published; 2. with all slices' (m, l) each thread scales its
-        // share of its O row to the common maximum and stages it in shared memory (Q and K buffers, idle now), column-major
-        // in 16-byte units; 3. pair q adds up columns [q, q+1) * head_dim / nsplit of all slices through distributed shared
-        // memory, divides by the common sum and writes bf16. A cluster barrier after 1 and after 2; the one at the end of
-        // the kernel keeps every CTA alive while a peer may still read its staging area.
+        // Pair q of the cluster holds slice q of the keys for the same 256 query rows; CTAs of equal rank inside their pairs hold the
+        // same 128 rows, and the one in pair q finishes columns [q, q + 1) * head_dim / nsplit of them. Every CTA sends each of the others
+        // its rows' (m, l) and those columns of its unnormalised O straight from tensor memory (st.async, counted on the owner's C_INBOX,
+        // into the idle Q and K buffers once their owner has said on C_MFREE that its MMAs are through), and combines what it
+        // receives with its own share. A warp's store is 512 contiguous bytes. (With (m, l) published first, O scaled to the common
+        // maximum and staged, and the owners reading it, a cluster barrier after either, the merge was 13 k cycles.)
         constexpr int NP = kTc2Parts;
-        const int ns = p.nsplit;
+        const int ns = p.nsplit, own = (int)(crank >> 1), cols_own = HD / ns;
         const int sw = warp - 2, part = sw >> 2;
         const int row = (warp & 3) * 32 + lane;
-        float2 *ml_own = reinterpret_cast<float2 *>(smem + L::OFF_STAGE);      // [128 rows]
-        float4 *stage = reinterpret_cast<float4 *>(smem + L::OFF_Q);           // [HD / 4][128 rows]
-        static_assert(L::OFF_K == L::OFF_Q + L::Q_BYTES && L::Q_BYTES + L::NKS * L::K_STAGE >= (uint32_t)HD * 128 * 4, "staging area of the merge");
-        // (the cluster barriers are warp-aligned instructions: the lanes of the producer warp that idled while lane 0 ran the
-        // loads must not reach them before lane 0 does, so the CTA meets here first)
-        __syncthreads();
-        if (warp >= 2 && part == 0) ml_own[row] = make_float2(fin_m, fin_l);
-        cluster_arrive();
-        cluster_wait();
-        float wgt[8], l_all = 0.f;
-        if (warp >= 2) {
-            float pm[8], mstar = -INFINITY;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                pm[q] = -INFINITY; wgt[q] = 0.f;
-                if (q < ns) {
-                    float lq;
-                    const uint32_t a = mapa(smem_u32(ml_own + row), (uint32_t)(2 * q) + rank);
-                    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(pm[q]), "=f"(lq) : "r"(a) : "memory");
-                    wgt[q] = lq;                                   // the sum for now
-                    if (!(lq > 0.f)) pm[q] = -INFINITY;            // a slice that saw nothing live has no say
-                    mstar = fmaxf(mstar, pm[q]);
+        const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
+        float2 *ml = reinterpret_cast<float2 *>(smem + L::OFF_STAGE);          // [slice][128 rows]
+        static_assert(L::OFF_K == L::OFF_Q + L::Q_BYTES && L::Q_BYTES + L::NKS * L::K_STAGE >= (uint32_t)HD * 128 * 4, "inbox [slice][column quad][128 rows]");
+        auto wait_cl = [&](int i, uint32_t code) -> bool {
+            if (mbar_try_wait_cluster(bar(i), 0)) return true;
+            const unsigned long long t_start = globaltimer_ns();
+            for (uint32_t n = 1;; ++n) {
+                if (mbar_try_wait_cluster(bar(i), 0)) return true;
+                if ((n & 255u) == 0u) {
+                    if (*abort_flag) return false;
+                    if (globaltimer_ns() - t_start > kWaitNs) break;
                 }
             }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const float e = (pm[q] == -INFINITY) ? 0.f : ex2(pm[q] - mstar);
-                l_all = fmaf(wgt[q], e, l_all);
-                wgt[q] = e;
-            }
-            float w_own = 0.f;
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (q == (int)(crank >> 1)) w_own = wgt[q];
-            {
-                // Only the columns that OTHER pairs reduce are staged; this pair's own columns stay in tensor memory until the
-                // reduction below. (The tensor-memory loads are warp-wide: every lane takes part, whatever its own row's
-                // weight; a row without weight in this slice, or a slice without tiles whose accumulator was never written,
-                // stages nothing.)
-                tc_fence_after();
-                const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-                constexpr int EC = HD / NP;
-                const bool mine = w_own > 0.f && fin_ok;
-                const int own_lo = (int)(crank >> 1) * (HD / ns), own_hi = own_lo + HD / ns;     // columns this pair reduces
+            *abort_flag = 1u;
+            atomicCAS(p.status, 0u, 0x80000000u | ((code + 32u) << 16) | (blockIdx.x & 0xFFFFu));
+            return false;
+        };
+        const int uu = u_start / ns, pair = uu % n_pairs, kvh = (uu / n_pairs) % p.Hkv, b = uu / (n_pairs * p.Hkv);
+        const int t0 = (2 * pair + (int)rank) * p.tile_tokens;
+        const int rows = max(0, min(128, (p.T - t0) * p.G));
+        const bool exists = row < rows;
+        if (threadIdx.x - 64 < ns) mbar_arrive_cluster(mapa(bar(C_MFREE), 2u * (threadIdx.x - 64) + rank));
+        if (part == 0 && exists) {
+            if (!(fin_l > 0.f)) fin_m = -INFINITY;             // a slice that saw nothing live has no say
+            const uint32_t at = smem_u32(ml + own * 128 + row);
+            for (int q = 0; q < ns; ++q)
+                if (q != own) st_async_v2(mapa(at, 2u * q + rank), mapa(bar(C_INBOX), 2u * q + rank), __float_as_uint(fin_m), __float_as_uint(fin_l));
+            ml[own * 128 + row] = make_float2(fin_m, fin_l);
+        }
+        tc_fence_after();
+        const bool free = wait_cl(C_MFREE, 16);
+        int turn = 0;
 #pragma unroll 1
-                for (int c = 0; c < EC / 32; ++c) {
-                    const int col0 = part * EC + c * 32;
-                    if (col0 >= own_lo && col0 < own_hi) continue;        // (uniform over the CTA; HD / ns is a multiple of 32)
-                    uint32_t o[32];
-                    tmem_ld32(tmem_base + lane_addr + kColO + col0, o);
-                    tmem_wait_ld();
-                    if (mine) {
+        for (int col0 = 0; col0 < HD && free; col0 += 32) {
+            const int owner = col0 / cols_own;                 // (uniform; cols_own is a multiple of 32)
+            if (owner == own || (turn++ % NP) != part) continue;
+            uint32_t o[32];
+            tmem_ld32(tmem_base + lane_addr + kColO + col0, o);
+            tmem_wait_ld();
+            if (!fin_ok || !(fin_l > 0.f)) {                   // (an accumulator that was never written sends zeros, a failed wait NaN)
 #pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            stage[(col0 / 4 + i) * 128 + row] =
-                                make_float4(__uint_as_float(o[4 * i]) * w_own, __uint_as_float(o[4 * i + 1]) * w_own,
-                                            __uint_as_float(o[4 * i + 2]) * w_own, __uint_as_float(o[4 * i + 3]) * w_own);
-                    }
-                }
+                for (int i = 0; i < 32; ++i) o[i] = fin_ok ? 0u : 0x7fc00000u;
+            }
+            if (exists) {
+                const uint32_t dst = mapa(base + L::OFF_Q + (uint32_t)((own * cols_own + col0 - owner * cols_own) / 4 * 128 + row) * 16u, 2u * owner + rank);
+                const uint32_t ib = mapa(bar(C_INBOX), 2u * owner + rank);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) st_async_v4(dst + i * (128 * 16), ib, o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
             }
         }
-        cluster_arrive();
-        cluster_wait();
-        if (warp >= 2) {
-            // this pair's columns [crank/2 * HD/ns, +HD/ns), split between the NP threads of the row: its own share comes
-            // straight from tensor memory, the other slices' shares from their staging areas
-            const int uu = u_start / p.nsplit, pair = uu % n_pairs, kvh = (uu / n_pairs) % p.Hkv, b = uu / (n_pairs * p.Hkv);
-            const int t_row = (2 * pair + (int)rank) * p.tile_tokens + row / p.G;
-            const int own = (int)(crank >> 1);
-            const int cols_thread = HD / ns / NP;                                       // columns per thread: 16, 32 or 64
-            const int col_0 = own * (HD / ns) + part * cols_thread;
-            const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-            const bool live = fin_ok && t_row < p.T && l_all > 0.f;
-            float w_own = 0.f;
+        const bool got = wait_cl(C_INBOX, 17);
+        asm volatile("bar.sync 1, %0;" ::"n"(128 * NP) : "memory");       // this CTA's own (m, l)
+        float wgt[4], l_all = 0.f, mstar = -INFINITY;
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (q == own) w_own = wgt[q];
-            if (!(fin_l > 0.f)) w_own = 0.f;                                            // an accumulator that was never written
-            const float inv = live ? 1.f / l_all : 0.f;
-            __nv_bfloat16 *orow = (__nv_bfloat16 *)p.out + (((size_t)b * p.T + (live ? t_row : 0)) * p.Hq + kvh * p.G + row % p.G) * HD + col_0;
-            tc_fence_after();
-#pragma unroll 1
-            for (int c0 = 0; c0 < cols_thread; c0 += 16) {
-                uint32_t o[16];
-                tmem_ld16(tmem_base + lane_addr + kColO + col_0 + c0, o);              // warp-wide, whatever the row's state
-                tmem_wait_ld();
-                if (!live) continue;
-                float acc[16];
+        for (int q = 0; q < 4; ++q) {
+            wgt[q] = 0.f;
+            if (q < ns) mstar = fmaxf(mstar, ml[q * 128 + row].x);
+        }
 #pragma unroll
-                for (int i = 0; i < 16; ++i) acc[i] = w_own > 0.f ? __uint_as_float(o[i]) * w_own : 0.f;
+        for (int q = 0; q < 4; ++q) {
+            if (q < ns) {
+                const float2 v = ml[q * 128 + row];
+                wgt[q] = v.x == -INFINITY ? 0.f : ex2(v.x - mstar);
+                l_all = fmaf(v.y, wgt[q], l_all);
+            }
+        }
+        const bool live = got && exists && l_all > 0.f;
+        const float inv = live ? 1.f / l_all : 0.f;
+        float w_own = 0.f;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    if (q < ns && q != own && wgt[q] > 0.f) {
-                        const uint32_t a = mapa(smem_u32(stage + ((col_0 + c0) / 4) * 128 + row), (uint32_t)(2 * q) + rank);
+        for (int q = 0; q < 4; ++q) {
+            wgt[q] *= inv;
+            if (q == own) w_own = wgt[q];
+        }
+        const int cols_thread = cols_own / NP;                 // columns per thread: 16, 32 or 64
+        const int c_first = part * cols_thread;                // inside this CTA's columns
+        __nv_bfloat16 *orow = (__nv_bfloat16 *)p.out + (((size_t)b * p.T + (live ? t0 + row / p.G : 0)) * p.Hq + kvh * p.G + row % p.G) * HD + own * cols_own + c_first;
+        const float4 *in = reinterpret_cast<const float4 *>(smem + L::OFF_Q) + row;
+#pragma unroll 2
+        for (int c0 = 0; c0 < cols_thread; c0 += 16) {
+            uint32_t o[16];
+            tmem_ld16(tmem_base + lane_addr + kColO + own * cols_own + c_first + c0, o);              // warp-wide, whatever the row's state
+            tmem_wait_ld();
+            if (!live) continue;
+            float acc[16];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            float4 v;
-                            asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a + j * 128 * 16) : "memory");
-                            acc[4 * j] += v.x; acc[4 * j + 1] += v.y; acc[4 * j + 2] += v.z; acc[4 * j + 3] += v.w;
-                        }
+            for (int i = 0; i < 16; ++i) acc[i] = w_own > 0.f ? __uint_as_float(o[i]) * w_own : 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (q < ns && q != own) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 v = in[(q * cols_own + c_first + c0 + 4 * j) / 4 * 128];
+                        acc[4 * j] = fmaf(v.x, wgt[q], acc[4 * j]); acc[4 * j + 1] = fmaf(v.y, wgt[q], acc[4 * j + 1]);
+                        acc[4 * j + 2] = fmaf(v.z, wgt[q], acc[4 * j + 2]); acc[4 * j + 3] = fmaf(v.w, wgt[q], acc[4 * j + 3]);
                     }
                 }
+            }
 #pragma unroll
-                for (int h8 = 0; h8 < 2; ++h8) {
-                    uint4 v;
-                    uint32_t *vv = reinterpret_cast<uint32_t *>(&v);
+            for (int h8 = 0; h8 < 2; ++h8) {
+                uint4 v;
+                uint32_t *vv = reinterpret_cast<uint32_t *>(&v);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        __nv_bfloat162 h = __floats2bfloat162_rn(acc[8 * h8 + 2 * k] * inv, acc[8 * h8 + 2 * k + 1] * inv);
-                        vv[k] = *reinterpret_cast<uint32_t *>(&h);
-                    }
-                    *reinterpret_cast<uint4 *>(orow + c0 + 8 * h8) = v;
+                for (int k = 0; k < 4; ++k) {
+                    __nv_bfloat162 h = __floats2bfloat162_rn(acc[8 * h8 + 2 * k], acc[8 * h8 + 2 * k + 1]);
+                    vv[k] = *reinterpret_cast<uint32_t *>(&h);
                 }
+                *reinterpret_cast<uint4 *>(orow + c0 + 8 * h8) = v;
             }
         }
     }
 
     tc_fence_before();
     __syncthreads();
-    cluster_arrive();
+    cluster_arrive_relaxed();     // (a release would wait for this thread's output stores)
     cluster_wait();   // neither CTA retires while its partner can still touch its shared memory or barriers
     if (warp == 1) tmem_dealloc2(tmem_base, kTmemCols);
     if (threadIdx.x == 64) TC2_TRACE(2, 15, 5);

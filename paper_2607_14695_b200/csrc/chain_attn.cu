@@ -77,19 +77,6 @@ struct CaParams {
     ChainPrefetch pf;
 };
 
-__device__ __forceinline__ void ca_st_async_v4(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];"
-                 ::"r"(addr), "r"(bar), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ void ca_st_async_v2(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b)
-{
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%2, %3}, [%1];" ::"r"(addr), "r"(bar), "r"(a), "r"(b) : "memory");
-}
-__device__ __forceinline__ void ca_st_async_b32(uint32_t addr, uint32_t bar, uint32_t a)
-{
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %2, [%1];" ::"r"(addr), "r"(bar), "r"(a) : "memory");
-}
 // lanes 0-15 of the warp's quarter, 64 columns: register 4 g + j of thread t is row t / 4 + (j & 2 ? 8 : 0), column 8 g + 2 (t % 4) + (j & 1)
 __device__ __forceinline__ void ca_tmem_ld_16x256b(uint32_t taddr, uint32_t (&r)[32])
 {
@@ -228,7 +215,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             // this CTA's Q K^T is through with the K tile: its peers may send their partial results over it
             wait(CB_S, 1);
             for (int r = 0; r < kCaSlices; ++r)
-                asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapa(bar(CB_FREE), (uint32_t)r)) : "memory");
+                mbar_arrive_cluster_release(mapa(bar(CB_FREE), (uint32_t)r));
         }
         __syncwarp();
         chain_prefetch(p.pf, blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y, lane);
@@ -353,8 +340,8 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 l += __shfl_xor_sync(0xffffffffu, l, 2);
                 if ((lane & 3) == 0 && row < rows) {
                     const uint32_t o = (uint32_t)(row / OWN), dst = mapa(base + L::ML + (uint32_t)(slice * OWN + row % OWN) * 16u, o), ib = mapa(bar(CB_INBOX), o);
-                    if (ROWS == 64 || group == 0) ca_st_async_v2(dst, ib, __float_as_uint(m * p.scale_log2), __float_as_uint(l));
-                    else ca_st_async_b32(dst + 8u, ib, __float_as_uint(l));
+                    if (ROWS == 64 || group == 0) st_async_v2(dst, ib, __float_as_uint(m * p.scale_log2), __float_as_uint(l));
+                    else st_async_b32(dst + 8u, ib, __float_as_uint(l));
                 }
             }
             fence_proxy_async_smem();
@@ -384,7 +371,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         const int quad = c * 8 + q;
                         if (quad * 4 < rows) {
                             const uint32_t o = (uint32_t)(quad / QUADS);
-                            ca_st_async_v4(mapa(base + L::K + (uint32_t)((slice * QUADS + quad % QUADS) * kCaHD + d) * 16u, o), mapa(bar(CB_INBOX), o), acc[4 * q], acc[4 * q + 1],
+                            st_async_v4(mapa(base + L::K + (uint32_t)((slice * QUADS + quad % QUADS) * kCaHD + d) * 16u, o), mapa(bar(CB_INBOX), o), acc[4 * q], acc[4 * q + 1],
                                            acc[4 * q + 2], acc[4 * q + 3]);
                         }
                     }
@@ -690,8 +677,8 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 #pragma unroll
             for (int o = 0; o < kC4Slices; ++o) {
                 const uint32_t dst = mapa(at, (uint32_t)o), ib = mapa(bar(C4_INBOX), (uint32_t)o);
-                if (group == 0) ca_st_async_v2(dst, ib, __float_as_uint(m * p.scale_log2), __float_as_uint(l0 + l1));
-                else ca_st_async_b32(dst + 8u, ib, __float_as_uint(l0 + l1));
+                if (group == 0) st_async_v2(dst, ib, __float_as_uint(m * p.scale_log2), __float_as_uint(l0 + l1));
+                else st_async_b32(dst + 8u, ib, __float_as_uint(l0 + l1));
             }
         }
         // V rows inside the contraction that hold no key: zero, so that weight 0 meets no stale NaN
@@ -715,7 +702,7 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         ok = wait(C4_O, 10) && ok;
         tc_fence_after();
         // this CTA's P V is through with its tiles: the peers may send their partial results over them
-        if (t < kC4Slices) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapa(bar(C4_FREE), (uint32_t)t)) : "memory");
+        if (t < kC4Slices) mbar_arrive_cluster_release(mapa(bar(C4_FREE), (uint32_t)t));
         const bool none = ext[0] == 0 && ext[1] == 0;
         if (wait_cl(C4_FREE, 11)) {
 #pragma unroll 1
@@ -734,7 +721,7 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     const uint32_t at = base + L::KV + (uint32_t)((slice * (kC4Cols / 4) + (cc & 1) * 8) * kC4Rows + row) * 16u;
                     const uint32_t dst = mapa(at, (uint32_t)owner), ib = mapa(bar(C4_INBOX), (uint32_t)owner);
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) ca_st_async_v4(dst + q * (kC4Rows * 16), ib, acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+                    for (int q = 0; q < 8; ++q) st_async_v4(dst + q * (kC4Rows * 16), ib, acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
                 }
             }
         }
