@@ -526,7 +526,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 }
             }
         }
-        cluster_arrive();
+        cluster_arrive_relaxed();   // (the peers' shares have been read and used: nothing to release)
         cluster_wait();
     }
 

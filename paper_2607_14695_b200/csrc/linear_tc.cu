@@ -444,8 +444,11 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
 
     tc_fence_before();
     __syncthreads();
-    cluster_arrive();
-    cluster_wait();   // no CTA retires while another can still touch its shared memory or barriers
+    cluster_arrive_relaxed();
+    // No CTA retires while another can still touch its shared memory or barriers. (Relaxed: what was read from a counterpart
+    // has been used above, and the output's visibility is the kernel boundary's matter; a releasing arrive would first wait
+    // for every output store. An expert layer of 13 x 33 rows 58.8 -> 57.7 us, of 16 x 50 69.7 -> 68.3.)
+    cluster_wait();
     if (warp == 1) tmem_dealloc2(tmem, BN);
     if (threadIdx.x == 64) LIN_TRACE(7);
 }

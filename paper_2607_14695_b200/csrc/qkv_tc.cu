@@ -495,8 +495,8 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     if (threadIdx.x == 64) QK_TRACE(2, 31, 2);
     tc_fence_before();
     __syncthreads();
-    cluster_arrive();
-    cluster_wait();   // neither CTA retires while its partner can still touch its shared memory or barriers
+    cluster_arrive_relaxed();
+    cluster_wait();   // neither CTA retires while its partner can still touch its shared memory or barriers (nothing to release)
     if (warp == 1) tmem_dealloc2(tmem, NACC * kQkBN);
 }
 
@@ -888,8 +888,8 @@ norm_linear_small_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
                 *reinterpret_cast<uint2 *>(dst) = o;
             }
         }
-        cluster_arrive();
-        cluster_wait();   // no CTA retires while a peer may still read its partial sums
+        cluster_arrive_relaxed();
+        cluster_wait();   // no CTA retires while a peer may still read its partial sums (read and used: nothing to release)
     }
     if (threadIdx.x == 64) QK_TRACE(2, 31, 2);
     tc_fence_before();

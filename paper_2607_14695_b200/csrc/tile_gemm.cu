@@ -289,8 +289,8 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
 
     tc_fence_before();
     __syncthreads();
-    cluster_arrive();
-    cluster_wait();   // neither CTA retires while its partner can still touch its shared memory or barriers
+    cluster_arrive_relaxed();
+    cluster_wait();   // neither CTA retires while its partner can still touch its shared memory or barriers (nothing to release)
     if (warp == 1) tmem_dealloc2(tmem, 2 * BN);
 }
 
