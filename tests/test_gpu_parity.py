@@ -1006,6 +1006,25 @@ def test_double_banked_static_prefix(U, impl):
     del keep, keep2
 
 
+@pytest.mark.parametrize("d,lens", [(64, [191, 192, 193]), (64, [384, 0, 385]), (256, [48, 47, 49]), (256, [1, 816, 31])])
+def test_prefix_copy_at_block_edges(U, d, lens):
+    """The prefix write moves 1536 16-byte units a block (192 rows of 64, 48 rows of 256): whole blocks, one row less, one more,
+    an empty prefix beside a long one. Bytes are compared exactly, and nothing is written behind a prefix."""
+    rb = U.rb
+    L, B, S_max = 2, 4, max(lens) + 3
+    cache = rb.Cache(L, B, 8, 1, d, S_max, 16, 8, rb.DTYPE_BF16, device=U.DEV)
+    g = torch.Generator(device=U.DEV); g.manual_seed(d)
+    src = [torch.randn(3, L, max(lens), 1, d, generator=g, device=U.DEV).to(torch.bfloat16) for _ in range(2)]
+    rb.reflex_cache_init_static(cache, [3, 0, 2], *src, S=lens)
+    want = [torch.zeros_like(cache.k_slab) for _ in range(2)]
+    for i, (b, S) in enumerate(zip([3, 0, 2], lens)):
+        for t, x in zip(want, src):
+            t[:, b, :S] = x[i, :, :S]
+    assert torch.equal(cache.k_slab, want[0]) and torch.equal(cache.v_slab, want[1])
+    sl, _, _, _ = rb.reflex_cache_get_state(cache)
+    assert sl == [lens[1], -1, lens[2], lens[0]]
+
+
 @pytest.mark.parametrize("frames,T", [(1, 75), (5, 50), (50, 25)])
 def test_context_window_and_chunk_sweep(U, frames, T):
     """Points of the paper's context-window (1 to 50 frames of 256 tokens in the sliding history) and action-chunk (25 to 100
