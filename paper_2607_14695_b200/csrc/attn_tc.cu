@@ -780,12 +780,13 @@ bool tc2_supported(const AttnParams &p) { return tc_supported(p) && (p.d == 128 
 // 21.7 unsplit (split in two: 21.6 to 40); at 4466 keys and 16 streams 41 us split in two, 51 unsplit, 47 in four.
 // The nsplit pairs that share a tile pair can merge inside one cluster (no partials, no merge launch) when the cluster stays
 // within the portable size of 8 CTAs, all clusters are resident at once with exactly one unit each, and a thread's share of
-// the columns is whole 16-byte stores. Measured against the split with partials: 4466 keys, 16 streams 41.2 -> 35.6 us
-// (two slices); 898 keys, 4 streams 18.5 -> 16.5 (four slices); one stream 15.5 merged in four against 14.4 with eight
-// slices and the merge kernel, and 2 streams 16.5 merged in four against 15.9 with partials. The model therefore charges
-// the in-cluster merge 6.6 us (three cluster barriers and the staged reduction keep every CTA of the cluster that long; 4 streams
-// x 4466 keys: 23.0 merged in four, 19.0 with eight slices and partials) and uses it only where the partials' round trip would cost more.
-static constexpr double kTc2MergedUs = 6.6;
+// the columns is whole 16-byte stores. What the model charges for that merge was fitted after the owners' shares came to be
+// pushed to them; it grows with the CTAs that push at the same time. Heads of 256, chunk of 50, merged against the other
+// choice, us: 898 keys, 3 streams 12.8 (four slices) against 13.9 unsplit, 8 streams 14.4 (two) against 15.2, 12 streams 15.7 (two) against
+// 15.3; 1122 keys, 8 streams 15.0 (two) against 16.8; 4466 keys, 4 streams 22.2 (four) against 19.2 (six to eight slices and partials),
+// 12 streams 32.1 (two) against 30.5 (three and partials), 16 streams 32.7 (two) against 41.2 with partials and 51 unsplit. Heads of
+// 128 are too short of columns or keys to change sides (14 shapes measured alike).
+static double tc2_merged_us(int units, int nsplit) { return 4.6 + 0.015 * units * nsplit; }
 static double tc2_partials_us(const AttnParams &p, int nsplit)   // merge launch + fp32 partials written and read back
 {
     const double per_split_bytes = (double)p.B * p.T * p.Hq * (p.d + 2) * sizeof(float);
@@ -803,7 +804,7 @@ static bool tc2_cluster_merge_ok(const AttnParams &p, int nsplit, int sm_count)
     // the most the device reports, measured 20.4 us where 12 took 17.5 and the unsplit kernel 19.5.
     const int active = tc2_active_clusters(p.d, 2 * nsplit);
     if (base_units > (nsplit == 4 ? active - active / 4 : active)) return false;
-    if (tc2_partials_us(p, nsplit) <= kTc2MergedUs) return false;
+    if (tc2_partials_us(p, nsplit) <= tc2_merged_us(base_units, nsplit)) return false;
     return (p.d / nsplit / kTc2Parts) % 16 == 0 && p.d / nsplit / kTc2Parts >= 16;   // a thread reduces whole 16-column pieces
 }
 
@@ -829,7 +830,7 @@ int tc2_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count)
         if (ns > 1 && !merged && per_split_bytes * ns > (double)partial_bytes) continue;
         const int waves = merged ? 1 : (units * ns + clusters - 1) / clusters;
         const double loop_us = 1.3 * waves * ((tiles + ns - 1) / ns);
-        const double split_us = ns == 1 ? 0.0 : (merged ? kTc2MergedUs : tc2_partials_us(p, ns));
+        const double split_us = ns == 1 ? 0.0 : (merged ? tc2_merged_us(units, ns) : tc2_partials_us(p, ns));
         if (loop_us + split_us < best_us - 0.05) { best_us = loop_us + split_us; best = ns; }
     }
     return best;
