@@ -2,8 +2,8 @@
 // (stacked weights) and B streams, bf16 weights and conditioning vectors.
 //
 // Both layers of the MLP are the same small GEMM, out[b][u] = act(bias[u] + sum_k W[u][k] vec[b][k]): one CTA takes 128
-// weight rows (the M of a tcgen05.mma, K-major A operand) and up to 64 streams (N, K-major B operand), loads both
-// operands whole with TMA (80 KB + 40 KB at the paper's widths), issues len/16 MMAs into a 64-column accumulator in
+// weight rows (the M of a tcgen05.mma, K-major A operand) and up to 32 streams (N, K-major B operand), loads both
+// operands whole with TMA (80 KB + 20 KB at the paper's widths), issues len/16 MMAs into a 32-column accumulator in
 // tensor memory and finishes with one thread per weight row. bf16 x bf16 products are exact in the fp32 accumulator. The
 // hidden activations go to the second layer as two bf16 arrays, hi = bf16(h) and lo = bf16(h - hi) (two passes of MMAs,
 // about 17 bits of h), in the space the fp32 hidden activations of the FMA kernels take.
@@ -26,23 +26,29 @@ using namespace ptx;
 namespace {
 
 constexpr int kGtUnits = 128;     // weight rows per CTA
-constexpr int kGtStreams = 64;    // streams per CTA
+constexpr int kGtStreams = 32;    // streams per group
+constexpr int kGtPerSm = 2;       // CTAs that fit on an SM
 constexpr int kGtMaxChunks = 5;   // 64-column chunks of the contraction axis held in shared memory (len <= 320)
 constexpr uint32_t kGtWaitNs = 1000000000u;
 
+// Shared memory holds just the chunks that the contraction has, so that two CTAs share an SM (100 KB and 97 KB for the layers of an
+// expert): its 37 x 8 second-layer CTAs are one wave instead of two, and they move in beside the first layer's. Both layers of the
+// MLP, 37 gates of 1024: 1 stream 11.3 -> 7.6 us, 13 11.9 -> 8.5, 64 14.6 -> 13.3; 4 gates and 64 streams 10.1 -> 7.6 (groups of 32
+// instead of 64 streams: twice the CTAs).
 struct GateTcSmem {
     static constexpr uint32_t A_CHUNK = kGtUnits * 128;      // 128 rows x 64 bf16
-    static constexpr uint32_t B_CHUNK = kGtStreams * 128;    // 64 rows x 64 bf16
-    static constexpr uint32_t OFF_A = 0;
-    static constexpr uint32_t OFF_B = kGtMaxChunks * A_CHUNK;                  // two passes (hi, lo) of B chunks
-    static constexpr uint32_t OFF_BAR = OFF_B + 2 * kGtMaxChunks * B_CHUNK;
-    static constexpr uint32_t TOTAL = OFF_BAR + 64 + 1024;                     // + slack for the 1024-byte alignment
+    static constexpr uint32_t B_CHUNK = kGtStreams * 128;    // 32 rows x 64 bf16
+    static constexpr uint32_t OFF_BAR = 0;
+    static constexpr uint32_t OFF_A = 1024;
+    static __host__ __device__ constexpr uint32_t off_b(int chunks) { return OFF_A + chunks * A_CHUNK; }                                  // one or two passes (hi, lo)
+    static __host__ __device__ constexpr uint32_t total(int chunks, int passes) { return off_b(chunks) + passes * chunks * B_CHUNK + 1024; }   // + slack for the alignment
 };
+static_assert(kGtPerSm * (GateTcSmem::total(kGtMaxChunks, 1) + 1024) <= 228 * 1024, "two first-layer CTAs per SM");
 
 // SILU: first layer (writes hi/lo bf16 hidden activations); else second layer (writes fp32 gates 1 + z). PASSES: 1 = one
 // bf16 vector per stream (tm_v0), 2 = hi and lo halves (tm_v0, tm_v1).
 template <bool SILU, int PASSES>
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(256, kGtPerSm)
 gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_v0, const __grid_constant__ CUtensorMap tm_v1,
                const __nv_bfloat16 *__restrict__ bias, float *out_f32, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, int B, int len, int units,
                int vec_rows_per_layer, uint32_t *status)
@@ -57,7 +63,8 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int layer = blockIdx.z, u0 = blockIdx.x * kGtUnits;
     const int chunks = (len + 63) / 64;
-    // A CTA keeps its 128 weight rows in shared memory and walks the groups of 64 streams that fall to it (blockIdx.y takes
+    const uint32_t off_b = S::off_b(chunks);
+    // A CTA keeps its 128 weight rows in shared memory and walks the groups of 32 streams that fall to it (blockIdx.y takes
     // a contiguous share of the groups): with many streams -- the conditioning vectors of all steps of a control tick
     // stacked -- the weights are fetched once per CTA instead of once per group, and the next group's vectors come in
     // while this group's results are stored.
@@ -83,7 +90,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
         __syncwarp();
         if (!SILU && ng > 0) load_weights();
     }
-    if (warp == 1) tmem_alloc(smem_u32((const void *)tmem_slot), 64);
+    if (warp == 1) tmem_alloc(smem_u32((const void *)tmem_slot), kGtStreams);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -102,11 +109,11 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
         if (status) atomicCAS(status, 0u, 0x80000000u | ((code + 64u) << 16) | (blockIdx.x & 0xFFFFu));
         return false;
     };
-    auto load_vectors = [&](int g) {   // the (up to) 64 vectors of group g, one or two bf16 arrays (the warp is converged)
+    auto load_vectors = [&](int g) {   // the (up to) 32 vectors of group g, one or two bf16 arrays (the warp is converged)
         for (int c = 0; c < chunks; ++c) {
-            tma_load_2d_elect(base + S::OFF_B + c * S::B_CHUNK, &tm_v0, bar_load, c * 64, layer * vec_rows_per_layer + g * kGtStreams);
+            tma_load_2d_elect(base + off_b + c * S::B_CHUNK, &tm_v0, bar_load, c * 64, layer * vec_rows_per_layer + g * kGtStreams);
             if (PASSES == 2)
-                tma_load_2d_elect(base + S::OFF_B + (kGtMaxChunks + c) * S::B_CHUNK, &tm_v1, bar_load, c * 64, layer * vec_rows_per_layer + g * kGtStreams);
+                tma_load_2d_elect(base + off_b + (chunks + c) * S::B_CHUNK, &tm_v1, bar_load, c * 64, layer * vec_rows_per_layer + g * kGtStreams);
         }
     };
 
@@ -134,7 +141,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
 #pragma unroll 1
                     for (int c = 0; c < chunks; ++c) {      // (columns past the contraction's end are zeros on both sides)
                         uint64_t ad = umma_desc_sw128(base + S::OFF_A + c * S::A_CHUNK, 16, 1024);
-                        uint64_t bd = umma_desc_sw128(base + S::OFF_B + (pass * kGtMaxChunks + c) * S::B_CHUNK, 16, 1024);
+                        uint64_t bd = umma_desc_sw128(base + off_b + (pass * chunks + c) * S::B_CHUNK, 16, 1024);
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {
                             umma_ss_elect(tmem, ad, bd, idesc, (pass > 0 || c > 0 || kk > 0) ? 1u : 0u);
@@ -153,13 +160,13 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
             mbar_expect_tx_elect(bar_load, (uint32_t)chunks * (PASSES * S::B_CHUNK));
             load_vectors(g_first + i + 1);
         }
-        // epilogue: thread = weight row (TMEM lane), columns = streams, the two warps of a lane quarter take 32 each in groups of eight.
+        // epilogue: thread = weight row (TMEM lane), columns = streams, the two warps of a lane quarter take half each in groups of eight.
         // Groups without a stream are skipped by a branch: as predicated code over all 64 columns the SiLU layer's epilogue took 4.7 us
         // for a single stream.
         const int nb = min(kGtStreams, B - b0);
 #pragma unroll 1
-        for (int g = 0; g < 4; ++g) {
-            const int n0 = half * 32 + g * 8;
+        for (int g = 0; g < kGtStreams / 16; ++g) {
+            const int n0 = half * (kGtStreams / 2) + g * 8;
             if (n0 >= nb) break;
             uint32_t acc[8];
             tmem_ld8(tmem + lane_addr + n0, acc);
@@ -188,7 +195,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem, 64);
+    if (warp == 1) tmem_dealloc(tmem, kGtStreams);
 }
 
 template <bool SILU, int PASSES>
@@ -197,18 +204,18 @@ cudaError_t launch_one(const CUtensorMap &mw, const CUtensorMap &mv0, const CUte
 {
     static std::atomic<unsigned long long> attr_set{0};
     cudaError_t e0 = once_per_device(attr_set, [] {
-        return cudaFuncSetAttribute(gate_tc_kernel<SILU, PASSES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GateTcSmem::TOTAL);
+        return cudaFuncSetAttribute(gate_tc_kernel<SILU, PASSES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GateTcSmem::total(kGtMaxChunks, PASSES));
     });
     if (e0 != cudaSuccess) return e0;
     cudaLaunchConfig_t cfg = {};
-    // groups of 64 streams are spread over blockIdx.y only as far as that adds CTAs the SMs can hold at once; beyond, a CTA
+    // groups of 32 streams are spread over blockIdx.y only as far as that adds CTAs the SMs can hold at once; beyond, a CTA
     // walks several groups with its weights resident
     const int ux = (units + kGtUnits - 1) / kGtUnits, n_groups = (B + kGtStreams - 1) / kGtStreams;
-    int gy = 148 / (ux * L);
+    int gy = 148 * kGtPerSm / (ux * L);
     gy = gy < 1 ? 1 : (gy > n_groups ? n_groups : gy);
     cfg.gridDim = dim3(ux, gy, L);
     cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = GateTcSmem::TOTAL;
+    cfg.dynamicSmemBytes = GateTcSmem::total((len + 63) / 64, PASSES);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
