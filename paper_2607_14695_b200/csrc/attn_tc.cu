@@ -647,13 +647,13 @@ cudaError_t launch_t(const CUtensorMap *mq, const CUtensorMap *mk, const CUtenso
     return e;
 }
 
-template <int HD>
+template <int HD, bool EARLY>
 cudaError_t launch2_t(const CUtensorMap *mq, const CUtensorMap *mk, const CUtensorMap *mv, const CUtensorMap *mkd,
                       const CUtensorMap *mvd, const CUtensorMap *mo, const TcParams &tp, dim3 grid, cudaStream_t st)
 {
     static std::atomic<unsigned long long> attr_set{0};
     cudaError_t e0 = once_per_device(attr_set, [] {
-        return cudaFuncSetAttribute(attn_tc2_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tc2Smem<HD>::TOTAL);
+        return cudaFuncSetAttribute(attn_tc2_kernel<HD, EARLY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tc2Smem<HD>::TOTAL);
     });
     if (e0 != cudaSuccess) return e0;
     // programmatic stream serialisation: the grid may be scheduled while the preceding kernel drains; it waits
@@ -670,7 +670,7 @@ cudaError_t launch2_t(const CUtensorMap *mq, const CUtensorMap *mk, const CUtens
     attr[1].val.clusterDim.x = 2u * (unsigned)(tp.cluster_merge ? tp.nsplit : 1); attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, attn_tc2_kernel<HD>, *mq, *mk, *mv, *mkd, *mvd, *mo, tp);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, attn_tc2_kernel<HD, EARLY>, *mq, *mk, *mv, *mkd, *mvd, *mo, tp);
     count_launch();
     return e;
 }
@@ -696,8 +696,8 @@ int tc2_active_clusters_t(int cluster_ctas)
     attr[0].val.clusterDim.x = (unsigned)cluster_ctas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaFuncSetAttribute(attn_tc2_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tc2Smem<HD>::TOTAL);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, attn_tc2_kernel<HD>, &cfg);
+    cudaError_t e = cudaFuncSetAttribute(attn_tc2_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tc2Smem<HD>::TOTAL);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, attn_tc2_kernel<HD, false>, &cfg);
     if (e != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
     cached[cluster_ctas] = n > 0 ? n : -1;
     return n > 0 ? n : 0;
@@ -877,9 +877,12 @@ cudaError_t launch_attention_tc(const AttnParams &p, uint32_t *status, bool two_
         int clusters = sm_count / 2;
         if (clusters > units) clusters = units;
         if (clusters < 1) clusters = 1;
+        // Inside an expert step the first two cached tiles go out ahead of the wait: the CTAs of a few streams sit beside the projection ahead
+        // of them for 4 to 6 us, those of many start when the first of its CTAs leave. Step of 9 x 50 rows 1017 -> 1012 us, 13 x 33 1027 ->
+        // 1017, 18 x 50 1230 -> 1221, 24 x 50 1491 -> 1482, 37 x 50 1737 -> 1726, 64 x 50 2356 -> 2353.
         dim3 grid2(2 * clusters, 1, 1);                      // with cluster_merge: units pairs = units / nsplit clusters of 2 * nsplit CTAs
-        if (p.d == 256) e = launch2_t<256>(&mq, &mk, &mv, &mkd, &mvd, &mo, tp, grid2, st);
-        else if (p.d == 128) e = launch2_t<128>(&mq, &mk, &mv, &mkd, &mvd, &mo, tp, grid2, st);
+        if (p.d == 256) e = (p.early ? launch2_t<256, true> : launch2_t<256, false>)(&mq, &mk, &mv, &mkd, &mvd, &mo, tp, grid2, st);
+        else if (p.d == 128) e = (p.early ? launch2_t<128, true> : launch2_t<128, false>)(&mq, &mk, &mv, &mkd, &mvd, &mo, tp, grid2, st);
         else return cudaErrorInvalidValue;
         if (e != cudaSuccess || p.nsplit == 1 || tp.cluster_merge) return e;
         return launch_attention_merge(p, st);

@@ -106,7 +106,8 @@ template <int HD> struct Tc2Smem {
 };
 
 // (18 warps are five on at least one of the four schedulers, whose 16 K registers then allow 96 per thread)
-template <int HD>
+template <int HD, bool EARLY>   // EARLY: inside an expert step, the first cached tiles are asked for ahead of the wait (an instance of its own: as
+                                 // run-time branches the same lines cost the grids that do not use them 0.7 % of a 64-stream step)
 __global__ void __launch_bounds__(kTc2Threads, 1)   // launched as clusters of 2 CTAs, or of 2 * nsplit (cluster_merge)
 attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kd,
@@ -208,7 +209,8 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (threadIdx.x == 64) TC2_TRACE(2, 15, 1);
     // Programmatic dependent launch: this grid may have been scheduled while the kernel ahead of it on the stream was still
     // running (its set-up above touches no global memory); from here on everything that kernel wrote is visible.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // (In an expert step the producer asks for cached keys first and waits after that.)
+    if (!(EARLY && warp == 0)) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     auto wait = [&](int i, uint32_t parity, uint32_t code) -> bool {
         if (mbar_try_wait(bar(i), parity)) return true;
@@ -252,9 +254,11 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 if (++c.jj == c.w.n_tiles) { c.u += u_stride; ++c.ui; settle(c); }
             };
             bool ok = true;
+            [[maybe_unused]] int ahead = 0;                 // tiles of the first unit whose loads went out ahead of the wait
             auto issue_k = [&](const Cursor &c) {
                 const Unit &w = c.w;
                 const int gi = c.g, st = gi % NKS;
+                if constexpr (EARLY) { if (gi < ahead) return; }
                 const uint32_t ph = (uint32_t)(gi / NKS - 1) & 1u;
                 const int h0 = 2 * (w.tile0 + c.jj), h1 = h0 + 1;
                 const int live = (h0 < w.H ? 1 : 0) + (h1 < w.H ? 1 : 0);
@@ -283,6 +287,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             auto issue_v = [&](const Cursor &c) {
                 const Unit &w = c.w;
                 const int gi = c.g, st = gi % NVS;
+                if constexpr (EARLY) { if (gi < ahead) return; }
                 const uint32_t ph = (uint32_t)(gi / NVS - 1) & 1u;
                 const int h0 = 2 * (w.tile0 + c.jj), h1 = h0 + 1;
                 const int live = (h0 < w.H ? 1 : 0) + (h1 < w.H ? 1 : 0);
@@ -300,6 +305,15 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             };
             Cursor ck, cv;
             ck.u = u_start; ck.ui = 0; ck.jj = 0; ck.g = 0;
+            if constexpr (EARLY) {
+                settle(ck);
+                const int n = ck.valid ? max(0, min(min(NKS, NVS), min(ck.w.n_tiles, (ck.w.g.ns + ck.w.g.nr) / 2 - ck.w.tile0))) : 0;
+                Cursor c = ck;
+                for (c.jj = c.g = 0; c.jj < n; ++c.jj, ++c.g) issue_k(c);
+                for (c.jj = c.g = 0; c.jj < n; ++c.jj, ++c.g) issue_v(c);
+                ahead = n;
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+            }
             // Where a Q tile lies follows from the unit's number alone: with unsplit keys (no unit is ever empty) the first
             // one is requested before the stream state, which everything else about the unit hangs on, has come in.
             const bool q_early = p.nsplit == 1 && u_start < n_units;
@@ -310,7 +324,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     tma2_load_4d(base + L::OFF_Q + ch * (128 * 128), &tm_q, bar(C_QFULL) & kPeerBitMask, ch * 64, kvh * p.G,
                                  (2 * pair + (int)rank) * p.tile_tokens, b);
             }
-            settle(ck);
+            if constexpr (!EARLY) settle(ck);
             cv = ck;
             if (kLead == 1 && ck.valid) { issue_k(ck); if (!q_early) issue_q(ck); advance(ck); }
             // At a unit boundary the pipe's completions come as QK(last - 1) PV(last - 2) QK(last): the next unit's first K

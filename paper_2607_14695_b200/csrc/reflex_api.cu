@@ -494,6 +494,7 @@ static int attention(reflex_cache_t *c, int layer, const void *q, const void *k_
     p.dyn_mask = dyn_mask;
     p.scale = scale > 0.f ? scale : 1.0f / sqrtf((float)d.d);
     p.dtype = d.dtype;
+    p.early = early ? 1 : 0;
     p.nsplit = 1;
     const bool tc_ok = tc_supported(p);
     const bool tc2_ok = tc2_supported(p);

@@ -58,6 +58,7 @@ struct AttnParams {
     float scale;
     int nsplit;
     int dtype;
+    int early;                     // inside an expert step: cached keys may be asked for before the wait for the preceding kernel
 };
 
 // Split-K partials in the workspace: for n = B * rows * nsplit (row, split) slots, first n rows of d floats with the

@@ -1122,6 +1122,21 @@ def test_expert_step_bf16_attention_of_a_few_streams(U, case):
     _expert_case(U, w, 512, 2e-2, "expert bf16, a few streams", streams=[0, 1, B // 2, B - 1], S_list=S_list)
 
 
+KEYS_AHEAD = [
+    # B, T, Hq, Hkv, d, S_max, prefix lengths, N: cached tiles asked for ahead of the wait: prefixes around a
+    # tile of 128 keys and its halves, none at all, a tile shared with the dynamic keys; split keys
+    (9, 33, 8, 1, 256, 300, [300, 0, 1, 63, 64, 65, 127, 128, 129], 64), (10, 40, 8, 2, 128, 260, [260, 192, 191, 193, 0, 5, 64, 128, 256, 259], 20),
+    (9, 33, 8, 1, 256, 1400, [1400, 1399, 0, 700, 1, 64, 128, 1281, 1345], 32),
+]
+
+
+@pytest.mark.parametrize("case", KEYS_AHEAD, ids=["B%d_T%d_h%dkv%d_d%d_S%d" % c[:6] for c in KEYS_AHEAD])
+def test_expert_step_bf16_cached_keys_ahead_of_the_wait(U, case):
+    B, T, Hq, Hkv, d, S_max, S_list, N = case
+    w = synth.CONFIGS["cfg2"].with_(B=B, L=2, T=T, Hq=Hq, Hkv=Hkv, d=d, D=512, S=S_max, S_max=S_max, N=N)
+    _expert_case(U, w, 512, 2e-2, "expert bf16, cached keys ahead", streams=[0, 1, 4, B - 1], S_list=S_list)
+
+
 def test_expert_step_bf16_batched(U):
     """The same two-layer step for 64 streams (3200 rows: the 256-row tiles of every projection kernel, the two-CTA attention
     in its batched form), three streams compared."""
