@@ -1,4 +1,4 @@
-// Internal interface of the chained expert step (chain_gemm.cu, chain_attn.cu, expert_step.cu).
+// Internal interface of the chained expert step (chain_gemm.cu, chain_attn.cu, tile_gemm.cu, linear_tc.cu; put together in reflex_api.cu).
 #pragma once
 
 #include <cuda_bf16.h>

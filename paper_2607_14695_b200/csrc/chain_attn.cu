@@ -795,7 +795,7 @@ static int chain_attn_rows(const AttnParams &p, bool early)
         if ((long long)p.B * p.Hkv * ((p.T + tt - 1) / tt) <= 14) return rows;
     }
     // Clusters of four while all of them fit, and only where the cached keys may come in ahead of the wait: 4 streams x 898 keys inside an
-    // expert step 15.8 -> 14.3 us (8 streams 16.9 -> 15.9); called by itself the two-CTA kernel's split takes 14.4 (15.4) against 14.6 (15.7).
+    // expert step 15.8 -> 14.3 us (8 streams 16.9 -> 15.9); called by itself the two-CTA kernel's split takes 13.7 (14.4) against 14.6 (15.7).
     const int tt = kC4Rows / G;
     return early && tt >= 1 && (long long)p.B * p.Hkv * ((p.T + tt - 1) / tt) <= 32 ? kC4Rows : 0;
 }

@@ -1,9 +1,8 @@
-"""A whole action-expert denoising step built from the library's calls: per layer the adaptive norm folded into the
+"""A whole action-expert denoising step in one call of the library (reflex_expert_step): per layer the adaptive norm folded into the
 packed Q/K/V projection, the partitioned attention, the output projection with its residual, the adaptive norm folded
 into the fused gate/up projections of the SwiGLU block and the down projection with its residual; then the velocity
-head and the Euler update of the action chunk (Sec. 2.1, Sec. 3.1-3.3). The output and down projections with their
-residual adds are reflex_linear_residual, and so are the two A-wide heads (input projection from the A = 32 action
-dimensions, velocity head back to them; no residual): every contraction of the step runs in this package's kernels.
+head and the Euler update of the action chunk (Sec. 2.1, Sec. 3.1-3.3). The call runs the
+same mathematics as the single entry points one after the other; every contraction is in this package's kernels.
 
 The paper does not print the expert's architecture; this is the usual pre-norm block of a pi0-class expert with both
 norms adaptive, no biases and no positional term (positions are outside the path), written down so that the fused calls
