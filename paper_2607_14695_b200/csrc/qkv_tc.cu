@@ -1063,6 +1063,8 @@ static cudaError_t launch_small(const CUtensorMap &mx, const CUtensorMap &mw, Qk
 
 // swiglu_F = 0: W = W_QKV, outputs q / k / v with nq and nk columns. swiglu_F = F > 0: W = [W_gate; W_up] ([2F][D]),
 // q = the [M][F] output SiLU(gate) * up; nq, nk, k, v unused.
+bool norm_swiglu_gates_fit(int R, int D) { return (size_t)((kQkBM - 1) / R + 2) * D * sizeof(float) <= QkSmem<2>::GATE_MAX; }
+
 cudaError_t launch_adarmsnorm_qkv(const void *x, const float *gate, const void *W, void *q, void *k, void *v, int B, int R, int D, int nq, int nk,
                                   int swiglu_F, float eps, int dtype, int impl, int sm_count, uint32_t *status, bool early, cudaStream_t st)
 {

@@ -548,11 +548,14 @@ static bool expert_chained(const reflex_cache_desc &d, const reflex_expert &e)
 }
 
 // ... or, for many rows, through the tile kernels on the same operands (tile_gemm.cu, linear_tc.cu). Up to 256 rows the single calls' few-rows
-// kernels split the two residual projections into more CTAs than tiles of 256 rows are (200 rows: 7.1 us each against 12 and 16).
+// kernels split the two residual projections into more CTAs than tiles of 256 rows are (200 rows: 7.1 us each against 12 and 16). Short chunks are the
+// exception: the gates of the streams under 128 rows then exceed what the single gate/up projection holds, and its plain kernel took
+// 8.5 ms a layer (8 x 20 rows: a step of 153 ms, 0.91 by the tiles).
 static bool expert_tiled(const reflex_cache_desc &d, const reflex_expert &e)
 {
     const int M = d.B * e.T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
-    if (d.dtype != REFLEX_DTYPE_BF16 || e.D % 256 != 0 || !(e.A == 8 || e.A == 16 || e.A == 32) || M <= 256 || e.T < 4) return false;      // (T: the gates of the streams under 128 rows fit the idle stages)
+    if (d.dtype != REFLEX_DTYPE_BF16 || e.D % 256 != 0 || !(e.A == 8 || e.A == 16 || e.A == 32) || e.T < 4) return false;      // (T: the gates of the streams under 128 rows fit the idle stages)
+    if (M <= 256 && norm_swiglu_gates_fit(e.T, e.D)) return false;
     return tile_proj_supported(CG_QKV, M, e.D, nq, nk, 0) && tile_proj_supported(CG_SWIGLU, M, e.D, 0, 0, e.F) && chain_proj_supported(CG_OUT, M, e.D, e.A) &&
            nq % 8 == 0 && e.F % 8 == 0;
 }

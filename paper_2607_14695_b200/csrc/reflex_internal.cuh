@@ -130,6 +130,8 @@ cudaError_t launch_chain_attn(const AttnParams &p, uint32_t *status, bool early,
 // 2 = tensor cores with 256-column tiles only
 bool norm_qkv_tc_supported(int dtype, int B, int R, int D, int nq, int nk);
 // swiglu_F > 0: W = [W_gate; W_up] and q receives SiLU(gate) * up, [B*R][F]
+// do the gates of the streams under 128 rows fit the shared memory of the tensor-core gate/up projections (the plain kernel takes the rest)?
+bool norm_swiglu_gates_fit(int R, int D);
 cudaError_t launch_adarmsnorm_qkv(const void *x, const float *gate, const void *W, void *q, void *k, void *v, int B, int R, int D, int nq, int nk,
                                   int swiglu_F, float eps, int dtype, int impl, int sm_count, uint32_t *status, bool early, cudaStream_t st);
 // plain projection with residual (linear_tc.cu): out [M][N] = res + a [M][K] W [N][K]^T. impl: 0 = tensor cores where supported,

@@ -1095,6 +1095,7 @@ def test_expert_step_bf16(U):
 CHAINS = [
     # B, T, F, A, Hq, Hkv, D: up to 128 rows ...
     (1, 50, 4096, 32, 8, 1, 1024), (2, 64, 1024, 8, 8, 1, 1024), (1, 1, 512, 16, 4, 1, 512), (3, 33, 1536, 32, 4, 2, 768), (1, 32, 328, 32, 8, 1, 1024),
+    (8, 20, 2048, 32, 8, 1, 1024),      # short chunks: the tiles below 256 rows
     # ... and more than 256: 128- and 256-column tiles, split contraction, ragged rows and widths, many streams under one tile
     (6, 50, 4096, 32, 8, 1, 1024), (13, 33, 1000, 16, 8, 1, 512), (67, 4, 328, 8, 4, 2, 256), (24, 50, 4104, 32, 8, 1, 1024), (5, 64, 1024, 32, 16, 1, 768),
 ]
