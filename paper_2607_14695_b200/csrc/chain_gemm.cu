@@ -347,8 +347,9 @@ chain_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                     }
                 }
                 const float tot = warp_sum4(sq[0], sq[1], sq[2], sq[3], lane);
-                // lanes 0, 8, 16, 24 hold the sums of rows 0, 1, 2, 3 of the quad
-                if ((lane & 7) == 0 && r + (lane >> 3) < p.M) p.ss_out[(size_t)(r + (lane >> 3)) * p.slots_out + (fg >> 5)] = tot;
+                // lanes 0, 8, 16, 24 hold the sums of rows 0, 1, 2, 3 of the quad. (The width is a multiple of 64: with tiles of 128 features the
+                // upper two warps of the last one may be past its end, and what would be their slots are the next row's.)
+                if ((lane & 7) == 0 && f_ok && r + (lane >> 3) < p.M) p.ss_out[(size_t)(r + (lane >> 3)) * p.slots_out + (fg >> 5)] = tot;
             } else {
                 const float4 rs = *reinterpret_cast<const float4 *>(rsm + q * 4);
                 const float rs4[4] = {rs.x, rs.y, rs.z, rs.w}, uu[4] = {u.x, u.y, u.z, u.w};

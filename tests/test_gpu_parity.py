@@ -1044,6 +1044,18 @@ def test_context_window_and_chunk_sweep(U, frames, T):
 # ------------------------------------------------------------------------------------------------
 # a whole action-expert denoising step chained from the library's calls
 # ------------------------------------------------------------------------------------------------
+def _with_guards(model):
+    """Every buffer of the step reallocated with 64 elements behind it that nothing may write; returns those."""
+    from paper_2607_14695_b200 import expert as ex
+    tails = {}
+    for n in ex._BUFFERS:
+        t = getattr(model, n)
+        buf = torch.full((t.numel() + 64,), 12345.0, dtype=t.dtype, device=t.device)
+        setattr(model, n, buf[:t.numel()].view(t.shape))
+        tails[n] = buf[t.numel():]
+    return tails
+
+
 def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None):
     from oracle import expert_oracle as eo
     from paper_2607_14695_b200 import expert as ex
@@ -1055,6 +1067,7 @@ def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None):
     W = ex.expert_weights(w, F, std_scale=0.5)
     dW = {n: U.to_dev(v, w.dtype) for n, v in W.items()}
     model = ex.ActionExpert(w, tw.g, dW, F, device=U.DEV)
+    tails = _with_guards(model)
     a0 = synth.normal(w, "noise", (w.B, w.T, w.A)).astype(np.float64)
     if w.dtype == synth.DTYPE_BF16:          # the step reads the chunk through a storage-dtype mirror: start from representable values
         a0 = synth.round_storage(a0.astype(np.float32), w.dtype).astype(np.float64)
@@ -1062,6 +1075,8 @@ def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None):
     a_gpu = torch.from_numpy(a0.astype(np.float32)).to(U.DEV)
     model.step(a_gpu, U.to_dev(cond, w.dtype), 1)
     rb.reflex_cache_check_status(tw.g)
+    for n, tail in tails.items():
+        assert torch.equal(tail, torch.full_like(tail, 12345.0)), f"{what}: written behind {n}"
     want_a, want_v = eo.expert_step(tw.o, W, a0, cond, w.K, w.Hq, w.Hkv, w.d, F, streams=streams)
     got_v = U.to_host(model.vel)
     if streams is not None:          # a sample of the (independent) streams
@@ -1096,6 +1111,8 @@ CHAINS = [
     # B, T, F, A, Hq, Hkv, D: up to 128 rows ...
     (1, 50, 4096, 32, 8, 1, 1024), (2, 64, 1024, 8, 8, 1, 1024), (1, 1, 512, 16, 4, 1, 512), (3, 33, 1536, 32, 4, 2, 768), (1, 32, 328, 32, 8, 1, 1024),
     (8, 20, 2048, 32, 8, 1, 1024),      # short chunks: the tiles below 256 rows
+    # model widths that end inside a tile of 128 features of a residual projection
+    (1, 50, 4096, 32, 8, 1, 960), (1, 8, 2048, 32, 8, 1, 960), (2, 33, 4096, 8, 4, 1, 960), (1, 50, 4096, 32, 8, 1, 1088), (1, 20, 512, 16, 4, 2, 320),
     # ... and more than 256: 128- and 256-column tiles, split contraction, ragged rows and widths, many streams under one tile
     (6, 50, 4096, 32, 8, 1, 1024), (13, 33, 1000, 16, 8, 1, 512), (67, 4, 328, 8, 4, 2, 256), (24, 50, 4104, 32, 8, 1, 1024), (5, 64, 1024, 32, 16, 1, 768),
 ]
