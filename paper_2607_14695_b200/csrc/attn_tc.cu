@@ -411,6 +411,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         } else if (p.cluster_merge) {
             fin_ok = ok;
             if (n_local > 0 && ok) { fin_m = (m_ref == -INFINITY) ? -INFINITY : m_ref * p.scale_log2; fin_l = l; }
+            if (!ok) fin_l = __int_as_float(0x7fc00000);      // (a wait that ran out: the row becomes NaN in every CTA that merges it)
         } else {
             const size_t slot = partial_slot(b, rows_total, t_row * p.Hq + hq, p.nsplit, split);
             float *po = partial_o(p.partials, slot, HD);
@@ -500,8 +501,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         if (warp >= 2) {
             const int t_row_m = t0 + row_m / p.G;
             const int c4_per = HD / 4 / ns, c4_0 = (int)my_rank * c4_per;           // this CTA's columns, in float4 units
-            if (t_row_m < p.T && l_all > 0.f) {
-                const float inv = 1.f / l_all;
+            if (t_row_m < p.T) {
+                // (the sum is positive unless a logit was not finite or a wait ran out: the row is NaN then, as in the unsplit form)
+                const float inv = l_all > 0.f ? 1.f / l_all : __int_as_float(0x7fc00000);
                 __nv_bfloat16 *orow = (__nv_bfloat16 *)p.out + (((size_t)b * p.T + t_row_m) * p.Hq + kvh * p.G + row_m % p.G) * HD + c4_0 * 4;
 #pragma unroll 1
                 for (int c4 = 0; c4 < c4_per; c4 += 2) {                            // 8 columns = one 16-byte store at a time

@@ -655,7 +655,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             if (p.cluster_merge) {
                 // the slices of this tile pair meet in the merge phase at the end of the kernel (this pair has no other unit)
                 fin_m = (m_ref == -INFINITY) ? -INFINITY : m_ref * p.scale_log2;
-                fin_l = l;
+                fin_l = ok ? l : __int_as_float(0x7fc00000);      // (after a wait that ran out the row becomes NaN in every CTA that merges it)
                 fin_ok = ok;
                 continue;
             }
@@ -852,8 +852,9 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 l_all = fmaf(v.y, wgt[q], l_all);
             }
         }
-        const bool live = got && exists && l_all > 0.f;
-        const float inv = live ? 1.f / l_all : 0.f;
+        // A row that exists is always written. Its sum is positive unless a logit was not finite or a wait ran out: it is NaN then, as
+        // in the unsplit form.
+        const float inv = got && l_all > 0.f ? 1.f / l_all : __int_as_float(0x7fc00000);
         float w_own = 0.f;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -862,17 +863,17 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         }
         const int cols_thread = cols_own / NP;                 // columns per thread: 16, 32 or 64
         const int c_first = part * cols_thread;                // inside this CTA's columns
-        __nv_bfloat16 *orow = (__nv_bfloat16 *)p.out + (((size_t)b * p.T + (live ? t0 + row / p.G : 0)) * p.Hq + kvh * p.G + row % p.G) * HD + own * cols_own + c_first;
+        __nv_bfloat16 *orow = (__nv_bfloat16 *)p.out + (((size_t)b * p.T + (exists ? t0 + row / p.G : 0)) * p.Hq + kvh * p.G + row % p.G) * HD + own * cols_own + c_first;
         const float4 *in = reinterpret_cast<const float4 *>(smem + L::OFF_Q) + row;
 #pragma unroll 2
         for (int c0 = 0; c0 < cols_thread; c0 += 16) {
             uint32_t o[16];
             tmem_ld16(tmem_base + lane_addr + kColO + own * cols_own + c_first + c0, o);              // warp-wide, whatever the row's state
             tmem_wait_ld();
-            if (!live) continue;
+            if (!exists) continue;
             float acc[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) acc[i] = w_own > 0.f ? __uint_as_float(o[i]) * w_own : 0.f;
+            for (int i = 0; i < 16; ++i) acc[i] = w_own == 0.f ? 0.f : __uint_as_float(o[i]) * w_own;      // (0: the accumulator may never have been written)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 if (q < ns && q != own) {

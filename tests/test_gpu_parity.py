@@ -362,6 +362,37 @@ def test_attention_of_few_streams(U, case):
         tw.attention(1, 2, T=T - 1, what="few streams, T < T_max")
 
 
+NON_FINITE = [
+    # B, Hq, Hkv, d, S, N, T: keys in one slice, slices merged in clusters of two to eight CTAs, slices merged by a second launch
+    (64, 8, 1, 256, 816, 32, 50), (1, 8, 1, 256, 816, 32, 50), (2, 8, 1, 256, 816, 32, 50), (3, 8, 1, 256, 816, 32, 50), (8, 8, 1, 256, 816, 32, 50),
+    (16, 8, 1, 256, 4160, 256, 50), (1, 8, 1, 256, 4160, 256, 50), (1, 8, 1, 128, 300, 48, 37), (1, 2, 1, 64, 64, 16, 8), (2, 8, 1, 64, 600, 16, 40),
+]
+
+
+@pytest.mark.parametrize("case", NON_FINITE, ids=["B%d_h%dkv%d_d%d_S%d_N%d_T%d" % c for c in NON_FINITE])
+def test_attention_of_a_row_that_is_not_finite(U, case):
+    """A query that holds a NaN or an infinity gives a row of NaN, whatever form takes the call, and changes no other row."""
+    rb = U.rb
+    B, Hq, Hkv, d, S, N, T = case
+    g = torch.Generator(device=U.DEV); g.manual_seed(3)
+    rnd = lambda *s: torch.randn(*s, generator=g, device=U.DEV).to(torch.bfloat16)
+    cache = rb.Cache(1, B, Hq, Hkv, d, S, N, T, rb.DTYPE_BF16, device=U.DEV)
+    rb.reflex_cache_init_static(cache, list(range(B)), rnd(B, 1, S, Hkv, d), rnd(B, 1, S, Hkv, d))
+    rb.reflex_cache_append_sliding(cache, list(range(B)), rnd(B, 1, N, Hkv, d), rnd(B, 1, N, Hkv, d))
+    q, k, v = rnd(B, T, Hq, d), rnd(B, T, Hkv, d), rnd(B, T, Hkv, d)
+    want = torch.full_like(q, 7.0)
+    rb.reflex_partitioned_attention(cache, 0, q, k, v, want)
+    at = (B - 1, T // 2, 1)
+    for bad in (float("nan"), float("inf")):
+        q2, out = q.clone(), torch.full_like(q, 7.0)
+        q2[at][3] = bad
+        rb.reflex_partitioned_attention(cache, 0, q2, k, v, out)
+        rb.reflex_cache_check_status(cache)
+        assert torch.isnan(out[at]).all(), (bad, out[at])
+        out[at] = want[at]
+        assert torch.equal(out, want), bad
+
+
 def _random_attention_cases(n, seed):
     """Seeded shapes across what the kernels branch on: head_dim, queries per KV head, KV heads, prefix lengths that differ per
     stream (0 included), ring capacity and fill (empty, partly filled, wrapped), dynamic tokens from 1 to beyond one tile."""
