@@ -382,7 +382,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         tc_fence_before();
         // ---- merge of this CTA's rows ----
         if (own > 0) {
-            ok = wait_cl(CB_INBOX, 10);
+            ok = wait_cl(CB_INBOX, 10);              // (after a wait that ran out the rows are marked invalid, a quiet NaN, not left stale)
             if (threadIdx.x == 64) CA_TRACE(7);
             float *wgt = reinterpret_cast<float *>(smem + L::WGT);
             if (t < kCaSlices * OWN) {               // eight neighbouring lanes: the slices of one row
@@ -411,7 +411,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const int r = slice * OWN + q2 * 4 + i, tk = r >> p.g_log2;
-                        if (ok && q2 * 4 + i < own) p.out[((size_t)(b * p.T + t0 + tk) * p.Hq + hkv * p.G + (r - (tk << p.g_log2))) * kCaHD + t] = __float2bfloat16_rn(o[i]);
+                        if (q2 * 4 + i < own) p.out[((size_t)(b * p.T + t0 + tk) * p.Hq + hkv * p.G + (r - (tk << p.g_log2))) * kCaHD + t] = __float2bfloat16_rn(ok ? o[i] : __int_as_float(0x7fc00000));
                     }
                 }
             }
@@ -742,7 +742,7 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 w[q] = ml[q].x == -INFINITY ? 0.f : ex2(ml[q].x - mm);
                 l = fmaf(w[q], ml[q].y + ml[q].z, l);
             }
-            const float inv = 1.f / l;
+            const float inv = ok ? 1.f / l : __int_as_float(0x7fc00000);      // (a wait that ran out: the row is marked invalid, not left stale)
 #pragma unroll
             for (int q = 0; q < kC4Slices; ++q) w[q] *= inv;
             const float4 *in = reinterpret_cast<const float4 *>(smem + L::KV) + mh * 8 * kC4Rows + mrow;
@@ -765,7 +765,7 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     __nv_bfloat162 hh = __floats2bfloat162_rn(a[2 * k], a[2 * k + 1]);
                     o[k] = *reinterpret_cast<uint32_t *>(&hh);
                 }
-                if (ok) *reinterpret_cast<uint4 *>(dst + q8 * 8) = make_uint4(o[0], o[1], o[2], o[3]);
+                *reinterpret_cast<uint4 *>(dst + q8 * 8) = make_uint4(o[0], o[1], o[2], o[3]);
             }
         }
     }

@@ -330,6 +330,7 @@ chain_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 }
             }
             float val[4] = {s.x, s.y, s.z, s.w};
+            if (!ok) val[0] = val[1] = val[2] = val[3] = __int_as_float(0x7fc00000);      // a wait ran out: sums may be missing
             const int r = row0 + (own_q0 + q) * 4;
             if constexpr (MODE == CG_RES) {
                 if (q != q_first) load_res(q);
