@@ -142,9 +142,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     volatile uint32_t *abort_flag = tmem_slot + 1;
 
     // programmatic dependent launch: scheduled, perhaps, before the kernel ahead on the stream has finished; nothing is read
-    // before it has. The kernel after this one may be scheduled once every CTA here has started (it waits the same way).
+    // before it has. The kernel after this one may be scheduled once every CTA here has its tensor memory: one that took the columns
+    // first would wait for this grid, and this grid for the columns.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int qt = blockIdx.x % p.n_qtiles;
     const int kvh = blockIdx.x / p.n_qtiles;
@@ -185,6 +185,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // bounded wait (about one second of wall time): false, and the abort flag raised, when the barrier never flips
     auto wait = [&](int i, uint32_t parity, uint32_t code) -> bool {

@@ -122,10 +122,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     const int own = max(0, min(OWN, rows - slice * OWN));            // query rows this CTA merges
     const bool last = slice == kCaSlices - 1;                        // ring and dynamic tokens
 
-    if (!p.early) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    }
+    if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (warp == 0) {
         if (lane == 0) {
             CA_TRACE(0);
@@ -182,10 +179,9 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     cluster_wait();              // the peers' barriers exist
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    if (p.early) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    }
+    if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // (not before this CTA has its tensor memory: a dependent that took the columns first would wait for this grid, and this grid for them)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (threadIdx.x == 0) CA_TRACE(1);
     auto wait_slow = [&](int i, uint32_t code) -> bool {

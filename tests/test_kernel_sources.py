@@ -1,0 +1,39 @@
+"""Rules that every kernel keeps and no run can show reliably, checked on the sources."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2607_14695_b200", "csrc")
+
+
+def _kernels():
+    """(file: name, parameters, body) of every __global__ function; comments taken out."""
+    out = []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh"))):
+        text = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(path).read(), flags=re.S)
+        for m in re.finditer(r"__global__\s+void\s+(?:__\w+__\((?:[^()]|\([^()]*\))*\)\s*)*(\w+)\s*\(([^{]*?)\)\s*\{", text):
+            depth, i = 1, m.end()
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[i], 0)
+                i += 1
+            out.append((f"{os.path.basename(path)}: {m.group(1)}", m.group(2), text[m.end():i]))
+    return out
+
+
+KERNELS = _kernels()
+
+
+def test_kernels_are_found():
+    names = {n.split(": ")[1] for n, _, _ in KERNELS}
+    assert {"chain_attn_kernel", "chain_attn128_kernel", "chain_gemm_kernel", "chain_in_kernel", "tile_gemm_kernel", "attn_tc2_kernel", "gate_kernel",
+            "flow_step_kernel", "init_static_kernel", "linear_res_tc_kernel"} <= names
+
+
+@pytest.mark.parametrize("kernel", [k for k in KERNELS if "tmem_alloc" in k[2]], ids=lambda k: k[0])
+def test_tensor_memory_is_taken_before_dependents_are_released(kernel):
+    """A dependent grid may move in as soon as it is released. If it takes tensor memory that this grid has yet to take, the two wait
+    for one another."""
+    _, _, body = kernel
+    assert body.index("tmem_alloc") < body.index("griddepcontrol.launch_dependents")
