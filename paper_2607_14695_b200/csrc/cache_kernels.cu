@@ -68,8 +68,7 @@ cudaError_t launch_state_init(StreamState *state, int64_t *total, uint32_t *stat
 constexpr int kCopyUnits = 6;
 
 __global__ void __launch_bounds__(256)
-init_static_kernel(uint4 *__restrict__ k_slab, uint4 *__restrict__ v_slab, const uint4 *__restrict__ k_src,
-                   const uint4 *__restrict__ v_src, StreamState *state, StreamBatch batch, int src_stream0, int L, int B,
+init_static_kernel(uint4 *k_slab, uint4 *v_slab, const uint4 *k_src, const uint4 *v_src, StreamState *state, StreamBatch batch, int src_stream0, int L, int B,
                    int rows_per_block /* ring_off + N */, int S_max, int S_src, int row_units, int to_other_bank)
 {
     wait_then_release();
@@ -119,8 +118,7 @@ cudaError_t launch_init_static(void *k_slab, void *v_slab, const void *k_src, co
 // L*m rows to slots (head + i) mod N, then takes a ticket; the last block to arrive publishes the new
 // state. No block waits for another, so there is no spin and nothing to time out.
 __global__ void __launch_bounds__(256)
-append_sliding_kernel(uint4 *__restrict__ k_slab, uint4 *__restrict__ v_slab, const uint4 *__restrict__ k_src,
-                      const uint4 *__restrict__ v_src, StreamState *state, int64_t *total, StreamBatch batch,
+append_sliding_kernel(uint4 *k_slab, uint4 *v_slab, const uint4 *k_src, const uint4 *v_src, StreamState *state, int64_t *total, StreamBatch batch,
                       int src_stream0, int L, int B, int ring_off, int N, int m, int row_units)
 {
     wait_then_release();

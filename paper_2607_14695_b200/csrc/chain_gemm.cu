@@ -510,8 +510,8 @@ constexpr int kCiRows = 4;       // rows at a time
 // for every four rows: 27 us for 3200 rows.)
 template <int A>
 __global__ void __launch_bounds__(256)
-chain_in_kernel(const float *__restrict__ a, const __nv_bfloat16 *__restrict__ W, const float *__restrict__ gate, __nv_bfloat16 *__restrict__ h,
-                __nv_bfloat16 *__restrict__ xg, float *__restrict__ ss_out, int M, int R, int D, int groups)
+chain_in_kernel(const float *a, const __nv_bfloat16 *W, const float *gate, __nv_bfloat16 *h, __nv_bfloat16 *xg, float *ss_out, int M, int R, int D,
+                int groups)
 {
     __shared__ __align__(16) float as[kCiRows][A];
     __shared__ float part[kCiRows][8];

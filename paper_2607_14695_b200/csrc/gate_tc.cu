@@ -50,7 +50,7 @@ static_assert(kGtPerSm * (GateTcSmem::total(kGtMaxChunks, 1) + 1024) <= 228 * 10
 template <bool SILU, int PASSES>
 __global__ void __launch_bounds__(256, kGtPerSm)
 gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_v0, const __grid_constant__ CUtensorMap tm_v1,
-               const __nv_bfloat16 *__restrict__ bias, float *out_f32, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, int B, int len, int units,
+               const __nv_bfloat16 *bias, float *out_f32, __nv_bfloat16 *out_hi, __nv_bfloat16 *out_lo, int B, int len, int units,
                int vec_rows_per_layer, uint32_t *status)
 {
     using S = GateTcSmem;

@@ -464,7 +464,7 @@ template <> __device__ __forceinline__ __nv_bfloat16 lin_from_f<__nv_bfloat16>(f
 
 template <typename T>
 __global__ void __launch_bounds__(256)
-linear_res_simt_kernel(const T *__restrict__ a, const T *__restrict__ W, const T *res, T *out, int K, int N)
+linear_res_simt_kernel(const T *a, const T *W, const T *res, T *out, int K, int N)
 {
     extern __shared__ float asm_row[];
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -93,8 +93,7 @@ __device__ void gate_columns(const T *__restrict__ W2, const T *__restrict__ b2,
 // grid = (column chunks, B, layers): writes gate_buf[layer][b][i]; every block computes the hidden layer for itself.
 template <typename T>
 __global__ void __launch_bounds__(256)
-gate_kernel(const T *__restrict__ cond, const T *__restrict__ W1, const T *__restrict__ b1, const T *__restrict__ W2,
-            const T *__restrict__ b2, float *__restrict__ gate_buf, int D, int Cd, int Hd, int cols_per_block)
+gate_kernel(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, float *gate_buf, int D, int Cd, int Hd, int cols_per_block)
 {
     extern __shared__ float smem[];
     float *c_s = smem, *hid_s = smem + Cd;
@@ -535,7 +534,7 @@ cudaError_t launch_adarmsnorm(const void *x, void *y, const void *cond, const vo
 
 // Euler update (Sec. 2.1; App. C): x <- x + dt * v on the fp32 master, optional low-precision mirror.
 template <typename T>
-__global__ void flow_step_kernel(float *__restrict__ x, const T *__restrict__ v, T *__restrict__ x_lowp, size_t n, float dt)
+__global__ void flow_step_kernel(float *x, const T *v, T *x_lowp, size_t n, float dt)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

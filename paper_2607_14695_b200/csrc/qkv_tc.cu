@@ -910,7 +910,7 @@ template <> __device__ __forceinline__ __nv_bfloat16 qk_from_f<__nv_bfloat16>(fl
 
 template <typename T>
 __global__ void __launch_bounds__(256)
-norm_qkv_simt_kernel(const T *__restrict__ x, const float *__restrict__ gate, const T *__restrict__ W, T *q, T *k, T *v,
+norm_qkv_simt_kernel(const T *x, const float *gate, const T *W, T *q, T *k, T *v,
                      int R, int D, int nq, int nk, int swiglu_F, float eps)
 {
     extern __shared__ float ysm[];    // [D] + 8 partial sums

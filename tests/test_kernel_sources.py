@@ -37,3 +37,13 @@ def test_tensor_memory_is_taken_before_dependents_are_released(kernel):
     for one another."""
     _, _, body = kernel
     assert body.index("tmem_alloc") < body.index("griddepcontrol.launch_dependents")
+
+
+@pytest.mark.parametrize("kernel", [k for k in KERNELS if re.search(r"griddepcontrol\.wait|wait_then_release", k[2])], ids=lambda k: k[0])
+def test_inputs_read_behind_the_wait_may_not_be_taken_for_constants(kernel):
+    """A programmatically launched grid may run beside the one that writes its inputs. A const __restrict__ parameter promises that
+    nobody writes it while the kernel runs, so its loads could be moved ahead of the wait. (The weights of the plain gate kernels, which
+    wait_prior marks, are read ahead of it on purpose: the launch in front of them writes none.)"""
+    _, params, _ = kernel
+    bad = re.findall(r"const [^,]*__restrict__ (\w+)", params)
+    assert not [b for b in bad if not ("wait_prior" in params and b in ("W", "bias"))], bad
