@@ -471,7 +471,7 @@ cudaError_t cg_launch_mode(int mode, const CgConfig &c, const CUtensorMap &mx, c
 bool chain_proj_supported(int mode, int M, int K, int N)
 {
     CgConfig c;
-    return M >= 1 && (M <= kCgMaxRows || mode == CG_OUT) && K % 8 == 0 && N % 8 == 0 && cg_choose(mode, M, K, N, c);
+    return M >= 1 && K >= 8 && N >= 8 && (M <= kCgMaxRows || mode == CG_OUT) && K % 8 == 0 && N % 8 == 0 && cg_choose(mode, M, K, N, c);
 }
 
 cudaError_t launch_chain_proj(const ChainProj &a, cudaStream_t st)

@@ -647,7 +647,14 @@ int reflex_expert_step(reflex_cache_t *c, const reflex_expert *ep, float *a, con
     }
     if (K < 1 || k < 0 || k >= K) return fail(REFLEX_ERR_INVALID_ARG, "step k=%d outside [0, K=%d)", k, K);
     if (e.T < 1 || e.T > d.T_max) return fail(REFLEX_ERR_SHAPE, "T=%d outside [1, T_max=%d]", e.T, d.T_max);
-    if (e.A < 1) return fail(REFLEX_ERR_SHAPE, "A=%d must be >= 1", e.A);
+    // the limits of the single calls, all of them before the first launch
+    auto bad = [](int n, int most) { return n < 8 || n % 8 != 0 || n > most; };
+    if (bad(e.D, 8192) || bad(e.F, 12288) || bad(e.A, 12288) || bad(e.Cd, 1024) || bad(e.Hd, 1024))
+        return fail(REFLEX_ERR_SHAPE, "D=%d (<= 8192), F=%d, A=%d (<= 12288), Cd=%d, Hd=%d (<= 1024) must be multiples of 8", e.D, e.F, e.A, e.Cd, e.Hd);
+    if (d.Hq * (long long)d.d > 12288 || (d.Hq + 2LL * d.Hkv) * d.d > 65536)
+        return fail(REFLEX_ERR_SHAPE, "Hq=%d, Hkv=%d, d=%d: need Hq d <= 12288, (Hq + 2 Hkv) d <= 65536", d.Hq, d.Hkv, d.d);
+    if (2LL * d.L + 1 > 65535) return fail(REFLEX_ERR_SHAPE, "L=%d: 2 L + 1 must be <= 65535", d.L);
+    if ((long long)d.B * e.T * (e.D > e.A ? e.D : e.A) > 0x3FFFFFFF) return fail(REFLEX_ERR_SHAPE, "B=%d, T=%d, D=%d, A=%d", d.B, e.T, e.D, e.A);
     if (!(e.eps >= 0.f)) return fail(REFLEX_ERR_INVALID_ARG, "eps must be >= 0");
     for (int b = 0; b < d.B; ++b)
         if (c->static_len[b] < 0) return fail(REFLEX_ERR_STATE, "stream %d: static prefix never initialised (reflex_cache_init_static, S = 0 allowed)", b);

@@ -1157,6 +1157,32 @@ def test_expert_step_bf16_chained(U, case):
     _expert_case(U, w, F, 2e-2, "expert bf16, chained", streams=None if B <= 6 else [0, B // 2, B - 1])
 
 
+@pytest.mark.parametrize("field,value", [("F", 0), ("F", -8), ("F", 12), ("F", 12296), ("D", 0), ("D", 100), ("D", 8200), ("A", 0), ("A", 12), ("Cd", 0), ("Cd", 1032),
+                                         ("Hd", 4), ("T", 0), ("T", 51), ("eps", -1.0)])
+def test_expert_step_refuses_before_it_launches(U, field, value):
+    """Widths that the single calls refuse are refused by the whole step, with nothing launched and nothing written."""
+    from paper_2607_14695_b200 import expert as ex
+    rb = U.rb
+    w = synth.CONFIGS["cfg2"].with_(B=1, L=1, T=50, S=64, S_max=64)
+    tw = U.Twin(w)
+    tw.init_static([0], [64])
+    model = ex.ActionExpert(w, tw.g, ex.random_weights_device(w, 512, U.DEV), 512, device=U.DEV)
+    d = rb.ExpertDesc(w.T, w.D, 512, w.A, w.Cd, w.Hd, 1e-6, 0)
+    for n in ex._WEIGHTS:
+        setattr(d, n, model.W[n].data_ptr())
+    for n in ex._BUFFERS:
+        getattr(model, n).fill_(7.0)
+        setattr(d, n, getattr(model, n).data_ptr())
+    setattr(d, field, value)
+    a, cond = torch.zeros((1, w.T, w.A), device=U.DEV), torch.zeros((1, w.Cd), dtype=torch.bfloat16, device=U.DEV)
+    before = rb.reflex_kernel_launch_count()
+    with pytest.raises(rb.ReflexError) as err:
+        rb.reflex_expert_step(tw.g, d, a, cond, 0, 10)
+    assert err.value.code == (rb.ERR_INVALID_ARG if field == "eps" else rb.ERR_SHAPE)
+    assert rb.reflex_kernel_launch_count() == before
+    assert all(bool((getattr(model, n) == 7.0).all()) for n in ex._BUFFERS)
+
+
 CLUSTERS_OF_FOUR = [
     # B, T, Hq, Hkv, S_max, prefix lengths, N: edges of the attention that merges four key slices per 128 rows (three to eight streams)
     (4, 50, 8, 1, 816, [816, 700, 0, 113], 32), (8, 64, 8, 1, 896, [896] * 8, 64), (6, 60, 4, 2, 300, [300, 1, 2, 7, 8, 299], 5),
