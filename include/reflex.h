@@ -309,11 +309,11 @@ int reflex_flow_step(void *x, const void *v, void *x_lowp, int B, int T, int A, 
  * Nothing inside the step writes weights or cache regions, so its kernels may ask for them ahead of their turn; the first kernel
  * waits for everything ahead of it on the stream. No other work on the device may write the weights or the cache regions that
  * are being read while a step runs (reflex_cache_stage_static, which writes the idle bank, may).
- * All tensors device, dense, 16-byte aligned, in the cache's dtype unless said otherwise; L, B, Hq, Hkv, d are the cache's. */
+ * All tensors device, dense, 16-byte aligned, in the cache's dtype unless said otherwise; B, Hq, Hkv, d are the cache's. */
 typedef struct {
     int32_t T, D, F, A, Cd, Hd;           /* tokens per stream, model / SwiGLU / action / conditioning / gate-MLP widths */
     float eps;
-    int32_t reserved;
+    int32_t L;                            /* layers, at most the cache's; 0 = all of the cache's                 */
     const void *W_in, *W_out;             /* [D][A], [A][D]                                                     */
     const void *Wqkv, *Wo, *Wgu, *Wd;     /* stacked over layers: [L][(Hq+2Hkv)d][D], [L][D][Hq d], [L][2F][D], [L][D][F] */
     const void *W1, *b1, *W2, *b2;        /* gate MLPs of the 2L + 1 norms, as reflex_adarmsnorm_gate takes them  */

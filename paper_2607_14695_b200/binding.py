@@ -35,7 +35,7 @@ EXPORTS = [
 
 class ExpertDesc(ctypes.Structure):
     """struct reflex_expert: the tensors of a whole expert step."""
-    _fields_ = ([(n, ctypes.c_int32) for n in ("T", "D", "F", "A", "Cd", "Hd")] + [("eps", ctypes.c_float), ("reserved", ctypes.c_int32)] +
+    _fields_ = ([(n, ctypes.c_int32) for n in ("T", "D", "F", "A", "Cd", "Hd")] + [("eps", ctypes.c_float), ("L", ctypes.c_int32)] +
                 [(n, ctypes.c_void_p) for n in ("W_in", "W_out", "Wqkv", "Wo", "Wgu", "Wd", "W1", "b1", "W2", "b2", "gates", "h", "y", "q", "k", "v", "o", "m",
                                                 "vel", "a_lowp", "row_sums")])
 

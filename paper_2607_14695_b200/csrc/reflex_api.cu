@@ -564,7 +564,7 @@ static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float 
 {
     const reflex_cache_desc &d = c->desc;
     typedef __nv_bfloat16 bf;
-    const int L = d.L, B = d.B, T = e.T, D = e.D, M = B * T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
+    const int L = e.L > 0 ? e.L : d.L, B = d.B, T = e.T, D = e.D, M = B * T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
     cudaStream_t st = (cudaStream_t)stream;
     auto proj = [&](const ChainProj &p) { return !tiled ? launch_chain_proj(p, st) : p.mode == CG_RES ? launch_tile_res(p, st) : launch_tile_proj(p, st); };
     auto slots_of = [&](int K) { return tiled ? tile_res_slots(M, K, D) : (D + 31) / 32; };
@@ -653,12 +653,13 @@ int reflex_expert_step(reflex_cache_t *c, const reflex_expert *ep, float *a, con
         return fail(REFLEX_ERR_SHAPE, "D=%d (<= 8192), F=%d, A=%d (<= 12288), Cd=%d, Hd=%d (<= 1024) must be multiples of 8", e.D, e.F, e.A, e.Cd, e.Hd);
     if (d.Hq * (long long)d.d > 12288 || (d.Hq + 2LL * d.Hkv) * d.d > 65536)
         return fail(REFLEX_ERR_SHAPE, "Hq=%d, Hkv=%d, d=%d: need Hq d <= 12288, (Hq + 2 Hkv) d <= 65536", d.Hq, d.Hkv, d.d);
+    if (e.L < 0 || e.L > d.L) return fail(REFLEX_ERR_SHAPE, "L=%d outside [0, %d]", e.L, d.L);
     if (2LL * d.L + 1 > 65535) return fail(REFLEX_ERR_SHAPE, "L=%d: 2 L + 1 must be <= 65535", d.L);
     if ((long long)d.B * e.T * (e.D > e.A ? e.D : e.A) > 0x3FFFFFFF) return fail(REFLEX_ERR_SHAPE, "B=%d, T=%d, D=%d, A=%d", d.B, e.T, e.D, e.A);
     if (!(e.eps >= 0.f)) return fail(REFLEX_ERR_INVALID_ARG, "eps must be >= 0");
     for (int b = 0; b < d.B; ++b)
         if (c->static_len[b] < 0) return fail(REFLEX_ERR_STATE, "stream %d: static prefix never initialised (reflex_cache_init_static, S = 0 allowed)", b);
-    const int L = d.L, B = d.B, T = e.T, D = e.D, M = B * T, nq = d.Hq * d.d, nk = d.Hkv * d.d, dt_ = d.dtype;
+    const int L = e.L > 0 ? e.L : d.L, B = d.B, T = e.T, D = e.D, M = B * T, nq = d.Hq * d.d, nk = d.Hkv * d.d, dt_ = d.dtype;
     int rc = reflex_adarmsnorm_gate(cond, e.W1, e.b1, e.W2, e.b2, e.gates, 2 * L + 1, B, D, e.Cd, e.Hd, dt_, stream);
     if (rc != REFLEX_OK) return rc;
     const bool chained = expert_chained(d, e);

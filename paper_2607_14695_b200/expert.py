@@ -48,7 +48,7 @@ class ActionExpert:
 
     def step(self, a: torch.Tensor, cond: torch.Tensor, k: int, stream=None):
         """One Euler step on the fp32 action chunk a [B][T][A] (updated in place); cond [B][Cd] in the storage dtype."""
-        d, w, W = rb.ExpertDesc(self.w.T, self.w.D, self.F, self.w.A, self.w.Cd, self.w.Hd, 1e-6, 0), self.w, self.W
+        d, w, W = rb.ExpertDesc(self.w.T, self.w.D, self.F, self.w.A, self.w.Cd, self.w.Hd, 1e-6, self.w.L), self.w, self.W
         for n in _WEIGHTS:
             if not W[n].is_contiguous():
                 raise ValueError(f"weight {n} must be contiguous")

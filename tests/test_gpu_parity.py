@@ -1087,11 +1087,11 @@ def _with_guards(model):
     return tails
 
 
-def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None):
+def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None, cache_layers=None):
     from oracle import expert_oracle as eo
     from paper_2607_14695_b200 import expert as ex
     rb = U.rb
-    tw = U.Twin(w, head0=[3] * w.B, poison=True)
+    tw = U.Twin(w.with_(L=cache_layers or w.L), head0=[3] * w.B, poison=True)
     tw.init_static(list(range(w.B)), S_list or [w.S] * w.B)
     for i in range(3):
         tw.append(list(range(w.B)), 2, i)
@@ -1158,7 +1158,7 @@ def test_expert_step_bf16_chained(U, case):
 
 
 @pytest.mark.parametrize("field,value", [("F", 0), ("F", -8), ("F", 12), ("F", 12296), ("D", 0), ("D", 100), ("D", 8200), ("A", 0), ("A", 12), ("Cd", 0), ("Cd", 1032),
-                                         ("Hd", 4), ("T", 0), ("T", 51), ("eps", -1.0)])
+                                         ("Hd", 4), ("T", 0), ("T", 51), ("L", 2), ("L", -1), ("eps", -1.0)])
 def test_expert_step_refuses_before_it_launches(U, field, value):
     """Widths that the single calls refuse are refused by the whole step, with nothing launched and nothing written."""
     from paper_2607_14695_b200 import expert as ex
@@ -1181,6 +1181,12 @@ def test_expert_step_refuses_before_it_launches(U, field, value):
     assert err.value.code == (rb.ERR_INVALID_ARG if field == "eps" else rb.ERR_SHAPE)
     assert rb.reflex_kernel_launch_count() == before
     assert all(bool((getattr(model, n) == 7.0).all()) for n in ex._BUFFERS)
+
+
+@pytest.mark.parametrize("B", [1, 6, 4])
+def test_expert_step_of_fewer_layers_than_the_cache(U, B):
+    w = synth.CONFIGS["cfg2"].with_(B=B, L=2, S=100, S_max=104)
+    _expert_case(U, w, 512, 2e-2, "expert of fewer layers than the cache", streams=[0, B - 1], cache_layers=4)
 
 
 CLUSTERS_OF_FOUR = [
