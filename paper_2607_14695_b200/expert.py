@@ -39,6 +39,9 @@ class ActionExpert:
         self.m = e(B, T, F)
         self.vel = e(B, T, w.A)
         self.a_lowp = e(B, T, w.A)
+        nq, nkv = w.Hq * w.d, w.Hkv * w.d
+        self.shapes = {"W_in": (D, w.A), "W_out": (w.A, D), "Wqkv": (w.L, nq + 2 * nkv, D), "Wo": (w.L, D, nq), "Wgu": (w.L, 2 * F, D), "Wd": (w.L, D, F),
+                       "W1": (n_norm, w.Hd, w.Cd), "b1": (n_norm, w.Hd), "W2": (n_norm, D, w.Hd), "b2": (n_norm, D)}
         self.row_sums = torch.empty((2 * B * T * ((D + 31) // 32),), dtype=torch.float32, device=self.dev)
 
     def gate(self, i: int):
@@ -48,8 +51,15 @@ class ActionExpert:
 
     def step(self, a: torch.Tensor, cond: torch.Tensor, k: int, stream=None):
         """One Euler step on the fp32 action chunk a [B][T][A] (updated in place); cond [B][Cd] in the storage dtype."""
-        d, w, W = rb.ExpertDesc(self.w.T, self.w.D, self.F, self.w.A, self.w.Cd, self.w.Hd, 1e-6, self.w.L), self.w, self.W
-        for n in _WEIGHTS:
+        w, W, c = self.w, self.W, self.cache.desc
+        if (c.B, c.Hq, c.Hkv, c.d, c.dtype) != (w.B, w.Hq, w.Hkv, w.d, w.dtype) or c.L < w.L:
+            raise ValueError("the cache has other streams, heads, head widths or storage, or fewer layers than the expert")
+        _want("a", a, (w.B, w.T, w.A), torch.float32, self.vel.device)
+        _want("cond", cond, (w.B, w.Cd), self.tdt, self.vel.device)
+        d = rb.ExpertDesc(w.T, w.D, self.F, w.A, w.Cd, w.Hd, 1e-6, w.L)
+        for n, shape in self.shapes.items():
+            more = n in _LAYERS and W[n].shape[:1] != shape[:1]         # (a stack may hold more layers than the expert uses)
+            _want(n, W[n][:w.L] if more else W[n], shape, self.tdt, self.vel.device)
             if not W[n].is_contiguous():
                 raise ValueError(f"weight {n} must be contiguous")
             setattr(d, n, W[n].data_ptr())
@@ -58,7 +68,13 @@ class ActionExpert:
         return rb.reflex_expert_step(self.cache, d, a, cond, k, w.K, stream=stream)
 
 
+def _want(name: str, t: torch.Tensor, shape: tuple, dtype: torch.dtype, device: torch.device):
+    if t.shape != shape or t.dtype != dtype or t.device != device:
+        raise ValueError(f"{name} must be {list(shape)} {dtype} on {device}, got {list(t.shape)} {t.dtype} on {t.device}")
+
+
 _BUFFERS = ("gates", "h", "y", "q", "k", "v", "o", "m", "vel", "a_lowp", "row_sums")
+_LAYERS = ("Wqkv", "Wo", "Wgu", "Wd")
 _WEIGHTS = ("W_in", "W_out", "Wqkv", "Wo", "Wgu", "Wd", "W1", "b1", "W2", "b2")
 
 
