@@ -56,16 +56,39 @@ class ActionExpert:
             raise ValueError("the cache has other streams, heads, head widths or storage, or fewer layers than the expert")
         _want("a", a, (w.B, w.T, w.A), torch.float32, self.vel.device)
         _want("cond", cond, (w.B, w.Cd), self.tdt, self.vel.device)
+        if not all(isinstance(W[n], torch.Tensor) and W[n].is_contiguous() for n in _WEIGHTS):
+            return self._step_by_calls(a, cond, k, stream)
         d = rb.ExpertDesc(w.T, w.D, self.F, w.A, w.Cd, w.Hd, 1e-6, w.L)
         for n, shape in self.shapes.items():
-            more = n in _LAYERS and W[n].shape[:1] != shape[:1]         # (a stack may hold more layers than the expert uses)
-            _want(n, W[n][:w.L] if more else W[n], shape, self.tdt, self.vel.device)
-            if not W[n].is_contiguous():
-                raise ValueError(f"weight {n} must be contiguous")
+            t = W[n]
+            if n in _LAYERS and t.shape[:1] != shape[:1]:
+                t = t[:w.L]                         # a stack may hold more layers than the expert uses
+            elif n in ("b1", "b2") and t.numel() == shape[0] * shape[1]:
+                t = t.view(shape)                   # biases in any shape
+            _want(n, t, shape, self.tdt, self.vel.device)
             setattr(d, n, W[n].data_ptr())
         for n in _BUFFERS:
             setattr(d, n, getattr(self, n).data_ptr())
         return rb.reflex_expert_step(self.cache, d, a, cond, k, w.K, stream=stream)
+
+    def _step_by_calls(self, a, cond, k, stream):
+        """The same step for weights that are not one dense stack (a list of layers, a slice of a wider tensor): the single calls in order."""
+        w, W = self.w, self.W
+        B, T, D = w.B, w.T, w.D
+        kw = dict(cache=self.cache, stream=stream)
+        rb.reflex_adarmsnorm_gate(cond, W["W1"], W["b1"], W["W2"], W["b2"], self.gates, stream=stream)   # all 2L + 1 gates
+        self.a_lowp.copy_(a)
+        rb.reflex_linear_residual(self.a_lowp.view(B * T, w.A), W["W_in"], None, self.h.view(B * T, D), **kw)
+        for l in range(w.L):
+            rb.reflex_adarmsnorm_qkv(self.h, self.gate(2 * l), W["Wqkv"][l], self.q, self.k, self.v, **kw)
+            rb.reflex_partitioned_attention(self.cache, l, self.q, self.k, self.v, self.o, stream=stream)
+            rb.reflex_linear_residual(self.o.view(B * T, w.Hq * w.d), W["Wo"][l], self.h, self.h, **kw)
+            rb.reflex_adarmsnorm_swiglu(self.h, self.gate(2 * l + 1), W["Wgu"][l], self.m, **kw)
+            rb.reflex_linear_residual(self.m.view(B * T, self.F), W["Wd"][l], self.h, self.h, **kw)
+        rb.reflex_adarmsnorm(self.h, self.y, None, None, None, None, None, gate_buf=self.gate(2 * w.L), stream=stream)
+        rb.reflex_linear_residual(self.y.view(B * T, D), W["W_out"], None, self.vel.view(B * T, w.A), **kw)
+        rb.reflex_flow_step(a, self.vel, None, k, w.K, stream=stream)
+        return a
 
 
 def _want(name: str, t: torch.Tensor, shape: tuple, dtype: torch.dtype, device: torch.device):

@@ -37,6 +37,9 @@ def test_step_passes_on_what_fits(calls):
     assert _model().step(a, torch.zeros(COND, dtype=torch.bfloat16), 0) is a
     assert _model(cache=dict(L=7)).step(a, torch.zeros(COND, dtype=torch.bfloat16), 0) is a
     assert [d.L for d in calls] == [W.L, W.L] and calls[0].F == F
+    m = _model()
+    m.W.update(b1=m.W["b1"].reshape(-1), Wo=torch.cat([m.W["Wo"]] * 2))
+    assert m.step(a, torch.zeros(COND, dtype=torch.bfloat16), 0) is a
 
 
 @pytest.mark.parametrize("a", [torch.zeros(1, W.T, W.A), torch.zeros(W.B, W.T - 1, W.A), torch.zeros(W.B * W.T, W.A), torch.zeros(CHUNK, dtype=torch.bfloat16),

@@ -1087,7 +1087,7 @@ def _with_guards(model):
     return tails
 
 
-def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None, cache_layers=None):
+def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None, cache_layers=None, weights=lambda dW: dW):
     from oracle import expert_oracle as eo
     from paper_2607_14695_b200 import expert as ex
     rb = U.rb
@@ -1097,7 +1097,7 @@ def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None, cache_layers=N
         tw.append(list(range(w.B)), 2, i)
     W = ex.expert_weights(w, F, std_scale=0.5)
     dW = {n: U.to_dev(v, w.dtype) for n, v in W.items()}
-    model = ex.ActionExpert(w, tw.g, dW, F, device=U.DEV)
+    model = ex.ActionExpert(w, tw.g, weights(dW), F, device=U.DEV)
     tails = _with_guards(model)
     a0 = synth.normal(w, "noise", (w.B, w.T, w.A)).astype(np.float64)
     if w.dtype == synth.DTYPE_BF16:          # the step reads the chunk through a storage-dtype mirror: start from representable values
@@ -1181,6 +1181,26 @@ def test_expert_step_refuses_before_it_launches(U, field, value):
     assert err.value.code == (rb.ERR_INVALID_ARG if field == "eps" else rb.ERR_SHAPE)
     assert rb.reflex_kernel_launch_count() == before
     assert all(bool((getattr(model, n) == 7.0).all()) for n in ex._BUFFERS)
+
+
+def _list_of_layers(dW):
+    return {n: [t.clone() for t in v] if n in ("Wqkv", "Wo", "Wgu", "Wd") else v for n, v in dW.items()}
+
+
+def _slice_of_wider(dW):
+    """Stacks with rows of other tensors between the layers."""
+    return {n: torch.cat([v, torch.full_like(v, float("nan"))], 1)[:, :v.shape[1]] if n in ("Wqkv", "Wo", "Wgu", "Wd") else v for n, v in dW.items()}
+
+
+def _more_layers(dW):
+    return {n: torch.cat([v, torch.full_like(v, float("nan"))], 0) if n in ("Wqkv", "Wo", "Wgu", "Wd") else v for n, v in dW.items()}
+
+
+@pytest.mark.parametrize("B", [1, 6, 4])       # chained, tiled and single calls
+@pytest.mark.parametrize("weights", [_list_of_layers, _slice_of_wider, _more_layers])
+def test_expert_step_weights_of_other_layouts(U, weights, B):
+    w = synth.CONFIGS["cfg2"].with_(B=B, L=2, S=100, S_max=104)
+    _expert_case(U, w, 512, 2e-2, "expert, weights of another layout", streams=[0, B - 1], weights=weights)
 
 
 @pytest.mark.parametrize("B", [1, 6, 4])
