@@ -74,8 +74,11 @@ int integer(PyObject *o)
 
 float real(PyObject *o)
 {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw Bad();
+    // (anything float() takes)
+    PyObject *n = PyFloat_Check(o) ? (Py_INCREF(o), o) : PyNumber_Float(o);
+    if (!n) throw Bad();
+    const double v = PyFloat_AS_DOUBLE(n);
+    Py_DECREF(n);
     return (float)v;
 }
 
@@ -106,7 +109,7 @@ std::vector<int32_t> ints(PyObject *o)
     PyObject *seq = PySequence_Fast(o, "expected a sequence of integers");
     if (!seq) throw Bad();
     const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);
-    v.reserve((size_t)n);
+    v.reserve((size_t)(n > 0 ? n : 1));      // (no elements is not the same as no list: data() is not NULL)
     try {
         for (Py_ssize_t i = 0; i < n; ++i) v.push_back(integer(PySequence_Fast_GET_ITEM(seq, i)));
     } catch (...) { Py_DECREF(seq); throw; }
@@ -114,15 +117,16 @@ std::vector<int32_t> ints(PyObject *o)
     return v;
 }
 
-// The call runs without the interpreter lock (a launch may block when the device's queue is full).
+// The call runs without the interpreter lock (a launch may block when the device's queue is full), which is taken again whatever way
+// the call ends.
 template <typename F>
 int unlocked(F &&f)
 {
-    int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = f();
-    Py_END_ALLOW_THREADS
-    return rc;
+    struct Unlocked {
+        PyThreadState *state = PyEval_SaveThread();
+        ~Unlocked() { PyEval_RestoreThread(state); }
+    } guard;
+    return f();
 }
 
 template <typename F>
@@ -147,6 +151,7 @@ PyObject *adarmsnorm(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return entry(n, 10, [&]() -> PyObject * {
         want_dims(a[0], 3);
+        if (a[3] != Py_None) want_dims(a[3], 2);
         const int B = dim(a[0], 0), R = dim(a[0], 1), D = dim(a[0], 2), Hd = a[3] == Py_None ? 0 : dim(a[3], 0), Cd = a[3] == Py_None ? 0 : dim(a[3], 1);
         const int dt = dtype(a[0]);
         const float eps = real(a[8]);
@@ -245,8 +250,8 @@ PyObject *write_static(PyObject *, PyObject *const *a, Py_ssize_t n)
         const int which = integer(a[0]), S_src = a[3] == Py_None ? 0 : dim(a[3], 2);
         reflex_cache_t *c = handle(a[1]);
         const std::vector<int32_t> ids = ints(a[2]), S = ints(a[5]);
-        if (a[5] != Py_None && S.size() != ids.size()) {
-            PyErr_SetString(PyExc_ValueError, "one prefix length per stream");
+        if (a[5] != Py_None && S.size() < ids.size()) {
+            PyErr_SetString(PyExc_ValueError, "a prefix length for every stream");
             throw Bad();
         }
         void *k = ptr(a[3]), *v = ptr(a[4]), *st = stream(a[6]);
