@@ -7,7 +7,7 @@
 //     weights, and a kernel of the chain only starts once its predecessor has passed its own wait, which the first kernel
 //     of the step does only when everything ahead of the step is complete: the loads see what the caller wrote.
 //   - the adaptive norm sits in the epilogue of the projection that PRODUCES the residual stream: it writes h, h * gamma of
-//     the norm that follows (bf16) and the sums of squares of its columns. The projection that reads the norm takes
+//     the norm that follows (bf16) and the sums of squares of its columns, both from h before its rounding. The projection takes
 //     h * gamma straight by TMA (no rewriting of operand tiles in shared memory) and applies 1 / RMS to its accumulator.
 //   - with the contraction split over the CTAs of a cluster, a CTA pushes its partial sums into the shared memory of the CTA
 //     that finishes the row (st.async, counted on that CTA's mbarrier): no cluster barrier between the last MMA and the
@@ -82,10 +82,6 @@ __device__ __forceinline__ uint2 pack4_bf16(float a, float b, float c, float d)
 {
     __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
     return make_uint2(*reinterpret_cast<uint32_t *>(&lo), *reinterpret_cast<uint32_t *>(&hi));
-}
-__device__ __forceinline__ float4 unpack4_bf16(uint2 v)
-{
-    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
 }
 
 // SiLU(g) * u with one special-function operation (tanh.approx, about 2^-11: a quarter of the spacing of the bf16 result)
@@ -339,10 +335,9 @@ chain_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 for (int i = 0; i < 4; ++i) {
                     sq[i] = 0.f;
                     if (f_ok && r + i < p.M) {
-                        const __nv_bfloat16 hv = __float2bfloat16_rn(val[i] + res4[i]);
-                        const float h = __bfloat162float(hv);
+                        const float h = val[i] + res4[i];           // (the norm takes the sum before its rounding: one rounding less)
                         const size_t o = (size_t)(r + i) * p.n_feat + fg;
-                        p.h[o] = hv;
+                        p.h[o] = __float2bfloat16_rn(h);
                         p.xg[o] = __float2bfloat16_rn(h * gate4[i]);
                         sq[i] = h * h;
                     }
@@ -556,12 +551,11 @@ chain_in_kernel(const float *a, const __nv_bfloat16 *W, const float *gate, __nv_
                                 acc[j] = fmaf(av[2 * i + 1], __uint_as_float(ww[i] & 0xFFFF0000u), fmaf(av[2 * i], __uint_as_float(ww[i] << 16), acc[j]));
                         }
                     }
-                    const uint2 hv = pack4_bf16(acc[0], acc[1], acc[2], acc[3]);
-                    const float4 h4 = unpack4_bf16(hv), g4 = *reinterpret_cast<const float4 *>(gate + (size_t)((row0 + r) / R) * D + f);
+                    const float4 g4 = *reinterpret_cast<const float4 *>(gate + (size_t)((row0 + r) / R) * D + f);
                     const size_t o = (size_t)(row0 + r) * D + f;
-                    *reinterpret_cast<uint2 *>(h + o) = hv;
-                    *reinterpret_cast<uint2 *>(xg + o) = pack4_bf16(h4.x * g4.x, h4.y * g4.y, h4.z * g4.z, h4.w * g4.w);
-                    ss = fmaf(h4.x, h4.x, fmaf(h4.y, h4.y, fmaf(h4.z, h4.z, h4.w * h4.w)));
+                    *reinterpret_cast<uint2 *>(h + o) = pack4_bf16(acc[0], acc[1], acc[2], acc[3]);
+                    *reinterpret_cast<uint2 *>(xg + o) = pack4_bf16(acc[0] * g4.x, acc[1] * g4.y, acc[2] * g4.z, acc[3] * g4.w);
+                    ss = fmaf(acc[0], acc[0], fmaf(acc[1], acc[1], fmaf(acc[2], acc[2], acc[3] * acc[3])));
                 }
                 for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
                 if ((threadIdx.x & 31) == 0) part[r][threadIdx.x >> 5] = fb == 0 ? ss : part[r][threadIdx.x >> 5] + ss;

@@ -1183,6 +1183,50 @@ def test_expert_step_refuses_before_it_launches(U, field, value):
     assert all(bool((getattr(model, n) == 7.0).all()) for n in ex._BUFFERS)
 
 
+def _expert_step_in_64_bits(w, W, F, cached_k, cached_v, a, cond):
+    """h and the velocity of one step in double precision on the GPU, by plain torch; cached_k, cached_v [B][L][keys][Hkv][d]."""
+    f = lambda t: t.double()
+    def norm(h, i):
+        z = f(cond) @ f(W["W1"][i]).T + f(W["b1"][i])
+        gate = 1 + (z * torch.sigmoid(z)) @ f(W["W2"][i]).T + f(W["b2"][i])
+        return h / torch.sqrt((h * h).mean(-1, keepdim=True) + 1e-6) * gate[:, None, :]
+    h, nq, nk = f(a.to(torch.bfloat16)) @ f(W["W_in"]).T, w.Hq * w.d, w.Hkv * w.d
+    for l in range(w.L):
+        q, k, v = (norm(h, 2 * l) @ f(W["Wqkv"][l]).T).split([nq, nk, nk], -1)
+        heads = lambda t, n: t.view(w.B, w.T, n, w.d).transpose(1, 2)
+        k, v = (torch.cat([f(c[:, l]).transpose(1, 2), heads(t, w.Hkv)], 2).repeat_interleave(w.Hq // w.Hkv, 1) for c, t in ((cached_k, k), (cached_v, v)))
+        o = torch.softmax(heads(q, w.Hq) @ k.transpose(2, 3) / w.d ** 0.5, -1) @ v
+        h = h + o.transpose(1, 2).reshape(w.B, w.T, nq) @ f(W["Wo"][l]).T
+        g, u = (norm(h, 2 * l + 1) @ f(W["Wgu"][l]).T).split(F, -1)
+        h = h + (g * torch.sigmoid(g) * u) @ f(W["Wd"][l]).T
+    return h, norm(h, 2 * w.L) @ f(W["W_out"]).T
+
+
+@pytest.mark.parametrize("B,T,F", [(1, 50, 2048), (2, 50, 4096), (1, 20, 3072), (6, 50, 2048)])
+def test_expert_step_precision_over_18_layers(U, B, T, F):
+    """How far 18 layers of bf16 activations are from 64 bits, mean of six seeds. With every norm taken from the residual sums before
+    their rounding it is 1.29 to 1.30e-2 on the residual stream, with norms of the rounded stream 1.33e-2; the means scatter by 1e-4
+    (20 tokens) and 3e-5 (50)."""
+    from paper_2607_14695_b200 import expert as ex
+    rb = U.rb
+    w = synth.CONFIGS["cfg2"].with_(B=B, L=18, T=T, S=300, S_max=300)
+    rel = []
+    for seed in range(6):
+        g = torch.Generator(device=U.DEV); g.manual_seed(seed)
+        r = lambda *s: torch.randn(*s, generator=g, device=U.DEV)
+        kv = [r(B, w.L, w.S + w.N, w.Hkv, w.d).to(torch.bfloat16) for _ in range(2)]
+        cache = rb.Cache(w.L, B, w.Hq, w.Hkv, w.d, w.S, w.N, T, w.dtype, device=U.DEV)
+        rb.reflex_cache_init_static(cache, list(range(B)), *(t[:, :, :w.S].contiguous() for t in kv))
+        rb.reflex_cache_append_sliding(cache, list(range(B)), *(t[:, :, w.S:].contiguous() for t in kv))
+        W = ex.random_weights_device(w, F, U.DEV, seed)
+        model = ex.ActionExpert(w, cache, W, F, device=U.DEV)
+        a, cond = r(B, T, w.A), r(B, w.Cd).to(torch.bfloat16)
+        want, _ = _expert_step_in_64_bits(w, W, F, *kv, a, cond)
+        model.step(a, cond, 0)
+        rel.append(float((model.h.double() - want).norm() / want.norm()))
+    assert np.mean(rel) <= 1.315e-2, rel
+
+
 def _list_of_layers(dW):
     return {n: [t.clone() for t in v] if n in ("Wqkv", "Wo", "Wgu", "Wd") else v for n, v in dW.items()}
 
