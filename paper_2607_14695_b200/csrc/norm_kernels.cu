@@ -68,30 +68,59 @@ __device__ __forceinline__ void dot_rows(const T *__restrict__ W, int len, int j
     }
 }
 
-// hidden = SiLU(W1 c + b1) for one stream into shared memory; c_s is scratch of Cd floats.
-template <typename T>
+// The same with four lanes per row, lane j taking elements j, j + 4, ...: the order of gate_layer_kernel's four partial sums, bit for bit.
+// For short rows: eight rows a warp, all loads of a row's next 32 elements in flight.
+template <typename T, typename F>
+__device__ __forceinline__ void dot_rows4(const T *W, int len, int j0, int j1, const float *v, F &&emit)
+{
+    const int sub = threadIdx.x >> 2, l = threadIdx.x & 3, step = blockDim.x >> 2;
+    for (int jj = j0; jj < j1; jj += step) {         // (uniform: every lane takes part in the shuffles)
+        const int j = jj + sub;
+        const T *w = W + (size_t)min(j, j1 - 1) * len;
+        float acc = 0.f;
+#pragma unroll 1
+        for (int e0 = 0; e0 < len; e0 += 32) {
+            float f[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) f[i] = e0 + 4 * i < len ? to_f<T>(w[e0 + 4 * i + l]) : 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (e0 + 4 * i < len) acc = fmaf(f[i], v[e0 + 4 * i + l], acc);
+        }
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if (l == 0 && j < j1) emit(j, acc);
+    }
+}
+
+// hidden = SiLU(W1 c + b1) for one stream into shared memory; c_s is scratch of Cd floats. SHORT: four lanes per row.
+template <typename T, bool SHORT = false>
 __device__ void gate_hidden(const T *__restrict__ cond_b, const T *__restrict__ W1, const T *__restrict__ b1, int Cd, int Hd,
                             float *c_s, float *hid_s)
 {
     for (int e = threadIdx.x; e < Cd; e += blockDim.x) c_s[e] = to_f<T>(cond_b[e]);
     __syncthreads();
-    dot_rows<T>(W1, Cd, 0, Hd, c_s, [&](int j, float acc) {
+    auto emit = [&](int j, float acc) {
         const float z = acc + to_f<T>(b1[j]);
         hid_s[j] = z / (1.f + expf(-z));
-    });
+    };
+    if constexpr (SHORT) dot_rows4<T>(W1, Cd, 0, Hd, c_s, emit);
+    else dot_rows<T>(W1, Cd, 0, Hd, c_s, emit);
     __syncthreads();
 }
 
 // gate[i] = 1 + b2[i] + W2[i] . hidden for columns [i0, i1).
-template <typename T>
+template <typename T, bool SHORT = false>
 __device__ void gate_columns(const T *__restrict__ W2, const T *__restrict__ b2, int Hd, int i0, int i1, const float *hid_s,
                              float *gate_out /* indexed by i - i0 */)
 {
-    dot_rows<T>(W2, Hd, i0, i1, hid_s, [&](int i, float acc) { gate_out[i - i0] = 1.f + (acc + to_f<T>(b2[i])); });
+    auto emit = [&](int i, float acc) { gate_out[i - i0] = 1.f + (acc + to_f<T>(b2[i])); };
+    if constexpr (SHORT) dot_rows4<T>(W2, Hd, i0, i1, hid_s, emit);
+    else dot_rows<T>(W2, Hd, i0, i1, hid_s, emit);
 }
 
 // grid = (column chunks, B, layers): writes gate_buf[layer][b][i]; every block computes the hidden layer for itself.
-template <typename T>
+template <typename T, bool SHORT>
 __global__ void __launch_bounds__(256)
 gate_kernel(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, float *gate_buf, int D, int Cd, int Hd, int cols_per_block)
 {
@@ -101,10 +130,10 @@ gate_kernel(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, f
     const size_t l = blockIdx.z;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    gate_hidden<T>(cond + (size_t)b * Cd, W1 + l * Hd * Cd, b1 + l * Hd, Cd, Hd, c_s, hid_s);
+    gate_hidden<T, SHORT>(cond + (size_t)b * Cd, W1 + l * Hd * Cd, b1 + l * Hd, Cd, Hd, c_s, hid_s);
     const int i0 = blockIdx.x * cols_per_block;
     const int i1 = min(D, i0 + cols_per_block);
-    gate_columns<T>(W2 + l * D * Hd, b2 + l * D, Hd, i0, i1, hid_s, gate_buf + (l * gridDim.y + b) * D + i0);
+    gate_columns<T, SHORT>(W2 + l * D * Hd, b2 + l * D, Hd, i0, i1, hid_s, gate_buf + (l * gridDim.y + b) * D + i0);
 }
 
 // grid = (row chunks, B); one warp per row. FUSED: the block computes its stream's gate itself.
@@ -375,9 +404,8 @@ static bool gate_scratch_fits(int Cd, int Hd)
     return smem_h <= 160 * 1024 && smem_g <= 160 * 1024;
 }
 
-// gamma_l(c) = 1 + W2_l SiLU(W1_l c + b1_l) + b2_l for L layers (stacked weights) and B streams: gates into
-// gate_buf[L][B][D], hidden activations into gate_buf + L*B*D ([L][B][Hd]). Two launches whatever L is.
-template <typename T>
+// One launch: a block per 64 columns, stream and layer.
+template <typename T, bool SHORT = false>
 static cudaError_t launch_gate_blocks(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, float *gate_buf, int L, int B,
                                       int D, int Cd, int Hd, cudaStream_t st)
 {
@@ -392,11 +420,25 @@ static cudaError_t launch_gate_blocks(const T *cond, const T *W1, const T *b1, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gate_kernel<T>, cond, W1, b1, W2, b2, gate_buf, D, Cd, Hd, cols);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gate_kernel<T, SHORT>, cond, W1, b1, W2, b2, gate_buf, D, Cd, Hd, cols);
     count_launch();
     return e;
 }
 
+// A small MLP in one launch, whose blocks compute the hidden layer each for themselves (same bits as the two launches). One layer: while a
+// block's 64 quads of lanes do the hidden layer in one round, 3.9 -> 2.8 us (128 columns, 40 -> 32 wide; 96 hidden units would be 4.2 ->
+// 4.6). Several layers: for one stream at any size (37 x 2048, 40 -> 32: 13.9 -> 6.4 us), for more streams, which the two launches
+// take 32 at a time, as long as the blocks are one round on the SMs (40 -> 32: 37 x 8 x 128 5.8 -> 5.0 us; 37 x 8 x 1024 would be 10 -> 23).
+static bool gate_one_launch(int L, int B, int D, int Cd, int Hd)
+{
+    if (Hd * Cd > 8192 || B > 8) return false;
+    const long long blocks = (long long)L * B * ((D + 63) / 64);
+    if (L == 1) return Hd <= 64 && Hd * Cd <= 4096 && blocks <= 300;
+    return B == 1 || blocks <= (Hd * Cd <= 2048 ? 600 : 300);
+}
+
+// gamma_l(c) = 1 + W2_l SiLU(W1_l c + b1_l) + b2_l for L layers (stacked weights) and B streams: gates into
+// gate_buf[L][B][D], hidden activations into gate_buf + L*B*D ([L][B][Hd]). One or two launches whatever L is.
 template <typename T>
 static cudaError_t launch_gate_t(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, float *gate_buf, int L, int B,
                                  int D, int Cd, int Hd, cudaStream_t st)
@@ -422,10 +464,7 @@ static cudaError_t launch_gate_t(const T *cond, const T *W1, const T *b1, const 
             if (e != cudaErrorInvalidValue) return e;   // invalid value: no tensor maps from this driver, fall through
         }
     }
-    // A small MLP for a few streams: one launch whose blocks compute the hidden layer each for themselves. Up to 8 K hidden products
-    // that costs a block less than the second launch (3.4 us for the two, tiny configuration). The rule does not depend on L: one call
-    // for L layers and L calls give the same bits.
-    if (Hd * Cd <= 8192 && B <= 8) return launch_gate_blocks<T>(cond, W1, b1, W2, b2, gate_buf, L, B, D, Cd, Hd, st);
+    if (gate_one_launch(L, B, D, Cd, Hd)) return launch_gate_blocks<T, true>(cond, W1, b1, W2, b2, gate_buf, L, B, D, Cd, Hd, st);
     const int groups = (B + kGateStreams - 1) / kGateStreams;
     const size_t tiled_h = (size_t)(kTileUnits + kGateStreams) * (Cd + 4) * 4, tiled_g = (size_t)(kTileUnits + kGateStreams) * (Hd + 4) * 4;
     if (L > 1 && tiled_h <= 200 * 1024 && tiled_g <= 200 * 1024) {

@@ -588,6 +588,30 @@ def test_10k_tick_stream_stays_finite(U, cfg):
     assert tot == [ticks] and ct == [w.N] and hd == [ticks % w.N]
 
 
+@pytest.mark.parametrize("dtype", [synth.DTYPE_F32, synth.DTYPE_BF16], ids=["fp32", "bf16"])
+@pytest.mark.parametrize("Cd,Hd", [(40, 32), (24, 64), (72, 24), (40, 96), (104, 72)])
+def test_small_gates_give_the_same_bits_in_every_form(U, dtype, Cd, Hd):
+    """A small MLP runs in one launch or in two, by layers, streams, columns and widths: a layer's gates are the same bits whatever
+    else the call computes, and those of any stream are those of the same stream among 32."""
+    rb, tdt = U.rb, U.rb.torch_dtype(dtype)
+    g = torch.Generator(device=U.DEV); g.manual_seed(Cd)
+    r = lambda *s: torch.randn(*s, generator=g, device=U.DEV).to(tdt)
+    L, D = 20, 200
+    cond, W1, b1, W2, b2 = r(32, Cd), r(L, Hd, Cd) * 0.2, r(L, Hd), r(L, D, Hd) * 0.2, r(L, D)
+    def gates(layers, n):
+        buf = torch.empty(len(W1[layers]) * n * (D + Hd), device=U.DEV)
+        rb.reflex_adarmsnorm_gate(cond[:n].contiguous(), W1[layers], b1[layers], W2[layers], b2[layers], buf)
+        return buf[:len(W1[layers]) * n * D].view(-1, n, D)
+    want = gates(slice(0, L), 32)
+    z = cond.double() @ W1.double().transpose(1, 2) + b1.double()[:, None]
+    exact = 1 + (z * torch.sigmoid(z)) @ W2.double().transpose(1, 2) + b2.double()[:, None]
+    assert (want.double() - exact).norm() <= 1e-6 * exact.norm()
+    for n in (1, 2, 5, 8, 9):
+        assert torch.equal(gates(slice(0, L), n), want[:, :n])
+        assert torch.equal(gates(slice(3, 5), n), want[3:5, :n])
+        assert torch.equal(gates(slice(7, 8), n), want[7:8, :n])
+
+
 def test_gate_for_all_layers_matches_per_layer_calls_and_oracle(U):
     """reflex_adarmsnorm_gate with L stacked layers == L single-layer calls (bitwise) == the oracle's gamma."""
     from oracle import reflex_oracle as orc
@@ -1325,3 +1349,35 @@ def test_bounded_wait_reports_and_context_survives(U):
     tw2.init_static([0], [w.S])
     tw2.append([0], 3, 0)
     tw2.attention(0, 0, what="after a reported timeout")
+
+
+# ------------------------------------------------------------------------------------------------
+# a rule of a dispatch that takes a call to a slower form shows as a call that costs much more than a larger one
+# ------------------------------------------------------------------------------------------------
+def _us(call, n=20):
+    """Microseconds of a call among others: the best of five graph replays of n calls."""
+    call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(n):
+            call()
+    best = float("inf")
+    for _ in range(5):
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        graph.replay()
+        end.record()
+        end.synchronize()
+        best = min(best, start.elapsed_time(end) * 1e3 / n)
+    return best
+
+
+@pytest.mark.parametrize("L,D,Cd,Hd", [(37, 1024, 40, 32), (37, 1024, 64, 128), (4, 2048, 64, 128)])
+def test_gates_of_eight_streams_cost_no_more_than_those_of_sixteen(U, L, D, Cd, Hd):
+    """(With a block per stream they cost 2 to 3 times as much. Bound: 1.3.)"""
+    def us(B):
+        cond, buf = torch.zeros((B, Cd), device=U.DEV), torch.empty(L * B * (D + Hd), device=U.DEV)
+        W1, b1, W2, b2 = (torch.zeros(s, device=U.DEV) for s in ((L, Hd, Cd), (L, Hd), (L, D, Hd), (L, D)))
+        return _us(lambda: U.rb.reflex_adarmsnorm_gate(cond, W1, b1, W2, b2, buf))
+    assert us(8) <= 1.3 * us(16)
