@@ -42,30 +42,40 @@ template <typename T> __device__ __forceinline__ float to_f(T v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-// emit(j, w_j . v) for j in [j0, j1): rows w_j of length len (a multiple of 8) in global memory, v in shared memory. 1 to 32 lanes per
-// row, eight elements a lane, so that a short row leaves no lane idle and a warp has several rows' loads in flight at once.
-template <typename T, typename F>
-__device__ __forceinline__ void dot_rows(const T *__restrict__ W, int len, int j0, int j1, const float *v, F &&emit)
+// emit(j, w_j . v) for j in [j0, j1): rows w_j of length len (a multiple of 8) in global memory, v in shared memory. G lanes per row, eight
+// elements a lane.
+template <int G, typename T, typename F>
+__device__ __forceinline__ void dot_rows_of(const T *W, int len, int j0, int j1, const float *v, F &&emit)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    int group = 32;
-    while (group > 1 && group * 4 >= len) group >>= 1;
-    const int per_warp = 32 / group, sub = lane / group, l = lane % group;
-    for (int jj = j0 + warp * per_warp; jj < j1; jj += nwarp * per_warp) {
+    constexpr int UNROLL = sizeof(T) == 4 ? 4 : 2;   // (1024 -> 512 wide, 200 streams x 128 columns: fp32 131 us by four, 143 by two; bf16 is 10 % faster by two)
+    const int sub = threadIdx.x / G, l = threadIdx.x % G, step = blockDim.x / G;
+    for (int jj = j0; jj < j1; jj += step) {         // (uniform: every lane takes part in the shuffles)
         const int j = jj + sub;
         float acc = 0.f;
         if (j < j1) {
             const T *w = W + (size_t)j * len;
-            for (int e = l * 8; e < len; e += group * 8) {
+#pragma unroll UNROLL
+            for (int e = l * 8; e < len; e += G * 8) {
                 float f[8];
                 Vec8<T>::load(w + e, f);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) acc = fmaf(f[i], v[e + i], acc);
             }
         }
-        for (int o = group / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (l == 0 && j < j1) emit(j, acc);
     }
+}
+// As many lanes as a row has use for, so that a warp has several short rows' loads in flight at once. (The number is a constant of the
+// loop, so that those of a long row are: chosen inside it at run time, the 1024- and 512-wide rows of 200 streams took 224 us instead of 131.)
+template <typename T, typename F>
+__device__ __forceinline__ void dot_rows(const T *W, int len, int j0, int j1, const float *v, F &&emit)
+{
+    if (len > 128) dot_rows_of<32, T>(W, len, j0, j1, v, emit);
+    else if (len > 64) dot_rows_of<16, T>(W, len, j0, j1, v, emit);
+    else if (len > 32) dot_rows_of<8, T>(W, len, j0, j1, v, emit);
+    else dot_rows_of<4, T>(W, len, j0, j1, v, emit);
 }
 
 // The same with four lanes per row, lane j taking elements j, j + 4, ...: the order of gate_layer_kernel's four partial sums, bit for bit.
@@ -128,8 +138,10 @@ gate_kernel(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, f
     float *c_s = smem, *hid_s = smem + Cd;
     const int b = blockIdx.y;
     const size_t l = blockIdx.z;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if constexpr (SHORT) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
     gate_hidden<T, SHORT>(cond + (size_t)b * Cd, W1 + l * Hd * Cd, b1 + l * Hd, Cd, Hd, c_s, hid_s);
     const int i0 = blockIdx.x * cols_per_block;
     const int i1 = min(D, i0 + cols_per_block);
@@ -404,7 +416,9 @@ static bool gate_scratch_fits(int Cd, int Hd)
     return smem_h <= 160 * 1024 && smem_g <= 160 * 1024;
 }
 
-// One launch: a block per 64 columns, stream and layer.
+// One launch: a block per 64 columns, stream and layer. SHORT takes part in programmatic dependent launch. The wide form, whose blocks run for
+// 60 us and more, does not: a grid that waits beside them spreads over the SMs as it finds them (norm of 13 x 50 rows x 2048, 512 -> 1024
+// wide: 189 us, 324 with both).
 template <typename T, bool SHORT = false>
 static cudaError_t launch_gate_blocks(const T *cond, const T *W1, const T *b1, const T *W2, const T *b2, float *gate_buf, int L, int B,
                                       int D, int Cd, int Hd, cudaStream_t st)
@@ -419,7 +433,7 @@ static cudaError_t launch_gate_blocks(const T *cond, const T *W1, const T *b1, c
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = SHORT ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, gate_kernel<T, SHORT>, cond, W1, b1, W2, b2, gate_buf, D, Cd, Hd, cols);
     count_launch();
     return e;

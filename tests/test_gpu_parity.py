@@ -1381,3 +1381,14 @@ def test_gates_of_eight_streams_cost_no_more_than_those_of_sixteen(U, L, D, Cd, 
         W1, b1, W2, b2 = (torch.zeros(s, device=U.DEV) for s in ((L, Hd, Cd), (L, Hd), (L, D, Hd), (L, D)))
         return _us(lambda: U.rb.reflex_adarmsnorm_gate(cond, W1, b1, W2, b2, buf))
     assert us(8) <= 1.3 * us(16)
+
+
+def test_wide_gates_of_twice_the_streams_cost_at_most_twice(U):
+    """200 streams x 128 columns, 1024 to 512 wide, are 400 blocks, which the SMs hold at once: 134 us against 110 for 100 streams. (224
+    while the lanes of a row were chosen inside its loop. Bound: 1.6.)"""
+    Cd, Hd, D = 1024, 512, 128
+    def us(B):
+        cond, buf = torch.zeros((B, Cd), device=U.DEV), torch.empty(B * (D + Hd), device=U.DEV)
+        W1, b1, W2, b2 = (torch.zeros(s, device=U.DEV) for s in ((1, Hd, Cd), (1, Hd), (1, D, Hd), (1, D)))
+        return _us(lambda: U.rb.reflex_adarmsnorm_gate(cond, W1, b1, W2, b2, buf))
+    assert us(200) <= 1.6 * us(100)
