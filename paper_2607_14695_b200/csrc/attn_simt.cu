@@ -48,11 +48,30 @@ template <int DPL> struct RowIO<float, DPL> {
     }
 };
 
+// Are a row's loads gathered before the first is used? In fp32 they are; in bf16, whose rows are half as many loads and have to be
+// converted, the plain loops are the faster ones (32 rows x 976 keys, heads of 32: 20.6 us, 42.5 gathered), but for the widest heads with
+// several warps per row (64 rows x 76 keys: 9.9 us, 8.1 gathered).
+template <typename T, int DPL, int WPR> constexpr bool kSimtGather = sizeof(T) == 4 || (DPL == 8 && WPR > 1);
+
 // dot of a K row (global, storage type) with a query row (shared, fp32), 8 elements per step; the loads of 64 elements in flight together
-template <typename T, int D>
+// where they are gathered
+template <typename T, int D, bool GATHER>
 __device__ __forceinline__ float dot_row(const T *__restrict__ k, const float *__restrict__ q_s)
 {
     constexpr int CH = D < 64 ? D : 64;
+    if constexpr (!GATHER) {
+        float acc0 = 0.f, acc1 = 0.f;
+        for (int e = 0; e < D; e += 8) {
+            float f[8];
+            RowIO<T, 8>::load(k + e, f);
+            const float4 qa = *reinterpret_cast<const float4 *>(q_s + e), qb = *reinterpret_cast<const float4 *>(q_s + e + 4);
+            acc0 = fmaf(f[0], qa.x, acc0); acc1 = fmaf(f[1], qa.y, acc1);
+            acc0 = fmaf(f[2], qa.z, acc0); acc1 = fmaf(f[3], qa.w, acc1);
+            acc0 = fmaf(f[4], qb.x, acc0); acc1 = fmaf(f[5], qb.y, acc1);
+            acc0 = fmaf(f[6], qb.z, acc0); acc1 = fmaf(f[7], qb.w, acc1);
+        }
+        return acc0 + acc1;
+    }
     float acc0 = 0.f, acc1 = 0.f;
 #pragma unroll 1
     for (int e0 = 0; e0 < D; e0 += CH) {
@@ -74,6 +93,9 @@ __device__ __forceinline__ float dot_row(const T *__restrict__ k, const float *_
 
 constexpr int kSimtWarps = 4;      // rows of a block, a warp each (WPR = 1)
 constexpr int kSimtRowWarps = 8;   // warps that share a row (WPR = kSimtRowWarps)
+// Does the grid take part in programmatic dependent launch? Not where many blocks run long: beside waiting blocks of the next grid they
+// spread unevenly over the SMs (bf16, 2400 rows x 626 keys, heads of 256: 302 us, 438 with it).
+template <typename T, int WPR> constexpr bool kSimtOverlap = WPR > 1 || sizeof(T) == 4;
 
 // WPR: warps per query row. 1: a block takes kSimtWarps rows, grid = (ceil(T Hq / kSimtWarps), B, nsplit). kSimtRowWarps: a block
 // takes one row, its warps every eighth tile of the slice, and merges their (m, l, acc) through shared memory, grid = (T Hq, B, nsplit).
@@ -85,10 +107,13 @@ __global__ void __launch_bounds__(WPR == 1 ? kSimtWarps * 32 : WPR * 32)
 attn_simt_kernel(AttnParams p)
 {
     constexpr int d = DPL * 32;
+    constexpr bool GATHER = kSimtGather<T, DPL, WPR>;
     constexpr int NB = DPL >= 8 ? 8 : DPL == 4 ? 16 : 32;      // V rows in flight
     __shared__ __align__(16) float q_s[WPR == 1 ? kSimtWarps : 1][d];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if constexpr (kSimtOverlap<T, WPR>) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b = blockIdx.y, split = blockIdx.z;
     const int rows = p.T * p.Hq;
@@ -160,9 +185,9 @@ attn_simt_kernel(AttnParams p)
                 }
             }
         };
-        load_v(0);
+        if constexpr (GATHER) load_v(0);
         float s = -INFINITY;
-        if (kp) s = dot_row<T, d>(kp, qs) * p.scale;
+        if (kp) s = dot_row<T, d, GATHER>(kp, qs) * p.scale;
         float tmax = s;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
@@ -177,6 +202,17 @@ attn_simt_kernel(AttnParams p)
         m = m_new;
 #pragma unroll
         for (int i = 0; i < DPL; ++i) acc[i] *= alpha;
+        if constexpr (!GATHER) {
+            for (int j = 0; j < 32; ++j) {
+                const float w = __shfl_sync(0xffffffffu, pj, j);
+                const unsigned long long va = __shfl_sync(0xffffffffu, vaddr, j);
+                if (va == 0ull) continue;
+                float v[DPL];
+                RowIO<T, DPL>::load((const T *)va + lane * DPL, v);
+#pragma unroll
+                for (int i = 0; i < DPL; ++i) acc[i] = fmaf(w, v[i], acc[i]);
+            }
+        } else
 #pragma unroll 1
         for (int j0 = 0; j0 < 32; j0 += NB) {
             if (j0 > 0) load_v(j0);
@@ -295,8 +331,17 @@ attn_merge_kernel(AttnParams p)
     RowIO<T, DPL>::store(out + lane * DPL, acc);
 }
 
-// Few rows: a block per row, its eight warps share the keys. The line lies where warps with a row each would no longer leave SMs idle.
-static bool simt_row_blocks(const AttnParams &p) { return (long long)p.T * p.Hq * p.B <= 2048; }
+// Few rows: a block per row, its eight warps share the keys. fp32: the line lies where warps with a row each would no longer leave SMs
+// idle. bf16, whose tiles are cheaper: while a warp has hardly more than one tile of 32 keys and the blocks are few (24 rows x 81 keys,
+// heads of 128: 17.2 -> 7.7 us; 512 x 80, heads of 256: 21.7 -> 13; but 384 x 380, heads of 256: 34 -> 48, and 4 x 825 18.3 -> 36, where
+// key slices go to more blocks). A single tile leaves nothing to share (fp32, 1536 rows x 32 keys: 18.4 us, 23.1 with a block per row).
+static bool simt_row_blocks(const AttnParams &p)
+{
+    const long long rows = (long long)p.T * p.Hq * p.B;
+    const int n_tiles = (p.S_max + p.N + p.T + 31) / 32;
+    if (p.dtype == REFLEX_DTYPE_F32) return rows <= (n_tiles < 2 ? 512 : 2048);
+    return n_tiles >= 2 && (n_tiles <= kSimtRowWarps ? rows <= 512 : rows <= 128 && n_tiles <= kSimtRowWarps * 3 / 2);
+}
 
 int simt_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count)
 {
@@ -327,7 +372,7 @@ static cudaError_t launch_simt_d(const AttnParams &p, cudaStream_t st)
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = (rb ? kSimtOverlap<T, kSimtRowWarps> : kSimtOverlap<T, 1>) ? 1 : 0;
     return rb ? cudaLaunchKernelEx(&cfg, attn_simt_kernel<T, DPL, kSimtRowWarps>, p) : cudaLaunchKernelEx(&cfg, attn_simt_kernel<T, DPL, 1>, p);
 }
 
