@@ -787,6 +787,9 @@ static int chain_attn_rows(const AttnParams &p, bool early)
     const int G = p.Hq / p.Hkv;
     for (int rows = 32; rows <= 64; rows *= 2) {
         if (rows % G != 0) continue;
+        // Called by itself on few keys the exchange of 64 rows costs more than the keys that the slices save (2 x 32 tokens x 112 keys
+        // 10.5 us, 8.8 by one CTA per tile; 66 keys 9.3 and 8.0; from 313 keys on 0.92 to 1.02 of it; of 32 rows 0.6 to 1.0 everywhere).
+        if (rows == 64 && !early && p.S_max + p.N + p.T < 288) continue;
         const int tt = rows / G;
         if ((long long)p.B * p.Hkv * ((p.T + tt - 1) / tt) <= 14) return rows;
     }
