@@ -128,19 +128,29 @@ append_sliding_kernel(uint4 *k_slab, uint4 *v_slab, const uint4 *k_src, const ui
     if (threadIdx.x == 0) s_head = ((volatile StreamState *)state)[b].head;
     __syncthreads();
     const int head = s_head;
-    const size_t units = (size_t)L * m * row_units;
-    const size_t src_base = (size_t)(src_stream0 + i) * L * m * row_units;
+    const unsigned units = (unsigned)L * m * row_units, step = gridDim.x * 256u;      // (16-byte units of one stream: 2^32 would be 64 GB)
+    const size_t src_base = (size_t)(src_stream0 + i) * units;
     const int rows_per_block = ring_off + N;
-    for (size_t u = (size_t)blockIdx.x * blockDim.x + threadIdx.x; u < units; u += (size_t)gridDim.x * blockDim.x) {
-        const int off = (int)(u % row_units);
-        const size_t r = u / row_units;
-        const int tok = (int)(r % m);
-        const int l = (int)(r / m);
-        int slot = head + tok;
-        if (slot >= N) slot -= N;
-        const size_t dst = (((size_t)l * B + b) * rows_per_block + ring_off + slot) * row_units + off;
-        k_slab[dst] = __ldcg(k_src + src_base + u);
-        v_slab[dst] = __ldcg(v_src + src_base + u);
+    // a thread's units of K and V are asked for together, four of each at a time (one by one, each pair was a round trip: 8 streams x
+    // 18 layers x 5 rows 5.7 us, 4.2 so)
+    for (unsigned u0 = blockIdx.x * 256u + threadIdx.x; u0 < units; u0 += 4u * step) {
+        uint4 k[4], v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned u = u0 + j * step;
+            if (u < units) { k[j] = __ldcg(k_src + src_base + u); v[j] = __ldcg(v_src + src_base + u); }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned u = u0 + j * step;
+            if (u >= units) break;
+            const unsigned r = u / (unsigned)row_units, off = u - r * row_units, l = r / (unsigned)m;
+            int slot = head + (int)(r - l * m);
+            if (slot >= N) slot -= N;
+            const size_t dst = (((size_t)l * B + b) * rows_per_block + ring_off + slot) * row_units + off;
+            k_slab[dst] = k[j];
+            v_slab[dst] = v[j];
+        }
     }
     __threadfence();
     __syncthreads();
