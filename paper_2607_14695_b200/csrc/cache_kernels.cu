@@ -128,21 +128,19 @@ append_sliding_kernel(uint4 *k_slab, uint4 *v_slab, const uint4 *k_src, const ui
     if (threadIdx.x == 0) s_head = ((volatile StreamState *)state)[b].head;
     __syncthreads();
     const int head = s_head;
-    const unsigned units = (unsigned)L * m * row_units, step = gridDim.x * 256u;      // (16-byte units of one stream: 2^32 would be 64 GB)
+    const unsigned units = (unsigned)L * m * row_units;              // 16-byte units of one stream (2^32 of them would be 64 GB)
     const size_t src_base = (size_t)(src_stream0 + i) * units;
     const int rows_per_block = ring_off + N;
-    // a thread's units of K and V are asked for together, four of each at a time (one by one, each pair was a round trip: 8 streams x
-    // 18 layers x 5 rows 5.7 us, 4.2 so)
-    for (unsigned u0 = blockIdx.x * 256u + threadIdx.x; u0 < units; u0 += 4u * step) {
-        uint4 k[4], v[4];
+    // A thread's units of K and V are asked for together, two of each at a time (8 streams x 18 layers x 5 rows: 5.7 us with one pair behind
+    // the other, 4.6 so; four of each are no faster there and slower, 8.4 us against 7.2, at 32 streams x 18 x 32).
+    for (unsigned u0 = blockIdx.x * 512u + threadIdx.x; u0 < units; u0 += gridDim.x * 512u) {
+        uint4 k[2], v[2];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const unsigned u = u0 + j * step;
-            if (u < units) { k[j] = __ldcg(k_src + src_base + u); v[j] = __ldcg(v_src + src_base + u); }
-        }
+        for (int j = 0; j < 2; ++j)
+            if (u0 + j * 256u < units) { k[j] = __ldcg(k_src + src_base + u0 + j * 256u); v[j] = __ldcg(v_src + src_base + u0 + j * 256u); }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const unsigned u = u0 + j * step;
+        for (int j = 0; j < 2; ++j) {
+            const unsigned u = u0 + j * 256u;
             if (u >= units) break;
             const unsigned r = u / (unsigned)row_units, off = u - r * row_units, l = r / (unsigned)m;
             int slot = head + (int)(r - l * m);
