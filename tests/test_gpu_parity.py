@@ -1080,6 +1080,25 @@ def test_prefix_copy_at_block_edges(U, d, lens):
     assert sl == [lens[1], -1, lens[2], lens[0]]
 
 
+@pytest.mark.parametrize("lens", [[400, 1, 0, 2, 399, 3], [0, 0, 0, 0, 0, 400], [400] + [1] * 69, [1] * 63 + [400] * 3, [0] * 70, [300, 200, 300, 200]], ids=str)
+def test_prefix_copy_of_uneven_lengths(U, lens):
+    """Lengths that differ, up to more streams than a launch takes: bytes exactly, nothing behind a prefix, every length taken over."""
+    rb = U.rb
+    L, n, S_max = 2, len(lens), 403
+    cache = rb.Cache(L, n + 1, 8, 1, 256, S_max, 4, 8, rb.DTYPE_BF16, device=U.DEV)
+    ids = [(7 * i + 1) % (n + 1) for i in range(n)] if (n + 1) % 7 else list(range(n, 0, -1))
+    g = torch.Generator(device=U.DEV); g.manual_seed(n)
+    src = [torch.randn(n, L, max(max(lens), 1), 1, 256, generator=g, device=U.DEV).to(torch.bfloat16) for _ in range(2)]
+    rb.reflex_cache_init_static(cache, ids, *src, S=lens)
+    want = [torch.zeros_like(cache.k_slab) for _ in range(2)]
+    for i, (b, S) in enumerate(zip(ids, lens)):
+        for t, x in zip(want, src):
+            t[:, b, :S] = x[i, :, :S]
+    assert torch.equal(cache.k_slab, want[0]) and torch.equal(cache.v_slab, want[1])
+    sl = rb.reflex_cache_get_state(cache)[0]
+    assert [sl[b] for b in ids] == lens and sum(s == -1 for s in sl) == 1
+
+
 @pytest.mark.parametrize("frames,T", [(1, 75), (5, 50), (50, 25)])
 def test_context_window_and_chunk_sweep(U, frames, T):
     """Points of the paper's context-window (1 to 50 frames of 256 tokens in the sliding history) and action-chunk (25 to 100
