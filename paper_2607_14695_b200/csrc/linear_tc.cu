@@ -499,7 +499,8 @@ cudaError_t launch_lin_simt(const void *a, const void *W, const void *res, void 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    // programmatic launch only while the blocks are few: beside those of the grid ahead more of them end up two to an SM
+    cfg.numAttrs = M <= 74 ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, linear_res_simt_kernel<T>, (const T *)a, (const T *)W, (const T *)res, (T *)out, K, N);
     count_launch();
     return e;

@@ -982,7 +982,9 @@ cudaError_t launch_simt(const void *x, const float *gate, const void *W, void *q
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    // Programmatic launch only while the blocks are few: beside those of the grid ahead that still run, more of them end up two to an SM and the
+    // launch takes twice as long (fp32 step of 8 x 16 rows 0.59 ms, 1.09 to 1.40 with it; bf16 gate/up of 300 rows x 2048 3.3 -> 13 ms).
+    cfg.numAttrs = M <= 74 ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, norm_qkv_simt_kernel<T>, (const T *)x, gate, (const T *)W, (T *)q, (T *)k, (T *)v, R, D, nq, nk, swiglu_F, eps);
     count_launch();
     return e;

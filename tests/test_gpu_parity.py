@@ -1444,3 +1444,27 @@ def test_attention_form_of_few_streams_is_no_slower_than_the_others(U, B, Hq, Hk
         return _us(lambda: rb.reflex_partitioned_attention(cache, 0, q, k, k, out))
     chosen, one, two = us(rb.ATTN_AUTO), us(rb.ATTN_TC), us(rb.ATTN_TC2)
     assert chosen <= 1.1 * min(one, two), (chosen, one, two)
+
+
+@pytest.mark.parametrize("dtype,B,T,D,F", [(synth.DTYPE_F32, 8, 16, 256, 512), (synth.DTYPE_F32, 8, 50, 256, 512), (synth.DTYPE_BF16, 6, 50, 2048, 512)],
+                         ids=["fp32_128", "fp32_400", "bf16_300"])
+def test_plain_projections_inside_a_step_cost_what_they_cost_alone(U, dtype, B, T, D, F):
+    """A step by single calls whose projections run as the plain kernels, in whole or in part, against these calls one by one. (With the
+    plain kernels launched programmatically their blocks shared SMs and the steps took 1.3 to 2 times as long here, now 1.02. Bound: 1.2.)"""
+    from paper_2607_14695_b200 import expert as ex
+    rb, tdt = U.rb, U.rb.torch_dtype(dtype)
+    L, d = 3, 64
+    w = synth.Workload("plain", 1, dtype, B=B, L=L, Hq=2, Hkv=1, d=d, S=64, S_max=64, N=16, T=T, D=D, Cd=40, Hd=32, A=24, K=10, m=0)
+    cache = rb.Cache(L, B, 2, 1, d, 64, 16, T, dtype, device=U.DEV)
+    kv = torch.randn((B, L, 64, 1, d), device=U.DEV).to(tdt)
+    rb.reflex_cache_init_static(cache, list(range(B)), kv, kv)
+    model = ex.ActionExpert(w, cache, ex.random_weights_device(w, F, U.DEV), F, device=U.DEV)
+    a, cond = torch.zeros((B, T, 24), device=U.DEV), torch.zeros((B, 40), device=U.DEV, dtype=tdt)
+    W, h = model.W, model.h
+    rows = lambda t: t.view(B * T, -1)
+    parts = [lambda: rb.reflex_adarmsnorm_qkv(h, model.gate(0), W["Wqkv"][0], model.q, model.k, model.v, cache=cache),
+             lambda: rb.reflex_linear_residual(rows(model.o), W["Wo"][0], h, h, cache=cache),
+             lambda: rb.reflex_adarmsnorm_swiglu(h, model.gate(0), W["Wgu"][0], model.m, cache=cache),
+             lambda: rb.reflex_linear_residual(rows(model.m), W["Wd"][0], h, h, cache=cache)]
+    alone, step = L * sum(_us(call, 3) for call in parts), _us(lambda: model.step(a, cond, 0), 3)
+    assert step <= 1.2 * alone
