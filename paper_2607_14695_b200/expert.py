@@ -56,17 +56,18 @@ class ActionExpert:
             raise ValueError("the cache has other streams, heads, head widths or storage, or fewer layers than the expert")
         _want("a", a, (w.B, w.T, w.A), torch.float32, self.vel.device)
         _want("cond", cond, (w.B, w.Cd), self.tdt, self.vel.device)
-        if not all(isinstance(W[n], torch.Tensor) and W[n].is_contiguous() for n in _WEIGHTS):
-            return self._step_by_calls(a, cond, k, stream)
-        d = rb.ExpertDesc(w.T, w.D, self.F, w.A, w.Cd, w.Hd, 1e-6, w.L)
+        d, dev = rb.ExpertDesc(w.T, w.D, self.F, w.A, w.Cd, w.Hd, 1e-6, w.L), self.vel.device
         for n, shape in self.shapes.items():
             t = W[n]
-            if n in _LAYERS and t.shape[:1] != shape[:1]:
-                t = t[:w.L]                         # a stack may hold more layers than the expert uses
-            elif n in ("b1", "b2") and t.numel() == shape[0] * shape[1]:
-                t = t.view(shape)                   # biases in any shape
-            _want(n, t, shape, self.tdt, self.vel.device)
-            setattr(d, n, W[n].data_ptr())
+            if not isinstance(t, torch.Tensor) or not t.is_contiguous():
+                return self._step_by_calls(a, cond, k, stream)
+            if t.shape != shape or t.dtype != self.tdt or t.device != dev:
+                if n in _LAYERS:
+                    t = t[:w.L]                         # a stack may hold more layers than the expert uses
+                elif n in ("b1", "b2") and t.numel() == shape[0] * shape[1]:
+                    t = t.view(shape)                   # biases in any shape
+                _want(n, t, shape, self.tdt, dev)
+            setattr(d, n, t.data_ptr())
         for n in _BUFFERS:
             setattr(d, n, getattr(self, n).data_ptr())
         return rb.reflex_expert_step(self.cache, d, a, cond, k, w.K, stream=stream)
