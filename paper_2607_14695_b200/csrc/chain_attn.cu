@@ -468,7 +468,6 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     const int rows = min(p.tt, p.T - t0) * p.G;                      // query rows of this CTA: (token, head in group)
     const bool last = slice == kC4Slices - 1;                        // its second tile: ring and dynamic tokens
 
-    if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (warp == 0) {
         if (lane == 0) {
             for (int i = 0; i < C4_COUNT; ++i) mbar_init(bar(i), i == C4_VREADY || i == C4_P ? 8u : i == C4_FREE ? (uint32_t)kC4Slices : 1u);
@@ -530,7 +529,7 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     cluster_wait();              // the peers' barriers exist
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");        // (this kernel is a step's only: K of the caches is on its way)
     // (not before this CTA has its tensor memory, all of it: a dependent that took some first would wait for this grid)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 

@@ -84,14 +84,6 @@ __device__ __forceinline__ uint2 pack4_bf16(float a, float b, float c, float d)
     return make_uint2(*reinterpret_cast<uint32_t *>(&lo), *reinterpret_cast<uint32_t *>(&hi));
 }
 
-// SiLU(g) * u with one special-function operation (tanh.approx, about 2^-11: a quarter of the spacing of the bf16 result)
-__device__ __forceinline__ float cg_silu_mul(float g, float u)
-{
-    float t;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * g));
-    return fmaf(t, 0.5f * g, 0.5f * g) * u;
-}
-
 // sum over the 32 lanes of four values: lane l ends with the total of value l / 8 (six shuffles instead of twenty)
 __device__ __forceinline__ float warp_sum4(float v0, float v1, float v2, float v3, int lane)
 {
@@ -352,7 +344,7 @@ chain_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     float o = val[i] * rs4[i];
-                    if constexpr (MODE == CG_SWIGLU) o = cg_silu_mul(o, uu[i] * rs4[i]);
+                    if constexpr (MODE == CG_SWIGLU) o = silu_mul(o, uu[i] * rs4[i]);
                     if (f_ok && r + i < p.M) {
                         const __nv_bfloat16 ov = __float2bfloat16_rn(o);
                         dst[(size_t)(r + i) * pitch] = ov;

@@ -86,17 +86,6 @@ __device__ long long g_qk_trace[3 * 32 * 8];
 #define QK_TRACE(role, step, ev) do { } while (0)
 #endif
 
-// SiLU(g) * u with one special-function operation per element: g / (1 + e^-g) = g (1 + tanh(g / 2)) / 2. The epilogue of the
-// gate/up kernel is bound by the special-function unit (16 results per clock and SM; 32 K elements per tile): with an
-// exponential and a reciprocal per element it took 7.7 k cycles of a 26 k-cycle tile. tanh.approx is accurate to about 2^-11,
-// a quarter of the spacing of the bf16 the result is rounded to.
-__device__ __forceinline__ float silu_mul(float g, float u)
-{
-    float t;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * g));
-    return fmaf(t, 0.5f * g, 0.5f * g) * u;
-}
-
 __device__ __forceinline__ void qk_tma_store_2d(const CUtensorMap *map, uint32_t src, int c0, int c1)
 {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");

@@ -508,8 +508,8 @@ static int attention(reflex_cache_t *c, int layer, const void *q, const void *k_
     } else if (c->attn_impl == REFLEX_ATTN_AUTO && chain_attn_supported(p, early, c->sm_count)) {
         e = launch_chain_attn(p, status, early, pf, (cudaStream_t)stream);
     } else {
-        // Batched shapes take the two-CTA kernel (with a key split when the streams alone do not fill the SM pairs);
-        // a single stream or a few take one CTA per query tile with a finer key split.
+        // the two-CTA kernel (with a key split when the streams alone do not fill the SM pairs); heads of 64 one CTA per query tile with
+        // a finer split
         const int split2 = tc2_ok ? tc2_choose_splits(p, c->lay.partial_bytes, c->sm_count) : 0;
         const bool two = c->attn_impl == REFLEX_ATTN_TC2 || (c->attn_impl == REFLEX_ATTN_AUTO && split2 >= 1);
         p.nsplit = two ? (split2 >= 1 ? split2 : 1) : tc_choose_splits(p, c->lay.partial_bytes, c->sm_count);
@@ -572,7 +572,7 @@ static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float 
     float *ss[2] = {e.row_sums, e.row_sums + (size_t)M * ((D + 31) / 32)};
     auto gate = [&](int i) { return (const float *)e.gates + (size_t)i * B * D; };
     // what a later kernel of the step reads is asked into the L2 one or two kernels ahead, so that the 34 MB of a layer come from
-    // memory while the chain is busy with latencies
+    // memory while the chain is busy with latencies (the tile form's projections are not, and take no part)
     auto range = [](ChainPrefetch &pf, int i, const void *base, size_t first, size_t n) {
         pf.ptr[i] = (const char *)base + first * 2; pf.bytes[i] = n * 2 & ~(size_t)15;
     };
@@ -596,7 +596,7 @@ static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float 
         ChainProj qkv = p;
         qkv.mode = CG_QKV; qkv.x = (const bf *)e.y; qkv.W = (const bf *)e.Wqkv; qkv.w_rows = L * (nq + 2 * nk); qkv.w_row0 = l * (nq + 2 * nk);
         qkv.K = D; qkv.N = nq + 2 * nk; qkv.ss_in = ss[0]; qkv.slots_in = slots; qkv.q = (bf *)e.q; qkv.k = (bf *)e.k; qkv.v = (bf *)e.v; qkv.nq = nq; qkv.nk = nk;
-        range(qkv.pf, 0, e.Wo, (size_t)l * D * nq, (size_t)D * nq);
+        if (!tiled) range(qkv.pf, 0, e.Wo, (size_t)l * D * nq, (size_t)D * nq);
         err = proj(qkv);
         if (err != cudaSuccess) return cuda_fail(err, "expert q/k/v projection launch");
         ChainPrefetch apf = {};
@@ -606,13 +606,13 @@ static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float 
         ChainProj o = p;
         o.mode = CG_RES; o.x = (const bf *)e.o; o.W = (const bf *)e.Wo; o.w_rows = L * D; o.w_row0 = l * D; o.K = nq; o.N = D; o.res = (const bf *)e.h;
         o.h = (bf *)e.h; o.xg = (bf *)e.y; o.gate = gate(2 * l + 1); o.ss_out = ss[1];
-        range(o.pf, 0, e.Wd, (size_t)l * D * e.F, (size_t)D * e.F);
+        if (!tiled) range(o.pf, 0, e.Wd, (size_t)l * D * e.F, (size_t)D * e.F);
         err = proj(o);
         if (err != cudaSuccess) return cuda_fail(err, "expert output projection launch");
         ChainProj gu = p;
         gu.mode = CG_SWIGLU; gu.x = (const bf *)e.y; gu.W = (const bf *)e.Wgu; gu.w_rows = L * 2 * e.F; gu.w_row0 = l * 2 * e.F; gu.K = D; gu.N = e.F;
         gu.h = (bf *)e.m; gu.ss_in = ss[1]; gu.slots_in = slots_of(nq);
-        if (l + 1 < L) {
+        if (!tiled && l + 1 < L) {
             range(gu.pf, 0, c->k_slab, (size_t)(l + 1) * kv_layer, kv_layer);
             range(gu.pf, 1, c->v_slab, (size_t)(l + 1) * kv_layer, kv_layer);
             range(gu.pf, 2, e.Wqkv, (size_t)(l + 1) * (nq + 2 * nk) * D, (size_t)(nq + 2 * nk) * D);

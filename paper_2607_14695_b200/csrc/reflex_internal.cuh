@@ -125,7 +125,6 @@ bool chain_attn_supported(const AttnParams &p, bool early, int sm_count);
 struct ChainPrefetch;
 cudaError_t launch_chain_attn(const AttnParams &p, uint32_t *status, bool early, const ChainPrefetch *pf, cudaStream_t st);
 // gate MLP of AdaRMSNorm on tcgen05 (bf16): false when the shapes or the driver do not allow it (the caller falls back)
-// early: inside an expert step weights and gates may be read before the preceding kernel on the stream is complete.
 // adaptive norm + packed Q/K/V projection (qkv_tc.cu). impl: 0 = tensor cores where supported, 1 = plain kernel,
 // 2 = tensor cores with 256-column tiles only
 bool norm_qkv_tc_supported(int dtype, int B, int R, int D, int nq, int nk);

@@ -54,14 +54,6 @@ struct TgParams {
     uint32_t *status;
 };
 
-// SiLU(g) * u with one special-function operation (tanh.approx, about 2^-11: a quarter of the spacing of the bf16 result)
-__device__ __forceinline__ float tg_silu_mul(float g, float u)
-{
-    float t;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * g));
-    return fmaf(t, 0.5f * g, 0.5f * g) * u;
-}
-
 __device__ __forceinline__ void tg_tma2_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t leader_bar, int c0, int c1)
 {
     asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
@@ -240,7 +232,7 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
                         tmem_ld32(tmem + lane_addr + buf * BN + BN / 2 + ch * 64 + gc * 32, up);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) acc[i] = __float_as_uint(tg_silu_mul(__uint_as_float(acc[i]) * rs, __uint_as_float(up[i]) * rs));
+                        for (int i = 0; i < 32; ++i) acc[i] = __float_as_uint(silu_mul(__uint_as_float(acc[i]) * rs, __uint_as_float(up[i]) * rs));
                     } else {
                         tmem_wait_ld();
 #pragma unroll
