@@ -1,6 +1,8 @@
 """GPU parity: the CUDA path (through the C ABI) against the CPU oracle, element by element on the
 same seeded inputs. Integer / byte work is compared exactly, floating point within the contract
 tolerances (bf16: max-abs 2e-2, mean-abs 2e-3 against the fp64 oracle; fp32 storage: 2e-5 / 2e-6)."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -1374,15 +1376,19 @@ def test_bounded_wait_reports_and_context_survives(U):
 # a rule of a dispatch that takes a call to a slower form shows as a call that costs much more than a larger one
 # ------------------------------------------------------------------------------------------------
 def _us(call, n=20):
-    """Microseconds of a call among others: the best of five graph replays of n calls."""
+    """Microseconds of a call among others: the best of nine graph replays of n calls, after 50 ms of them (an idle GPU's clock rises)."""
     call()
     torch.cuda.synchronize()
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph):
         for _ in range(n):
             call()
+    until = time.perf_counter() + 0.05
+    while time.perf_counter() < until:
+        graph.replay()
+        torch.cuda.synchronize()
     best = float("inf")
-    for _ in range(5):
+    for _ in range(9):
         start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         start.record()
         graph.replay()
