@@ -132,8 +132,15 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             mbar_expect_tx(bar(CB_INBOX), (uint32_t)(kCaSlices * (((own + 3) / 4) * kCaHD * 16 + own * (ROWS == 64 ? 8 : 12))));
         }
         __syncwarp();
+        cluster_arrive();
+        asm volatile("bar.arrive 4, %0;" ::"n"(kCaThreads) : "memory");
+    } else {
+        if (warp == 1) tmem_alloc(smem_u32((const void *)tmem_slot), 256);
+        else if (warp == 2 && lane == 0) { prefetch_tmap(&tm_q); prefetch_tmap(&tm_kd); prefetch_tmap(&tm_vd); }
+        __syncwarp();
+        tc_fence_before();
+        cluster_arrive();
     }
-    if (warp == 1) tmem_alloc(smem_u32((const void *)tmem_slot), 256);
     // ---- geometry of the slice ----
     const StreamState ss = p.state[b];
     const int S = max(ss.static_len, 0), count = min(ss.count, p.N);
@@ -154,34 +161,29 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         live_lo = ca_bits(0, ext);
         live_hi = ca_bits(-64, ext - 64);
     }
+    // The producer goes from its barriers straight to its loads, the hand-shakes of block and cluster are the other warps' business: a CTA that
+    // starts late, for lack of room beside the preceding kernel, has its first operands that much sooner.
     if (warp == 0) {
         // K and V of the cached regions (a whole box each; rows past the slice are masked)
         const uint32_t kv_bytes = last ? (uint32_t)((count > 0 ? p.N : 0) + p.T) * (kCaHD * 2) : n_static > 0 ? (uint32_t)p.box * (kCaHD * 2) : 0u;
+        const bool some = last ? count > 0 : n_static > 0;
+        const CUtensorMap *mk = last ? &tm_kr : &tm_ks, *mv = last ? &tm_vr : &tm_vs;
+        const int r0 = row_base + (last ? p.ring_off : ss.bank * p.S_max + k0);
         mbar_expect_tx_elect(bar(CB_K), kv_bytes);
-        const bool ring = last && count > 0;
-        if (ring || n_static > 0) {
-            const CUtensorMap *mk = last ? &tm_kr : &tm_ks, *mv = last ? &tm_vr : &tm_vs;
-            const int r0 = row_base + (last ? p.ring_off : ss.bank * p.S_max + k0);
-            if (lane == 0)
-                for (int c = 0; c < 4; ++c) tma_load_3d(base + L::K + c * (kCaKeys * 128), mk, bar(CB_K), c * 64, hkv, r0);
-            __syncwarp();
-            mbar_expect_tx_elect(bar(CB_V), kv_bytes);
-            if (lane == 0)
-                for (int c = 0; c < 4; ++c) tma_load_3d(base + L::V + c * (kCaKeys * 128), mv, bar(CB_V), c * 64, hkv, r0);
-            __syncwarp();
-        } else {
-            mbar_expect_tx_elect(bar(CB_V), kv_bytes);
-        }
+        if (some)
+            for (int c = 0; c < 4; ++c) tma_load_3d_elect(base + L::K + c * (kCaKeys * 128), mk, bar(CB_K), c * 64, hkv, r0);
+        mbar_expect_tx_elect(bar(CB_V), kv_bytes);
+        if (some)
+            for (int c = 0; c < 4; ++c) tma_load_3d_elect(base + L::V + c * (kCaKeys * 128), mv, bar(CB_V), c * 64, hkv, r0);
+    } else {
+        asm volatile("bar.sync 4, %0;" ::"n"(kCaThreads) : "memory");
+        cluster_wait();              // the peers' barriers exist
+        tc_fence_after();
     }
-    tc_fence_before();
-    __syncthreads();
-    cluster_arrive();
-    cluster_wait();              // the peers' barriers exist
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
     if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     // (not before this CTA has its tensor memory: a dependent that took the columns first would wait for this grid, and this grid for them)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (warp != 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t tmem = warp == 0 ? 0u : *tmem_slot;
 
     if (threadIdx.x == 0) CA_TRACE(1);
     auto wait_slow = [&](int i, uint32_t code) -> bool {
@@ -201,13 +203,14 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     auto wait_cl = [&](int i, uint32_t code) -> bool { return mbar_try_wait_cluster(bar(i), 0) || wait_slow(i, code); };
 
     if (warp == 0) {
+        mbar_expect_tx_elect(bar(CB_Q), ROWS * kCaHD * 2);
+        for (int c = 0; c < 4; ++c) tma_load_4d_elect(base + L::Q + c * L::Q_CHUNK, &tm_q, bar(CB_Q), c * 64, hkv * p.G, t0, b);
+        if (last) {
+            for (int c = 0; c < 4; ++c) tma_load_3d_elect(base + L::K + c * (kCaKeys * 128) + p.dyn_row * 128, &tm_kd, bar(CB_K), c * 64, hkv, b * p.T);
+            for (int c = 0; c < 4; ++c) tma_load_3d_elect(base + L::V + c * (kCaKeys * 128) + p.dyn_row * 128, &tm_vd, bar(CB_V), c * 64, hkv, b * p.T);
+        }
+        cluster_wait();              // the peers' barriers exist
         if (lane == 0) {
-            mbar_expect_tx(bar(CB_Q), ROWS * kCaHD * 2);
-            for (int c = 0; c < 4; ++c) tma_load_4d(base + L::Q + c * L::Q_CHUNK, &tm_q, bar(CB_Q), c * 64, hkv * p.G, t0, b);
-            if (last) {
-                for (int c = 0; c < 4; ++c) tma_load_3d(base + L::K + c * (kCaKeys * 128) + p.dyn_row * 128, &tm_kd, bar(CB_K), c * 64, hkv, b * p.T);
-                for (int c = 0; c < 4; ++c) tma_load_3d(base + L::V + c * (kCaKeys * 128) + p.dyn_row * 128, &tm_vd, bar(CB_V), c * 64, hkv, b * p.T);
-            }
             // this CTA's Q K^T is through with the K tile: its peers may send their partial results over it
             wait(CB_S, 1);
             for (int r = 0; r < kCaSlices; ++r)
@@ -476,8 +479,15 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             mbar_expect_tx(bar(C4_INBOX), (uint32_t)(kC4Slices * rows * (kC4Cols * 4 + 12)));
         }
         __syncwarp();
+        cluster_arrive();
+        asm volatile("bar.arrive 1, %0;" ::"n"(kCaThreads) : "memory");
+    } else {
+        if (warp == 1) tmem_alloc(smem_u32((const void *)tmem_slot), 512);
+        else if (warp == 2 && lane == 0) { prefetch_tmap(&tm_q); prefetch_tmap(&tm_kd); prefetch_tmap(&tm_vs); prefetch_tmap(&tm_vd); }
+        __syncwarp();
+        tc_fence_before();
+        cluster_arrive();
     }
-    if (warp == 1) tmem_alloc(smem_u32((const void *)tmem_slot), 512);
     // ---- geometry: seven tiles divide the static prefix, the eighth holds ring slots and dynamic tokens ----
     const StreamState ss = p.state[b];
     const int S = max(ss.static_len, 0), count = min(ss.count, p.N);
@@ -504,34 +514,33 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         if (t == 1 && last) return (uint32_t)((count > 0 ? p.N : 0) + p.T) * (kCaHD * 2);
         return ext[t] > 0 ? (uint32_t)p.box * (kCaHD * 2) : 0u;
     };
-    // the cached part of tile t of K or V (a whole box; rows past the slice are masked); one lane issues
+    // the cached part of tile t of K or V (a whole box; rows past the slice are masked)
     auto load_cached = [&](int t, bool v) {
         const bool ring = t == 1 && last;
         if (ring ? count == 0 : ext[t] == 0) return;
         const CUtensorMap *m = ring ? (v ? &tm_vr : &tm_kr) : (v ? &tm_vs : &tm_ks);
         const int r0 = row_base + (ring ? p.ring_off : ss.bank * p.S_max + (2 * slice + t) * per);
-        for (int c = 0; c < 4; ++c) tma_load_3d(base + L::KV + t * L::TILE + c * (kCaKeys * 128), m, bar((v ? C4_V : C4_K) + t), c * 64, hkv, r0);
+        for (int c = 0; c < 4; ++c) tma_load_3d_elect(base + L::KV + t * L::TILE + c * (kCaKeys * 128), m, bar((v ? C4_V : C4_K) + t), c * 64, hkv, r0);
     };
     auto load_dyn = [&](bool v) {
         for (int c = 0; c < 4; ++c)
-            tma_load_3d(base + L::KV + L::TILE + c * (kCaKeys * 128) + p.dyn_row * 128, v ? &tm_vd : &tm_kd, bar((v ? C4_V : C4_K) + 1), c * 64, hkv, b * p.T);
+            tma_load_3d_elect(base + L::KV + L::TILE + c * (kCaKeys * 128) + p.dyn_row * 128, v ? &tm_vd : &tm_kd, bar((v ? C4_V : C4_K) + 1), c * 64, hkv, b * p.T);
     };
-    if (warp == 0 && lane == 0) {
+    // (This kernel is a step's only: K of the caches comes ahead of the wait. The roles part as in chain_attn_kernel.)
+    if (warp == 0) {
         for (int t = 0; t < 2; ++t) {
-            mbar_expect_tx(bar(C4_K + t), kv_bytes(t));
+            mbar_expect_tx_elect(bar(C4_K + t), kv_bytes(t));
             load_cached(t, false);
         }
+    } else {
+        asm volatile("bar.sync 1, %0;" ::"n"(kCaThreads) : "memory");
+        cluster_wait();              // the peers' barriers exist
+        tc_fence_after();
     }
-    __syncwarp();
-    tc_fence_before();
-    __syncthreads();
-    cluster_arrive();
-    cluster_wait();              // the peers' barriers exist
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-    asm volatile("griddepcontrol.wait;" ::: "memory");        // (this kernel is a step's only: K of the caches is on its way)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // (not before this CTA has its tensor memory, all of it: a dependent that took some first would wait for this grid)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (warp != 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t tmem = warp == 0 ? 0u : *tmem_slot;
 
     auto wait_slow = [&](int i, uint32_t code) -> bool {
         const unsigned long long t_start = globaltimer_ns();
@@ -550,24 +559,23 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     auto wait_cl = [&](int i, uint32_t code) -> bool { return mbar_try_wait_cluster(bar(i), 0) || wait_slow(i, code); };
 
     if (warp == 0) {
-        if (lane == 0) {
-            mbar_expect_tx(bar(C4_Q), kC4Rows * kCaHD * 2);
-            for (int c = 0; c < 4; ++c) tma_load_4d(base + L::QP + c * (kC4Rows * 128), &tm_q, bar(C4_Q), c * 64, hkv * p.G, t0, b);
-            if (last) load_dyn(false);
-            for (int t = 0; t < 2; ++t) {          // V comes when K is through: into the L2 until then
-                const bool ring = t == 1 && last;
-                if (ring ? count == 0 : ext[t] == 0) continue;
-                const int r0 = row_base + (ring ? p.ring_off : ss.bank * p.S_max + (2 * slice + t) * per);
-                for (int c = 0; c < 4; ++c) tma_prefetch_3d(ring ? &tm_vr : &tm_vs, c * 64, hkv, r0);
-            }
-            for (int t = 0; t < 2; ++t) {
-                mbar_expect_tx(bar(C4_V + t), kv_bytes(t));
-                if (!wait(C4_S + t, 1)) break;
-                load_cached(t, true);
-                if (t == 1 && last) load_dyn(true);
-            }
+        mbar_expect_tx_elect(bar(C4_Q), kC4Rows * kCaHD * 2);
+        for (int c = 0; c < 4; ++c) tma_load_4d_elect(base + L::QP + c * (kC4Rows * 128), &tm_q, bar(C4_Q), c * 64, hkv * p.G, t0, b);
+        if (last) load_dyn(false);
+        for (int t = 0; t < 2; ++t) {              // V comes when K is through: into the L2 until then
+            const bool ring = t == 1 && last;
+            if (ring ? count == 0 : ext[t] == 0) continue;
+            const int r0 = row_base + (ring ? p.ring_off : ss.bank * p.S_max + (2 * slice + t) * per);
+            if (lane < 4) tma_prefetch_3d(ring ? &tm_vr : &tm_vs, lane * 64, hkv, r0);
+            __syncwarp();
         }
-        __syncwarp();
+        for (int t = 0; t < 2; ++t) {
+            mbar_expect_tx_elect(bar(C4_V + t), kv_bytes(t));
+            if (!__all_sync(0xffffffffu, wait(C4_S + t, 1))) break;
+            load_cached(t, true);
+            if (t == 1 && last) load_dyn(true);
+        }
+        cluster_wait();
     } else if (warp == 1) {
         constexpr uint32_t idesc_qk = umma_idesc_bf16(kC4Rows, kCaKeys, false);
         constexpr uint32_t idesc_pv = umma_idesc_bf16(kC4Rows, kCaHD, true);
