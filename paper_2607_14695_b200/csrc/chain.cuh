@@ -56,7 +56,7 @@ struct ChainProj {
 // Do the chain's projections take this shape (all CTAs of the launch on the SMs at once)?
 bool chain_proj_supported(int mode, int M, int K, int N);
 cudaError_t launch_chain_proj(const ChainProj &p, cudaStream_t st);
-// The same projections for many rows: CG_QKV and CG_SWIGLU (tile_gemm.cu), CG_RES (linear_tc.cu; N a multiple of 256, tile_res_slots
+// The same projections for many rows: CG_QKV and CG_SWIGLU (tile_gemm.cu), CG_RES (linear_half.cu, linear_tc.cu; N a multiple of 256, tile_res_slots
 // partial sums of squares per row)
 bool tile_proj_supported(int mode, int M, int K, int nq, int nk, int F);
 cudaError_t launch_tile_proj(const ChainProj &p, cudaStream_t st);

@@ -15,7 +15,7 @@
 // The contraction is long (2048 or 4096) and the output small (3200 x 1024 at 64 streams): 52 tiles on 74 SM pairs in
 // one wave, so the kernel is not persistent.
 //
-// Few rows (at most 128 in all): the weights-as-A-operand kernel of the fused projections with the gate stage switched off
+// A few hundred rows: pair tiles of 128 rows (linear_half.cu). Few rows (at most 128 in all): the weights-as-A-operand kernel of the fused projections with the gate stage switched off
 // (qkv_tc.cu). Any other dtype or shape: a plain kernel, one block per row, fp32 FMAs.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -23,6 +23,7 @@
 #include <stdint.h>
 
 #include "chain.cuh"
+#include "linear_half.cuh"
 #include "reflex_internal.cuh"
 #include "sm100_ptx.cuh"
 
@@ -572,6 +573,12 @@ static cudaError_t launch_tiles(LinParams p, const void *a, const void *W, const
 // CG_RES of ChainProj for many rows: the residual projection together with what the norm behind it needs
 cudaError_t launch_tile_res(const ChainProj &a, cudaStream_t st)
 {
+    if (linear_half_columns(a.B * a.R, a.K, a.N)) {
+        LinearHalf h = {};
+        h.a = a.x; h.W = a.W + (size_t)a.w_row0 * a.K; h.res = a.res; h.out = a.h; h.xg = a.xg; h.gate = a.gate; h.ss_out = a.ss_out;
+        h.M = a.B * a.R; h.K = a.K; h.N = a.N; h.R = a.R; h.B = a.B; h.early_w = true; h.status = a.status;
+        return launch_linear_half(h, st);
+    }
     LinParams p = {};
     p.M = a.B * a.R; p.K = a.K; p.N = a.N; p.status = a.status; p.early_w = 1; p.gate = a.gate; p.ss_out = a.ss_out; p.R = a.R; p.B = a.B;
     return launch_tiles(p, a.x, a.W + (size_t)a.w_row0 * a.K, a.res, a.h, a.xg, st);
@@ -579,6 +586,7 @@ cudaError_t launch_tile_res(const ChainProj &a, cudaStream_t st)
 
 int tile_res_slots(int M, int K, int N)
 {
+    if (const int slots = linear_half_slots(M, K, N)) return slots;
     int bn, ks;
     lin_tiles(M, K, N, bn, ks);
     return N / bn * 2 * (ks == 2 ? 2 : 1);
@@ -594,6 +602,11 @@ cudaError_t launch_linear_residual(const void *a, const void *W, const void *res
         return dtype == REFLEX_DTYPE_BF16 ? launch_lin_simt<__nv_bfloat16>(a, W, res, out, M, K, N, st) : launch_lin_simt<float>(a, W, res, out, M, K, N, st);
     }
     if (impl == 0 && linear_small_takes(M, K, N)) return launch_linear_small(a, W, res, out, M, K, N, status, early_w, st);
+    if (impl == 0 && linear_half_columns(M, K, N)) {
+        LinearHalf h = {};
+        h.a = a; h.W = W; h.res = res; h.out = out; h.M = M; h.K = K; h.N = N; h.R = M; h.B = 1; h.early_w = early_w; h.status = status;
+        return launch_linear_half(h, st);
+    }
     LinParams p = {};
     p.M = M; p.K = K; p.N = N; p.status = status; p.early_w = early_w ? 1 : 0;
     return launch_tiles(p, a, W, res, out, nullptr, st);

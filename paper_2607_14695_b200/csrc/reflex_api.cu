@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "chain.cuh"
+#include "linear_half.cuh"
 #include "reflex_internal.cuh"
 
 using namespace reflex;
@@ -547,15 +548,17 @@ static bool expert_chained(const reflex_cache_desc &d, const reflex_expert &e)
            chain_proj_supported(CG_RES, M, e.F, e.D) && chain_proj_supported(CG_OUT, M, e.D, e.A);
 }
 
-// ... or, for many rows, through the tile kernels on the same operands (tile_gemm.cu, linear_tc.cu). Up to 256 rows the single calls' few-rows
-// kernels split the two residual projections into more CTAs than tiles of 256 rows are (200 rows: 7.1 us each against 12 and 16). Short chunks are the
-// exception: the gates of the streams under 128 rows then exceed what the single gate/up projection holds, and its plain kernel took
-// 8.5 ms a layer (8 x 20 rows: a step of 153 ms, 0.91 by the tiles).
+// ... or, for more rows, through the tile kernels on the same operands (tile_gemm.cu, linear_half.cu, linear_tc.cu). Up to 256 rows only where
+// both residual projections go as pair tiles of 128 rows (a contraction of 2048 or more): as tiles of 256 rows they are too few CTAs, and the single
+// calls' few-rows kernels were ahead (200 rows: 7.1 us each against 12 and 16). Short chunks are the exception: the gates of the streams under
+// 128 rows then exceed what the single gate/up projection holds, and its plain kernel took 8.5 ms a layer (8 x 20 rows: a step of 153 ms, 0.91
+// by the tiles).
 static bool expert_tiled(const reflex_cache_desc &d, const reflex_expert &e)
 {
     const int M = d.B * e.T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
     if (d.dtype != REFLEX_DTYPE_BF16 || e.D % 256 != 0 || !(e.A == 8 || e.A == 16 || e.A == 32) || e.T < 4) return false;      // (T: the gates of the streams under 128 rows fit the idle stages)
-    if (M <= 256 && norm_swiglu_gates_fit(e.T, e.D)) return false;
+    const bool halves = linear_half_columns(M, nq, e.D) && linear_half_columns(M, e.F, e.D);
+    if (M <= 256 && !halves && norm_swiglu_gates_fit(e.T, e.D)) return false;
     return tile_proj_supported(CG_QKV, M, e.D, nq, nk, 0) && tile_proj_supported(CG_SWIGLU, M, e.D, 0, 0, e.F) && chain_proj_supported(CG_OUT, M, e.D, e.A) &&
            nq % 8 == 0 && e.F % 8 == 0;
 }

@@ -1002,6 +1002,14 @@ def test_linear_residual_bf16_mid_size_rows(U, M, K, N, residual):
     _linear_case(U, synth.DTYPE_BF16, M, K, N, 0, f"linear {M}x{K}->{N}", residual=residual, rows=rows, seed=73)
 
 
+@pytest.mark.parametrize("M,K,N,residual", [(257, 2048, 1024, True), (320, 2168, 1000, True), (512, 4096, 1024, False), (385, 2176, 40, True)])
+def test_linear_residual_bf16_pair_tiles_of_128_rows(U, M, K, N, residual):
+    """64 rows per CTA, halves of the contraction that meet by rows: last rows and columns inside a tile, a contraction that ends inside a
+    chunk, tiles of 64 and of 128 columns, every third row compared and the edges of all row groups."""
+    rows = sorted(set(range(0, M, 3)) | {r for e in range(0, M, 32) for r in (e, e - 1) if 0 <= r < M} | {M - 1})
+    _linear_case(U, synth.DTYPE_BF16, M, K, N, 0, "pair tiles of 128 rows", residual=residual, rows=rows)
+
+
 def test_linear_residual_error_paths(U):
     rb = U.rb
     z = lambda *s: torch.zeros(s, dtype=torch.bfloat16, device=U.DEV)
@@ -1283,6 +1291,19 @@ def _slice_of_wider(dW):
 
 def _more_layers(dW):
     return {n: torch.cat([v, torch.full_like(v, float("nan"))], 0) if n in ("Wqkv", "Wo", "Wgu", "Wd") else v for n, v in dW.items()}
+
+
+PAIR_TILES = [
+    # B, T, F, Hq, D: rows around the tiles of 128, contractions of 2048 and more, streams of four rows under a CTA's 32
+    (3, 43, 2048, 8, 1024), (64, 4, 2048, 8, 512), (4, 50, 2168, 8, 1024), (8, 64, 4096, 8, 1024), (6, 43, 2048, 16, 768), (21, 18, 2176, 8, 256),
+]
+
+
+@pytest.mark.parametrize("case", PAIR_TILES, ids=["B%d_T%d_F%d_h%d_D%d" % c for c in PAIR_TILES])
+def test_expert_step_bf16_pair_tiles_of_128_rows(U, case):
+    B, T, F, Hq, D = case
+    w = synth.CONFIGS["cfg2"].with_(B=B, L=2, T=T, Hq=Hq, D=D, S=100, S_max=104)
+    _expert_case(U, w, F, 2e-2, "expert bf16, pair tiles of 128 rows", streams=sorted({0, 1, B // 2, B - 1}))
 
 
 @pytest.mark.parametrize("B", [1, 6, 4])       # chained, tiled and single calls
