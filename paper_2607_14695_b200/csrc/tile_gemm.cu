@@ -9,6 +9,8 @@
 // and SM from the L2; at 300-800 rows the fixed part of a launch (first loads, last epilogue).
 // Measured inside an expert step against the kernels that gate x in shared memory (D = 1024, F = 4096): gate/up 43.5 -> 34.4 us at 3200
 // rows and 15.6 -> 10.0 at 429, Q/K/V 16.5 -> 15.1 and 7.6 -> 6.6; the residual projections in front pay 1.5 to 2.3 us each for h * gamma.
+// At a few hundred rows a launch lasts as long as one CTA takes to take its operands in, at 50 to 58 bytes per cycle: pair tiles of 128 rows
+// (BM = 64) where they lower that (tg_shape). Expert steps of 150 rows 770 -> 761 us, 200 rows 775 -> 770, 300 rows (F = 3072) 815 -> 789.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -25,24 +27,26 @@ using namespace ptx;
 namespace {
 
 constexpr int kTgThreads = 64 + 256;      // producer warp, MMA warp, eight epilogue warps (two threads per row)
-constexpr int kTgBM = 128;                // rows per CTA
 constexpr int kTgBK = 64;
 constexpr unsigned long long kTgWaitNs = 1000000000ull;
 
-template <int BN>
+template <int BN, int BM>
 struct TgSmem {
-    static constexpr int NST = BN == 256 ? 5 : 6;
-    static constexpr uint32_t A_STAGE = kTgBM * 128;
+    static constexpr int NST = BM == 64 ? (BN == 256 ? 7 : BN == 128 ? 10 : 13) : BN == 256 ? 5 : 6;
+    static constexpr uint32_t A_STAGE = BM * 128;
     static constexpr uint32_t B_STAGE = (BN / 2) * 128;
-    static constexpr uint32_t CHUNK = kTgBM * 128;                // 128 rows x 64 output columns
+    static constexpr uint32_t CHUNK = BM * 128;                   // BM rows x 64 output columns
     static constexpr uint32_t OFF_A = 0;
     static constexpr uint32_t OFF_B = OFF_A + NST * A_STAGE;
-    static constexpr uint32_t OFF_OUT = OFF_B + NST * B_STAGE;    // [half][2] chunks on their way out
+    static constexpr uint32_t OFF_OUT = OFF_B + NST * B_STAGE;    // [half][2] chunks on their way out (BM = 64: [2][chunks of a tile])
     static constexpr uint32_t OFF_BAR = OFF_OUT + 4 * CHUNK;
     static constexpr uint32_t TOTAL = OFF_BAR + 512 + 1024;
     static_assert(TOTAL <= 227u * 1024u, "shared memory budget");
     static constexpr int T_FULL = 0, T_EMPTY = NST, T_ACC = 2 * NST, T_ACCFREE = T_ACC + 2, T_COUNT = T_ACCFREE + 2;
+    static_assert(8 * T_COUNT + 8 <= 512, "barrier area");
 };
+
+struct TgShape { int bm, bn; };
 
 struct TgParams {
     int M, K, m_tiles, n_tiles;
@@ -65,12 +69,14 @@ __device__ __forceinline__ void tg_tma_store_2d(const CUtensorMap *map, uint32_t
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");
 }
 
-template <bool SWIGLU, int BN>
+// BM = 128 or 64 rows per CTA. An accumulator of 2 x 64 rows fills all lanes of either CTA: lanes 0-63 hold its 64 rows for the first half of
+// the accumulator's columns, lanes 64-127 for the second, so its CTAs each bring gate and up rows of their own half of the output columns.
+template <bool SWIGLU, int BN, int BM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTgThreads, 1)
 tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_q,
                  const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const TgParams p)
 {
-    using S = TgSmem<BN>;
+    using S = TgSmem<BN, BM>;
     constexpr int NST = S::NST;
     constexpr int OUT_N = SWIGLU ? BN / 2 : BN;        // output columns of a tile
     extern __shared__ uint8_t smem_raw[];
@@ -86,7 +92,7 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
     const int total = p.m_tiles * p.n_tiles;
     const int my_tiles = pair < total ? (total - pair + n_pairs - 1) / n_pairs : 0;
     // row tiles fastest: the pairs working at the same time share weight rows in the L2
-    auto tile_m0 = [&](int it) -> int { return ((pair + it * n_pairs) % p.m_tiles) * (2 * kTgBM) + (int)rank * kTgBM; };
+    auto tile_m0 = [&](int it) -> int { return ((pair + it * n_pairs) % p.m_tiles) * (2 * BM) + (int)rank * BM; };
     auto tile_n0 = [&](int it) -> int { return ((pair + it * n_pairs) / p.m_tiles) * OUT_N; };
     const int nk_steps = (p.K + kTgBK - 1) / kTgBK;
 
@@ -114,6 +120,13 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
     auto load_w = [&](int s, int ks, int n0) {
         // both CTAs' loads complete on the leader's barrier
         if (rank == 0) mbar_expect_tx(bar(S::T_FULL + s), 2 * (S::A_STAGE + S::B_STAGE));
+        if constexpr (SWIGLU && BM == 64) {
+#pragma unroll
+            for (int up = 0; up < 2; ++up)
+                tg_tma2_load_2d(base + S::OFF_B + s * S::B_STAGE + up * (S::B_STAGE / 2), &tm_w, bar(S::T_FULL + s) & kPeerBitMask, ks * kTgBK,
+                                p.w_row0 + up * p.F + n0 + (int)rank * (BN / 4));
+            return;
+        }
         const int row = SWIGLU ? p.w_row0 + (int)rank * p.F + n0 : p.w_row0 + n0 + (int)rank * (BN / 2);
         tg_tma2_load_2d(base + S::OFF_B + s * S::B_STAGE, &tm_w, bar(S::T_FULL + s) & kPeerBitMask, ks * kTgBK, row);
     };
@@ -160,7 +173,7 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader CTA; the warp stays converged, one elected lane issues) ----------------
         if (rank == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(2 * kTgBM, BN, false);
+            constexpr uint32_t idesc = umma_idesc_bf16(2 * BM, BN, false);
             bool ok = true;
             int s = 0;
             uint32_t ph = 0u;
@@ -185,6 +198,88 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
                 umma2_commit_mc_elect(bar(S::T_ACC + buf), (uint16_t)3);   // also after a wait that ran out: the epilogue must not wait for nothing
             }
         }
+    } else if constexpr (BM == 64) {
+        // ---------------- epilogue: thread = one row, a quarter of the tile's output columns ----------------
+        const int quarter = warp & 3, half = quarter >> 1, part = (warp - 2) >> 2;
+        const int row = (quarter & 1) * 32 + lane;
+        constexpr int CW = OUT_N / 2, CPT = CW / 2;                   // output columns of a lane half, of a thread (32 or 16)
+        constexpr int CHUNKS = OUT_N / 64;
+        const int col0 = half * CW + part * CPT, ch = col0 / 64, p0 = (col0 & 63) / 8;
+        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + part * CPT;
+        const uint32_t leader_free = mapa(bar(S::T_ACCFREE), 0);
+        const bool issuer = lane == 0 && part == 0 && (CHUNKS == 2 ? (quarter & 1) == 0 : quarter == 0);
+        auto meet = [&] {                                             // the threads that fill a chunk
+            if constexpr (CHUNKS == 2) asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
+            else asm volatile("bar.sync 1, 256;" ::: "memory");
+        };
+        bool ok = true;
+#pragma unroll 1
+        for (int it = 0; it < my_tiles; ++it) {
+            const int m0 = tile_m0(it), n0 = tile_n0(it), buf = it & 1;
+            float ss = 0.f;
+            {
+                const int r = m0 + row < p.M ? m0 + row : p.M - 1;
+                const float *src = p.ss_in + (size_t)r * p.slots;
+                if ((p.slots & 3) == 0) {
+                    for (int j = 0; j < p.slots; j += 4) { const float4 v = *reinterpret_cast<const float4 *>(src + j); ss += (v.x + v.y) + (v.z + v.w); }
+                } else {
+                    for (int j = 0; j < p.slots; ++j) ss += src[j];
+                }
+            }
+            const float rs = rsqrtf(ss * p.inv_D + p.eps);
+            ok = wait(S::T_ACC + buf, (uint32_t)(it >> 1) & 1u, 4) && ok;
+            tc_fence_after();
+            uint32_t acc[CPT];
+            if constexpr (CPT == 32) tmem_ld32(taddr + buf * BN, acc);
+            else tmem_ld16(taddr + buf * BN, acc);
+            if constexpr (SWIGLU) {
+                uint32_t up[CPT];
+                if constexpr (CPT == 32) tmem_ld32(taddr + buf * BN + CW, up);
+                else tmem_ld16(taddr + buf * BN + CW, up);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < CPT; ++i) acc[i] = __float_as_uint(silu_mul(__uint_as_float(acc[i]) * rs, __uint_as_float(up[i]) * rs));
+            } else {
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < CPT; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * rs);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(leader_free + 8u * (uint32_t)buf);
+            // this tile's staging chunk may still be read by the store issued two tiles ago
+            if (issuer) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            if (it > 1) meet();
+            const uint32_t stage_off = S::OFF_OUT + (uint32_t)(buf * CHUNKS + ch) * S::CHUNK;
+            uint8_t *rowp = smem + stage_off + row * 128;
+#pragma unroll
+            for (int i = 0; i < CPT / 8; ++i) {
+                uint4 o;
+                uint32_t *oo = reinterpret_cast<uint32_t *>(&o);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(acc[8 * i + 2 * k]), __uint_as_float(acc[8 * i + 2 * k + 1]));
+                    oo[k] = *reinterpret_cast<uint32_t *>(&h);
+                }
+                *reinterpret_cast<uint4 *>(rowp + (((p0 + i) ^ (row & 7)) << 4)) = o;      // 128-byte swizzle of the TMA box
+            }
+            fence_proxy_async_smem();
+            meet();
+            if (issuer) {
+                const int n = n0 + ch * 64;
+                if (ok && m0 < p.M) {
+                    if constexpr (SWIGLU) {
+                        if (n < p.F) tg_tma_store_2d(&tm_q, base + stage_off, n, m0);
+                    } else {              // (the widths are multiples of 64: a chunk lies in one tensor)
+                        if (n < p.nq) tg_tma_store_2d(&tm_q, base + stage_off, n, m0);
+                        else if (n < p.nq + p.nk) tg_tma_store_2d(&tm_k, base + stage_off, n - p.nq, m0);
+                        else if (n < p.nq + 2 * p.nk) tg_tma_store_2d(&tm_v, base + stage_off, n - p.nq - p.nk, m0);
+                    }
+                }
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
+        }
+        if (issuer) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // (the writes are complete when the grid is)
     } else {
         // ---------------- epilogue: thread (row, half); chunks of 64 output columns ----------------
         const int quarter = warp & 3;                 // the TMEM lane quarter this warp may read
@@ -286,12 +381,12 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
     if (warp == 1) tmem_dealloc2(tmem, 2 * BN);
 }
 
-template <bool SWIGLU, int BN>
+template <bool SWIGLU, int BN, int BM>
 cudaError_t launch_tg(const CUtensorMap *m, TgParams p, int n_out, cudaStream_t st)
 {
     static std::atomic<unsigned long long> attr_set{0};
     cudaError_t e = once_per_device(attr_set, [] {
-        return cudaFuncSetAttribute(tile_gemm_kernel<SWIGLU, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TgSmem<BN>::TOTAL);
+        return cudaFuncSetAttribute(tile_gemm_kernel<SWIGLU, BN, BM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TgSmem<BN, BM>::TOTAL);
     });
     if (e != cudaSuccess) return e;
     constexpr int OUT_N = SWIGLU ? BN / 2 : BN;
@@ -300,19 +395,33 @@ cudaError_t launch_tg(const CUtensorMap *m, TgParams p, int n_out, cudaStream_t 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2u * (unsigned)(tiles < 74 ? tiles : 74));
     cfg.blockDim = dim3(kTgThreads);
-    cfg.dynamicSmemBytes = TgSmem<BN>::TOTAL;
+    cfg.dynamicSmemBytes = TgSmem<BN, BM>::TOTAL;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, tile_gemm_kernel<SWIGLU, BN>, m[0], m[1], m[2], m[3], m[4], p);
+    e = cudaLaunchKernelEx(&cfg, tile_gemm_kernel<SWIGLU, BN, BM>, m[0], m[1], m[2], m[3], m[4], p);
     count_launch();
     return e;
 }
 
 }  // namespace
+
+// The tile of a problem: the one whose CTAs take in the least, waves over the 74 SM pairs times the rows of x and W that a CTA loads per step.
+static TgShape tg_shape(int M, int cols, bool swiglu)
+{
+    static const TgShape kShapes[] = {{128, 256}, {128, 128}, {64, 256}, {64, 128}, {64, 64}};
+    TgShape best = kShapes[0];
+    int best_cost = 0x7fffffff;
+    for (const TgShape &t : kShapes) {
+        if ((t.bm == 64) && (swiglu ? t.bn == 64 : t.bn == 256)) continue;       // (not built)
+        const int tiles = ((M + 2 * t.bm - 1) / (2 * t.bm)) * ((cols + t.bn - 1) / t.bn), cost = (tiles + 73) / 74 * (t.bm + t.bn / 2);
+        if (cost < best_cost) { best_cost = cost; best = t; }
+    }
+    return best;
+}
 
 bool tile_proj_supported(int mode, int M, int K, int nq, int nk, int F)
 {
@@ -325,21 +434,23 @@ cudaError_t launch_tile_proj(const ChainProj &a, cudaStream_t st)
 {
     const bool swiglu = a.mode == CG_SWIGLU;
     TgParams p = {};
-    p.M = a.B * a.R; p.K = a.K; p.m_tiles = (p.M + 2 * kTgBM - 1) / (2 * kTgBM); p.w_row0 = a.w_row0; p.F = a.N; p.nq = a.nq; p.nk = a.nk;
+    p.M = a.B * a.R; p.K = a.K; p.w_row0 = a.w_row0; p.F = a.N; p.nq = a.nq; p.nk = a.nk;
     p.ss_in = a.ss_in; p.slots = a.slots_in; p.inv_D = 1.f / (float)a.D; p.eps = a.eps; p.status = a.status;
-    // 256 accumulator columns per tile unless they would leave more than half of the SM pairs without one
     const int cols = swiglu ? 2 * a.N : a.N;
-    const bool narrow = p.m_tiles * ((cols + 255) / 256) * 2 <= 74;
+    const TgShape t = tg_shape(p.M, cols, swiglu);
+    p.m_tiles = (p.M + 2 * t.bm - 1) / (2 * t.bm);
     CUtensorMap m[5];
-    if (!tensor_map_2d_bf16(&m[0], a.x, a.K, p.M, kTgBM) || !tensor_map_2d_bf16(&m[1], a.W, a.K, a.w_rows, narrow ? 64 : 128)) return cudaErrorInvalidValue;
+    if (!tensor_map_2d_bf16(&m[0], a.x, a.K, p.M, t.bm) || !tensor_map_2d_bf16(&m[1], a.W, a.K, a.w_rows, swiglu && t.bm == 64 ? t.bn / 4 : t.bn / 2)) return cudaErrorInvalidValue;
     if (swiglu) {
-        if (!tensor_map_2d_bf16(&m[2], a.h, a.N, p.M, kTgBM)) return cudaErrorInvalidValue;
+        if (!tensor_map_2d_bf16(&m[2], a.h, a.N, p.M, t.bm)) return cudaErrorInvalidValue;
         m[3] = m[4] = m[2];
-        return narrow ? launch_tg<true, 128>(m, p, a.N, st) : launch_tg<true, 256>(m, p, a.N, st);
+        if (t.bm == 64) return t.bn == 128 ? launch_tg<true, 128, 64>(m, p, a.N, st) : launch_tg<true, 256, 64>(m, p, a.N, st);
+        return t.bn == 128 ? launch_tg<true, 128, 128>(m, p, a.N, st) : launch_tg<true, 256, 128>(m, p, a.N, st);
     }
-    if (!tensor_map_2d_bf16(&m[2], a.q, a.nq, p.M, kTgBM) || !tensor_map_2d_bf16(&m[3], a.k, a.nk, p.M, kTgBM) || !tensor_map_2d_bf16(&m[4], a.v, a.nk, p.M, kTgBM))
+    if (!tensor_map_2d_bf16(&m[2], a.q, a.nq, p.M, t.bm) || !tensor_map_2d_bf16(&m[3], a.k, a.nk, p.M, t.bm) || !tensor_map_2d_bf16(&m[4], a.v, a.nk, p.M, t.bm))
         return cudaErrorInvalidValue;
-    return narrow ? launch_tg<false, 128>(m, p, a.N, st) : launch_tg<false, 256>(m, p, a.N, st);
+    if (t.bm == 64) return t.bn == 64 ? launch_tg<false, 64, 64>(m, p, a.N, st) : launch_tg<false, 128, 64>(m, p, a.N, st);
+    return t.bn == 128 ? launch_tg<false, 128, 128>(m, p, a.N, st) : launch_tg<false, 256, 128>(m, p, a.N, st);
 }
 
 }  // namespace reflex

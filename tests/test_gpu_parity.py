@@ -1296,6 +1296,7 @@ def _more_layers(dW):
 PAIR_TILES = [
     # B, T, F, Hq, D: rows around the tiles of 128, contractions of 2048 and more, streams of four rows under a CTA's 32
     (3, 43, 2048, 8, 1024), (64, 4, 2048, 8, 512), (4, 50, 2168, 8, 1024), (8, 64, 4096, 8, 1024), (6, 43, 2048, 16, 768), (21, 18, 2176, 8, 256),
+    (6, 43, 3072, 8, 1024),      # gate/up in pair tiles of 128 rows x 256 columns
 ]
 
 
