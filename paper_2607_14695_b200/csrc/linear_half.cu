@@ -311,7 +311,7 @@ cudaError_t lh_launch(const CUtensorMap *m, const LhParams &p, cudaStream_t st)
 int linear_half_columns(int M, int K, int N)
 {
     const int chunks = (K + 63) / 64, m_tiles = (M + 127) / 128;
-    if (M <= 128 || chunks % 2 != 0 || chunks < 32) return 0;
+    if (M <= 64 || chunks % 2 != 0 || chunks < 32) return 0;
     for (int bn = 64; bn <= 128; bn *= 2)
         if (m_tiles * ((N + bn - 1) / bn) <= 32) return bn;
     return 0;

@@ -548,34 +548,57 @@ static bool expert_chained(const reflex_cache_desc &d, const reflex_expert &e)
            chain_proj_supported(CG_RES, M, e.F, e.D) && chain_proj_supported(CG_OUT, M, e.D, e.A);
 }
 
+// Both residual projections as pair tiles of 128 rows (linear_half.cu): 65 to 512 rows, contractions of 2048 or more.
+static bool expert_halves(const reflex_cache_desc &d, const reflex_expert &e)
+{
+    return linear_half_columns(d.B * e.T, d.Hq * d.d, e.D) && linear_half_columns(d.B * e.T, e.F, e.D);
+}
+
 // ... or, for more rows, through the tile kernels on the same operands (tile_gemm.cu, linear_half.cu, linear_tc.cu). Up to 256 rows only where
-// both residual projections go as pair tiles of 128 rows (a contraction of 2048 or more): as tiles of 256 rows they are too few CTAs, and the single
-// calls' few-rows kernels were ahead (200 rows: 7.1 us each against 12 and 16). Short chunks are the exception: the gates of the streams under
-// 128 rows then exceed what the single gate/up projection holds, and its plain kernel took 8.5 ms a layer (8 x 20 rows: a step of 153 ms, 0.91
-// by the tiles).
+// both residual projections go as pair tiles of 128 rows: as tiles of 256 rows they are too few CTAs, and the single calls' few-rows kernels
+// were ahead (200 rows: 7.1 us each against 12 and 16). Short chunks are the exception: the gates of the streams under 128 rows then exceed
+// what the single gate/up projection holds, and its plain kernel took 8.5 ms a layer (8 x 20 rows: a step of 153 ms, 0.91 by the tiles).
 static bool expert_tiled(const reflex_cache_desc &d, const reflex_expert &e)
 {
     const int M = d.B * e.T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
     if (d.dtype != REFLEX_DTYPE_BF16 || e.D % 256 != 0 || !(e.A == 8 || e.A == 16 || e.A == 32) || e.T < 4) return false;      // (T: the gates of the streams under 128 rows fit the idle stages)
-    const bool halves = linear_half_columns(M, nq, e.D) && linear_half_columns(M, e.F, e.D);
-    if (M <= 256 && !halves && norm_swiglu_gates_fit(e.T, e.D)) return false;
+    if (M <= 256 && !expert_halves(d, e) && norm_swiglu_gates_fit(e.T, e.D)) return false;
     return tile_proj_supported(CG_QKV, M, e.D, nq, nk, 0) && tile_proj_supported(CG_SWIGLU, M, e.D, 0, 0, e.F) && chain_proj_supported(CG_OUT, M, e.D, e.A) &&
            nq % 8 == 0 && e.F % 8 == 0;
 }
 
-static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float *a, float dt, bool tiled, void *stream)
+// Which of a step's projections go through the tile kernels instead of the chained ones.
+struct StepForm { bool qkv, gu, res; };
+
+// Pair tiles take in 64 rows of x and of W per step, whatever of them is live; the chained kernels split the contraction and pay for the exchange.
+// Whole steps (D = 1024, us, chained / Q/K/V and gate/up by tiles / all by tiles): 50 rows 570 / 572 / 623, 56 rows 588 / 578 / 624, 64 rows
+// 638 / 621 / 655, 72 rows 796 / 737 / 655, 100 rows 741 / 661 / 662 (F = 2048: 676 / 614 / 583), 120 rows 800 / 733 / 715. A gate/up projection whose tiles
+// leave half of the SM pairs idle is ahead with fewer rows too: F = 2048, 33 rows 513 -> 504, 50 rows 530 -> 518 (F = 3072: 548 -> 550).
+static StepForm step_form(const reflex_cache_desc &d, const reflex_expert &e, bool chained)
+{
+    const int M = d.B * e.T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
+    if (!chained || (expert_halves(d, e) && expert_tiled(d, e))) return {true, true, true};
+    const bool half_idle = e.F >= 1536 && (2 * e.F + 127) / 128 <= 37;
+    return {M > 52 && tile_proj_supported(CG_QKV, M, e.D, nq, nk, 0), (M > 52 || half_idle) && tile_proj_supported(CG_SWIGLU, M, e.D, 0, 0, e.F), false};
+}
+
+static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float *a, float dt, const StepForm form, void *stream)
 {
     const reflex_cache_desc &d = c->desc;
     typedef __nv_bfloat16 bf;
     const int L = e.L > 0 ? e.L : d.L, B = d.B, T = e.T, D = e.D, M = B * T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
     cudaStream_t st = (cudaStream_t)stream;
-    auto proj = [&](const ChainProj &p) { return !tiled ? launch_chain_proj(p, st) : p.mode == CG_RES ? launch_tile_res(p, st) : launch_tile_proj(p, st); };
+    const bool tiled = form.res;
+    auto proj = [&](const ChainProj &p) {
+        if (p.mode == CG_RES) return form.res ? launch_tile_res(p, st) : launch_chain_proj(p, st);
+        return (p.mode == CG_QKV ? form.qkv : form.gu) ? launch_tile_proj(p, st) : launch_chain_proj(p, st);
+    };
     auto slots_of = [&](int K) { return tiled ? tile_res_slots(M, K, D) : (D + 31) / 32; };
     // partial sums of squares of the residual rows: two areas, so that a projection never writes the one its predecessor reads
     float *ss[2] = {e.row_sums, e.row_sums + (size_t)M * ((D + 31) / 32)};
     auto gate = [&](int i) { return (const float *)e.gates + (size_t)i * B * D; };
     // what a later kernel of the step reads is asked into the L2 one or two kernels ahead, so that the 34 MB of a layer come from
-    // memory while the chain is busy with latencies (the tile form's projections are not, and take no part)
+    // memory while the chain is busy with latencies (the tile kernels are not, and take no part)
     auto range = [](ChainPrefetch &pf, int i, const void *base, size_t first, size_t n) {
         pf.ptr[i] = (const char *)base + first * 2; pf.bytes[i] = n * 2 & ~(size_t)15;
     };
@@ -666,7 +689,7 @@ int reflex_expert_step(reflex_cache_t *c, const reflex_expert *ep, float *a, con
     int rc = reflex_adarmsnorm_gate(cond, e.W1, e.b1, e.W2, e.b2, e.gates, 2 * L + 1, B, D, e.Cd, e.Hd, dt_, stream);
     if (rc != REFLEX_OK) return rc;
     const bool chained = expert_chained(d, e);
-    if (chained || expert_tiled(d, e)) return expert_step_chained(c, e, a, -1.0f / (float)K, !chained, stream);
+    if (chained || expert_tiled(d, e)) return expert_step_chained(c, e, a, -1.0f / (float)K, step_form(d, e, chained), stream);
     // any other dtype, shape or row count: the single calls in order, allowed to read weights and gates ahead of the preceding kernel (nothing in
     // the step writes weights; the gates are complete before the input projection starts)
     const size_t es = elem_size(dt_);

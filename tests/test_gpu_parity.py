@@ -1297,6 +1297,8 @@ PAIR_TILES = [
     # B, T, F, Hq, D: rows around the tiles of 128, contractions of 2048 and more, streams of four rows under a CTA's 32
     (3, 43, 2048, 8, 1024), (64, 4, 2048, 8, 512), (4, 50, 2168, 8, 1024), (8, 64, 4096, 8, 1024), (6, 43, 2048, 16, 768), (21, 18, 2176, 8, 256),
     (6, 43, 3072, 8, 1024),      # gate/up in pair tiles of 128 rows x 256 columns
+    # the fewest rows, all of one pair tile, and the chained residual projections between tiles
+    (13, 5, 2048, 8, 1024), (2, 64, 4096, 8, 1024), (1, 53, 4096, 8, 1024), (2, 32, 4096, 8, 1024), (1, 33, 2048, 8, 1024), (1, 60, 1000, 4, 320),
 ]
 
 
@@ -1304,7 +1306,7 @@ PAIR_TILES = [
 def test_expert_step_bf16_pair_tiles_of_128_rows(U, case):
     B, T, F, Hq, D = case
     w = synth.CONFIGS["cfg2"].with_(B=B, L=2, T=T, Hq=Hq, D=D, S=100, S_max=104)
-    _expert_case(U, w, F, 2e-2, "expert bf16, pair tiles of 128 rows", streams=sorted({0, 1, B // 2, B - 1}))
+    _expert_case(U, w, F, 2e-2, "expert bf16, pair tiles of 128 rows", streams=sorted({0, B // 2, B - 1}))
 
 
 @pytest.mark.parametrize("B", [1, 6, 4])       # chained, tiled and single calls
