@@ -17,6 +17,7 @@
 // drains, so a mistake cannot hang the device.
 #include <cuda.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -541,6 +542,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 }  // namespace reflex
 
 #include "attn_tc2.cuh"
+#include "attn_pair.cuh"
 
 namespace reflex {
 
@@ -674,6 +676,29 @@ cudaError_t launch2_t(const CUtensorMap *mq, const CUtensorMap *mk, const CUtens
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     cudaError_t e = cudaLaunchKernelEx(&cfg, attn_tc2_kernel<HD, EARLY>, *mq, *mk, *mv, *mkd, *mvd, *mo, tp);
+    count_launch();
+    return e;
+}
+
+template <int HD, bool EARLY>
+cudaError_t launch_pair_t(const CUtensorMap *m, const TcParams &tp, int units, cudaStream_t st)
+{
+    static std::atomic<unsigned long long> attr_set{0};
+    cudaError_t e = once_per_device(attr_set, [] { return cudaFuncSetAttribute(attn_pair_kernel<HD, EARLY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ApSmem<HD>::TOTAL); });
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2u * (unsigned)(units * tp.nsplit));
+    cfg.blockDim = dim3(kApThreads);
+    cfg.dynamicSmemBytes = ApSmem<HD>::TOTAL;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2u * (unsigned)(tp.cluster_merge ? tp.nsplit : 1); attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    e = cudaLaunchKernelEx(&cfg, attn_pair_kernel<HD, EARLY>, m[0], m[1], m[2], m[3], m[4], m[5], tp);
     count_launch();
     return e;
 }
@@ -837,6 +862,80 @@ int tc2_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count)
         if (loop_us + split_us < best_us - 0.05) { best_us = loop_us + split_us; best = ns; }
     }
     return best;
+}
+
+static int pair_units(const AttnParams &p)
+{
+    const int G = p.Hq / p.Hkv;
+    if (G > kApRows || kApRows % G != 0) return 0;
+    const int tt = kApRows / G;
+    return ((p.T + tt - 1) / tt + 1) / 2 * p.Hkv * p.B;
+}
+
+// What a launch of units of 256 rows takes, us: fitted to graph replays (heads of 256: 13.9 us for 4 streams of 898 keys in one slice, 16.4 for 18, 33.1
+// for 16 of 4466 keys in two, 22.7 for 8 of 3306).
+static double tc2_us(const AttnParams &p, int nsplit, int sm_count)
+{
+    const int G = p.Hq / p.Hkv, units = ((p.T + kBM / G - 1) / (kBM / G) + 1) / 2 * p.Hkv * p.B;
+    const int tiles = ((p.S_max + kBN - 1) / kBN + (p.N + kBN - 1) / kBN + (p.T + kBN - 1) / kBN + 1) / 2, clusters = sm_count / 2 > 0 ? sm_count / 2 : 1;
+    const bool merged = tc2_cluster_merge_ok(p, nsplit, sm_count);
+    const int waves = merged ? 1 : (units * nsplit + clusters - 1) / clusters;
+    const double split = nsplit <= 1 ? 0.0 : merged ? tc2_merged_us(units, nsplit) : tc2_partials_us(p, nsplit);
+    return 4.4 + 0.03 * std::min(units * nsplit, clusters) + (p.d == 256 ? 1.17 : 0.95) * waves * ((tiles + nsplit - 1) / nsplit) + split;
+}
+
+// Key slices of the 128-row units where they are the faster two-CTA form; 0: units of 256 rows. One wave is all they may be; a tile of 128 keys takes
+// them 1.05 us and one of 256 rows 1.17, a merge inside a cluster 2.3 us and more with the CTAs that push at the same time, partials and the
+// merge launch 1.2 us and 0.37 per 400 rows and slice. Measured against the form of before, one call, graph replay, us: 898 keys x 50 tokens, 2 streams
+// 10.6 -> 8.8 (four slices), 4 streams 13.7 -> 10.6 (two), 8 streams 14.4 -> 11.4 (two), 16 streams 16.2 -> 13.6 (one); 24 streams x 33 tokens 17.5 -> 14.6;
+// heads of 128, 6 streams x 4 KV heads 9.2 -> 7.5; one stream x 2111 keys 13.2 -> 10.8, 4 streams x 2082 keys 17.1 -> 14.3. 16 streams x 4466 keys
+// stay with units of 256 rows in two slices (33.1 against 40.8).
+int pair_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count, bool &merged)
+{
+    const int units = pair_units(p), clusters = sm_count / 2;
+    merged = false;
+    if (units == 0 || units > clusters || !tc2_supported(p)) return 0;
+    const int tiles = ((p.S_max + kBN - 1) / kBN + (p.N + kBN - 1) / kBN + (p.T + kBN - 1) / kBN + 1) / 2;
+    const double rows = (double)p.B * p.T * p.Hq, per_split_bytes = rows * (p.d + 2) * sizeof(float);
+    const int ns2 = tc2_choose_splits(p, partial_bytes, sm_count);
+    double best_us = tc2_us(p, ns2 < 1 ? 1 : ns2, sm_count) - 0.1;
+    int best = 0;
+    static const int kSlices[] = {1, 2, 3, 4, 6, 8, 12, 16, 18};
+    for (const int ns : kSlices) {
+        if (ns > tiles || units * ns > clusters) break;
+        for (int m = ns == 2 || ns == 4 ? 1 : 0; m >= 0; --m) {
+            // (clusters of eight with a margin: the last ones find room late, 16.0 us with 16 of them against 9.3 with 12)
+            const int active = m ? tc2_active_clusters(p.d, 2 * ns) : 0;
+            if (m && units > (ns == 4 ? active - active / 6 : active)) continue;
+            if (!m && ns > 1 && per_split_bytes * ns > (double)partial_bytes) continue;
+            const double split = ns == 1 ? 0.0 : m ? 2.2 + 0.1 * (ns - 2) + 0.015 * units * ns : 1.2 + 0.37 * rows * ns / 400.0 * p.d / 256.0;
+            const double us = 4.0 + (ns == 1 ? 0.02 * units : 0.0) + (p.d == 256 ? 1.05 : 0.85) * ((tiles + ns - 1) / ns) + split;
+            if (us < best_us) { best_us = us; best = ns; merged = m != 0; }
+        }
+    }
+    return best;
+}
+
+cudaError_t launch_attention_pair(const AttnParams &p, uint32_t *status, int nsplit, bool merged, cudaStream_t st)
+{
+    const int G = p.Hq / p.Hkv, rows_slab = p.L * p.B * (p.ring_off + p.N), tt = kApRows / G;
+    CUtensorMap m[6];
+    if (!tensor_map_q_bf16(&m[0], p.q, p.B, p.T, p.Hq, p.d, G, tt) || !cache().get(&m[1], p.k_slab, 0, rows_slab, p.Hkv, p.d, 0, mk_slab) ||
+        !cache().get(&m[2], p.v_slab, 0, rows_slab, p.Hkv, p.d, 0, mk_slab) || !cache().get(&m[3], p.k_dyn, 0, p.B * p.T, p.Hkv, p.d, 0, mk_slab) ||
+        !cache().get(&m[4], p.v_dyn, 0, p.B * p.T, p.Hkv, p.d, 0, mk_slab) || !tensor_map_q_bf16(&m[5], p.out, p.B, p.T, p.Hq, p.d, G, tt))
+        return cudaErrorInvalidValue;
+    TcParams tp = {};
+    tp.state = p.state; tp.out = p.out; tp.partials = p.partials; tp.status = status;
+    tp.B = p.B; tp.L = p.L; tp.Hq = p.Hq; tp.Hkv = p.Hkv; tp.G = G; tp.S_max = p.S_max; tp.N = p.N; tp.T = p.T; tp.layer = p.layer; tp.ring_off = p.ring_off;
+    tp.dyn_mask = p.dyn_mask; tp.scale = p.scale; tp.scale_log2 = p.scale * 1.4426950408889634f;
+    tp.nsplit = nsplit; tp.tile_tokens = tt; tp.live_rows = kApRows; tp.n_qtiles = ((p.T + tt - 1) / tt + 1) / 2; tp.cluster_merge = merged && nsplit > 1 ? 1 : 0;
+    const int units = pair_units(p);
+    cudaError_t e;
+    if (p.d == 256) e = (p.early ? launch_pair_t<256, true> : launch_pair_t<256, false>)(m, tp, units, st);
+    else if (p.d == 128) e = (p.early ? launch_pair_t<128, true> : launch_pair_t<128, false>)(m, tp, units, st);
+    else return cudaErrorInvalidValue;
+    if (e != cudaSuccess || nsplit == 1 || tp.cluster_merge) return e;
+    return launch_attention_merge(p, st);
 }
 
 cudaError_t launch_attention_tc(const AttnParams &p, uint32_t *status, bool two_cta, int sm_count, cudaStream_t st)
