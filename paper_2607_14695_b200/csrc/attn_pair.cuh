@@ -33,8 +33,9 @@ template <int HD> struct ApSmem {
     static constexpr uint32_t OFF_K = OFF_Q + Q_BYTES;                // later the inbox of a merge, or the partial tile on its way out
     static constexpr uint32_t OFF_V = OFF_K + NKS * K_STAGE;
     static constexpr uint32_t OFF_P = OFF_V + NVS * V_STAGE;
-    static constexpr uint32_t OFF_MAX = OFF_P + 2 * P_BUF;            // [2 buffers][64 rows][4] row maxima; the sums use the buffer the last tile did not
-    static constexpr uint32_t OFF_ML = OFF_MAX + 2 * kApRows * 16;    // [4 slices][64 rows] (m, l)
+    static constexpr uint32_t OFF_MAX = OFF_P + 2 * P_BUF;            // [2 buffers][64 rows][4] row maxima
+    static constexpr uint32_t OFF_SUM = OFF_MAX + 2 * kApRows * 16;   // [2 accumulators][64 rows][4] row sums
+    static constexpr uint32_t OFF_ML = OFF_SUM + 2 * kApRows * 16;    // [4 slices][64 rows] (m, l)
     static constexpr uint32_t OFF_BAR = OFF_ML + 4 * kApRows * 8;
     static constexpr uint32_t TOTAL = OFF_BAR + 256 + 1024;
     static_assert(TOTAL <= 227u * 1024u, "shared memory budget");
@@ -44,15 +45,19 @@ template <int HD> struct ApSmem {
     static_assert(8 * C_COUNT + 8 <= 256, "barrier area");
 };
 
-template <int HD, bool EARLY>      // EARLY: inside an expert step, the first cached tiles are asked for ahead of the wait
+// EARLY: inside an expert step, the first cached tiles are asked for ahead of the wait.
+// DUAL: even and odd tiles have an accumulator each, with a reference maximum and a sum of its own. The key that sets a reference has weight 1, which
+// bf16 holds exactly, and twice as many references are twice as many such keys: 898 keys in four slices 2.24e-3 -> 2.13e-3 from 64 bits, what the eight
+// slices of chain_attn_kernel give. Split launches take it, they stand where finer slices stood; it costs them 0.3 to 0.5 us. Unsplit ones
+// are as far from 64 bits as units of 256 rows, 2.32e-3 (2.29e-3 with DUAL, for 1 us).
+template <int HD, bool EARLY, bool DUAL>
 __global__ void __launch_bounds__(kApThreads, 1)      // clusters of 2 CTAs, or of 2 * nsplit (cluster_merge)
 attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                  const __grid_constant__ CUtensorMap tm_kd, const __grid_constant__ CUtensorMap tm_vd, const __grid_constant__ CUtensorMap tm_o, const TcParams p)
 {
     using L = ApSmem<HD>;
     constexpr int CH = L::CH, VCH = L::VCH, NKS = L::NKS, NVS = L::NVS;
-    constexpr uint32_t kColO = 0, kColS = HD / 2, kTmemCols = 256;       // O: HD / 2 columns; S: two buffers of 64
-    static_assert(HD / 2 + 128 <= (int)kTmemCols, "tensor memory");
+    constexpr uint32_t kColO = 0, kColS = DUAL ? HD : HD / 2, kTmemCols = kColS + 128 <= 256 ? 256 : 512;       // O: HD / 2 columns an accumulator; S: two buffers of 64
     constexpr int OC = HD / 4;                                           // a thread's columns of O
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -202,7 +207,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 const int ksteps = 2 * (tile0 + j) + 1 < H ? 8 : 4;
 #pragma unroll 4
                 for (int kk = 0; kk < ksteps; ++kk) {
-                    umma2_ss_elect(tmem + kColO, pd, vd, idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
+                    umma2_ss_elect(tmem + kColO + (DUAL ? buf * (HD / 2) : 0), pd, vd, idesc_pv, (j > (DUAL ? 1 : 0) || kk > 0) ? 1u : 0u);
                     umma_desc_advance(pd, (kk & 3) == 3 ? kApRows * 128 - 96 : 32);
                     umma_desc_advance(vd, 16 * 128);
                 }
@@ -219,7 +224,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         float *xmax = reinterpret_cast<float *>(smem + L::OFF_MAX);
         const Ex2PolyConsts pk = ex2_poly_consts();
         bool ok = true;
-        float m_ref = -INFINITY, l = 0.f;
+        float m_ref = -INFINITY, l = 0.f, m_oth = -INFINITY, l_oth = 0.f;      // of this tile's accumulator and of the other one
         for (int j = 0; j < n; ++j) {
             const int buf = j & 1, st = j % NVS, h = 2 * (tile0 + j) + half;
             const bool dead = h >= H;                         // a half past the last key: its threads only take part in the row exchange
@@ -277,7 +282,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 const float4 v = *reinterpret_cast<const float4 *>(xmax + (buf * kApRows + row) * 4);
                 mx = fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
             }
-            if (j == 0) {
+            if (j < (DUAL ? 2 : 1)) {
                 m_ref = mx;
             } else {
                 const bool grow = (mx - m_ref) * p.scale_log2 > kRescaleThreshold;
@@ -286,16 +291,16 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                     const float alpha = grow ? ex2((m_ref - mx) * p.scale_log2) : 1.f;
                     if (grow) m_ref = mx;
                     l *= alpha;
-                    ok = ok && wait(L::C_PVDONE + (buf ^ 1), (uint32_t)((j - 1) >> 1) & 1u, 8);
+                    ok = ok && (DUAL ? wait(L::C_PVDONE + buf, (uint32_t)((j - 2) >> 1) & 1u, 8) : wait(L::C_PVDONE + (buf ^ 1), (uint32_t)((j - 1) >> 1) & 1u, 8));
                     tc_fence_after();
 #pragma unroll 1
                     for (int c = 0; c < OC / 32; ++c) {
                         uint32_t o[32];
-                        tmem_ld32(taddr + kColO + part * OC + c * 32, o);
+                        tmem_ld32(taddr + kColO + (DUAL ? buf * (HD / 2) : 0) + part * OC + c * 32, o);
                         tmem_wait_ld();
 #pragma unroll
                         for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                        tmem_st32(taddr + kColO + part * OC + c * 32, o);
+                        tmem_st32(taddr + kColO + (DUAL ? buf * (HD / 2) : 0) + part * OC + c * 32, o);
                     }
                     tmem_wait_st();
                 }
@@ -338,27 +343,65 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(leader_pfull + 8u * (uint32_t)buf);
+            if constexpr (DUAL) {
+                const float m_tmp = m_ref, l_tmp = l;
+                m_ref = m_oth; l = l_oth; m_oth = m_tmp; l_oth = l_tmp;
+            }
         }
         // ---- epilogue ----
         if (n > 0) ok = ok && wait(L::C_PVDONE + ((n - 1) & 1), (uint32_t)((n - 1) >> 1) & 1u, 10);
+        if (DUAL && n > 1) ok = ok && wait(L::C_PVDONE + (n & 1), (uint32_t)((n - 2) >> 1) & 1u, 10);
         if (*abort_flag) ok = false;
         tc_fence_after();
-        float *xsum = xmax + (n & 1) * (kApRows * 4);                  // (the last tile used the other one)
-        xsum[row * 4 + half * 2 + part] = l;
+        float *xsum = reinterpret_cast<float *>(smem + L::OFF_SUM);    // [accumulator][64 rows][4]
+        const bool odd = DUAL && (n & 1) != 0;                         // m_ref and l are the second accumulator's
+        xsum[row * 4 + half * 2 + part] = odd ? l_oth : l;
+        if constexpr (DUAL) xsum[(kApRows + row) * 4 + half * 2 + part] = odd ? l : l_oth;
         asm volatile("bar.sync 1, 256;" ::: "memory");
+        float w0 = 1.f, w1 = 0.f;                                      // the two become one
         {
             const float4 v = *reinterpret_cast<const float4 *>(xsum + row * 4);
             l = (v.x + v.y) + (v.z + v.w);
         }
+        if constexpr (DUAL) {
+            const float m0 = odd ? m_oth : m_ref, m1 = odd ? m_ref : m_oth;
+            m_ref = fmaxf(m0, m1);
+            w0 = m0 == -INFINITY ? 0.f : ex2((m0 - m_ref) * p.scale_log2);
+            w1 = m1 == -INFINITY ? 0.f : ex2((m1 - m_ref) * p.scale_log2);
+            const float4 u = *reinterpret_cast<const float4 *>(xsum + (kApRows + row) * 4);
+            l = fmaf(w0, l, w1 * ((u.x + u.y) + (u.z + u.w)));
+        }
+        // 32 columns of the row's unnormalised O (an accumulator that was never written counts as zero; after a failed wait NaN)
+        auto load_o = [&](int c, float (&o)[32]) {
+            uint32_t a[32];
+            tmem_ld32(taddr + kColO + part * OC + c * 32, a);
+            if constexpr (DUAL) {
+                uint32_t b2[32];
+                tmem_ld32(taddr + kColO + HD / 2 + part * OC + c * 32, b2);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    o[i] = n > 0 ? __uint_as_float(a[i]) * w0 : 0.f;
+                    if (n > 1) o[i] = fmaf(__uint_as_float(b2[i]), w1, o[i]);
+                }
+            } else {
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) o[i] = n > 0 ? __uint_as_float(a[i]) : 0.f;
+            }
+            if (!ok) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) o[i] = __int_as_float(0x7fc00000);
+            }
+        };
         const int col0 = half * (HD / 2) + part * OC;                  // this thread's first column of O
         if (ns == 1) {
             // O / l through the idle Q buffer, laid out like it, and TMA stores
             const float inv = ok ? 1.f / l : __int_as_float(0x7fc00000);
 #pragma unroll
             for (int c = 0; c < OC / 32; ++c) {
-                uint32_t o[32];
-                tmem_ld32(taddr + kColO + part * OC + c * 32, o);
-                tmem_wait_ld();
+                float o[32];
+                load_o(c, o);
                 const int col = col0 + c * 32;
                 uint8_t *srow = smem + L::OFF_Q + (col / 64) * (kApRows * 128) + row * 128;
 #pragma unroll
@@ -367,7 +410,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                     uint32_t *vv = reinterpret_cast<uint32_t *>(&v);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(o[8 * i + 2 * k]) * inv, __uint_as_float(o[8 * i + 2 * k + 1]) * inv);
+                        __nv_bfloat162 hh = __floats2bfloat162_rn(o[8 * i + 2 * k] * inv, o[8 * i + 2 * k + 1] * inv);
                         vv[k] = *reinterpret_cast<uint32_t *>(&hh);
                     }
                     *reinterpret_cast<uint4 *>(srow + ((((col & 63) / 8 + i) ^ (row & 7)) << 4)) = v;
@@ -399,19 +442,14 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             const uint32_t dst = mapa(base + slot, 2u * owner + rank), ib = mapa(bar(L::C_INBOX), 2u * owner + rank);
 #pragma unroll
             for (int c = 0; c < OC / 32; ++c) {
-                uint32_t o[32];
-                tmem_ld32(taddr + kColO + part * OC + c * 32, o);
-                tmem_wait_ld();
-                if (!ok || n == 0) {                                   // (an accumulator that was never written sends zeros, a failed wait NaN)
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) o[i] = ok ? 0u : 0x7fc00000u;
-                }
+                float o[32];
+                load_o(c, o);
                 if (exists && free) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const uint32_t at = (uint32_t)(c * 8 + i) * (kApRows * 16);
-                        if (owner == split) *reinterpret_cast<uint4 *>(smem + slot + at) = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
-                        else st_async_v4(dst + at, ib, o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                        if (owner == split) *reinterpret_cast<float4 *>(smem + slot + at) = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                        else st_async_v4(dst + at, ib, __float_as_uint(o[4 * i]), __float_as_uint(o[4 * i + 1]), __float_as_uint(o[4 * i + 2]), __float_as_uint(o[4 * i + 3]));
                     }
                 }
             }
@@ -473,21 +511,20 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             }
             if (n > 0) {
                 constexpr int PR = HD / 4;                             // 16-byte pieces per row, swizzled: piece i of row r at i ^ (r % 32)
-                uint4 *stage = reinterpret_cast<uint4 *>(smem + L::OFF_K);
+                float4 *stage = reinterpret_cast<float4 *>(smem + L::OFF_K);
 #pragma unroll
                 for (int c = 0; c < OC / 32; ++c) {
-                    uint32_t o[32];
-                    tmem_ld32(taddr + kColO + part * OC + c * 32, o);
-                    tmem_wait_ld();
+                    float o[32];
+                    load_o(c, o);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) stage[row * PR + (((col0 + c * 32) / 4 + i) ^ (row & 31))] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                    for (int i = 0; i < 8; ++i) stage[row * PR + (((col0 + c * 32) / 4 + i) ^ (row & 31))] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
                 }
                 asm volatile("bar.sync 1, 256;" ::: "memory");
 #pragma unroll 2
                 for (int rr = 0; rr < kApRows / 8; ++rr) {
                     const int r = (warp - 2) * (kApRows / 8) + rr;
                     if (r >= rows) continue;
-                    uint4 *dst = reinterpret_cast<uint4 *>(partial_o(p.partials, slot_of(r), HD));
+                    float4 *dst = reinterpret_cast<float4 *>(partial_o(p.partials, slot_of(r), HD));
 #pragma unroll
                     for (int i = 0; i < PR / 32; ++i) dst[i * 32 + lane] = stage[r * PR + ((i * 32 + lane) ^ (r & 31))];
                 }

@@ -680,11 +680,11 @@ cudaError_t launch2_t(const CUtensorMap *mq, const CUtensorMap *mk, const CUtens
     return e;
 }
 
-template <int HD, bool EARLY>
+template <int HD, bool EARLY, bool DUAL>
 cudaError_t launch_pair_t(const CUtensorMap *m, const TcParams &tp, int units, cudaStream_t st)
 {
     static std::atomic<unsigned long long> attr_set{0};
-    cudaError_t e = once_per_device(attr_set, [] { return cudaFuncSetAttribute(attn_pair_kernel<HD, EARLY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ApSmem<HD>::TOTAL); });
+    cudaError_t e = once_per_device(attr_set, [] { return cudaFuncSetAttribute(attn_pair_kernel<HD, EARLY, DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ApSmem<HD>::TOTAL); });
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2u * (unsigned)(units * tp.nsplit));
@@ -698,7 +698,7 @@ cudaError_t launch_pair_t(const CUtensorMap *m, const TcParams &tp, int units, c
     attr[1].val.clusterDim.x = 2u * (unsigned)(tp.cluster_merge ? tp.nsplit : 1); attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    e = cudaLaunchKernelEx(&cfg, attn_pair_kernel<HD, EARLY>, m[0], m[1], m[2], m[3], m[4], m[5], tp);
+    e = cudaLaunchKernelEx(&cfg, attn_pair_kernel<HD, EARLY, DUAL>, m[0], m[1], m[2], m[3], m[4], m[5], tp);
     count_launch();
     return e;
 }
@@ -931,8 +931,8 @@ cudaError_t launch_attention_pair(const AttnParams &p, uint32_t *status, int nsp
     tp.nsplit = nsplit; tp.tile_tokens = tt; tp.live_rows = kApRows; tp.n_qtiles = ((p.T + tt - 1) / tt + 1) / 2; tp.cluster_merge = merged && nsplit > 1 ? 1 : 0;
     const int units = pair_units(p);
     cudaError_t e;
-    if (p.d == 256) e = (p.early ? launch_pair_t<256, true> : launch_pair_t<256, false>)(m, tp, units, st);
-    else if (p.d == 128) e = (p.early ? launch_pair_t<128, true> : launch_pair_t<128, false>)(m, tp, units, st);
+    if (p.d == 256) e = (nsplit == 1 ? (p.early ? launch_pair_t<256, true, false> : launch_pair_t<256, false, false>) : (p.early ? launch_pair_t<256, true, true> : launch_pair_t<256, false, true>))(m, tp, units, st);
+    else if (p.d == 128) e = (nsplit == 1 ? (p.early ? launch_pair_t<128, true, false> : launch_pair_t<128, false, false>) : (p.early ? launch_pair_t<128, true, true> : launch_pair_t<128, false, true>))(m, tp, units, st);
     else return cudaErrorInvalidValue;
     if (e != cudaSuccess || nsplit == 1 || tp.cluster_merge) return e;
     return launch_attention_merge(p, st);
