@@ -269,11 +269,12 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 float m4[4] = {s[0], s[1], s[2], s[3]};
 #pragma unroll
                 for (int c = 4; c < 28; c += 8) {
-                    m4[0] = max3_f32(m4[0], s[c], s[c + 1]); m4[1] = max3_f32(m4[1], s[c + 2], s[c + 3]);
-                    m4[2] = max3_f32(m4[2], s[c + 4], s[c + 5]); m4[3] = max3_f32(m4[3], s[c + 6], s[c + 7]);
+                    m4[0] = max3_nan_f32(m4[0], s[c], s[c + 1]); m4[1] = max3_nan_f32(m4[1], s[c + 2], s[c + 3]);
+                    m4[2] = max3_nan_f32(m4[2], s[c + 4], s[c + 5]); m4[3] = max3_nan_f32(m4[3], s[c + 6], s[c + 7]);
                 }
-                m4[0] = max3_f32(m4[0], s[28], s[29]); m4[1] = max3_f32(m4[1], s[30], s[31]);
-                mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+                m4[0] = max3_nan_f32(m4[0], s[28], s[29]); m4[1] = max3_nan_f32(m4[1], s[30], s[31]);
+                mx = max_nan_f32(max_nan_f32(m4[0], m4[1]), max_nan_f32(m4[2], m4[3]));
+                if (!(mx < INFINITY)) l = __int_as_float(0x7fc00000);      // a logit that is NaN or +inf makes the row NaN (the polynomial below would lose it)
             }
             // the threads of a row agree on its maximum
             xmax[(buf * kApRows + row) * 4 + half * 2 + part] = mx;
@@ -397,7 +398,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         const int col0 = half * (HD / 2) + part * OC;                  // this thread's first column of O
         if (ns == 1) {
             // O / l through the idle Q buffer, laid out like it, and TMA stores
-            const float inv = ok ? 1.f / l : __int_as_float(0x7fc00000);
+            const float inv = ok && m_ref != -INFINITY ? 1.f / l : __int_as_float(0x7fc00000);      // (NaN too where every logit is -inf)
 #pragma unroll
             for (int c = 0; c < OC / 32; ++c) {
                 float o[32];

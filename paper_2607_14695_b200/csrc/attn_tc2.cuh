@@ -515,14 +515,15 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 float mx4[4] = {s[0], s[1], s[2], s[3]};
 #pragma unroll
                 for (int c = 4; c + 7 < KT; c += 8) {
-                    mx4[0] = max3_f32(mx4[0], s[c], s[c + 1]); mx4[1] = max3_f32(mx4[1], s[c + 2], s[c + 3]);
-                    mx4[2] = max3_f32(mx4[2], s[c + 4], s[c + 5]); mx4[3] = max3_f32(mx4[3], s[c + 6], s[c + 7]);
+                    mx4[0] = max3_nan_f32(mx4[0], s[c], s[c + 1]); mx4[1] = max3_nan_f32(mx4[1], s[c + 2], s[c + 3]);
+                    mx4[2] = max3_nan_f32(mx4[2], s[c + 4], s[c + 5]); mx4[3] = max3_nan_f32(mx4[3], s[c + 6], s[c + 7]);
                 }
                 static_assert((KT - 4) % 8 == 4 || (KT - 4) % 8 == 0, "tail of the maximum loop");
                 if constexpr ((KT - 4) % 8 == 4) {
-                    mx4[0] = max3_f32(mx4[0], s[KT - 4], s[KT - 3]); mx4[1] = max3_f32(mx4[1], s[KT - 2], s[KT - 1]);
+                    mx4[0] = max3_nan_f32(mx4[0], s[KT - 4], s[KT - 3]); mx4[1] = max3_nan_f32(mx4[1], s[KT - 2], s[KT - 1]);
                 }
-                mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+                mx = max_nan_f32(max_nan_f32(mx4[0], mx4[1]), max_nan_f32(mx4[2], mx4[3]));
+                if (!(mx < INFINITY)) l = __int_as_float(0x7fc00000);      // a logit that is NaN or +inf makes the row NaN (the polynomial below would lose it)
                 }
                 // meet the threads that hold the other keys of this row: every one of them publishes its maximum and takes the
                 // largest of the NP published values, so all agree. Past this barrier every thread of the row has its logits
@@ -726,7 +727,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             // and TMA stores: the threads are done once the tile sits in shared memory, and the store drains underneath the
             // next unit. (Stores straight from registers kept every thread until its 64 KB were accepted by a memory system
             // that all clusters hit at the same moment: 4.4 k cycles per unit.)
-            const float inv = 1.f / l;
+            const float inv = m_ref == -INFINITY ? __int_as_float(0x7fc00000) : 1.f / l;      // (NaN where every logit is -inf)
             const bool store_unit = w.t0 < p.T;   // an idle partner tile (odd tile count) has nothing to write
             // Rounds of 64 columns, alternating between the two 16 KB halves of the staging area: the TMA store of one round
             // reads its half while the threads convert the next round into the other (one store of 32 KB per 128 columns made

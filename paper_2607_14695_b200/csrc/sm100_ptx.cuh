@@ -303,9 +303,13 @@ __device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c
 __device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) { uint64_t d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
 __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) { uint64_t d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
 __device__ __forceinline__ float max3_f32(float a, float b, float c) { float d; asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c)); return d; }
+// ... and maxima that are NaN where an argument is
+__device__ __forceinline__ float max3_nan_f32(float a, float b, float c) { float d; asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c)); return d; }
+__device__ __forceinline__ float max_nan_f32(float a, float b) { float d; asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b)); return d; }
 
 // 2^x for a packed pair on the FMA pipe (same scheme as ex2_fma, the arithmetic in f32x2 instructions): arguments are
-// clamped at -125, so anything below gives 2^-125 (2.4e-38) instead of 0; the caller zeroes what must be exactly 0.
+// clamped at -125, so anything below, and a NaN, gives 2^-125 (2.4e-38); the caller zeroes what must be exactly 0 and takes a NaN from
+// the maximum of the arguments (max3_nan_f32).
 struct Ex2PolyConsts { uint64_t magic, neg_magic, neg_one, c3, c2, c1, c0; };
 __device__ __forceinline__ Ex2PolyConsts ex2_poly_consts()
 {

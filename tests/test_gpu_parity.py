@@ -395,6 +395,48 @@ def test_attention_of_a_row_that_is_not_finite(U, case):
         assert torch.equal(out, want), bad
 
 
+NON_FINITE_KEYS = NON_FINITE + [
+    # ... and: one stream in more rows than fit clusters of eight, key halves that end inside a tile, units of 128 rows unsplit, many units
+    (1, 8, 1, 256, 816, 32, 60), (2, 8, 1, 256, 300, 5, 50), (16, 8, 1, 256, 816, 32, 50), (13, 8, 1, 256, 777, 32, 33), (6, 16, 4, 128, 300, 48, 37),
+    (40, 8, 2, 128, 300, 48, 20),
+]
+
+
+@pytest.mark.parametrize("case", NON_FINITE_KEYS, ids=["B%d_h%dkv%d_d%d_S%d_N%d_T%d" % c for c in NON_FINITE_KEYS])
+def test_attention_over_a_key_that_is_not_finite(U, case):
+    """A key that holds a NaN gives NaN in every row that sees it, one that holds an infinity in every row where its logit is +inf, wherever the key
+    lies in a tile; a row whose logits are all -inf is NaN as well (0 / 0). Other streams keep their bits."""
+    rb = U.rb
+    B, Hq, Hkv, d, S, N, T = case
+    G = Hq // Hkv
+    g = torch.Generator(device=U.DEV); g.manual_seed(5)
+    rnd = lambda *s: torch.randn(*s, generator=g, device=U.DEV).to(torch.bfloat16)
+    cache = rb.Cache(1, B, Hq, Hkv, d, S, N, T, rb.DTYPE_BF16, device=U.DEV)
+    ks, vs, kr, vr = rnd(B, 1, S, Hkv, d), rnd(B, 1, S, Hkv, d), rnd(B, 1, N, Hkv, d), rnd(B, 1, N, Hkv, d)
+    q, k, v = rnd(B, T, Hq, d), rnd(B, T, Hkv, d), rnd(B, T, Hkv, d)
+    rb.reflex_cache_append_sliding(cache, list(range(B)), kr, vr)
+
+    def attend(q, ks, k):
+        rb.reflex_cache_init_static(cache, list(range(B)), ks, vs)
+        out = torch.full_like(q, 7.0)
+        rb.reflex_partitioned_attention(cache, 0, q, k, v, out)
+        rb.reflex_cache_check_status(cache)
+        return out
+
+    want = attend(q, ks, k)
+    for key in sorted({0, 1, 2, 5, 7, 8, 15, S // 2, S // 2 + 1, S - 2, S - 1}):
+        for bad in (float("nan"), float("inf")):
+            k2 = ks.clone()
+            k2[B - 1, 0, key, 0, 3] = bad
+            out = attend(q, k2, k)
+            hit = q[B - 1, :, :G, 3] > 0 if bad == float("inf") else torch.ones((T, G), dtype=torch.bool, device=U.DEV)
+            assert torch.isnan(out[B - 1, :, :G][hit]).all(), (key, bad)
+            assert torch.equal(out[:B - 1], want[:B - 1]), (key, bad)
+    big = lambda t, x: t.index_fill(-1, torch.tensor([3], device=U.DEV), x)
+    rb.reflex_cache_append_sliding(cache, list(range(B)), big(kr, 3e38), vr)
+    assert torch.isnan(attend(big(q, -3e38), big(ks, 3e38), big(k, 3e38))).all()
+
+
 def _random_attention_cases(n, seed):
     """Seeded shapes across what the kernels branch on: head_dim, queries per KV head, KV heads, prefix lengths that differ per
     stream (0 included), ring capacity and fill (empty, partly filled, wrapped), dynamic tokens from 1 to beyond one tile."""
