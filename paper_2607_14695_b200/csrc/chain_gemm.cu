@@ -208,8 +208,10 @@ chain_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         const uint32_t idesc = umma_idesc_bf16(FT, 0, false) | ((uint32_t)(p.NT >> 3) << 17);
         int s = 0;
         uint32_t ph = 0, acc = 0;
+        bool ok = true;
         for (int st = 0; st < steps; ++st) {
-            if (!wait(CG_FULL + s, ph, 2)) break;
+            ok = wait(CG_FULL + s, ph, 2);
+            if (!ok) break;
             if (st == 0 && lane == 0) CG_TRACE(3);
             if (st == steps - 1 && lane == 0) CG_TRACE(1);
             tc_fence_after();
@@ -227,7 +229,7 @@ chain_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             if (st + p.stages < steps) umma_commit_elect(bar(CG_EMPTY + s));
             if (++s == p.stages) { s = 0; ph ^= 1u; }
         }
-        umma_commit_elect(bar(CG_ACC));      // also after a wait that ran out: nobody waits for nothing
+        if (ok) umma_commit_elect(bar(CG_ACC));
     } else {
         const int t = threadIdx.x - 64, quarter = warp & 3, group = (warp - 2) >> 2;
         // ---- what finishing needs beside the sums, while the operands are on their way ----

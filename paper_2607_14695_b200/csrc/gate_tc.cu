@@ -151,7 +151,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
                     }
                 }
             }
-            umma_commit_elect(bar_mma);   // also when the load never came: the other warps must not wait for nothing
+            if (ok) umma_commit_elect(bar_mma);   // (when the load never came, the other warps learn of it by their own wait)
         }
         ok = wait(bar_mma, ph, 2) && ok;
         tc_fence_after();

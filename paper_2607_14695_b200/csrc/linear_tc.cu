@@ -263,7 +263,7 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
                 umma2_commit_mc_elect(bar(S::C_EMPTY + s), pair_mask);
                 if (++s == NST) { s = 0; ph ^= 1u; }
             }
-            umma2_commit_mc_elect(bar(S::C_ACC), pair_mask);   // also after a wait that ran out: the epilogue warps must not wait for nothing
+            if (ok) umma2_commit_mc_elect(bar(S::C_ACC), pair_mask);   // (not after a wait that ran out: the other CTA knows of it by its own wait alone)
         }
     } else {
         // ---------------- epilogue: two threads per row, each owns BN / 2 columns ----------------

@@ -284,7 +284,7 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                     umma2_commit_mc_elect(bar(Q_EMPTY + s), (uint16_t)3);
                     if (lane == 0) QK_TRACE(1, ks, 3);
                 }
-                umma2_commit_mc_elect(bar(Q_ACC), (uint16_t)3);   // also after a wait that ran out: the epilogue warps must not wait for nothing
+                if (ok) umma2_commit_mc_elect(bar(Q_ACC), (uint16_t)3);   // (not after a wait that ran out: the other CTA knows of it by its own wait alone)
             }
         }
     } else {
@@ -363,7 +363,7 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         ok = wait(Q_ACC, (uint32_t)it & 1u, 5) && ok;
         if (threadIdx.x == 64) QK_TRACE(2, 31, 1);
         tc_fence_after();
-        const float rs = rsqrtf(ss / (float)p.D + p.eps);
+        const float rs = ok ? rsqrtf(ss / (float)p.D + p.eps) : __int_as_float(0x7fc00000);      // a wait ran out: the tile is marked invalid, not left stale
         if (p.tma_out) {
             // The tile goes out through shared memory and TMA stores. The stage ring is idle now (every load has been consumed and
             // every MMA has completed): accumulator j is staged in the x stages (j = 0) or the weight stages (j = 1) as four
@@ -415,7 +415,7 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                     }
                     fence_proxy_async_smem();
                     asm volatile("bar.sync %0, 128;" ::"r"(2 + half) : "memory");   // the chunk's 128 threads
-                    if (quarter == 0 && lane == 0 && ok && m0 < p.M) {
+                    if (quarter == 0 && lane == 0 && m0 < p.M) {
                         const int n = n0 + j * kQkBN + ch * 64;     // first output column of the chunk (chunks never straddle Q, K and V:
                                                                     // the launcher takes this path only when their widths are multiples of 64)
                         const uint32_t src = base + stage_off + ch * (128 * 128);
@@ -482,7 +482,7 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                 else if (n < p.nq + p.nk) { dst0 = p.k + (n - p.nq); pitch = (size_t)p.nk; }
                 else if (n < n_out) { dst0 = p.v + (n - p.nq - p.nk); pitch = (size_t)p.nk; }
                 const int w8 = warp - 2;                    // 0..7: rows w8, w8 + 8, ...
-                if (ok && dst0) {
+                if (dst0) {
 #pragma unroll 4
                     for (int r = w8; r < kQkBM; r += 8) {
                         if (m0 + r >= p.M) break;
@@ -672,7 +672,7 @@ norm_linear_small_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
             }
             umma_commit_elect(bar(S_EMPTY + s));
         }
-        umma_commit_elect(bar(S_ACC));    // also after a wait that ran out: the epilogue warps must not wait for nothing
+        if (ok) umma_commit_elect(bar(S_ACC));
     } else {
         // ---------------- gate multiply (B operand) and epilogue ----------------
         const int tid = threadIdx.x - 64;              // 0..255
@@ -797,12 +797,12 @@ norm_linear_small_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
                 }
                 continue;
             }
-            if (!ok || f >= n_feat) continue;
+            if (f >= n_feat) continue;
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
                 const int r = c * 32 + i, rg = row0 + r;
                 if (rg < p.M) {                     // (no early exit: the accumulator stays in registers)
-                    const float rs = rsm[r];
+                    const float rs = ok ? rsm[r] : __int_as_float(0x7fc00000);
                     float val = __uint_as_float(acc[i]) * rs;
                     if (swiglu) { const float u = __uint_as_float(up[i]) * rs; val = silu_mul(val, u); }
                     if constexpr (PLAIN) { if (p.res) val += __bfloat162float(p.res[(size_t)rg * pitch + f]); }

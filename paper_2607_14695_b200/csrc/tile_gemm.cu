@@ -195,7 +195,7 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
                     umma2_commit_mc_elect(bar(S::T_EMPTY + s), (uint16_t)3);
                     if (++s == NST) { s = 0; ph ^= 1u; }
                 }
-                umma2_commit_mc_elect(bar(S::T_ACC + buf), (uint16_t)3);   // also after a wait that ran out: the epilogue must not wait for nothing
+                if (ok) umma2_commit_mc_elect(bar(S::T_ACC + buf), (uint16_t)3);   // (not after a wait that ran out: the other CTA knows of it by its own wait alone)
             }
         }
     } else if constexpr (BM == 64) {
@@ -226,8 +226,9 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
                     for (int j = 0; j < p.slots; ++j) ss += src[j];
                 }
             }
-            const float rs = rsqrtf(ss * p.inv_D + p.eps);
+            float rs = rsqrtf(ss * p.inv_D + p.eps);
             ok = wait(S::T_ACC + buf, (uint32_t)(it >> 1) & 1u, 4) && ok;
+            if (!ok) rs = __int_as_float(0x7fc00000);      // a wait ran out: the tile is marked invalid, not left stale
             tc_fence_after();
             uint32_t acc[CPT];
             if constexpr (CPT == 32) tmem_ld32(taddr + buf * BN, acc);
@@ -267,7 +268,7 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
             meet();
             if (issuer) {
                 const int n = n0 + ch * 64;
-                if (ok && m0 < p.M) {
+                if (m0 < p.M) {
                     if constexpr (SWIGLU) {
                         if (n < p.F) tg_tma_store_2d(&tm_q, base + stage_off, n, m0);
                     } else {              // (the widths are multiples of 64: a chunk lies in one tensor)
@@ -305,8 +306,9 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
                     for (int j = 0; j < p.slots; ++j) ss += src[j];
                 }
             }
-            const float rs = rsqrtf(ss * p.inv_D + p.eps);
+            float rs = rsqrtf(ss * p.inv_D + p.eps);
             ok = wait(S::T_ACC + buf, (uint32_t)(it >> 1) & 1u, 4) && ok;
+            if (!ok) rs = __int_as_float(0x7fc00000);      // a wait ran out: the tile is marked invalid, not left stale
             tc_fence_after();
 #pragma unroll
             for (int cc = 0; cc < CPT; ++cc) {
@@ -357,7 +359,7 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
                 else asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
                 if (issuer) {
                     const int n = n0 + ch * 64;
-                    if (ok && m0 < p.M) {
+                    if (m0 < p.M) {
                         if constexpr (SWIGLU) {
                             if (n < p.F) tg_tma_store_2d(&tm_q, base + stage_off, n, m0);
                         } else {              // (the widths are multiples of 64: a chunk lies in one tensor)

@@ -47,3 +47,23 @@ def test_inputs_read_behind_the_wait_may_not_be_taken_for_constants(kernel):
     _, params, _ = kernel
     bad = re.findall(r"const [^,]*__restrict__ (\w+)", params)
     assert not [b for b in bad if not ("wait_prior" in params and b in ("W", "bias"))], bad
+
+
+PROJECTIONS = [k for k in KERNELS if k[0].split(":")[0] in ("tile_gemm.cu", "linear_half.cu", "linear_tc.cu", "qkv_tc.cu", "chain_gemm.cu", "gate_tc.cu") and "commit" in k[2]]
+
+
+@pytest.mark.parametrize("kernel", PROJECTIONS, ids=lambda k: k[0])
+def test_sums_are_announced_only_when_complete(kernel):
+    """After a wait that ran out a contraction is not complete. The warps that read the accumulator (in a pair those of the other CTA, which sees nothing
+    of the failed wait) may take it for complete only by the barrier that the last commit arrives on: no commit, no result but NaN."""
+    commits = re.findall(r"([^;{}]*)\bumma2?_commit\w*\(bar\w*(?:\((?:S::)?(\w+))?", kernel[2])
+    last = [before for before, name in commits if name.endswith("_ACC") or not name]
+    assert last and all(re.search(r"if \(ok\)\s*$", b) for b in last), last
+
+
+@pytest.mark.parametrize("kernel", PROJECTIONS, ids=lambda k: k[0])
+def test_a_tile_of_a_failed_wait_is_written_as_nan(kernel):
+    """A store that is left out keeps what the last call wrote: the result is written whatever the waits said, and is NaN where one ran out."""
+    _, _, body = kernel
+    assert "0x7fc00000" in body
+    assert not re.search(r"if \([^()]*\bok && (?:m0|dst)|if \(!ok \|\| f >=", body)
