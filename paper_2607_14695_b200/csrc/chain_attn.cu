@@ -1,15 +1,15 @@
-// Partitioned attention (Eq. 1) for one stream, or two of few tokens: one launch, keys split over the eight CTAs of a cluster.
+// Partitioned attention (Eq. 1) for one or two streams: one launch, keys split over the eight CTAs of a cluster.
 //
 // What bounds a single stream is latency: 368 MFLOP and 0.9 MB of K/V per layer, spread over the chip, are a microsecond of work
 // in a chain of dependent steps. The batched kernel's key split needs a second launch and 64-128 KB of fp32 partials per CTA through
 // global memory: 12.4 us per layer inside an expert step (898 keys, 50 tokens, 8 heads). This kernel takes about 8.
-//   - A CTA owns 32 query rows -- (token, head of the group) pairs -- and one of eight slices of the keys, at most 128, so that its
+//   - A CTA owns 32 (64) query rows -- (token, head of the group) pairs -- and one of eight slices of the keys, at most 128, so that its
 //     partial O is 32 x 256 and goes to its seven peers through distributed shared memory.
 //   - Seven slices divide the static prefix, the eighth holds ring slots and dynamic tokens. Static and ring keys are asked for before
 //     the wait for the preceding kernel when the caller vouches for them (early: nothing in an expert step writes cache regions);
 //     only Q and the dynamic tokens come after it.
 //   - S = Q K^T with M = 64 (rows in lanes 0-15 of every lane quarter), read as 16x256b fragments: a thread holds two rows and the
-//     row maximum is two shuffles. The two warps of a lane quarter take 64 keys each.
+//     row maximum is two shuffles. With 32 rows the two warps of a lane quarter take 64 keys each.
 //   - O^T = V^T P^T with the head dimension as M (V as the MN-major A operand): a thread holds one column of O for all rows, so that
 //     four rows of it are one 16-byte st.async and a warp's store is 512 contiguous bytes of the owner's inbox. CTA r of the cluster
 //     owns an eighth of the rows: it receives the slices' unnormalised O and (m, l), counted on one mbarrier, and writes the merged
@@ -38,21 +38,20 @@ constexpr int kCaThreads = 64 + 256;
 constexpr int kCaHD = 256;
 constexpr unsigned long long kCaWaitNs = 1000000000ull;
 
-constexpr int kCaRows = 32;                // query rows -- (token, head of the KV head's group) pairs -- of a CTA at most
-
-struct CaSmem {
-    static constexpr int OWN = kCaRows / kCaSlices;                 // rows a CTA of the cluster merges: one quad
-    static constexpr uint32_t Q_CHUNK = kCaRows * 128;
-    static constexpr uint32_t Q = 0;                             // 4 chunks of [kCaRows][128 B] (the MMA reads kCaM rows: the rest is whatever follows)
-    static constexpr uint32_t K = Q + 4 * Q_CHUNK;               // 4 chunks of [128 keys][128 B]; later the inbox [8 slices][256][4] fp32
+// ROWS: query rows -- (token, head of the KV head's group) pairs -- of a CTA at most, 32 or 64
+template <int ROWS> struct CaSmem {
+    static constexpr int OWN = ROWS / kCaSlices;                 // rows a CTA of the cluster merges: one or two quads
+    static constexpr uint32_t Q_CHUNK = ROWS * 128;
+    static constexpr uint32_t Q = 0;                             // 4 chunks of [ROWS][128 B] (the MMA reads kCaM rows: the rest is whatever follows)
+    static constexpr uint32_t K = Q + 4 * Q_CHUNK;               // 4 chunks of [128 keys][128 B]; later the inbox [8 slices][OWN / 4 quads][256][4] fp32
     static constexpr uint32_t V = K + 4 * kCaKeys * 128;
-    static constexpr uint32_t P = V + 4 * kCaKeys * 128;         // 2 chunks of [kCaRows][64 keys]
-    static constexpr uint32_t MX = P + 2 * kCaRows * 128;           // [2 key halves][32 rows] row maxima
+    static constexpr uint32_t P = V + 4 * kCaKeys * 128;         // 2 chunks of [ROWS][64 keys]
+    static constexpr uint32_t MX = P + 2 * ROWS * 128;           // [2 key halves][32 rows] row maxima
     static constexpr uint32_t ML = MX + 256;                     // [8 slices][OWN] (m, l, l of the second key half, -)
     static constexpr uint32_t WGT = ML + kCaSlices * OWN * 16;   // [8 slices][OWN] weights of the merge
     static constexpr uint32_t BAR = WGT + kCaSlices * OWN * 4;
     static constexpr uint32_t TOTAL = BAR + 128 + 1024;
-    static_assert(OWN == 4 && kCaSlices * kCaHD * 16 <= 4 * kCaKeys * 128, "inbox fits in the K tile");
+    static_assert(kCaSlices * (OWN / 4) * kCaHD * 16 <= 4 * kCaKeys * 128, "inbox fits in the K tile");
     static_assert(TOTAL <= 227u * 1024u, "shared memory budget");
 };
 enum { CB_Q = 0, CB_K, CB_V, CB_S, CB_VREADY, CB_P, CB_O, CB_FREE, CB_INBOX, CB_COUNT };
@@ -73,7 +72,7 @@ struct CaParams {
     int dyn_row;         // tile row of the first dynamic token in the last slice
     int early;
     int g_log2;
-    int units, tt;       // tiles of a stream and KV head; tokens of a tile: kCaRows / G
+    int units, tt;       // tiles of a stream and KV head; tokens of a tile: ROWS / G
     float scale_log2;
     ChainPrefetch pf;
 };
@@ -100,13 +99,14 @@ __device__ __forceinline__ uint64_t ca_bits(int lo, int hi)
     return (hi >= 64 ? ~0ull : (1ull << hi) - 1ull) & ~((1ull << lo) - 1ull);
 }
 
+template <int ROWS>
 __global__ void __cluster_dims__(kCaSlices, 1, 1) __launch_bounds__(kCaThreads, 1)
 chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_ks, const __grid_constant__ CUtensorMap tm_vs,
                   const __grid_constant__ CUtensorMap tm_kr, const __grid_constant__ CUtensorMap tm_vr, const __grid_constant__ CUtensorMap tm_kd,
                   const __grid_constant__ CUtensorMap tm_vd, const CaParams p)
 {
-    using L = CaSmem;
-    constexpr int OWN = L::OWN;
+    using L = CaSmem<ROWS>;
+    constexpr int OWN = L::OWN, QUADS = OWN / 4;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t base = (raw_addr + 1023u) & ~1023u;
@@ -129,7 +129,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             for (int i = 0; i < CB_COUNT; ++i) mbar_init(bar(i), i == CB_VREADY || i == CB_P ? 4u : i == CB_FREE ? (uint32_t)kCaSlices : 1u);
             *abort_flag = 0u;
             fence_mbar_init();
-            mbar_expect_tx(bar(CB_INBOX), (uint32_t)(kCaSlices * (((own + 3) / 4) * kCaHD * 16 + own * 12)));
+            mbar_expect_tx(bar(CB_INBOX), (uint32_t)(kCaSlices * (((own + 3) / 4) * kCaHD * 16 + own * (ROWS == 64 ? 8 : 12))));
         }
         __syncwarp();
         cluster_arrive();
@@ -203,7 +203,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     auto wait_cl = [&](int i, uint32_t code) -> bool { return mbar_try_wait_cluster(bar(i), 0) || wait_slow(i, code); };
 
     if (warp == 0) {
-        mbar_expect_tx_elect(bar(CB_Q), kCaRows * kCaHD * 2);
+        mbar_expect_tx_elect(bar(CB_Q), ROWS * kCaHD * 2);
         for (int c = 0; c < 4; ++c) tma_load_4d_elect(base + L::Q + c * L::Q_CHUNK, &tm_q, bar(CB_Q), c * 64, hkv * p.G, t0, b);
         if (last) {
             for (int c = 0; c < 4; ++c) tma_load_3d_elect(base + L::K + c * (kCaKeys * 128) + p.dyn_row * 128, &tm_kd, bar(CB_K), c * 64, hkv, b * p.T);
@@ -220,7 +220,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         chain_prefetch(p.pf, blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y, lane);
     } else if (warp == 1) {
         constexpr uint32_t idesc_qk = umma_idesc_bf16(kCaM, kCaKeys, false);
-        constexpr uint32_t idesc_pv = umma_idesc_bf16(128, kCaRows, false) | (1u << 15);     // A is MN-major
+        constexpr uint32_t idesc_pv = umma_idesc_bf16(128, ROWS, false) | (1u << 15);     // A is MN-major
         bool ok = wait(CB_K, 2) && wait(CB_Q, 3);
         if (lane == 0) CA_TRACE(2);
         if (ok && ext > 0) {
@@ -243,10 +243,10 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             tc_fence_after();
             const int steps = (ext + 15) / 16;
             for (int kk = 0; kk < steps; ++kk) {
-                const uint64_t bd = umma_desc_sw128(base + L::P + (kk >> 2) * (kCaRows * 128) + (kk & 3) * 32, 16, 1024);
+                const uint64_t bd = umma_desc_sw128(base + L::P + (kk >> 2) * (ROWS * 128) + (kk & 3) * 32, 16, 1024);
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
-                    umma_ss_elect(tmem + 128 + h * kCaRows, umma_desc_sw128(base + L::V + h * (2 * kCaKeys * 128) + kk * (16 * 128), kCaKeys * 128, 1024), bd, idesc_pv,
+                    umma_ss_elect(tmem + 128 + h * ROWS, umma_desc_sw128(base + L::V + h * (2 * kCaKeys * 128) + kk * (16 * 128), kCaKeys * 128, 1024), bd, idesc_pv,
                                   kk > 0 ? 1u : 0u);
             }
         }
@@ -254,14 +254,15 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     } else {
         const int t = threadIdx.x - 64, quarter = warp & 3, group = (warp - 2) >> 2;
         bool ok = true;
-        // Four warps run the softmax, the other four clear V. The rows sit in lane quarters 0 and 1; the two warps of a quarter take 64 keys each.
-        const bool softmax = quarter < 2;
+        // Four warps run the softmax, the other four clear V. 64 rows: warps of group 0, one lane quarter (16 rows) each, all 128
+        // keys. 32 rows: they sit in lane quarters 0 and 1; the two warps of a quarter take 64 keys each.
+        const bool softmax = ROWS == 64 ? group == 0 : quarter < 2;
         if (!softmax) {
             // V rows inside the contraction that hold no key: zero, so that weight 0 meets no stale NaN
             ok = wait(CB_V, 6);
             const int ext16 = (ext + 15) & ~15;
             uint64_t dead[2] = {~live_lo & ca_bits(0, ext16), ~live_hi & ca_bits(0, ext16 - 64)};
-            const int chunk = (quarter & 1) + 2 * group;
+            const int chunk = ROWS == 64 ? quarter : (quarter & 1) + 2 * group;
             uint8_t *v = smem + L::V + chunk * (kCaKeys * 128) + lane * 4;
 #pragma unroll
             for (int w = 0; w < 2; ++w)
@@ -274,31 +275,41 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(CB_VREADY));
         } else {
+            constexpr int NW = ROWS == 64 ? 2 : 1;      // 64-key halves per warp
+            const int w0 = ROWS == 64 ? 0 : group;
             ok = wait(CB_S, 7);
-            if (threadIdx.x == 128) CA_TRACE(3);
+            if (threadIdx.x == 64 + (ROWS == 64 ? 0 : 64)) CA_TRACE(3);
             tc_fence_after();
-            uint32_t s[32];
-            ca_tmem_ld_16x256b(tmem + ((uint32_t)(quarter * 32) << 16) + group * 64, s);
+            uint32_t s[NW][32];
+            const uint32_t addr = tmem + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll
+            for (int w = 0; w < NW; ++w) ca_tmem_ld_16x256b(addr + (w0 + w) * 64, s[w]);
             tmem_wait_ld();
-            const uint64_t live = group == 0 ? live_lo : live_hi;
-            if (live != ~0ull) {
-                const uint64_t ml = live >> (2 * (lane & 3));      // bit 8 g + j: this thread's column j of group g
+            const uint64_t full = ~0ull;
+            if (live_lo != full || live_hi != full) {
+                const int sh = 2 * (lane & 3);
 #pragma unroll
-                for (int g = 0; g < 8; ++g)
+                for (int w = 0; w < NW; ++w) {
+                    const uint64_t ml = (w0 + w == 0 ? live_lo : live_hi) >> sh;      // bit 8 g + j: this thread's column j of group g
 #pragma unroll
-                    for (int j = 0; j < 2; ++j)
-                        if (!((ml >> (8 * g + j)) & 1ull)) { s[4 * g + j] = 0xff800000u; s[4 * g + 2 + j] = 0xff800000u; }
+                    for (int g = 0; g < 8; ++g)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j)
+                            if (!((ml >> (8 * g + j)) & 1ull)) { s[w][4 * g + j] = 0xff800000u; s[w][4 * g + 2 + j] = 0xff800000u; }
+                }
             }
             float mrow[2];                            // the thread's two rows
 #pragma unroll
             for (int hr = 0; hr < 2; ++hr) {
                 float m = -INFINITY;
 #pragma unroll
-                for (int g = 0; g < 8; ++g) m = max3_f32(m, __uint_as_float(s[4 * g + 2 * hr]), __uint_as_float(s[4 * g + 2 * hr + 1]));
+                for (int w = 0; w < NW; ++w)
+#pragma unroll
+                    for (int g = 0; g < 8; ++g) m = max3_f32(m, __uint_as_float(s[w][4 * g + 2 * hr]), __uint_as_float(s[w][4 * g + 2 * hr + 1]));
                 m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
                 mrow[hr] = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
             }
-            {
+            if constexpr (ROWS == 32) {
                 // the row's maximum over both halves of the keys
                 float *mx = reinterpret_cast<float *>(smem + L::MX);
                 const int r = quarter * 16 + (lane >> 2);
@@ -312,21 +323,23 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 const float m = mrow[hr];
                 const float ref = m == -INFINITY ? 0.f : -m * p.scale_log2;
                 const int row = quarter * 16 + hr * 8 + (lane >> 2);
-                uint8_t *pr = smem + L::P + group * (kCaRows * 128) + row * 128 + (lane & 3) * 4;
+                uint8_t *pr = smem + L::P + w0 * (ROWS * 128) + row * 128 + (lane & 3) * 4;
                 float l = 0.f;
 #pragma unroll
-                for (int g = 0; g < 8; ++g) {
-                    const float p0 = ex2(fmaf(__uint_as_float(s[4 * g + 2 * hr]), p.scale_log2, ref));
-                    const float p1 = ex2(fmaf(__uint_as_float(s[4 * g + 2 * hr + 1]), p.scale_log2, ref));
-                    l += p0 + p1;
-                    __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1);
-                    *reinterpret_cast<uint32_t *>(pr + ((g ^ (row & 7)) << 4)) = *reinterpret_cast<uint32_t *>(&pp);
-                }
+                for (int w = 0; w < NW; ++w)
+#pragma unroll
+                    for (int g = 0; g < 8; ++g) {
+                        const float p0 = ex2(fmaf(__uint_as_float(s[w][4 * g + 2 * hr]), p.scale_log2, ref));
+                        const float p1 = ex2(fmaf(__uint_as_float(s[w][4 * g + 2 * hr + 1]), p.scale_log2, ref));
+                        l += p0 + p1;
+                        __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1);
+                        *reinterpret_cast<uint32_t *>(pr + w * (ROWS * 128) + ((g ^ (row & 7)) << 4)) = *reinterpret_cast<uint32_t *>(&pp);
+                    }
                 l += __shfl_xor_sync(0xffffffffu, l, 1);
                 l += __shfl_xor_sync(0xffffffffu, l, 2);
                 if ((lane & 3) == 0 && row < rows) {
                     const uint32_t o = (uint32_t)(row / OWN), dst = mapa(base + L::ML + (uint32_t)(slice * OWN + row % OWN) * 16u, o), ib = mapa(bar(CB_INBOX), o);
-                    if (group == 0) st_async_v2(dst, ib, __float_as_uint(m * p.scale_log2), __float_as_uint(l));
+                    if (ROWS == 64 || group == 0) st_async_v2(dst, ib, __float_as_uint(m * p.scale_log2), __float_as_uint(l));
                     else st_async_b32(dst + 8u, ib, __float_as_uint(l));
                 }
             }
@@ -334,7 +347,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(CB_P));
-            if (threadIdx.x == 128) CA_TRACE(4);
+            if (threadIdx.x == 64 + (ROWS == 64 ? 0 : 64)) CA_TRACE(4);
         }
         // ---- partial O^T to the owners of the rows ----
         ok = wait(CB_O, 8) && ok;
@@ -342,18 +355,27 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         tc_fence_after();
         const int d = group * 128 + quarter * 32 + lane;
         if (wait_cl(CB_FREE, 9)) {
-            uint32_t acc[32];
-            tmem_ld32(tmem + 128 + group * kCaRows + ((uint32_t)(quarter * 32) << 16), acc);
-            tmem_wait_ld();
-            if (!ok || ext == 0) {
 #pragma unroll
-                for (int i = 0; i < 32; ++i) acc[i] = ok ? 0u : 0x7fc00000u;
+            for (int c = 0; c < ROWS / 32; ++c) {
+                if (c * 32 < rows) {
+                    uint32_t acc[32];
+                    tmem_ld32(tmem + 128 + group * ROWS + ((uint32_t)(quarter * 32) << 16) + c * 32, acc);
+                    tmem_wait_ld();
+                    if (!ok || ext == 0) {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) acc[i] = ok ? 0u : 0x7fc00000u;
+                    }
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const int quad = c * 8 + q;
+                        if (quad * 4 < rows) {
+                            const uint32_t o = (uint32_t)(quad / QUADS);
+                            st_async_v4(mapa(base + L::K + (uint32_t)((slice * QUADS + quad % QUADS) * kCaHD + d) * 16u, o), mapa(bar(CB_INBOX), o), acc[4 * q], acc[4 * q + 1],
+                                           acc[4 * q + 2], acc[4 * q + 3]);
+                        }
+                    }
+                }
             }
-#pragma unroll
-            for (int q = 0; q < 8; ++q)                  // (a CTA of the cluster merges one quad of rows)
-                if (q * 4 < rows)
-                    st_async_v4(mapa(base + L::K + (uint32_t)(slice * kCaHD + d) * 16u, (uint32_t)q), mapa(bar(CB_INBOX), (uint32_t)q), acc[4 * q], acc[4 * q + 1], acc[4 * q + 2],
-                                acc[4 * q + 3]);
         }
         if (threadIdx.x == 64) CA_TRACE(6);
         tc_fence_before();
@@ -368,24 +390,29 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 float m = v.x;
                 for (int o = 1; o < 8; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
                 const float w = v.x == -INFINITY ? 0.f : ex2(v.x - m);
-                float l = w * (v.y + v.z);
+                float l = w * (ROWS == 64 ? v.y : v.y + v.z);
                 for (int o = 1; o < 8; o <<= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
                 wgt[q * OWN + r] = w / l;
             }
             asm volatile("bar.sync 1, 256;" ::: "memory");
             const float4 *in = reinterpret_cast<const float4 *>(smem + L::K);
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int q = 0; q < kCaSlices; ++q) {
-                const float4 v = in[q * kCaHD + t];
-                const float4 w = *reinterpret_cast<const float4 *>(wgt + q * OWN);
-                a.x = fmaf(v.x, w.x, a.x); a.y = fmaf(v.y, w.y, a.y); a.z = fmaf(v.z, w.z, a.z); a.w = fmaf(v.w, w.w, a.w);
-            }
-            const float o[4] = {a.x, a.y, a.z, a.w};
+            for (int q2 = 0; q2 < QUADS; ++q2) {
+                if (q2 * 4 < own) {
+                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int r = slice * OWN + i, tk = r >> p.g_log2;
-                if (i < own) p.out[((size_t)(b * p.T + t0 + tk) * p.Hq + hkv * p.G + (r - (tk << p.g_log2))) * kCaHD + t] = __float2bfloat16_rn(ok ? o[i] : __int_as_float(0x7fc00000));
+                    for (int q = 0; q < kCaSlices; ++q) {
+                        const float4 v = in[(q * QUADS + q2) * kCaHD + t];
+                        const float4 w = *reinterpret_cast<const float4 *>(wgt + q * OWN + q2 * 4);
+                        a.x = fmaf(v.x, w.x, a.x); a.y = fmaf(v.y, w.y, a.y); a.z = fmaf(v.z, w.z, a.z); a.w = fmaf(v.w, w.w, a.w);
+                    }
+                    const float o[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int r = slice * OWN + q2 * 4 + i, tk = r >> p.g_log2;
+                        if (q2 * 4 + i < own) p.out[((size_t)(b * p.T + t0 + tk) * p.Hq + hkv * p.G + (r - (tk << p.g_log2))) * kCaHD + t] = __float2bfloat16_rn(ok ? o[i] : __int_as_float(0x7fc00000));
+                    }
+                }
             }
         }
     }
@@ -403,7 +430,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     if (threadIdx.x == 0) CA_TRACE(9);
 }
 
-// ---- groups of 128 heads: 128 rows per CTA, two tiles of keys, clusters of four --------------------------------------------------
+// ---- a few streams: 128 rows per CTA, two tiles of keys, clusters of four --------------------------------------------------
 // The same scheme for more row tiles than clusters of eight fit the device (it holds 33 clusters of four at once): a CTA owns 128 query
 // rows and a quarter of the keys as two tiles of at most 128. Both tiles' logits fit tensor memory beside O (2 x 128 + 256 columns), so
 // the softmax needs no running rescale; P goes back over the logits it came from and is the A operand of P V from there. Shared
@@ -759,14 +786,24 @@ chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 
 }  // namespace
 
-// Rows of a CTA: 32 while the clusters of eight fit the device at once (it holds 15: they need their SMs in one GPC; a cluster too many starts when
-// another has finished). More rows go to the pairs of CTAs of attn_pair.cuh: 64 rows here took 10.6 us for two streams x 898 keys where those take 8.8,
-// clusters of four with 128 rows 13.7 to 15.4 for 4 to 8 streams where those take 10.6 to 11.4. The latter are left with what those do not
-// take, groups of 128 heads, inside a step.
+// Rows of a CTA: 32 while the clusters of eight fit the device at once, else 64 where the call stands by itself (0: too many streams). What a CTA
+// sends through distributed shared memory is 1 KB per row at some 20 bytes per cycle. The device holds 15 clusters of eight (they need their SMs in
+// one GPC); a cluster too many starts when another has finished.
+// 64 rows would be faster as units of 128 (attn_pair.cuh): two streams x 382 keys 8.1 us against 10.6 here, x 898 keys 9.1 against 11.3. But the key
+// that sets a slice's reference has weight 1, which bf16 holds exactly, and those have fewer slices and references than the eight here: 382 keys are
+// 2.14e-3 from 64 bits there and 2.07e-3 here, 296 keys 2.26e-3 and 2.05e-3, 898 keys 2.13e-3 in both. Inside a step that distance does not
+// show (layer output 3.46e-3 from 64 bits with either), so the units of 128 rows take it.
 static int chain_attn_rows(const AttnParams &p, bool early)
 {
     const int G = p.Hq / p.Hkv;
-    if (32 % G == 0 && (long long)p.B * p.Hkv * ((p.T + 32 / G - 1) / (32 / G)) <= 14) return 32;
+    for (int rows = 32; rows <= (early ? 32 : 64); rows *= 2) {
+        if (rows % G != 0) continue;
+        // On few keys the exchange of 64 rows costs more than the keys that the slices save (2 x 32 tokens x 112 keys 10.5 us, 8.8 by one CTA
+        // per tile; 66 keys 9.3 and 8.0; from 313 keys on 0.92 to 1.02 of it; of 32 rows 0.6 to 1.0 everywhere).
+        if (rows == 64 && p.S_max + p.N + p.T < 288) continue;
+        const int tt = rows / G;
+        if ((long long)p.B * p.Hkv * ((p.T + tt - 1) / tt) <= 14) return rows;
+    }
     return early && G == kC4Rows && (long long)p.B * p.Hkv * p.T <= 32 ? kC4Rows : 0;
 }
 
@@ -817,10 +854,10 @@ cudaError_t launch_chain_attn(const AttnParams &a, uint32_t *status, bool early,
     p.units = (a.T + tt - 1) / tt; p.tt = tt;
     p.scale_log2 = a.scale * 1.4426950408889634f;
     p.pf = pf ? *pf : ChainPrefetch{};
-    static std::atomic<unsigned long long> set32{0}, set128{0};
+    static std::atomic<unsigned long long> set32{0}, set64{0}, set128{0};
     const dim3 grid((unsigned)((tile == kC4Rows ? kC4Slices : kCaSlices) * a.Hkv * p.units), (unsigned)a.B);
     if (tile == kC4Rows) return launch_rows(chain_attn128_kernel, C4Smem::TOTAL, set128, m, p, grid, st);
-    return launch_rows(chain_attn_kernel, CaSmem::TOTAL, set32, m, p, grid, st);
+    return tile == 32 ? launch_rows(chain_attn_kernel<32>, CaSmem<32>::TOTAL, set32, m, p, grid, st) : launch_rows(chain_attn_kernel<64>, CaSmem<64>::TOTAL, set64, m, p, grid, st);
 }
 
 }  // namespace reflex

@@ -437,6 +437,29 @@ def test_attention_over_a_key_that_is_not_finite(U, case):
     assert torch.isnan(attend(big(q, -3e38), big(ks, 3e38), big(k, 3e38))).all()
 
 
+@pytest.mark.parametrize("B,T,S,most", [(1, 57, 200, 2.08e-3), (2, 50, 300, 2.10e-3), (1, 64, 400, 2.12e-3), (2, 32, 500, 2.13e-3)])
+def test_attention_of_few_streams_keeps_a_reference_per_eighth_of_the_keys(U, B, T, S, most):
+    """The key that sets the reference maximum has weight 1, which bf16 holds exactly. With eight slices of the keys, each with its own reference, these
+    calls are 2.05e-3, 2.07e-3, 2.10e-3 and 2.11e-3 from 64 bits (2-norms), with one to five references 2.26e-3, 2.14e-3, 2.14e-3 and 2.15e-3. The bounds
+    lie 1 % above the former: over 100,000 outputs the inputs change the distance by less than 0.2 %."""
+    rb, Hq, d, N = U.rb, 8, 256, 32
+    off = []
+    for seed in range(4):
+        g = torch.Generator(device=U.DEV); g.manual_seed(seed)
+        rnd = lambda *s: torch.randn(*s, generator=g, device=U.DEV).to(torch.bfloat16)
+        cache = rb.Cache(1, B, Hq, 1, d, S, N, T, rb.DTYPE_BF16, device=U.DEV)
+        ks, vs, kn, vn = rnd(B, 1, S, 1, d), rnd(B, 1, S, 1, d), rnd(B, 1, N, 1, d), rnd(B, 1, N, 1, d)
+        rb.reflex_cache_init_static(cache, list(range(B)), ks, vs)
+        rb.reflex_cache_append_sliding(cache, list(range(B)), kn, vn)
+        q, k, v = rnd(B, T, Hq, d), rnd(B, T, 1, d), rnd(B, T, 1, d)
+        K, V = (torch.cat([x[:, 0, :, 0], y[:, 0, :, 0], z[:, :, 0]], 1).double() for x, y, z in ((ks, kn, k), (vs, vn, v)))
+        want = torch.softmax(torch.einsum("bthd,bsd->bhts", q.double(), K) / d ** 0.5, -1) @ V[:, None]
+        out = torch.empty_like(q)
+        rb.reflex_partitioned_attention(cache, 0, q, k, v, out)
+        off.append(((out.double() - want.transpose(1, 2)).norm() / want.norm()).item())
+    assert sum(off) / len(off) <= most, off
+
+
 def _random_attention_cases(n, seed):
     """Seeded shapes across what the kernels branch on: head_dim, queries per KV head, KV heads, prefix lengths that differ per
     stream (0 included), ring capacity and fill (empty, partly filled, wrapped), dynamic tokens from 1 to beyond one tile."""
