@@ -430,360 +430,6 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     if (threadIdx.x == 0) CA_TRACE(9);
 }
 
-// ---- a few streams: 128 rows per CTA, two tiles of keys, clusters of four --------------------------------------------------
-// The same scheme for more row tiles than clusters of eight fit the device (it holds 33 clusters of four at once): a CTA owns 128 query
-// rows and a quarter of the keys as two tiles of at most 128. Both tiles' logits fit tensor memory beside O (2 x 128 + 256 columns), so
-// the softmax needs no running rescale; P goes back over the logits it came from and is the A operand of P V from there. Shared
-// memory is used twice: V's tiles land where K's were once their Q K^T is complete, and the peers' partial results over V when the own
-// P V is complete. O is not transposed here (with V^T as an MN-major A operand an MMA took 135 cycles instead of 64): CTA r of the cluster merges columns [64 r, 64 r + 64) of all rows, so
-// that a warp still sends 512 contiguous bytes. The exchange, 96 KB a CTA at some 18 bytes per cycle, is the longest part.
-constexpr int kC4Slices = 4, kC4Rows = 128, kC4Cols = kCaHD / kC4Slices;
-struct C4Smem {
-    static constexpr uint32_t QP = 0;                                  // Q: 4 chunks of [128 rows][128 B]
-    static constexpr uint32_t KV = 4 * kC4Rows * 128;                  // two tiles of 4 chunks [128 keys][128 B]; later the inbox [4 slices][16 column quads][128 rows][4] fp32
-    static constexpr uint32_t TILE = 4 * kCaKeys * 128;
-    static constexpr uint32_t MX = KV + 2 * TILE;                      // [2 tiles][128 rows] row maxima
-    static constexpr uint32_t ML = MX + 2 * kC4Rows * 4;               // [4 slices][128 rows] (m, l of tile 0, l of tile 1, -)
-    static constexpr uint32_t BAR = ML + kC4Slices * kC4Rows * 16;
-    static constexpr uint32_t TOTAL = BAR + 160 + 1024;
-    static_assert(kC4Slices * (kC4Cols / 4) * kC4Rows * 16 <= 2 * TILE, "inbox fits over the V tiles");
-    static_assert(TOTAL <= 227u * 1024u, "shared memory budget");
-};
-enum { C4_Q = 0, C4_K, C4_V = C4_K + 2, C4_S = C4_V + 2, C4_VREADY = C4_S + 2, C4_P, C4_O, C4_FREE, C4_INBOX, C4_COUNT };
-
-__global__ void __cluster_dims__(kC4Slices, 1, 1) __launch_bounds__(kCaThreads, 1)
-chain_attn128_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_ks, const __grid_constant__ CUtensorMap tm_vs,
-                     const __grid_constant__ CUtensorMap tm_kr, const __grid_constant__ CUtensorMap tm_vr, const __grid_constant__ CUtensorMap tm_kd,
-                     const __grid_constant__ CUtensorMap tm_vd, const CaParams p)
-{
-    using L = C4Smem;
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t raw_addr = smem_u32(smem_raw);
-    const uint32_t base = (raw_addr + 1023u) & ~1023u;
-    uint8_t *smem = smem_raw + (base - raw_addr);
-    auto bar = [&](int i) -> uint32_t { return base + L::BAR + 8u * (uint32_t)i; };
-    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + L::BAR + 8 * C4_COUNT);
-    volatile uint32_t *abort_flag = tmem_slot + 1;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int slice = (int)cluster_ctarank();
-    const int unit = blockIdx.x >> 2, b = blockIdx.y;
-    const int hkv = p.Hkv == 1 ? 0 : unit / p.units, t0 = (unit - hkv * p.units) * p.tt;   // KV head, first token
-    const int rows = min(p.tt, p.T - t0) * p.G;                      // query rows of this CTA: (token, head in group)
-    const bool last = slice == kC4Slices - 1;                        // its second tile: ring and dynamic tokens
-
-    if (warp == 0) {
-        if (lane == 0) {
-            for (int i = 0; i < C4_COUNT; ++i) mbar_init(bar(i), i == C4_VREADY || i == C4_P ? 8u : i == C4_FREE ? (uint32_t)kC4Slices : 1u);
-            *abort_flag = 0u;
-            fence_mbar_init();
-            mbar_expect_tx(bar(C4_INBOX), (uint32_t)(kC4Slices * rows * (kC4Cols * 4 + 12)));
-        }
-        __syncwarp();
-        cluster_arrive();
-        asm volatile("bar.arrive 1, %0;" ::"n"(kCaThreads) : "memory");
-    } else {
-        if (warp == 1) tmem_alloc(smem_u32((const void *)tmem_slot), 512);
-        else if (warp == 2 && lane == 0) { prefetch_tmap(&tm_q); prefetch_tmap(&tm_kd); prefetch_tmap(&tm_vs); prefetch_tmap(&tm_vd); }
-        __syncwarp();
-        tc_fence_before();
-        cluster_arrive();
-    }
-    // ---- geometry: seven tiles divide the static prefix, the eighth holds ring slots and dynamic tokens ----
-    const StreamState ss = p.state[b];
-    const int S = max(ss.static_len, 0), count = min(ss.count, p.N);
-    const int row_base = (p.layer * p.B + b) * (p.ring_off + p.N);
-    const int per = (S + 6) / 7;
-    int ext[2];                     // tile rows that may hold keys
-    uint64_t live[2][2];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        if (t == 1 && last) {
-            ext[t] = p.dyn_row + p.T;
-            int oldest = (ss.head - ss.count) % p.N;                  // live ring slots: the circular run of `count` from here
-            if (oldest < 0) oldest += p.N;
-            const int end = oldest + count;
-            live[t][0] = ca_bits(oldest, min(end, p.N)) | (end > p.N ? ca_bits(0, end - p.N) : 0ull) | ca_bits(p.dyn_row, ext[t]);
-            live[t][1] = ca_bits(p.dyn_row - 64, ext[t] - 64);
-        } else {
-            ext[t] = max(0, min(per, S - (2 * slice + t) * per));
-            live[t][0] = ca_bits(0, ext[t]);
-            live[t][1] = ca_bits(-64, ext[t] - 64);
-        }
-    }
-    auto kv_bytes = [&](int t) -> uint32_t {
-        if (t == 1 && last) return (uint32_t)((count > 0 ? p.N : 0) + p.T) * (kCaHD * 2);
-        return ext[t] > 0 ? (uint32_t)p.box * (kCaHD * 2) : 0u;
-    };
-    // the cached part of tile t of K or V (a whole box; rows past the slice are masked)
-    auto load_cached = [&](int t, bool v) {
-        const bool ring = t == 1 && last;
-        if (ring ? count == 0 : ext[t] == 0) return;
-        const CUtensorMap *m = ring ? (v ? &tm_vr : &tm_kr) : (v ? &tm_vs : &tm_ks);
-        const int r0 = row_base + (ring ? p.ring_off : ss.bank * p.S_max + (2 * slice + t) * per);
-        for (int c = 0; c < 4; ++c) tma_load_3d_elect(base + L::KV + t * L::TILE + c * (kCaKeys * 128), m, bar((v ? C4_V : C4_K) + t), c * 64, hkv, r0);
-    };
-    auto load_dyn = [&](bool v) {
-        for (int c = 0; c < 4; ++c)
-            tma_load_3d_elect(base + L::KV + L::TILE + c * (kCaKeys * 128) + p.dyn_row * 128, v ? &tm_vd : &tm_kd, bar((v ? C4_V : C4_K) + 1), c * 64, hkv, b * p.T);
-    };
-    // (This kernel is a step's only: K of the caches comes ahead of the wait. The roles part as in chain_attn_kernel.)
-    if (warp == 0) {
-        for (int t = 0; t < 2; ++t) {
-            mbar_expect_tx_elect(bar(C4_K + t), kv_bytes(t));
-            load_cached(t, false);
-        }
-    } else {
-        asm volatile("bar.sync 1, %0;" ::"n"(kCaThreads) : "memory");
-        cluster_wait();              // the peers' barriers exist
-        tc_fence_after();
-    }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // (not before this CTA has its tensor memory, all of it: a dependent that took some first would wait for this grid)
-    if (warp != 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const uint32_t tmem = warp == 0 ? 0u : *tmem_slot;
-
-    auto wait_slow = [&](int i, uint32_t code) -> bool {
-        const unsigned long long t_start = globaltimer_ns();
-        for (uint32_t n = 1;; ++n) {
-            if (mbar_try_wait_cluster(bar(i), 0)) return true;
-            if ((n & 255u) == 0u) {
-                if (*abort_flag) return false;
-                if (globaltimer_ns() - t_start > kCaWaitNs) break;
-            }
-        }
-        *abort_flag = 1u;
-        if (p.status) atomicCAS(p.status, 0u, 0x80000000u | ((code + 80u) << 16) | (blockIdx.x & 0xFFFFu));
-        return false;
-    };
-    auto wait = [&](int i, uint32_t code) -> bool { return mbar_try_wait(bar(i), 0) || wait_slow(i, code); };
-    auto wait_cl = [&](int i, uint32_t code) -> bool { return mbar_try_wait_cluster(bar(i), 0) || wait_slow(i, code); };
-
-    if (warp == 0) {
-        mbar_expect_tx_elect(bar(C4_Q), kC4Rows * kCaHD * 2);
-        for (int c = 0; c < 4; ++c) tma_load_4d_elect(base + L::QP + c * (kC4Rows * 128), &tm_q, bar(C4_Q), c * 64, hkv * p.G, t0, b);
-        if (last) load_dyn(false);
-        for (int t = 0; t < 2; ++t) {              // V comes when K is through: into the L2 until then
-            const bool ring = t == 1 && last;
-            if (ring ? count == 0 : ext[t] == 0) continue;
-            const int r0 = row_base + (ring ? p.ring_off : ss.bank * p.S_max + (2 * slice + t) * per);
-            if (lane < 4) tma_prefetch_3d(ring ? &tm_vr : &tm_vs, lane * 64, hkv, r0);
-            __syncwarp();
-        }
-        for (int t = 0; t < 2; ++t) {
-            mbar_expect_tx_elect(bar(C4_V + t), kv_bytes(t));
-            if (!__all_sync(0xffffffffu, wait(C4_S + t, 1))) break;
-            load_cached(t, true);
-            if (t == 1 && last) load_dyn(true);
-        }
-        cluster_wait();
-    } else if (warp == 1) {
-        constexpr uint32_t idesc_qk = umma_idesc_bf16(kC4Rows, kCaKeys, false);
-        constexpr uint32_t idesc_pv = umma_idesc_bf16(kC4Rows, kCaHD, true);
-        bool ok = wait(C4_Q, 3);
-#pragma unroll 1
-        for (int t = 0; t < 2; ++t) {
-            ok = ok && wait(C4_K + t, 4);
-            if (ok && ext[t] > 0) {
-                tc_fence_after();
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint64_t ad = umma_desc_sw128(base + L::QP + c * (kC4Rows * 128), 16, 1024);
-                    uint64_t bd = umma_desc_sw128(base + L::KV + t * L::TILE + c * (kCaKeys * 128), 16, 1024);
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        umma_ss_elect(tmem + t * kCaKeys, ad, bd, idesc_qk, (c > 0 || kk > 0) ? 1u : 0u);
-                        umma_desc_advance(ad, 32);
-                        umma_desc_advance(bd, 32);
-                    }
-                }
-            }
-            umma_commit_elect(bar(C4_S + t));      // also after a wait that ran out: nobody waits for nothing
-        }
-        ok = ok && wait(C4_VREADY, 5) && wait(C4_P, 6);
-        if (ok) {
-            tc_fence_after();
-            uint32_t acc = 0u;
-#pragma unroll 1
-            for (int t = 0; t < 2; ++t) {
-                const int steps = (ext[t] + 15) / 16;
-#pragma unroll 1
-                for (int kk = 0; kk < steps; ++kk) {
-                    umma_ts_elect(tmem + 256, tmem + t * kCaKeys + kk * 8,
-                                  umma_desc_sw128(base + L::KV + t * L::TILE + kk * (16 * 128), kCaKeys * 128, 1024), idesc_pv, acc);
-                    acc = 1u;
-                }
-            }
-        }
-        umma_commit_elect(bar(C4_O));
-    } else {
-        const int t = threadIdx.x - 64, quarter = warp & 3, group = (warp - 2) >> 2;
-        const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-        const int row = quarter * 32 + lane;
-        // ---- softmax: group g takes tile g, a thread one row of it (its 128 logits, read twice) ----
-        const uint64_t lv[2] = {group ? live[1][0] : live[0][0], group ? live[1][1] : live[0][1]};
-        const uint32_t s_addr = tmem + lane_addr + group * kCaKeys;
-        bool ok = wait(C4_S + group, 7);
-        tc_fence_after();
-        float m = -INFINITY;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            uint32_t s[32];
-            tmem_ld32(s_addr + c * 32, s);
-            tmem_wait_ld();
-            const uint32_t mk = (uint32_t)(lv[c >> 1] >> ((c & 1) * 32));
-            if (mk != 0xFFFFFFFFu) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i)
-                    if (!((mk >> i) & 1u)) s[i] = 0xff800000u;
-            }
-#pragma unroll
-            for (int i = 0; i < 32; i += 2) m = max3_f32(m, __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
-        }
-        float *mx = reinterpret_cast<float *>(smem + L::MX);
-        mx[group * kC4Rows + row] = m;
-        asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");       // the two warps of these rows
-        m = fmaxf(m, mx[(group ^ 1) * kC4Rows + row]);
-        const float ref = m == -INFINITY ? 0.f : -m * p.scale_log2;
-        const Ex2PolyConsts kc = ex2_poly_consts();
-        float l0 = 0.f, l1 = 0.f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            uint32_t s[32];
-            tmem_ld32(s_addr + c * 32, s);
-            tmem_wait_ld();
-            const uint32_t mk = (uint32_t)(lv[c >> 1] >> ((c & 1) * 32));
-            uint32_t o[16];                     // P of these 32 keys, over logits that have been read
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int i = q * 8 + 2 * k;
-                    const float x0 = fmaf(__uint_as_float(s[i]), p.scale_log2, ref), x1 = fmaf(__uint_as_float(s[i + 1]), p.scale_log2, ref);
-                    float p0, p1;
-                    if (k == 3) ex2_poly_f32x2(x0, x1, kc, p0, p1);           // a quarter of them on the FMA pipe
-                    else { p0 = ex2(x0); p1 = ex2(x1); }
-                    if (!((mk >> i) & 1u)) p0 = 0.f;
-                    if (!((mk >> (i + 1)) & 1u)) p1 = 0.f;
-                    l0 += p0; l1 += p1;
-                    __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1);
-                    o[q * 4 + k] = *reinterpret_cast<uint32_t *>(&pp);
-                }
-            }
-            tmem_st16(s_addr + c * 16, o);
-        }
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(C4_P));
-        if (row < rows) {
-            const uint32_t at = base + L::ML + (uint32_t)(slice * kC4Rows + row) * 16u;
-#pragma unroll
-            for (int o = 0; o < kC4Slices; ++o) {
-                const uint32_t dst = mapa(at, (uint32_t)o), ib = mapa(bar(C4_INBOX), (uint32_t)o);
-                if (group == 0) st_async_v2(dst, ib, __float_as_uint(m * p.scale_log2), __float_as_uint(l0 + l1));
-                else st_async_b32(dst + 8u, ib, __float_as_uint(l0 + l1));
-            }
-        }
-        // V rows inside the contraction that hold no key: zero, so that weight 0 meets no stale NaN
-        {
-            ok = wait(C4_V + group, 9) && ok;
-            const int ext16 = ((group ? ext[1] : ext[0]) + 15) & ~15;
-            uint64_t dead[2] = {~lv[0] & ca_bits(0, ext16), ~lv[1] & ca_bits(0, ext16 - 64)};
-            uint8_t *v = smem + L::KV + group * L::TILE + quarter * (kCaKeys * 128) + lane * 4;
-#pragma unroll
-            for (int w = 0; w < 2; ++w)
-                while (dead[w]) {
-                    const int r = __ffsll((long long)dead[w]) - 1;
-                    dead[w] &= dead[w] - 1;
-                    *reinterpret_cast<uint32_t *>(v + (w * 64 + r) * 128) = 0u;
-                }
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(C4_VREADY));
-        }
-        // ---- partial O to the owners of the columns: group g sends columns [128 g, 128 g + 128) of its rows ----
-        ok = wait(C4_O, 10) && ok;
-        tc_fence_after();
-        // this CTA's P V is through with its tiles: the peers may send their partial results over them
-        if (t < kC4Slices) mbar_arrive_cluster_release(mapa(bar(C4_FREE), (uint32_t)t));
-        const bool none = ext[0] == 0 && ext[1] == 0;
-        if (wait_cl(C4_FREE, 11)) {
-#pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
-                const int o = (slice + 1 + c) & 1;                    // (the four CTAs start with different owners)
-                const int cc = c ^ (o << 1);                          // 32-column piece of the group's 128
-                const int owner = group * 2 + (cc >> 1);
-                uint32_t acc[32];
-                tmem_ld32(tmem + 256 + lane_addr + group * 128 + cc * 32, acc);
-                tmem_wait_ld();
-                if (!ok || none) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) acc[i] = ok ? 0u : 0x7fc00000u;
-                }
-                if (row < rows) {
-                    const uint32_t at = base + L::KV + (uint32_t)((slice * (kC4Cols / 4) + (cc & 1) * 8) * kC4Rows + row) * 16u;
-                    const uint32_t dst = mapa(at, (uint32_t)owner), ib = mapa(bar(C4_INBOX), (uint32_t)owner);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) st_async_v4(dst + q * (kC4Rows * 16), ib, acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
-                }
-            }
-        }
-        tc_fence_before();
-        // ---- merge of this CTA's 64 columns: thread = (row, 32 columns) ----
-        ok = wait_cl(C4_INBOX, 12);
-        const int mrow = t & 127, mh = t >> 7;
-        if (mrow < rows) {
-            float w[kC4Slices], mm = -INFINITY, l = 0.f;
-            float4 ml[kC4Slices];
-#pragma unroll
-            for (int q = 0; q < kC4Slices; ++q) {
-                ml[q] = reinterpret_cast<const float4 *>(smem + L::ML)[q * kC4Rows + mrow];
-                mm = fmaxf(mm, ml[q].x);
-            }
-#pragma unroll
-            for (int q = 0; q < kC4Slices; ++q) {
-                w[q] = ml[q].x == -INFINITY ? 0.f : ex2(ml[q].x - mm);
-                l = fmaf(w[q], ml[q].y + ml[q].z, l);
-            }
-            const float inv = ok ? 1.f / l : __int_as_float(0x7fc00000);      // (a wait that ran out: the row is marked invalid, not left stale)
-#pragma unroll
-            for (int q = 0; q < kC4Slices; ++q) w[q] *= inv;
-            const float4 *in = reinterpret_cast<const float4 *>(smem + L::KV) + mh * 8 * kC4Rows + mrow;
-            const int tk = mrow >> p.g_log2;
-            __nv_bfloat16 *dst = p.out + ((size_t)(b * p.T + t0 + tk) * p.Hq + hkv * p.G + (mrow - (tk << p.g_log2))) * kCaHD + slice * kC4Cols + mh * 32;
-#pragma unroll
-            for (int q8 = 0; q8 < 4; ++q8) {             // eight columns
-                float a[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) a[i] = 0.f;
-#pragma unroll
-                for (int q = 0; q < kC4Slices; ++q) {
-                    const float4 v0 = in[(q * (kC4Cols / 4) + q8 * 2) * kC4Rows], v1 = in[(q * (kC4Cols / 4) + q8 * 2 + 1) * kC4Rows];
-                    a[0] = fmaf(v0.x, w[q], a[0]); a[1] = fmaf(v0.y, w[q], a[1]); a[2] = fmaf(v0.z, w[q], a[2]); a[3] = fmaf(v0.w, w[q], a[3]);
-                    a[4] = fmaf(v1.x, w[q], a[4]); a[5] = fmaf(v1.y, w[q], a[5]); a[6] = fmaf(v1.z, w[q], a[6]); a[7] = fmaf(v1.w, w[q], a[7]);
-                }
-                uint32_t o[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    __nv_bfloat162 hh = __floats2bfloat162_rn(a[2 * k], a[2 * k + 1]);
-                    o[k] = *reinterpret_cast<uint32_t *>(&hh);
-                }
-                *reinterpret_cast<uint4 *>(dst + q8 * 8) = make_uint4(o[0], o[1], o[2], o[3]);
-            }
-        }
-    }
-    __syncwarp();
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem, 512);
-    // Everything its peers send to a CTA has arrived before it leaves: their C4_FREE arrivals, their partial results. After a wait that
-    // ran out that is not known: it stays until its peers' waits have run out as well.
-    if (*abort_flag) {
-        const unsigned long long ta = globaltimer_ns();
-        while (globaltimer_ns() - ta < 6ull * kCaWaitNs) __nanosleep(1000);
-    }
-}
-
 }  // namespace
 
 // Rows of a CTA: 32 while the clusters of eight fit the device at once, else 64 where the call stands by itself (0: too many streams). What a CTA
@@ -804,7 +450,7 @@ static int chain_attn_rows(const AttnParams &p, bool early)
         const int tt = rows / G;
         if ((long long)p.B * p.Hkv * ((p.T + tt - 1) / tt) <= 14) return rows;
     }
-    return early && G == kC4Rows && (long long)p.B * p.Hkv * p.T <= 32 ? kC4Rows : 0;
+    return 0;
 }
 
 bool chain_attn_supported(const AttnParams &p, bool early, int sm_count)
@@ -854,9 +500,8 @@ cudaError_t launch_chain_attn(const AttnParams &a, uint32_t *status, bool early,
     p.units = (a.T + tt - 1) / tt; p.tt = tt;
     p.scale_log2 = a.scale * 1.4426950408889634f;
     p.pf = pf ? *pf : ChainPrefetch{};
-    static std::atomic<unsigned long long> set32{0}, set64{0}, set128{0};
-    const dim3 grid((unsigned)((tile == kC4Rows ? kC4Slices : kCaSlices) * a.Hkv * p.units), (unsigned)a.B);
-    if (tile == kC4Rows) return launch_rows(chain_attn128_kernel, C4Smem::TOTAL, set128, m, p, grid, st);
+    static std::atomic<unsigned long long> set32{0}, set64{0};
+    const dim3 grid((unsigned)(kCaSlices * a.Hkv * p.units), (unsigned)a.B);
     return tile == 32 ? launch_rows(chain_attn_kernel<32>, CaSmem<32>::TOTAL, set32, m, p, grid, st) : launch_rows(chain_attn_kernel<64>, CaSmem<64>::TOTAL, set64, m, p, grid, st);
 }
 

@@ -122,8 +122,8 @@ cudaError_t launch_attention_tc(const AttnParams &p, uint32_t *status, bool two_
 // units of 128 rows (attn_pair.cuh): key slices where they are the faster form, 0 otherwise; merged: inside clusters
 int pair_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count, bool &merged);
 cudaError_t launch_attention_pair(const AttnParams &p, uint32_t *status, int nsplit, bool merged, cudaStream_t st);
-// a few streams (chain_attn.cu): key slices merged inside clusters of eight or four. early: the caller
-// vouches that the cached regions are not written by work that may still be running
+// a few streams (chain_attn.cu): key slices merged inside clusters of eight. early: the caller vouches that the cached regions are not
+// written by work that may still be running
 bool chain_attn_supported(const AttnParams &p, bool early, int sm_count);
 struct ChainPrefetch;
 cudaError_t launch_chain_attn(const AttnParams &p, uint32_t *status, bool early, const ChainPrefetch *pf, cudaStream_t st);

@@ -109,10 +109,6 @@ __device__ __forceinline__ float silu_mul(float g, float u)
     return fmaf(t, 0.5f * g, 0.5f * g) * u;
 }
 // L2 prefetch of one box of a tiled tensor map (no shared-memory destination, no completion barrier)
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap *map, int c0, int c1, int c2)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2) : "memory");
-}
 __device__ __forceinline__ void tma_prefetch_2d_elect(const CUtensorMap *map, int c0, int c1)
 {
     asm volatile(
@@ -120,10 +116,6 @@ __device__ __forceinline__ void tma_prefetch_2d_elect(const CUtensorMap *map, in
         "elect.sync _|q, 0xffffffff;\n\t"
         "@q cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];\n\t}"
         ::"l"(map), "r"(c0), "r"(c1) : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap *map, int c0, int c1, int c2, int c3)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap *map)
 {
@@ -188,17 +180,6 @@ __device__ __forceinline__ void umma_ss_elect(uint32_t tmem_d, uint64_t desc_a, 
         "elect.sync _|q, 0xffffffff;\n\t"
         "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// A operand in tensor memory (lanes = rows; a 32-bit column holds two consecutive bf16 of the contraction)
-__device__ __forceinline__ void umma_ts_elect(uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "elect.sync _|q, 0xffffffff;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 __device__ __forceinline__ void umma_commit_elect(uint32_t bar)

@@ -1387,14 +1387,14 @@ def test_expert_step_of_fewer_layers_than_the_cache(U, B):
     _expert_case(U, w, 512, 2e-2, "expert of fewer layers than the cache", streams=[0, B - 1], cache_layers=4)
 
 
-CLUSTERS_OF_FOUR = [
-    # B, T, Hq, Hkv, S_max, prefix lengths, N: edges of the attention that merges four key slices per 128 rows (three to eight streams)
+A_FEW_STREAMS = [
+    # B, T, Hq, Hkv, S_max, prefix lengths, N: edges of the attention in units of 128 rows whose key slices merge in clusters (three to eight streams)
     (4, 50, 8, 1, 816, [816, 700, 0, 113], 32), (8, 64, 8, 1, 896, [896] * 8, 64), (6, 60, 4, 2, 300, [300, 1, 2, 7, 8, 299], 5),
     (5, 33, 16, 1, 64, [64] * 5, 4),
 ]
 
 
-@pytest.mark.parametrize("case", CLUSTERS_OF_FOUR, ids=["B%d_T%d_h%dkv%d_S%d" % c[:5] for c in CLUSTERS_OF_FOUR])
+@pytest.mark.parametrize("case", A_FEW_STREAMS, ids=["B%d_T%d_h%dkv%d_S%d" % c[:5] for c in A_FEW_STREAMS])
 def test_expert_step_bf16_attention_of_a_few_streams(U, case):
     B, T, Hq, Hkv, S_max, S_list, N = case
     w = synth.CONFIGS["cfg2"].with_(B=B, L=1, T=T, Hq=Hq, Hkv=Hkv, D=512, S=S_max, S_max=S_max, N=N)

@@ -27,8 +27,14 @@ KERNELS = _kernels()
 
 def test_kernels_are_found():
     names = {n.split(": ")[1] for n, _, _ in KERNELS}
-    assert {"chain_attn_kernel", "chain_attn128_kernel", "chain_gemm_kernel", "chain_in_kernel", "tile_gemm_kernel", "attn_tc2_kernel", "gate_kernel",
-            "flow_step_kernel", "init_static_kernel", "linear_res_tc_kernel"} <= names
+    assert {"chain_attn_kernel", "attn_pair_kernel", "chain_gemm_kernel", "chain_in_kernel", "tile_gemm_kernel", "attn_tc2_kernel", "gate_kernel",
+            "flow_step_kernel", "init_static_kernel", "linear_half_kernel", "linear_res_tc_kernel"} <= names
+
+
+def test_attention_kernels_are_the_ones_a_call_can_reach():
+    """(Clusters of four with 128 rows per CTA were left with groups of 128 heads of 256 inside a step, which refuses more than 12288 / 256 heads.)"""
+    assert {n.split(": ")[1] for n, _, _ in KERNELS if re.search(r"(attn|attention)_?\w*kernel", n)} == {
+        "attn_merge_kernel", "attn_pair_kernel", "attn_simt_kernel", "attn_tc2_kernel", "attn_tc_kernel", "chain_attn_kernel"}
 
 
 @pytest.mark.parametrize("kernel", [k for k in KERNELS if "tmem_alloc" in k[2]], ids=lambda k: k[0])
