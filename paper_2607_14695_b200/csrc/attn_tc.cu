@@ -890,6 +890,13 @@ static double tc2_us(const AttnParams &p, int nsplit, int sm_count)
 // 10.6 -> 8.8 (four slices), 4 streams 13.7 -> 10.6 (two), 8 streams 14.4 -> 11.4 (two), 16 streams 16.2 -> 13.6 (one); 24 streams x 33 tokens 17.5 -> 14.6;
 // heads of 128, 6 streams x 4 KV heads 9.2 -> 7.5; one stream x 2111 keys 13.2 -> 10.8, 4 streams x 2082 keys 17.1 -> 14.3. 16 streams x 4466 keys
 // stay with units of 256 rows in two slices (33.1 against 40.8).
+// References per row of a launch in ns slices: two accumulators in a slice of two tiles or more, one accumulator in all without a split.
+static int pair_references(int tiles, int ns)
+{
+    const int per = (tiles + ns - 1) / ns, full = tiles / per;
+    return ns == 1 ? 1 : full * std::min(2, per) + std::min(2, tiles - full * per);
+}
+
 int pair_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count, bool &merged)
 {
     const int units = pair_units(p), clusters = sm_count / 2;
@@ -903,6 +910,9 @@ int pair_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count, 
     static const int kSlices[] = {1, 2, 3, 4, 6, 8, 12, 16, 18};
     for (const int ns : kSlices) {
         if (ns > tiles || units * ns > clusters) break;
+        // The key that sets a reference has weight 1, which bf16 holds exactly, and units of 256 rows have one reference per slice: fewer of them are
+        // farther from 64 bits (10 streams of 33 tokens, 4 heads of 128, 552 keys: 2.30e-3 with one, 2.14e-3 with five).
+        if (pair_references(tiles, ns) < ns2) continue;
         for (int m = ns == 2 || ns == 4 ? 1 : 0; m >= 0; --m) {
             // (clusters of eight with a margin: the last ones find room late, 16.0 us with 16 of them against 9.3 with 12)
             const int active = m ? tc2_active_clusters(p.d, 2 * ns) : 0;
