@@ -285,12 +285,11 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 #pragma unroll
             for (int w = 0; w < NW; ++w) ca_tmem_ld_16x256b(addr + (w0 + w) * 64, s[w]);
             tmem_wait_ld();
-            const uint64_t full = ~0ull;
-            if (live_lo != full || live_hi != full) {
-                const int sh = 2 * (lane & 3);
 #pragma unroll
-                for (int w = 0; w < NW; ++w) {
-                    const uint64_t ml = (w0 + w == 0 ? live_lo : live_hi) >> sh;      // bit 8 g + j: this thread's column j of group g
+            for (int w = 0; w < NW; ++w) {
+                const uint64_t live = w0 + w == 0 ? live_lo : live_hi;
+                if (live != ~0ull) {
+                    const uint64_t ml = live >> (2 * (lane & 3));      // bit 8 g + j: this thread's column j of group g
 #pragma unroll
                     for (int g = 0; g < 8; ++g)
 #pragma unroll
@@ -357,7 +356,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         if (wait_cl(CB_FREE, 9)) {
 #pragma unroll
             for (int c = 0; c < ROWS / 32; ++c) {
-                if (c * 32 < rows) {
+                if (ROWS == 32 || c * 32 < rows) {
                     uint32_t acc[32];
                     tmem_ld32(tmem + 128 + group * ROWS + ((uint32_t)(quarter * 32) << 16) + c * 32, acc);
                     tmem_wait_ld();
@@ -398,7 +397,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             const float4 *in = reinterpret_cast<const float4 *>(smem + L::K);
 #pragma unroll
             for (int q2 = 0; q2 < QUADS; ++q2) {
-                if (q2 * 4 < own) {
+                if (QUADS == 1 || q2 * 4 < own) {
                     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                     for (int q = 0; q < kCaSlices; ++q) {
