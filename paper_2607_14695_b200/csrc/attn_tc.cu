@@ -872,24 +872,29 @@ static int pair_units(const AttnParams &p)
     return ((p.T + tt - 1) / tt + 1) / 2 * p.Hkv * p.B;
 }
 
-// What a launch of units of 256 rows takes, us: fitted to graph replays (heads of 256: 13.9 us for 4 streams of 898 keys in one slice, 16.4 for 18, 33.1
-// for 16 of 4466 keys in two, 22.7 for 8 of 3306).
+// What a launch takes, us, in units of 256 rows and of 128: fitted to 1700 graph replays of single calls (204 shapes of 1 to 36 streams, 4 to 100 tokens,
+// 100 to 13,700 keys, heads of 128 and 256, with every number of slices that fits; rms of the fits 2 to 6 %). Heads of 128 take 0.83 of the fixed parts
+// and 0.915 of the time of a tile of 128 keys. A kilorow is 1000 rows of fp32 partials 256 wide.
 static double tc2_us(const AttnParams &p, int nsplit, int sm_count)
 {
-    const int G = p.Hq / p.Hkv, units = ((p.T + kBM / G - 1) / (kBM / G) + 1) / 2 * p.Hkv * p.B;
-    const int tiles = ((p.S_max + kBN - 1) / kBN + (p.N + kBN - 1) / kBN + (p.T + kBN - 1) / kBN + 1) / 2, clusters = sm_count / 2 > 0 ? sm_count / 2 : 1;
-    const bool merged = tc2_cluster_merge_ok(p, nsplit, sm_count);
-    const int waves = merged ? 1 : (units * nsplit + clusters - 1) / clusters;
-    const double split = nsplit <= 1 ? 0.0 : merged ? tc2_merged_us(units, nsplit) : tc2_partials_us(p, nsplit);
-    return 4.4 + 0.03 * std::min(units * nsplit, clusters) + (p.d == 256 ? 1.17 : 0.95) * waves * ((tiles + nsplit - 1) / nsplit) + split;
+    const int G = p.Hq / p.Hkv, units = ((p.T + kBM / G - 1) / (kBM / G) + 1) / 2 * p.Hkv * p.B, clusters = sm_count / 2 > 0 ? sm_count / 2 : 1;
+    const int tiles = ((p.S_max + kBN - 1) / kBN + (p.N + kBN - 1) / kBN + (p.T + kBN - 1) / kBN + 1) / 2, per = (tiles + nsplit - 1) / nsplit;
+    const double fixed = p.d == 256 ? 1.0 : 0.83, tile = p.d == 256 ? 1.0 : 0.915;
+    if (nsplit > 1 && tc2_cluster_merge_ok(p, nsplit, sm_count)) return 9.3 * fixed + 1.15 * tile * per + 0.033 * units * nsplit;
+    const int walked = per * ((units * nsplit + clusters - 1) / clusters);      // tiles of the busiest SM pair
+    if (nsplit <= 1) return 5.8 * fixed + 1.19 * tile * walked + 0.045 * std::min(units, clusters);
+    const double kilorows = 1e-3 * p.B * p.T * p.Hq * nsplit * p.d / 256.0;
+    return 9.2 * fixed + 1.27 * tile * walked + 0.025 * std::min(units * nsplit, clusters) + 0.25 * kilorows;
+}
+static double pair_us(const AttnParams &p, int units, int tiles, int ns, bool merged)
+{
+    const double fixed = p.d == 256 ? 1.0 : 0.83, per = (p.d == 256 ? 1.0 : 0.915) * ((tiles + ns - 1) / ns);
+    if (ns == 1) return 4.5 * fixed + 1.04 * per + 0.022 * units;
+    if (merged) return ns == 2 ? 6.4 * fixed + 1.0 * per + 0.04 * units : 6.2 * fixed + 1.01 * per + 0.112 * units;
+    const double kilorows = 1e-3 * p.B * p.T * p.Hq * ns * p.d / 256.0;          // (the merge launch hides some)
+    return 7.75 * fixed + 1.03 * per + 0.028 * units * ns + 0.25 * std::max(0.0, kilorows - 4.4);
 }
 
-// Key slices of the 128-row units where they are the faster two-CTA form; 0: units of 256 rows. One wave is all they may be; a tile of 128 keys takes
-// them 1.05 us and one of 256 rows 1.17, a merge inside a cluster 2.3 us and more with the CTAs that push at the same time, partials and the
-// merge launch 1.2 us and 0.37 per 400 rows and slice. Measured against the form of before, one call, graph replay, us: 898 keys x 50 tokens, 2 streams
-// 10.6 -> 8.8 (four slices), 4 streams 13.7 -> 10.6 (two), 8 streams 14.4 -> 11.4 (two), 16 streams 16.2 -> 13.6 (one); 24 streams x 33 tokens 17.5 -> 14.6;
-// heads of 128, 6 streams x 4 KV heads 9.2 -> 7.5; one stream x 2111 keys 13.2 -> 10.8, 4 streams x 2082 keys 17.1 -> 14.3. 16 streams x 4466 keys
-// stay with units of 256 rows in two slices (33.1 against 40.8).
 // References per row of a launch in ns slices: two accumulators in a slice of two tiles or more, one accumulator in all without a split.
 static int pair_references(int tiles, int ns)
 {
@@ -897,29 +902,34 @@ static int pair_references(int tiles, int ns)
     return ns == 1 ? 1 : full * std::min(2, per) + std::min(2, tiles - full * per);
 }
 
-int pair_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count, bool &merged)
+// Key slices of the 128-row units where those are the faster two-CTA form; 0: units of 256 rows, in the tc2_slices that tc2_choose_splits picked. One wave is
+// all they may be. Over the 191 shapes above that no cluster of eight takes, the choice is within 0.3 % (geometric mean; at most 8.5 %) of the fastest of all
+// forms and slices, units of 256 rows alone 21.7 %. One call against those, us: 898 keys x 50 tokens, 2 streams 12.6 -> 9.1 (four slices), 4 streams
+// 13.7 -> 10.9 (two), 8 streams 14.3 -> 11.8 (two), 16 streams 15.7 -> 13.7 (one); 24 streams x 33 tokens 17.6 -> 14.6; heads of 128, 2 KV heads, 14 tokens x 341
+// keys 8.9 -> 7.1 (four); one stream x 2082 keys 13.5 -> 11.2; 16 tokens x 13,632 keys 18.9 -> 14.9 (32). 12 streams x 4466 keys stay with
+// units of 256 rows in three slices.
+int pair_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count, int tc2_slices, bool &merged)
 {
     const int units = pair_units(p), clusters = sm_count / 2;
     merged = false;
     if (units == 0 || units > clusters || !tc2_supported(p)) return 0;
     const int tiles = ((p.S_max + kBN - 1) / kBN + (p.N + kBN - 1) / kBN + (p.T + kBN - 1) / kBN + 1) / 2;
-    const double rows = (double)p.B * p.T * p.Hq, per_split_bytes = rows * (p.d + 2) * sizeof(float);
-    const int ns2 = tc2_choose_splits(p, partial_bytes, sm_count);
-    double best_us = tc2_us(p, ns2 < 1 ? 1 : ns2, sm_count) - 0.1;
+    const double per_split_bytes = (double)p.B * p.T * p.Hq * (p.d + 2) * sizeof(float);
+    double best_us = tc2_us(p, std::max(1, tc2_slices), sm_count) - 0.1;
     int best = 0;
-    static const int kSlices[] = {1, 2, 3, 4, 6, 8, 12, 16, 18};
+    static constexpr int kSlices[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 28, 32};
+    static_assert(kSlices[13] <= kMaxSplits, "the merge kernel has a lane per slice");
     for (const int ns : kSlices) {
         if (ns > tiles || units * ns > clusters) break;
         // The key that sets a reference has weight 1, which bf16 holds exactly, and units of 256 rows have one reference per slice: fewer of them are
         // farther from 64 bits (10 streams of 33 tokens, 4 heads of 128, 552 keys: 2.30e-3 with one, 2.14e-3 with five).
-        if (pair_references(tiles, ns) < ns2) continue;
+        if (pair_references(tiles, ns) < tc2_slices) continue;
         for (int m = ns == 2 || ns == 4 ? 1 : 0; m >= 0; --m) {
-            // (clusters of eight with a margin: the last ones find room late, 16.0 us with 16 of them against 9.3 with 12)
+            // (clusters of eight with a margin: the last ones find room late, 16.7 us with 16 of them against 9.6 with 12)
             const int active = m ? tc2_active_clusters(p.d, 2 * ns) : 0;
             if (m && units > (ns == 4 ? active - active / 6 : active)) continue;
             if (!m && ns > 1 && per_split_bytes * ns > (double)partial_bytes) continue;
-            const double split = ns == 1 ? 0.0 : m ? 2.2 + 0.1 * (ns - 2) + 0.015 * units * ns : 1.2 + 0.37 * rows * ns / 400.0 * p.d / 256.0;
-            const double us = 4.0 + (ns == 1 ? 0.02 * units : 0.0) + (p.d == 256 ? 1.05 : 0.85) * ((tiles + ns - 1) / ns) + split;
+            const double us = pair_us(p, units, tiles, ns, m != 0);
             if (us < best_us) { best_us = us; best = ns; merged = m != 0; }
         }
     }

@@ -502,23 +502,26 @@ static int attention(reflex_cache_t *c, int layer, const void *q, const void *k_
     if ((c->attn_impl == REFLEX_ATTN_TC && !tc_ok) || (c->attn_impl == REFLEX_ATTN_TC2 && !tc2_ok))
         return fail(REFLEX_ERR_NOT_IMPLEMENTED, "tensor-core attention needs bf16, 128 %% (Hq/Hkv) == 0 and d in {64,128,256} (two-CTA form: {128,256})");
     cudaError_t e;
-    bool pair_merged = false;
     uint32_t *status = (uint32_t *)(c->ws + c->lay.status_off);
     if (c->attn_impl == REFLEX_ATTN_SIMT || !tc_ok) {
         p.nsplit = simt_choose_splits(p, c->lay.partial_bytes, c->sm_count);
         e = launch_attention_simt(p, (cudaStream_t)stream);
     } else if (c->attn_impl == REFLEX_ATTN_AUTO && chain_attn_supported(p, early, c->sm_count)) {
         e = launch_chain_attn(p, status, early, pf, (cudaStream_t)stream);
-    } else if (const int ns = c->attn_impl == REFLEX_ATTN_AUTO ? pair_choose_splits(p, c->lay.partial_bytes, c->sm_count, pair_merged) : 0) {
-        p.nsplit = ns;
-        e = launch_attention_pair(p, status, ns, pair_merged, (cudaStream_t)stream);
     } else {
-        // the two-CTA kernel (with a key split when the streams alone do not fill the SM pairs); heads of 64 one CTA per query tile with
-        // a finer split
+        // the two-CTA kernels in units of 128 or of 256 rows (with a key split when the streams alone do not fill the SM pairs); heads of 64 one CTA per
+        // query tile with a finer split
+        const bool choose = c->attn_impl == REFLEX_ATTN_AUTO && tc2_ok;
         const int split2 = tc2_ok ? tc2_choose_splits(p, c->lay.partial_bytes, c->sm_count) : 0;
-        const bool two = c->attn_impl == REFLEX_ATTN_TC2 || (c->attn_impl == REFLEX_ATTN_AUTO && split2 >= 1);
-        p.nsplit = two ? (split2 >= 1 ? split2 : 1) : tc_choose_splits(p, c->lay.partial_bytes, c->sm_count);
-        e = launch_attention_tc(p, status, two, c->sm_count, (cudaStream_t)stream);
+        bool merged = false;
+        p.nsplit = choose ? pair_choose_splits(p, c->lay.partial_bytes, c->sm_count, split2, merged) : 0;
+        if (p.nsplit > 0) {
+            e = launch_attention_pair(p, status, p.nsplit, merged, (cudaStream_t)stream);
+        } else {
+            const bool two = choose || c->attn_impl == REFLEX_ATTN_TC2;
+            p.nsplit = two ? split2 : tc_choose_splits(p, c->lay.partial_bytes, c->sm_count);
+            e = launch_attention_tc(p, status, two, c->sm_count, (cudaStream_t)stream);
+        }
     }
     if (e != cudaSuccess) return cuda_fail(e, "attention launch");
     return REFLEX_OK;

@@ -1575,3 +1575,19 @@ def test_plain_projections_inside_a_step_cost_what_they_cost_alone(U, dtype, B, 
              lambda: rb.reflex_linear_residual(rows(model.m), W["Wd"][0], h, h, cache=cache)]
     alone, step = L * sum(_us(call, 3) for call in parts), _us(lambda: model.step(a, cond, 0), 3)
     assert step <= 1.2 * alone
+
+
+@pytest.mark.parametrize("B,T,Hq,Hkv,d,S,N", [(6, 10, 8, 4, 256, 133, 82), (11, 15, 4, 2, 128, 149, 41)])
+def test_attention_as_chosen_costs_no_more_than_in_units_of_256_rows(U, B, T, Hq, Hkv, d, S, N):
+    """Few keys in many units: three slices and a merge launch cost 1.04 and 1.06 of one launch of 256-row units, one slice of 128-row units 0.75 and 0.80.
+    Bound: 1.02."""
+    def us(impl):
+        cache = U.rb.Cache(1, B, Hq, Hkv, d, S, N, T, U.rb.DTYPE_BF16, device=U.DEV)
+        U.rb.reflex_cache_set_attention_impl(cache, impl)
+        z = lambda *s: torch.randn(s, device=U.DEV).to(torch.bfloat16)
+        U.rb.reflex_cache_init_static(cache, list(range(B)), z(B, 1, S, Hkv, d), z(B, 1, S, Hkv, d))
+        U.rb.reflex_cache_append_sliding(cache, list(range(B)), z(B, 1, N, Hkv, d), z(B, 1, N, Hkv, d))
+        q, k, v = z(B, T, Hq, d), z(B, T, Hkv, d), z(B, T, Hkv, d)
+        out = torch.empty_like(q)
+        return _us(lambda: U.rb.reflex_partitioned_attention(cache, 0, q, k, v, out))
+    assert us(U.rb.ATTN_AUTO) <= 1.02 * us(U.rb.ATTN_TC2)
