@@ -764,6 +764,7 @@ norm_linear_small_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
         asm volatile("bar.sync 1, 256;" ::: "memory");
         if (threadIdx.x == 64) QK_TRACE(2, 31, 0);
         ok = wait(S_ACC, 0u, 5) && ok;
+        const float invalid = ok ? -0.f : __int_as_float(0x7fc00000);      // (adding it changes nothing, or makes the tile NaN after a wait that ran out)
         if (threadIdx.x == 64) QK_TRACE(2, 31, 1);
         tc_fence_after();
         // epilogue: thread = output feature (TMEM lane), columns = rows of x; the two warps of a lane quarter take alternate
@@ -802,8 +803,8 @@ norm_linear_small_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
             for (int i = 0; i < 32; ++i) {
                 const int r = c * 32 + i, rg = row0 + r;
                 if (rg < p.M) {                     // (no early exit: the accumulator stays in registers)
-                    const float rs = ok ? rsm[r] : __int_as_float(0x7fc00000);
-                    float val = __uint_as_float(acc[i]) * rs;
+                    const float rs = rsm[r];
+                    float val = fmaf(__uint_as_float(acc[i]), rs, invalid);
                     if (swiglu) { const float u = __uint_as_float(up[i]) * rs; val = silu_mul(val, u); }
                     if constexpr (PLAIN) { if (p.res) val += __bfloat162float(p.res[(size_t)rg * pitch + f]); }
                     dst0[(size_t)rg * pitch] = __float2bfloat16_rn(val);    // a warp writes 64 contiguous bytes per row
