@@ -929,7 +929,9 @@ int pair_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count, 
             const int active = m ? tc2_active_clusters(p.d, 2 * ns) : 0;
             if (m && units > (ns == 4 ? active - active / 6 : active)) continue;
             if (!m && ns > 1 && per_split_bytes * ns > (double)partial_bytes) continue;
-            const double us = pair_us(p, units, tiles, ns, m != 0);
+            // (inside a step the first keys come ahead of the wait, which leaves slices less to save: 4 x 50 tokens x 482 keys, D = 512, a layer 0.4 us
+            // longer in two slices, where single calls take the same)
+            const double us = pair_us(p, units, tiles, ns, m != 0) + (p.early && ns > 1 ? 0.4 : 0.0);
             if (us < best_us) { best_us = us; best = ns; merged = m != 0; }
         }
     }
