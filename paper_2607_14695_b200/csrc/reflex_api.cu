@@ -555,7 +555,8 @@ static bool expert_chained(const reflex_cache_desc &d, const reflex_expert &e)
            chain_proj_supported(CG_RES, M, e.F, e.D) && chain_proj_supported(CG_OUT, M, e.D, e.A);
 }
 
-// Both residual projections as pair tiles of 128 rows (linear_half.cu): 65 to 512 rows, contractions of 2048 or more.
+// Both residual projections as pair tiles of 128 rows (linear_half.cu): 65 rows or more in at most 32 tiles (512 rows x 1024 columns), contractions of
+// 2048 or more.
 static bool expert_halves(const reflex_cache_desc &d, const reflex_expert &e)
 {
     return linear_half_columns(d.B * e.T, d.Hq * d.d, e.D) && linear_half_columns(d.B * e.T, e.F, e.D);
@@ -577,16 +578,24 @@ static bool expert_tiled(const reflex_cache_desc &d, const reflex_expert &e)
 // Which of a step's projections go through the tile kernels instead of the chained ones.
 struct StepForm { bool qkv, gu, res; };
 
-// Pair tiles take in 64 rows of x and of W per step, whatever of them is live; the chained kernels split the contraction and pay for the exchange.
-// Whole steps (D = 1024, us, chained / Q/K/V and gate/up by tiles / all by tiles): 50 rows 570 / 572 / 623, 56 rows 588 / 578 / 624, 64 rows
-// 638 / 621 / 655, 72 rows 796 / 737 / 655, 100 rows 741 / 661 / 662 (F = 2048: 676 / 614 / 583), 120 rows 800 / 733 / 715. A gate/up projection whose tiles
-// leave half of the SM pairs idle is ahead with fewer rows too: F = 2048, 33 rows 513 -> 504, 50 rows 530 -> 518 (F = 3072: 548 -> 550).
+// Pair tiles take in 64 rows of x and of W per step, whatever of them is live, and walk the whole contraction; the chained kernels split it and pay for the
+// exchange. So tiles are ahead with many rows, short contractions (D) and enough weight rows for all SMs (F). Whole steps over the chained form, for D of
+// 256 to 4096 and F of 512 to 12288, each with 4 to 128 rows (1000 shapes, keys 482 to 498, four layers):
+//   all by tiles (65 rows on)   0.71 to 0.95 for F <= 6 D; 0.95 to 1.06 above, where the residual projections have few tiles and a long contraction, and
+//                               tiles for the other two alone are 0.84 to 0.90
+//   Q/K/V by tiles              53 to 64 rows: 0.97 to 1.01 for D <= 1024, 1.01 to 1.06 up to 2048; from 72 rows 0.92 to 1.01. D > 2048: 0.99 to 1.12
+//   gate/up by tiles            53 rows on: 0.89 to 1.01 for D <= 512, for D <= 1024 and F >= 4/3 D or 65 rows, or for F >= 6144; else up to 1.11
+//                               4 to 52 rows, tiles that leave half of the SM pairs idle: 0.93 to 1.02 for D <= 768; D = 1024: 0.95 to 1.01 for F >= 2176
+//                               and, above 32 rows, for F >= 1792, else 1.00 to 1.04; larger D up to 1.11
 static StepForm step_form(const reflex_cache_desc &d, const reflex_expert &e, bool chained)
 {
     const int M = d.B * e.T, nq = d.Hq * d.d, nk = d.Hkv * d.d;
-    if (!chained || (expert_halves(d, e) && expert_tiled(d, e))) return {true, true, true};
+    if (!chained || (expert_halves(d, e) && expert_tiled(d, e) && e.F <= 6 * e.D)) return {true, true, true};
     const bool half_idle = e.F >= 1536 && (2 * e.F + 127) / 128 <= 37;
-    return {M > 52 && tile_proj_supported(CG_QKV, M, e.D, nq, nk, 0), (M > 52 || half_idle) && tile_proj_supported(CG_SWIGLU, M, e.D, 0, 0, e.F), false};
+    const bool qkv = M > (e.D <= 1024 ? 52 : 64) && e.D <= 2048;
+    const bool gu = M > 52 ? e.D <= 512 || (e.D <= 1024 && (M > 64 || 3 * e.F >= 4 * e.D)) || e.F >= 6144
+                           : half_idle && (e.D <= 768 || (e.D <= 1024 && e.F >= (M > 32 ? 1792 : 2176)));
+    return {qkv && tile_proj_supported(CG_QKV, M, e.D, nq, nk, 0), gu && tile_proj_supported(CG_SWIGLU, M, e.D, 0, 0, e.F), false};
 }
 
 static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float *a, float dt, const StepForm form, void *stream)

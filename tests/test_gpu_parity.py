@@ -1591,3 +1591,23 @@ def test_attention_as_chosen_costs_no_more_than_in_units_of_256_rows(U, B, T, Hq
         out = torch.empty_like(q)
         return _us(lambda: U.rb.reflex_partitioned_attention(cache, 0, q, k, v, out))
     assert us(U.rb.ATTN_AUTO) <= 1.02 * us(U.rb.ATTN_TC2)
+
+
+def _step_us(U, T, D, F, B=1):
+    from paper_2607_14695_b200.expert import ActionExpert, random_weights_device
+    w = synth.CONFIGS["cfg2"].with_(B=B, L=4, T=T, D=D, S=400, S_max=400)
+    cache = U.rb.Cache(w.L, w.B, w.Hq, w.Hkv, w.d, w.S_max, w.N, w.T, w.dtype, device=U.DEV)
+    U.rb.reflex_cache_init_static(cache, list(range(B)), *[torch.randn((B, w.L, w.S, w.Hkv, w.d), device=U.DEV).to(torch.bfloat16) for _ in range(2)])
+    expert = ActionExpert(w, cache, random_weights_device(w, F, U.DEV), F, U.DEV)
+    a, cond = torch.zeros((B, T, w.A), device=U.DEV), torch.zeros((B, w.Cd), dtype=torch.bfloat16, device=U.DEV)
+    return _us(lambda: expert.step(a, cond, 0), 1)
+
+
+@pytest.mark.parametrize("small,large,most", [
+    ((53, 2048, 512), (52, 2048, 512), 1.08),        # Q/K/V and gate/up by tiles 1.17, chained 1.00
+    ((40, 2048, 1536), (40, 2048, 1528), 1.04),      # gate/up by tiles 1.08, chained 1.00
+    ((40, 256, 8192, 2), (50, 256, 4096, 2), 1.14),  # residual projections of 256 columns by tiles 1.21, chained 1.07
+])
+def test_expert_step_by_tiles_costs_no_more_than_chained(U, small, large, most):
+    """(rows, D, F, streams) on either side of a line of the dispatch. Bounds between what both sides of the line cost chained and by tiles."""
+    assert _step_us(U, *small) <= most * _step_us(U, *large)
