@@ -123,7 +123,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             }
         }
         *abort_flag = 1u;
-        atomicCAS(p.status, 0u, 0x80000000u | ((code + 112u) << 16) | (blockIdx.x & 0xFFFFu));
+        raise_status(p.status, kSiteAttnPair + code);
         return false;
     };
     auto wait = [&](int i, uint32_t parity, uint32_t code) -> bool { return mbar_try_wait(bar(i), parity) || wait_slow(i, parity, code); };

@@ -200,7 +200,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             }
         }
         *abort_flag = 1u;
-        atomicCAS(p.status, 0u, 0x80000000u | (code << 16) | (blockIdx.x & 0xFFFFu));
+        raise_status(p.status, kSiteAttnTc + code);
         return false;
     };
 

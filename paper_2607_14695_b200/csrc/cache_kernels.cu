@@ -224,7 +224,7 @@ cudaError_t launch_commit_static(StreamState *state, const StreamBatch &batch, i
 // Self-test of the bounded-wait convention every kernel of the library follows: one thread waits on an mbarrier that
 // nothing will ever complete, with a time limit, and on expiry records the wait site in the status word and returns.
 // Nothing here can hang: the limit is clamped by the launcher, and the loop leaves on its own.
-__global__ void wait_limit_probe_kernel(uint32_t *status, unsigned long long limit_ns, uint32_t code)
+__global__ void wait_limit_probe_kernel(uint32_t *status, unsigned long long limit_ns)
 {
     __shared__ __align__(8) unsigned long long probe_bar;
     using namespace ptx;
@@ -238,13 +238,13 @@ __global__ void wait_limit_probe_kernel(uint32_t *status, unsigned long long lim
             if (mbar_try_wait(bar, 0)) done = true;                                   // (never: nothing arrives)
             else if ((n & 63u) == 0u && globaltimer_ns() - t_start > limit_ns) break;
         }
-        if (!done) atomicCAS(status, 0u, 0x80000000u | (code << 16) | (blockIdx.x & 0xFFFFu));
+        if (!done) raise_status(status, kSiteProbe);
     }
 }
 
 cudaError_t launch_wait_limit_probe(uint32_t *status, unsigned long long limit_ns, cudaStream_t st)
 {
-    wait_limit_probe_kernel<<<1, 32, 0, st>>>(status, limit_ns, 127u);
+    wait_limit_probe_kernel<<<1, 32, 0, st>>>(status, limit_ns);
     count_launch();
     return cudaGetLastError();
 }

@@ -187,7 +187,7 @@ chain_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             }
         }
         *abort_flag = 1u;
-        if (p.status) atomicCAS(p.status, 0u, 0x80000000u | ((code + 80u) << 16) | (blockIdx.x & 0xFFFFu));
+        raise_status(p.status, kSiteChainGemm + code);
         return false;
     };
     auto wait = [&](int i, uint32_t parity, uint32_t code) -> bool { return mbar_try_wait(bar(i), parity) || wait_slow(i, parity, code); };

@@ -137,7 +137,7 @@ linear_half_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
             }
         }
         *abort_flag = 1u;
-        if (p.status) atomicCAS(p.status, 0u, 0x80000000u | ((code + 96u) << 16) | (blockIdx.x & 0xFFFFu));
+        raise_status(p.status, kSiteLinearHalf + code);
         return false;
     };
     auto wait = [&](int i, uint32_t parity, uint32_t code) -> bool { return mbar_try_wait(bar(i), parity) || wait_slow(i, parity, code); };

@@ -204,7 +204,7 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             }
         }
         *abort_flag = 1u;
-        if (p.status) atomicCAS(p.status, 0u, 0x80000000u | ((code + 80u) << 16) | (blockIdx.x & 0xFFFFu));
+        raise_status(p.status, kSiteLinear + code);
         return false;
     };
 

@@ -204,7 +204,7 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             }
         }
         *abort_flag = 1u;
-        if (p.status) atomicCAS(p.status, 0u, 0x80000000u | ((code + 96u) << 16) | (blockIdx.x & 0xFFFFu));
+        raise_status(p.status, kSiteQkv + code);
         return false;
     };
 
@@ -626,7 +626,7 @@ norm_linear_small_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
             }
         }
         *abort_flag = 1u;
-        if (p.status) atomicCAS(p.status, 0u, 0x80000000u | ((code + 112u) << 16) | (blockIdx.x & 0xFFFFu));
+        raise_status(p.status, kSiteFewRows + code);
         return false;
     };
 

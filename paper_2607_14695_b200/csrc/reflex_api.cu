@@ -227,6 +227,18 @@ int reflex_cache_slot_map(reflex_cache_t *c, int b, int32_t *slot_of_age)
     return REFLEX_OK;
 }
 
+static const char *wait_site_kernel(uint32_t site)
+{
+    static const struct { uint32_t end; const char *name; } kKernels[] = {
+        {kSiteAttnTc2, "attn_tc_kernel"}, {kSiteGate, "attn_tc2_kernel"}, {kSiteProbe, "gate_tc_kernel"}, {kSiteQkv, "wait_limit_probe_kernel"},
+        {kSiteFewRows, "norm_qkv_tc_kernel"}, {kSiteLinear, "norm_linear_small_kernel"}, {kSiteTileGemm, "linear_res_tc_kernel"},
+        {kSiteChainGemm, "tile_gemm_kernel"}, {kSiteChainAttn, "chain_gemm_kernel"}, {kSiteLinearHalf, "chain_attn_kernel"},
+        {kSiteAttnPair, "linear_half_kernel"}, {kSiteEnd, "attn_pair_kernel"}};
+    for (const auto &k : kKernels)
+        if (site < k.end) return k.name;
+    return "unknown";
+}
+
 int reflex_cache_check_status(reflex_cache_t *c, void *stream)
 {
     if (!c) return fail(REFLEX_ERR_INVALID_ARG, "cache is NULL");
@@ -236,8 +248,8 @@ int reflex_cache_check_status(reflex_cache_t *c, void *stream)
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "status read-back");
     if (word != 0u)
-        return fail(REFLEX_ERR_TIMEOUT, "a device-side wait ran out (status 0x%08x: wait site %u, block %u); results of that launch are invalid",
-                    word, (word >> 16) & 0x7FFFu, word & 0xFFFFu);
+        return fail(REFLEX_ERR_TIMEOUT, "a device-side wait ran out (status 0x%08x: wait site %u, %s, block %u); results of that launch are invalid",
+                    word, (word >> 16) & 0x7FFFu, wait_site_kernel((word >> 16) & 0x7FFFu), word & 0xFFFFu);
     return REFLEX_OK;
 }
 

@@ -33,6 +33,17 @@ struct WorkspaceLayout {
     size_t bytes;
 };
 
+// Wait sites of the status word: a kernel's own numbers (from 1) behind a base of its own, so that a report names the kernel (wait_site_kernel)
+enum WaitSites : uint32_t {
+    kSiteAttnTc = 0, kSiteAttnTc2 = 32, kSiteGate = 64, kSiteProbe = 127, kSiteQkv = 128, kSiteFewRows = 144, kSiteLinear = 160, kSiteTileGemm = 176,
+    kSiteChainGemm = 192, kSiteChainAttn = 208, kSiteLinearHalf = 224, kSiteAttnPair = 240, kSiteEnd = 256
+};
+// The first wait that runs out leaves its site and block (a NULL status: nobody to tell)
+__device__ __forceinline__ void raise_status(uint32_t *status, uint32_t site)
+{
+    if (status) atomicCAS(status, 0u, 0x80000000u | site << 16 | (blockIdx.x & 0xFFFFu));
+}
+
 constexpr int kMaxSplits = 32;
 constexpr int kStreamsPerLaunch = 64;  // stream ids / lengths passed by value per launch
 

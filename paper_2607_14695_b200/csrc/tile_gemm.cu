@@ -148,7 +148,7 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
             }
         }
         *abort_flag = 1u;
-        if (p.status) atomicCAS(p.status, 0u, 0x80000000u | ((code + 48u) << 16) | (blockIdx.x & 0xFFFFu));
+        raise_status(p.status, kSiteTileGemm + code);
         return false;
     };
 

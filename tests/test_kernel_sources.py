@@ -73,3 +73,19 @@ def test_a_tile_of_a_failed_wait_is_written_as_nan(kernel):
     _, _, body = kernel
     assert "0x7fc00000" in body
     assert not re.search(r"if \([^()]*\bok && (?:m0|dst)|if \(!ok \|\| f >=", body)
+
+
+def test_a_reported_wait_names_its_kernel():
+    """The status word holds a number for every wait: kernels count theirs from bases of their own, far enough apart."""
+    header = open(os.path.join(CSRC, "reflex_internal.cuh")).read()
+    sites = {n: int(v) for n, v in re.findall(r"(kSite\w+) = (\d+)", header)}
+    used = {}
+    for name, _, body in KERNELS:
+        assert "atomicCAS(p.status" not in body and "atomicCAS(status" not in body, name
+        for base in set(re.findall(r"raise_status\([\w.]+, (kSite\w+)", body)):
+            last = max([int(c) for c in re.findall(r"\bwait(?:_slow|_cl)?\([^;]*?, (\d+)u?\)", body)] + [int(c) for c in re.findall(base + r" \+ (\d+)u", body)] + [0])
+            used[base] = (name, last)
+    assert len(used) == len({n for n, _ in used.values()}) == 12, used       # one base a kernel, no two kernels on one
+    bases = sorted(sites[b] for b in used) + [sites["kSiteEnd"]]
+    for base, (name, last) in used.items():
+        assert sites[base] + last < min(b for b in bases if b > sites[base]), name
