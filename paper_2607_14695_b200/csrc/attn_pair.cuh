@@ -123,7 +123,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             }
         }
         *abort_flag = 1u;
-        raise_status(p.status, kSiteAttnPair + code);
+        atomicCAS(p.status, 0u, status_word(kSiteAttnPair + code));
         return false;
     };
     auto wait = [&](int i, uint32_t parity, uint32_t code) -> bool { return mbar_try_wait(bar(i), parity) || wait_slow(i, parity, code); };

@@ -200,7 +200,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             }
         }
         *abort_flag = 1u;
-        raise_status(p.status, kSiteAttnTc + code);
+        atomicCAS(p.status, 0u, status_word(kSiteAttnTc + code));
         return false;
     };
 

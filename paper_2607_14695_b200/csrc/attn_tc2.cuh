@@ -136,7 +136,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if ((base - raw_addr) + L::NEED > L::TOTAL) {
         // the dynamic shared-memory window starts too far from a 1024-byte boundary to hold the tiles: same for every
         // CTA of the launch, so all of them leave here, before any barrier, cluster or TMEM state exists
-        if (threadIdx.x == 0) raise_status(p.status, kSiteAttnTc2 + 31u);
+        if (threadIdx.x == 0) atomicCAS(p.status, 0u, status_word(kSiteAttnTc2 + 31u));
         return;
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -223,7 +223,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             }
         }
         *abort_flag = 1u;
-        raise_status(p.status, kSiteAttnTc2 + code);
+        atomicCAS(p.status, 0u, status_word(kSiteAttnTc2 + code));
         return false;
     };
 
@@ -801,7 +801,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 }
             }
             *abort_flag = 1u;
-            raise_status(p.status, kSiteAttnTc2 + code);
+            atomicCAS(p.status, 0u, status_word(kSiteAttnTc2 + code));
             return false;
         };
         const int uu = u_start / ns, pair = uu % n_pairs, kvh = (uu / n_pairs) % p.Hkv, b = uu / (n_pairs * p.Hkv);

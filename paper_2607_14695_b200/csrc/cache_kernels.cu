@@ -238,7 +238,7 @@ __global__ void wait_limit_probe_kernel(uint32_t *status, unsigned long long lim
             if (mbar_try_wait(bar, 0)) done = true;                                   // (never: nothing arrives)
             else if ((n & 63u) == 0u && globaltimer_ns() - t_start > limit_ns) break;
         }
-        if (!done) raise_status(status, kSiteProbe);
+        if (!done) atomicCAS(status, 0u, status_word(kSiteProbe));
     }
 }
 

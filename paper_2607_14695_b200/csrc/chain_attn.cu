@@ -196,7 +196,7 @@ chain_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             }
         }
         *abort_flag = 1u;
-        raise_status(p.status, kSiteChainAttn + code);
+        if (p.status) atomicCAS(p.status, 0u, status_word(kSiteChainAttn + code));
         return false;
     };
     auto wait = [&](int i, uint32_t code) -> bool { return mbar_try_wait(bar(i), 0) || wait_slow(i, code); };

@@ -187,7 +187,7 @@ chain_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             }
         }
         *abort_flag = 1u;
-        raise_status(p.status, kSiteChainGemm + code);
+        if (p.status) atomicCAS(p.status, 0u, status_word(kSiteChainGemm + code));
         return false;
     };
     auto wait = [&](int i, uint32_t parity, uint32_t code) -> bool { return mbar_try_wait(bar(i), parity) || wait_slow(i, parity, code); };

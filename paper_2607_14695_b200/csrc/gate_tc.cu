@@ -106,7 +106,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
             if (mbar_try_wait(bar, parity)) return true;
             if ((n & 255u) == 0u && globaltimer_ns() - t_start > kGtWaitNs) break;
         }
-        raise_status(status, kSiteGate + code);
+        if (status) atomicCAS(status, 0u, status_word(kSiteGate + code));
         return false;
     };
     auto load_vectors = [&](int g) {   // the (up to) 32 vectors of group g, one or two bf16 arrays (the warp is converged)

@@ -137,7 +137,7 @@ linear_half_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
             }
         }
         *abort_flag = 1u;
-        raise_status(p.status, kSiteLinearHalf + code);
+        if (p.status) atomicCAS(p.status, 0u, status_word(kSiteLinearHalf + code));
         return false;
     };
     auto wait = [&](int i, uint32_t parity, uint32_t code) -> bool { return mbar_try_wait(bar(i), parity) || wait_slow(i, parity, code); };

@@ -204,7 +204,7 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             }
         }
         *abort_flag = 1u;
-        raise_status(p.status, kSiteLinear + code);
+        if (p.status) atomicCAS(p.status, 0u, status_word(kSiteLinear + code));
         return false;
     };
 

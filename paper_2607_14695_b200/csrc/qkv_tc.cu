@@ -204,7 +204,7 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             }
         }
         *abort_flag = 1u;
-        raise_status(p.status, kSiteQkv + code);
+        if (p.status) atomicCAS(p.status, 0u, status_word(kSiteQkv + code));
         return false;
     };
 
@@ -626,7 +626,7 @@ norm_linear_small_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
             }
         }
         *abort_flag = 1u;
-        raise_status(p.status, kSiteFewRows + code);
+        if (p.status) atomicCAS(p.status, 0u, status_word(kSiteFewRows + code));
         return false;
     };
 

@@ -38,11 +38,8 @@ enum WaitSites : uint32_t {
     kSiteAttnTc = 0, kSiteAttnTc2 = 32, kSiteGate = 64, kSiteProbe = 127, kSiteQkv = 128, kSiteFewRows = 144, kSiteLinear = 160, kSiteTileGemm = 176,
     kSiteChainGemm = 192, kSiteChainAttn = 208, kSiteLinearHalf = 224, kSiteAttnPair = 240, kSiteEnd = 256
 };
-// The first wait that runs out leaves its site and block (a NULL status: nobody to tell)
-__device__ __forceinline__ void raise_status(uint32_t *status, uint32_t site)
-{
-    if (status) atomicCAS(status, 0u, 0x80000000u | site << 16 | (blockIdx.x & 0xFFFFu));
-}
+// (what the first wait that runs out leaves in the status word)
+__device__ __forceinline__ uint32_t status_word(uint32_t site) { return 0x80000000u | (site << 16) | (blockIdx.x & 0xFFFFu); }
 
 constexpr int kMaxSplits = 32;
 constexpr int kStreamsPerLaunch = 64;  // stream ids / lengths passed by value per launch

@@ -148,7 +148,7 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
             }
         }
         *abort_flag = 1u;
-        raise_status(p.status, kSiteTileGemm + code);
+        if (p.status) atomicCAS(p.status, 0u, status_word(kSiteTileGemm + code));
         return false;
     };
 

@@ -81,8 +81,8 @@ def test_a_reported_wait_names_its_kernel():
     sites = {n: int(v) for n, v in re.findall(r"(kSite\w+) = (\d+)", header)}
     used = {}
     for name, _, body in KERNELS:
-        assert "atomicCAS(p.status" not in body and "atomicCAS(status" not in body, name
-        for base in set(re.findall(r"raise_status\([\w.]+, (kSite\w+)", body)):
+        assert len(re.findall(r"atomicCAS\((?:p\.)?status,", body)) == len(re.findall(r"atomicCAS\((?:p\.)?status, 0u, status_word\(kSite", body)), name
+        for base in set(re.findall(r"status_word\((kSite\w+)", body)):
             last = max([int(c) for c in re.findall(r"\bwait(?:_slow|_cl)?\([^;]*?, (\d+)u?\)", body)] + [int(c) for c in re.findall(base + r" \+ (\d+)u", body)] + [0])
             used[base] = (name, last)
     assert len(used) == len({n for n, _ in used.values()}) == 12, used       # one base a kernel, no two kernels on one
