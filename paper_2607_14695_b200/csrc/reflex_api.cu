@@ -626,7 +626,8 @@ static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float 
     float *ss[2] = {e.row_sums, e.row_sums + (size_t)M * ((D + 31) / 32)};
     auto gate = [&](int i) { return (const float *)e.gates + (size_t)i * B * D; };
     // what a later kernel of the step reads is asked into the L2 one or two kernels ahead, so that the 34 MB of a layer come from
-    // memory while the chain is busy with latencies (the tile kernels are not, and take no part)
+    // memory while the chain is busy with latencies. The tile kernels and the attention in units of 128 or 256 rows are not, and take no part: steps of
+    // 1 x 57 to 64 and 2 x 29 to 32 tokens, whose attention went from clusters of eight to units of 128 rows, are 6 % faster without its part.
     auto range = [](ChainPrefetch &pf, int i, const void *base, size_t first, size_t n) {
         pf.ptr[i] = (const char *)base + first * 2; pf.bytes[i] = n * 2 & ~(size_t)15;
     };
@@ -650,23 +651,23 @@ static int expert_step_chained(reflex_cache_t *c, const reflex_expert &e, float 
         ChainProj qkv = p;
         qkv.mode = CG_QKV; qkv.x = (const bf *)e.y; qkv.W = (const bf *)e.Wqkv; qkv.w_rows = L * (nq + 2 * nk); qkv.w_row0 = l * (nq + 2 * nk);
         qkv.K = D; qkv.N = nq + 2 * nk; qkv.ss_in = ss[0]; qkv.slots_in = slots; qkv.q = (bf *)e.q; qkv.k = (bf *)e.k; qkv.v = (bf *)e.v; qkv.nq = nq; qkv.nk = nk;
-        if (!tiled) range(qkv.pf, 0, e.Wo, (size_t)l * D * nq, (size_t)D * nq);
+        if (!form.qkv) range(qkv.pf, 0, e.Wo, (size_t)l * D * nq, (size_t)D * nq);
         err = proj(qkv);
         if (err != cudaSuccess) return cuda_fail(err, "expert q/k/v projection launch");
-        ChainPrefetch apf = {};
+        ChainPrefetch apf = {};       // (for chain_attn_kernel)
         range(apf, 0, e.Wgu, (size_t)l * 2 * e.F * D, (size_t)2 * e.F * D);
         const int rc = attention(c, l, e.q, e.k, e.v, e.o, T, 0.f, 0, true, &apf, stream);
         if (rc != REFLEX_OK) return rc;
         ChainProj o = p;
         o.mode = CG_RES; o.x = (const bf *)e.o; o.W = (const bf *)e.Wo; o.w_rows = L * D; o.w_row0 = l * D; o.K = nq; o.N = D; o.res = (const bf *)e.h;
         o.h = (bf *)e.h; o.xg = (bf *)e.y; o.gate = gate(2 * l + 1); o.ss_out = ss[1];
-        if (!tiled) range(o.pf, 0, e.Wd, (size_t)l * D * e.F, (size_t)D * e.F);
+        if (!form.res) range(o.pf, 0, e.Wd, (size_t)l * D * e.F, (size_t)D * e.F);
         err = proj(o);
         if (err != cudaSuccess) return cuda_fail(err, "expert output projection launch");
         ChainProj gu = p;
         gu.mode = CG_SWIGLU; gu.x = (const bf *)e.y; gu.W = (const bf *)e.Wgu; gu.w_rows = L * 2 * e.F; gu.w_row0 = l * 2 * e.F; gu.K = D; gu.N = e.F;
         gu.h = (bf *)e.m; gu.ss_in = ss[1]; gu.slots_in = slots_of(nq);
-        if (!tiled && l + 1 < L) {
+        if (!form.gu && l + 1 < L) {
             range(gu.pf, 0, c->k_slab, (size_t)(l + 1) * kv_layer, kv_layer);
             range(gu.pf, 1, c->v_slab, (size_t)(l + 1) * kv_layer, kv_layer);
             range(gu.pf, 2, e.Wqkv, (size_t)(l + 1) * (nq + 2 * nk) * D, (size_t)(nq + 2 * nk) * D);
