@@ -48,8 +48,8 @@ template <int HD> struct ApSmem {
 // EARLY: inside an expert step, the first cached tiles are asked for ahead of the wait.
 // DUAL: even and odd tiles have an accumulator each, with a reference maximum and a sum of its own. The key that sets a reference has weight 1, which
 // bf16 holds exactly, and twice as many references are twice as many such keys: 898 keys in four slices 2.24e-3 -> 2.13e-3 from 64 bits, what the eight
-// slices of chain_attn_kernel give. Split launches take it, they stand where finer slices stood; it costs them 0.3 to 0.5 us. Unsplit ones
-// are as far from 64 bits as units of 256 rows, 2.32e-3 (2.29e-3 with DUAL, for 1 us).
+// slices of chain_attn_kernel give. Split launches take it, they stand where finer slices stood, and unsplit ones where units of 256 rows would be cut
+// into slices; it costs a launch 0.1 to 0.5 us.
 template <int HD, bool EARLY, bool DUAL>
 __global__ void __launch_bounds__(kApThreads, 1)      // clusters of 2 CTAs, or of 2 * nsplit (cluster_merge)
 attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,

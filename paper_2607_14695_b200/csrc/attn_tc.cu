@@ -889,17 +889,18 @@ static double tc2_us(const AttnParams &p, int nsplit, int sm_count)
 static double pair_us(const AttnParams &p, int units, int tiles, int ns, bool merged)
 {
     const double fixed = p.d == 256 ? 1.0 : 0.83, per = (p.d == 256 ? 1.0 : 0.915) * ((tiles + ns - 1) / ns);
-    if (ns == 1) return 4.5 * fixed + 1.04 * per + 0.022 * units;
+    if (ns == 1) return 4.6 * fixed + 1.04 * per + 0.022 * units;
     if (merged) return ns == 2 ? 6.4 * fixed + 1.0 * per + 0.04 * units : 6.2 * fixed + 1.01 * per + 0.112 * units;
-    const double kilorows = 1e-3 * p.B * p.T * p.Hq * ns * p.d / 256.0;          // (the merge launch hides some)
-    return 7.75 * fixed + 1.03 * per + 0.028 * units * ns + 0.25 * std::max(0.0, kilorows - 4.4);
+    // the merge launch: many rows, or many slices of few rows, outlast what the attention's last CTAs hide of it
+    const double kilorows = 1e-3 * p.B * p.T * p.Hq * p.d / 256.0;
+    return 7.75 * fixed + 1.03 * per + 0.028 * units * ns + 1.6 * std::max(0.0, kilorows - 2.3) + 0.25 * std::max(0.0, kilorows * ns - 4.4) + 0.08 * std::max(0, ns - 12);
 }
 
-// References per row of a launch in ns slices: two accumulators in a slice of two tiles or more, one accumulator in all without a split.
+// References per row of a launch in ns slices with two accumulators each
 static int pair_references(int tiles, int ns)
 {
     const int per = (tiles + ns - 1) / ns, full = tiles / per;
-    return ns == 1 ? 1 : full * std::min(2, per) + std::min(2, tiles - full * per);
+    return full * std::min(2, per) + std::min(2, tiles - full * per);
 }
 
 // Key slices of the 128-row units where those are the faster two-CTA form; 0: units of 256 rows, in the tc2_slices that tc2_choose_splits picked. One wave is
@@ -922,10 +923,11 @@ int pair_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count, 
     for (const int ns : kSlices) {
         if (ns > tiles || units * ns > clusters) break;
         // The key that sets a reference has weight 1, which bf16 holds exactly, and units of 256 rows have one reference per slice: fewer of them are
-        // farther from 64 bits (10 streams of 33 tokens, 4 heads of 128, 552 keys: 2.30e-3 with one, 2.14e-3 with five).
+        // farther from 64 bits (10 streams of 33 tokens, 4 heads of 128, 552 keys: 2.30e-3 with one, 2.14e-3 with five). So does one slice here take its
+        // second accumulator (0.1 to 0.25 us) where those would be cut.
         if (pair_references(tiles, ns) < tc2_slices) continue;
         for (int m = ns == 2 || ns == 4 ? 1 : 0; m >= 0; --m) {
-            // (clusters of eight with a margin: the last ones find room late, 16.7 us with 16 of them against 9.6 with 12)
+            // (the device holds 33 clusters of four and 15 of eight at once; one more waits for a whole cluster to end: 15.1 -> 26.5 us, 11.2 -> 20.7)
             const int active = m ? tc2_active_clusters(p.d, 2 * ns) : 0;
             if (m && units > (ns == 4 ? active - active / 6 : active)) continue;
             if (!m && ns > 1 && per_split_bytes * ns > (double)partial_bytes) continue;
@@ -938,7 +940,7 @@ int pair_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count, 
     return best;
 }
 
-cudaError_t launch_attention_pair(const AttnParams &p, uint32_t *status, int nsplit, bool merged, cudaStream_t st)
+cudaError_t launch_attention_pair(const AttnParams &p, uint32_t *status, int nsplit, bool merged, bool dual, cudaStream_t st)
 {
     const int G = p.Hq / p.Hkv, rows_slab = p.L * p.B * (p.ring_off + p.N), tt = kApRows / G;
     CUtensorMap m[6];
@@ -953,8 +955,8 @@ cudaError_t launch_attention_pair(const AttnParams &p, uint32_t *status, int nsp
     tp.nsplit = nsplit; tp.tile_tokens = tt; tp.live_rows = kApRows; tp.n_qtiles = ((p.T + tt - 1) / tt + 1) / 2; tp.cluster_merge = merged && nsplit > 1 ? 1 : 0;
     const int units = pair_units(p);
     cudaError_t e;
-    if (p.d == 256) e = (nsplit == 1 ? (p.early ? launch_pair_t<256, true, false> : launch_pair_t<256, false, false>) : (p.early ? launch_pair_t<256, true, true> : launch_pair_t<256, false, true>))(m, tp, units, st);
-    else if (p.d == 128) e = (nsplit == 1 ? (p.early ? launch_pair_t<128, true, false> : launch_pair_t<128, false, false>) : (p.early ? launch_pair_t<128, true, true> : launch_pair_t<128, false, true>))(m, tp, units, st);
+    if (p.d == 256) e = (!dual ? (p.early ? launch_pair_t<256, true, false> : launch_pair_t<256, false, false>) : (p.early ? launch_pair_t<256, true, true> : launch_pair_t<256, false, true>))(m, tp, units, st);
+    else if (p.d == 128) e = (!dual ? (p.early ? launch_pair_t<128, true, false> : launch_pair_t<128, false, false>) : (p.early ? launch_pair_t<128, true, true> : launch_pair_t<128, false, true>))(m, tp, units, st);
     else return cudaErrorInvalidValue;
     if (e != cudaSuccess || nsplit == 1 || tp.cluster_merge) return e;
     return launch_attention_merge(p, st);

@@ -528,7 +528,7 @@ static int attention(reflex_cache_t *c, int layer, const void *q, const void *k_
         bool merged = false;
         p.nsplit = choose ? pair_choose_splits(p, c->lay.partial_bytes, c->sm_count, split2, merged) : 0;
         if (p.nsplit > 0) {
-            e = launch_attention_pair(p, status, p.nsplit, merged, (cudaStream_t)stream);
+            e = launch_attention_pair(p, status, p.nsplit, merged, p.nsplit > 1 || split2 > 1, (cudaStream_t)stream);
         } else {
             const bool two = choose || c->attn_impl == REFLEX_ATTN_TC2;
             p.nsplit = two ? split2 : tc_choose_splits(p, c->lay.partial_bytes, c->sm_count);

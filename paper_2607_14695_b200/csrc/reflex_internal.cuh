@@ -127,9 +127,10 @@ int tc_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count);
 bool tc2_supported(const AttnParams &p);
 int tc2_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count);
 cudaError_t launch_attention_tc(const AttnParams &p, uint32_t *status, bool two_cta, int sm_count, cudaStream_t st);
-// units of 128 rows (attn_pair.cuh): key slices where they are the faster form than tc2_slices of units of 256, 0 otherwise; merged: inside clusters
+// units of 128 rows (attn_pair.cuh): key slices where they are the faster form than tc2_slices of units of 256, 0 otherwise; merged: inside clusters;
+// dual: two accumulators
 int pair_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count, int tc2_slices, bool &merged);
-cudaError_t launch_attention_pair(const AttnParams &p, uint32_t *status, int nsplit, bool merged, cudaStream_t st);
+cudaError_t launch_attention_pair(const AttnParams &p, uint32_t *status, int nsplit, bool merged, bool dual, cudaStream_t st);
 // a few streams (chain_attn.cu): key slices merged inside clusters of eight. early: the caller vouches that the cached regions are not
 // written by work that may still be running
 bool chain_attn_supported(const AttnParams &p, bool early, int sm_count);
