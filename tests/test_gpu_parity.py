@@ -537,6 +537,33 @@ def test_wide_logits_exercise_the_lazy_rescale(U, impl):
         tw.attention(0, 2, dyn_mask=1, q_scale=q_scale, rel_clause=True, what=f"wide logits x{q_scale} causal {impl}")
 
 
+UNITS_OF_128 = [
+    # B, Hq, Hkv, d, S, N, T, launches: units of 128 rows in every form, three key tiles or more for an accumulator, last units with few rows
+    (16, 8, 1, 256, 816, 32, 50, 1), (6, 16, 4, 128, 300, 48, 37, 1),          # one slice, one accumulator
+    (9, 8, 1, 256, 1093, 32, 50, 1),                                           # one slice, two accumulators
+    (8, 8, 1, 256, 816, 32, 50, 1), (7, 8, 4, 128, 681, 115, 43, 1),           # two slices merged in a cluster
+    (3, 8, 1, 256, 2000, 32, 50, 1), (2, 16, 1, 128, 1823, 39, 41, 1),         # four slices merged in a cluster
+    (1, 8, 1, 256, 4160, 256, 50, 2), (1, 2, 1, 128, 1823, 39, 41, 2),         # slices that leave partials, and the launch that merges them
+]
+
+
+@pytest.mark.parametrize("case", UNITS_OF_128, ids=["B%d_h%dkv%d_d%d_S%d_N%d_T%d" % c[:7] for c in UNITS_OF_128])
+def test_wide_logits_in_units_of_128_rows(U, case):
+    """As above for the library's choice: row maxima that keep growing rescale O in tensor memory while the next Q K^T is in flight, each
+    accumulator behind its own P V; both masks, prefixes of different lengths, ring partly filled and wrapped."""
+    B, Hq, Hkv, d, S, N, T, launches = case
+    w = synth.Workload("wide128", 33, synth.DTYPE_BF16, B=B, L=1, Hq=Hq, Hkv=Hkv, d=d, S=S, S_max=S, N=N, T=T, D=64, Cd=8, Hd=8, A=4, K=2)
+    tw = U.Twin(w, head0=[(5 * b + 3) % N for b in range(B)], poison=True)
+    tw.init_static(list(range(B)), [S - (b * 131) % S for b in range(B)])
+    for i in range(3):
+        tw.append([b for b in range(B) if not (b % 4 == 2 and i >= 1)], N // 2, i)
+    for q_scale in (6.0, 20.0):
+        for mask in (0, 1):
+            before = U.rb.reflex_kernel_launch_count()
+            tw.attention(0, 1 + mask, dyn_mask=mask, q_scale=q_scale, rel_clause=True, streams=sorted({0, min(2, B - 1), B - 1}), what=f"units of 128, x{q_scale} mask {mask}")
+            assert U.rb.reflex_kernel_launch_count() - before == launches
+
+
 def test_two_cta_kernel_many_units_head_dim_128(U):
     """More work units than SM pairs at head_dim 128 (four K and four V stages), two KV heads, several key tiles per unit:
     the persistent loop crosses unit boundaries with every stage and buffer rotation."""
@@ -1218,7 +1245,7 @@ def _with_guards(model):
     return tails
 
 
-def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None, cache_layers=None, weights=lambda dW: dW):
+def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None, cache_layers=None, weights=lambda dW: dW, impl=None):
     from oracle import expert_oracle as eo
     from paper_2607_14695_b200 import expert as ex
     rb = U.rb
@@ -1226,6 +1253,8 @@ def _expert_case(U, w, F, tol_v, what, streams=None, S_list=None, cache_layers=N
     tw.init_static(list(range(w.B)), S_list or [w.S] * w.B)
     for i in range(3):
         tw.append(list(range(w.B)), 2, i)
+    if impl is not None:
+        rb.reflex_cache_set_attention_impl(tw.g, impl)
     W = ex.expert_weights(w, F, std_scale=0.5)
     dW = {n: U.to_dev(v, w.dtype) for n, v in W.items()}
     model = ex.ActionExpert(w, tw.g, weights(dW), F, device=U.DEV)
@@ -1401,7 +1430,7 @@ def test_expert_step_of_fewer_layers_than_the_cache(U, B):
 
 
 A_FEW_STREAMS = [
-    # B, T, Hq, Hkv, S_max, prefix lengths, N: edges of the attention in units of 128 rows whose key slices merge in clusters (three to eight streams)
+    # B, T, Hq, Hkv, S_max, prefix lengths, N: edges of the attention of three to eight streams, units of 128 rows in one slice or in slices merged in clusters
     (4, 50, 8, 1, 816, [816, 700, 0, 113], 32), (8, 64, 8, 1, 896, [896] * 8, 64), (6, 60, 4, 2, 300, [300, 1, 2, 7, 8, 299], 5),
     (5, 33, 16, 1, 64, [64] * 5, 4),
 ]
@@ -1427,6 +1456,28 @@ def test_expert_step_bf16_cached_keys_ahead_of_the_wait(U, case):
     B, T, Hq, Hkv, d, S_max, S_list, N = case
     w = synth.CONFIGS["cfg2"].with_(B=B, L=2, T=T, Hq=Hq, Hkv=Hkv, d=d, D=512, S=S_max, S_max=S_max, N=N)
     _expert_case(U, w, 512, 2e-2, "expert bf16, cached keys ahead", streams=[0, 1, 4, B - 1], S_list=S_list)
+
+
+@pytest.mark.parametrize("case", KEYS_AHEAD, ids=["B%d_T%d_h%dkv%d_d%d_S%d" % c[:6] for c in KEYS_AHEAD])
+def test_expert_step_bf16_cached_keys_ahead_of_the_wait_in_units_of_256_rows(U, case):
+    """The same steps through units of 256 rows, which the library takes only where units of 128 do not fit the SM pairs at once."""
+    B, T, Hq, Hkv, d, S_max, S_list, N = case
+    w = synth.CONFIGS["cfg2"].with_(B=B, L=2, T=T, Hq=Hq, Hkv=Hkv, d=d, D=512, S=S_max, S_max=S_max, N=N)
+    _expert_case(U, w, 512, 2e-2, "expert bf16, cached keys ahead, units of 256", streams=[0, 1, 4, B - 1], S_list=S_list, impl=U.rb.ATTN_TC2)
+
+
+MANY_UNITS_AHEAD = [
+    # B, T, Hq, Hkv, d, S_max, N: more units of 128 rows than SM pairs, with the prefixes above
+    (40, 33, 8, 1, 256, 300, 64), (42, 20, 8, 2, 128, 260, 20),
+]
+
+
+@pytest.mark.parametrize("case", MANY_UNITS_AHEAD, ids=["B%d_T%d_h%dkv%d_d%d_S%d" % c[:6] for c in MANY_UNITS_AHEAD])
+def test_expert_step_bf16_cached_keys_ahead_of_the_wait_in_many_units(U, case):
+    B, T, Hq, Hkv, d, S_max, N = case
+    S_list = [[S_max, 0, 1, 63, 64, 65, 127, 128, 129, S_max - 1, 191, 192, 193][b % 13] for b in range(B)]
+    w = synth.CONFIGS["cfg2"].with_(B=B, L=2, T=T, Hq=Hq, Hkv=Hkv, d=d, D=512, S=S_max, S_max=S_max, N=N)
+    _expert_case(U, w, 512, 2e-2, "expert bf16, cached keys ahead, many units", streams=[0, 1, 4, 8, 12, B - 1], S_list=S_list)
 
 
 def test_expert_step_bf16_batched(U):
