@@ -64,17 +64,6 @@ struct LhParams {
     uint32_t *status;
 };
 
-__device__ __forceinline__ void lh_tma2_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t leader_bar, int c0, int c1)
-{
-    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 ::"r"(dst), "l"(map), "r"(leader_bar), "r"(c0), "r"(c1)
-                 : "memory");
-}
-__device__ __forceinline__ void lh_tma_store_2d(const CUtensorMap *map, uint32_t src, int c0, int c1)
-{
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");
-}
-
 template <int BN>
 __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kLhThreads, 1)
 linear_half_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_res,
@@ -118,7 +107,7 @@ linear_half_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
     auto load_w = [&](int s, int ks) {
         // both CTAs' loads complete on the leader's barrier
         if (rank == 0) mbar_expect_tx(bar(S::C_FULL + s), 2 * (S::A_STAGE + S::B_STAGE));
-        lh_tma2_load_2d(base + S::OFF_B + s * S::B_STAGE, &tm_w, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * 64, n0 + (int)rank * (BN / 2));
+        tma2_load_2d(base + S::OFF_B + s * S::B_STAGE, &tm_w, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * 64, n0 + (int)rank * (BN / 2));
     };
     // inside an expert step the weights of the first steps are asked for ahead of the wait for the preceding kernel
     const int head = p.early_w ? min(steps, NST) : 0;
@@ -152,7 +141,7 @@ linear_half_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
                 if (ks >= NST) ok = wait(S::C_EMPTY + s, ph, 1);
                 if (!ok) break;
                 if (ks >= head) load_w(s, ks);
-                lh_tma2_load_2d(base + S::OFF_A + s * S::A_STAGE, &tm_a, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * 64, m0);
+                tma2_load_2d(base + S::OFF_A + s * S::A_STAGE, &tm_a, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * 64, m0);
                 if (++s == NST) { s = 0; ph ^= 1u; }
             }
             if (p.has_res) {
@@ -263,8 +252,8 @@ linear_half_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
 #pragma unroll
                     for (int c = 0; c < BN / 64; ++c) {
                         if (n0 + c * 64 < p.N) {
-                            lh_tma_store_2d(&tm_out, base + S::OFF_RES + c * S::CHUNK, n0 + c * 64, mo);
-                            if (p.gate) lh_tma_store_2d(&tm_xg, base + S::OFF_XG + c * S::CHUNK, n0 + c * 64, mo);
+                            tma_store_2d(&tm_out, base + S::OFF_RES + c * S::CHUNK, n0 + c * 64, mo);
+                            if (p.gate) tma_store_2d(&tm_xg, base + S::OFF_XG + c * S::CHUNK, n0 + c * 64, mo);
                         }
                     }
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");

@@ -75,12 +75,6 @@ __device__ unsigned long long g_lin_trace[512 * 8];
 #define LIN_TRACE(ev) do { } while (0)
 #endif
 
-__device__ __forceinline__ void lin_tma2_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t leader_bar, int c0, int c1)
-{
-    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 ::"r"(dst), "l"(map), "r"(leader_bar), "r"(c0), "r"(c1)
-                 : "memory");
-}
 __device__ __forceinline__ float lin_sum2(uint64_t v) { float a, b; unpack_f32x2(v, a, b); return a + b; }
 
 // The gates of the streams under a CTA's 128 rows, columns [n0, n0 + W), on their way to shared memory: the first ones in registers before
@@ -126,10 +120,6 @@ __device__ __forceinline__ void lin_gated_piece(const uint64_t (&v)[4], const fl
         o[k] = *reinterpret_cast<uint32_t *>(&x);
     }
     *reinterpret_cast<uint4 *>(dst) = make_uint4(o[0], o[1], o[2], o[3]);
-}
-__device__ __forceinline__ void lin_tma_store_2d(const CUtensorMap *map, uint32_t src, int c0, int c1)
-{
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");
 }
 
 // KS = 2 (128-column tiles only): the cluster holds the two pairs that share an output tile, each taking half of the contraction;
@@ -182,7 +172,7 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     auto load_w = [&](int s, int ks) {
         // both CTAs' loads complete on the leader's barrier: the issuing thread there waits for all four at once
         if (rank == 0) mbar_expect_tx(bar(S::C_FULL + s), 2 * (S::A_STAGE + S::B_STAGE));
-        lin_tma2_load_2d(base + S::OFF_B + s * S::B_STAGE, &tm_w, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * kLinBK, n0 + (int)rank * (BN / 2));
+        tma2_load_2d(base + S::OFF_B + s * S::B_STAGE, &tm_w, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * kLinBK, n0 + (int)rank * (BN / 2));
     };
     // inside an expert step (early_w) the weights of the first steps are asked for before the wait for the preceding kernel
     const int head = p.early_w ? (nk_steps < NST ? nk_steps : NST) : 0;
@@ -222,7 +212,7 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
                 if (ks >= NST) ok = wait(S::C_EMPTY + s, ph, 1);
                 if (!ok) break;
                 if (ks >= head) load_w(s, ks);
-                lin_tma2_load_2d(base + S::OFF_A + s * S::A_STAGE, &tm_a, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * kLinBK, m0);
+                tma2_load_2d(base + S::OFF_A + s * S::A_STAGE, &tm_a, bar(S::C_FULL + s) & kPeerBitMask, (k_first + ks) * kLinBK, m0);
                 if (++s == NST) { s = 0; ph ^= 1u; }
             }
             if (ok) {
@@ -358,8 +348,8 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             fence_proxy_async_smem();
             asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
             if (quarter == 0 && lane == 0 && m0 < p.M && n0 + ch * 64 < p.N) {
-                lin_tma_store_2d(&tm_out, base + S::OFF_RES + ch * S::CHUNK, n0 + ch * 64, m0);
-                if (p.gate) lin_tma_store_2d(&tm_xg, base + S::OFF_A + ch * S::CHUNK, n0 + ch * 64, m0);
+                tma_store_2d(&tm_out, base + S::OFF_RES + ch * S::CHUNK, n0 + ch * 64, m0);
+                if (p.gate) tma_store_2d(&tm_xg, base + S::OFF_A + ch * S::CHUNK, n0 + ch * 64, m0);
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
         }
@@ -439,8 +429,8 @@ linear_res_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             asm volatile("bar.sync 1, 256;" ::: "memory");     // the chunk's 256 threads
             if (warp == 2 && lane == 0) {
                 if (m0 < p.M && n0 + kq * 64 < p.N) {
-                    lin_tma_store_2d(&tm_out, base + S::OFF_RES + kq * S::CHUNK, n0 + kq * 64, m0);
-                    if (p.gate) lin_tma_store_2d(&tm_xg, base + S::OFF_B, n0 + kq * 64, m0);
+                    tma_store_2d(&tm_out, base + S::OFF_RES + kq * S::CHUNK, n0 + kq * 64, m0);
+                    if (p.gate) tma_store_2d(&tm_xg, base + S::OFF_B, n0 + kq * 64, m0);
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
                 asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");

@@ -86,18 +86,6 @@ __device__ long long g_qk_trace[3 * 32 * 8];
 #define QK_TRACE(role, step, ev) do { } while (0)
 #endif
 
-__device__ __forceinline__ void qk_tma_store_2d(const CUtensorMap *map, uint32_t src, int c0, int c1)
-{
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");
-}
-
-__device__ __forceinline__ void tma2_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t leader_bar, int c0, int c1)
-{
-    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 ::"r"(dst), "l"(map), "r"(leader_bar), "r"(c0), "r"(c1)
-                 : "memory");
-}
-
 // n4 groups of four gates to shared memory by 256 threads, four loads of a thread in flight (one by one, each was a round trip to the L2 in
 // front of the next: 0.3 to 0.6 us of a Q/K/V or gate/up projection).
 __device__ __forceinline__ void qk_copy_gates(float4 *dst, const float4 *src, int n4, int t)
@@ -419,10 +407,10 @@ norm_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                         const int n = n0 + j * kQkBN + ch * 64;     // first output column of the chunk (chunks never straddle Q, K and V:
                                                                     // the launcher takes this path only when their widths are multiples of 64)
                         const uint32_t src = base + stage_off + ch * (128 * 128);
-                        if (swiglu) { if (n < p.swiglu_F) qk_tma_store_2d(&tm_q, src, n, m0); }
-                        else if (n < p.nq) qk_tma_store_2d(&tm_q, src, n, m0);
-                        else if (n < p.nq + p.nk) qk_tma_store_2d(&tm_k, src, n - p.nq, m0);
-                        else if (n < n_out) qk_tma_store_2d(&tm_v, src, n - p.nq - p.nk, m0);
+                        if (swiglu) { if (n < p.swiglu_F) tma_store_2d(&tm_q, src, n, m0); }
+                        else if (n < p.nq) tma_store_2d(&tm_q, src, n, m0);
+                        else if (n < p.nq + p.nk) tma_store_2d(&tm_k, src, n - p.nq, m0);
+                        else if (n < n_out) tma_store_2d(&tm_v, src, n - p.nq - p.nk, m0);
                         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
                 }

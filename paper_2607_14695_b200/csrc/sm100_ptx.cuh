@@ -108,6 +108,11 @@ __device__ __forceinline__ float silu_mul(float g, float u)
     asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * g));
     return fmaf(t, 0.5f * g, 0.5f * g) * u;
 }
+// TMA tiled store; the issuing thread commits the group
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t src, int c0, int c1)
+{
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");
+}
 // L2 prefetch of one box of a tiled tensor map (no shared-memory destination, no completion barrier)
 __device__ __forceinline__ void tma_prefetch_2d_elect(const CUtensorMap *map, int c0, int c1)
 {
@@ -388,6 +393,12 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
     return ok != 0;
 }
 // TMA loads whose completion is signalled on the pair leader's mbarrier (no multicast)
+__device__ __forceinline__ void tma2_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t leader_bar, int c0, int c1)
+{
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+                 ::"r"(dst), "l"(map), "r"(leader_bar), "r"(c0), "r"(c1)
+                 : "memory");
+}
 __device__ __forceinline__ void tma2_load_3d(uint32_t dst, const CUtensorMap *map, uint32_t leader_bar, int c0, int c1, int c2)
 {
     asm volatile("cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"

@@ -58,17 +58,6 @@ struct TgParams {
     uint32_t *status;
 };
 
-__device__ __forceinline__ void tg_tma2_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t leader_bar, int c0, int c1)
-{
-    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 ::"r"(dst), "l"(map), "r"(leader_bar), "r"(c0), "r"(c1)
-                 : "memory");
-}
-__device__ __forceinline__ void tg_tma_store_2d(const CUtensorMap *map, uint32_t src, int c0, int c1)
-{
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");
-}
-
 // BM = 128 or 64 rows per CTA. An accumulator of 2 x 64 rows fills all lanes of either CTA: lanes 0-63 hold its 64 rows for the first half of
 // the accumulator's columns, lanes 64-127 for the second, so its CTAs each bring gate and up rows of their own half of the output columns.
 template <bool SWIGLU, int BN, int BM>
@@ -123,12 +112,12 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
         if constexpr (SWIGLU && BM == 64) {
 #pragma unroll
             for (int up = 0; up < 2; ++up)
-                tg_tma2_load_2d(base + S::OFF_B + s * S::B_STAGE + up * (S::B_STAGE / 2), &tm_w, bar(S::T_FULL + s) & kPeerBitMask, ks * kTgBK,
+                tma2_load_2d(base + S::OFF_B + s * S::B_STAGE + up * (S::B_STAGE / 2), &tm_w, bar(S::T_FULL + s) & kPeerBitMask, ks * kTgBK,
                                 p.w_row0 + up * p.F + n0 + (int)rank * (BN / 4));
             return;
         }
         const int row = SWIGLU ? p.w_row0 + (int)rank * p.F + n0 : p.w_row0 + n0 + (int)rank * (BN / 2);
-        tg_tma2_load_2d(base + S::OFF_B + s * S::B_STAGE, &tm_w, bar(S::T_FULL + s) & kPeerBitMask, ks * kTgBK, row);
+        tma2_load_2d(base + S::OFF_B + s * S::B_STAGE, &tm_w, bar(S::T_FULL + s) & kPeerBitMask, ks * kTgBK, row);
     };
     // the weights of the first steps are asked for before the wait for the preceding kernel: nothing in a step writes weights
     const int head = my_tiles > 0 ? (nk_steps < NST ? nk_steps : NST) : 0;
@@ -165,7 +154,7 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
                     if (it > 0 || ks >= NST) ok = wait(S::T_EMPTY + s, ph, 1);
                     if (!ok) break;
                     if (!first) load_w(s, ks, n0);
-                    tg_tma2_load_2d(base + S::OFF_A + s * S::A_STAGE, &tm_x, bar(S::T_FULL + s) & kPeerBitMask, ks * kTgBK, m0);
+                    tma2_load_2d(base + S::OFF_A + s * S::A_STAGE, &tm_x, bar(S::T_FULL + s) & kPeerBitMask, ks * kTgBK, m0);
                     if (++s == NST) { s = 0; ph ^= 1u; }
                 }
             }
@@ -270,11 +259,11 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
                 const int n = n0 + ch * 64;
                 if (m0 < p.M) {
                     if constexpr (SWIGLU) {
-                        if (n < p.F) tg_tma_store_2d(&tm_q, base + stage_off, n, m0);
+                        if (n < p.F) tma_store_2d(&tm_q, base + stage_off, n, m0);
                     } else {              // (the widths are multiples of 64: a chunk lies in one tensor)
-                        if (n < p.nq) tg_tma_store_2d(&tm_q, base + stage_off, n, m0);
-                        else if (n < p.nq + p.nk) tg_tma_store_2d(&tm_k, base + stage_off, n - p.nq, m0);
-                        else if (n < p.nq + 2 * p.nk) tg_tma_store_2d(&tm_v, base + stage_off, n - p.nq - p.nk, m0);
+                        if (n < p.nq) tma_store_2d(&tm_q, base + stage_off, n, m0);
+                        else if (n < p.nq + p.nk) tma_store_2d(&tm_k, base + stage_off, n - p.nq, m0);
+                        else if (n < p.nq + 2 * p.nk) tma_store_2d(&tm_v, base + stage_off, n - p.nq - p.nk, m0);
                     }
                 }
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -361,11 +350,11 @@ tile_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
                     const int n = n0 + ch * 64;
                     if (m0 < p.M) {
                         if constexpr (SWIGLU) {
-                            if (n < p.F) tg_tma_store_2d(&tm_q, base + stage_off, n, m0);
+                            if (n < p.F) tma_store_2d(&tm_q, base + stage_off, n, m0);
                         } else {              // (the widths are multiples of 64: a chunk lies in one tensor)
-                            if (n < p.nq) tg_tma_store_2d(&tm_q, base + stage_off, n, m0);
-                            else if (n < p.nq + p.nk) tg_tma_store_2d(&tm_k, base + stage_off, n - p.nq, m0);
-                            else if (n < p.nq + 2 * p.nk) tg_tma_store_2d(&tm_v, base + stage_off, n - p.nq - p.nk, m0);
+                            if (n < p.nq) tma_store_2d(&tm_q, base + stage_off, n, m0);
+                            else if (n < p.nq + p.nk) tma_store_2d(&tm_k, base + stage_off, n - p.nq, m0);
+                            else if (n < p.nq + 2 * p.nk) tma_store_2d(&tm_v, base + stage_off, n - p.nq - p.nk, m0);
                         }
                     }
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
