@@ -262,7 +262,8 @@ int reflex_adarmsnorm_swiglu(reflex_cache_t *cache, const void *x, const float *
  *   out      device [M][N] dtype (written); may be the same buffer as res (in-place update of the residual stream),
  *            must not overlap a
  *   impl     0: tensor cores when dtype is bf16 (256 x 256 output tiles per pair of SMs; 256 x 128 where those would leave
- *               most pairs idle, a contraction of 2048 or more then split over two pairs of a cluster while they fit;
+ *               most pairs idle, a contraction of 2048 or more then split over two pairs of a cluster while they fit; tiles of
+ *               128 rows, the contraction in two halves, where M > 64 and K >= 2048 leave at most 32 of them;
  *               a kernel with the weights as the stationary operand when K % 64 == 0 and M <= 128, or M <= 256 in groups
  *               of 64 rows for K >= 2048),
  *               else the plain kernel; 1: the plain kernel (fp32 FMAs, K <= 12288); 2: like 0 but always the 256-row tiles

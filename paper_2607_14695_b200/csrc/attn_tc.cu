@@ -905,7 +905,7 @@ static int pair_references(int tiles, int ns)
 
 // Key slices of the 128-row units where those are the faster two-CTA form; 0: units of 256 rows, in the tc2_slices that tc2_choose_splits picked. One wave is
 // all they may be. Over the 191 shapes above that no cluster of eight takes, the choice is within 0.3 % (geometric mean; at most 8.5 %) of the fastest of all
-// forms and slices, units of 256 rows alone 21.7 %. One call against those, us: 898 keys x 50 tokens, 2 streams 12.6 -> 9.1 (four slices), 4 streams
+// forms and slices, units of 256 rows alone 21.7 %. One call against those, us: 898 keys x 50 tokens, 3 streams 12.8 -> 9.5 (four slices), 4 streams
 // 13.7 -> 10.9 (two), 8 streams 14.3 -> 11.8 (two), 16 streams 15.7 -> 13.7 (one); 24 streams x 33 tokens 17.6 -> 14.6; heads of 128, 2 KV heads, 14 tokens x 341
 // keys 8.9 -> 7.1 (four); one stream x 2082 keys 13.5 -> 11.2; 16 tokens x 13,632 keys 18.9 -> 14.9 (32). 12 streams x 4466 keys stay with
 // units of 256 rows in three slices.

@@ -6,7 +6,8 @@
 // each; a cluster is the two pairs that share a tile's contraction. 64-column tiles while those still are at most 32 clusters (up to 256
 // rows of 1024 columns), 128-column tiles above.
 // Measured against the tiles of 256 rows, contraction split the same way (graph replay, in place, 1024 columns): 264 rows x 2048 7.9 -> 6.2 us, x 4096
-// 11.2 -> 9.3; 429 rows 7.9 -> 6.5 and 11.3 -> 9.8; 512 rows 7.9 -> 6.5 and 11.4 -> 9.9.
+// 11.2 -> 9.3; 429 rows 7.9 -> 6.5 and 11.3 -> 9.8; 512 rows 7.9 -> 6.5 and 11.4 -> 9.9. Narrow outputs of more rows in as many tiles are served alike: 4000
+// rows x 4096 -> 64 columns 10.8 -> 8.9, 2000 x 4096 -> 256 11.0 -> 9.2; of 45 shapes of 512 to 4000 rows x 2048 to 12288 -> 32 to 1024 none is slower.
 //
 // An accumulator of 128 rows over a pair fills all lanes of either CTA: lanes 0-63 hold its 64 rows for the first half of the columns, lanes
 // 64-127 for the second. The halves of the contraction meet by rows: either CTA of the two with equal rank finishes 32 of their 64 rows, the
