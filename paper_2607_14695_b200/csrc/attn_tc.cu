@@ -836,6 +836,7 @@ static bool tc2_cluster_merge_ok(const AttnParams &p, int nsplit, int sm_count)
     return (p.d / nsplit / kTc2Parts) % 16 == 0 && p.d / nsplit / kTc2Parts >= 16;   // a thread reduces whole 16-column pieces
 }
 
+// (The picks also say how exact a call has to be, pair_choose_splits. Where units of 128 rows compete they are priced by tc2_us, which was fitted to them.)
 int tc2_choose_splits(const AttnParams &p, size_t partial_bytes, int sm_count)
 {
     const int G = p.Hq / p.Hkv;
